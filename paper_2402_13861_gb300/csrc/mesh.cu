@@ -2,6 +2,7 @@
 // float32 point evaluation of the MLP, and the library's own marching-cubes case table.
 #include "internal.cuh"
 #include "linearise.cuh"
+#include "sgemm.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -161,8 +162,6 @@ isx_status mc_upload_table(int device) {
 // ---- float32 MLP evaluation at points -----------------------------------------------------------
 namespace {
 
-constexpr int kEvalPts = 32;
-
 // Points come either as xyz triples or as lattice ids of the (R+1)^3 grid (coordinates
 // -1 + 2 i / R, computed directly).
 __device__ __forceinline__ void point_xyz(const float* xyz, const uint32_t* ids, int R, int64_t i, float p[3]) {
@@ -193,57 +192,113 @@ struct MlpView {
   float bout;
 };
 
-__global__ void __launch_bounds__(256) k_eval_fp32(MlpView m, const float* xyz, const uint32_t* ids, int R,
-                                                   int64_t n, float* out) {
-  extern __shared__ float sm[];
-  const int w = m.w;
-  float* A = sm;                       // [kEvalPts][w]
-  float* B = sm + kEvalPts * w;        // [kEvalPts][w]
-  __shared__ float pts[kEvalPts][3];
-  int64_t p0 = (int64_t)blockIdx.x * kEvalPts;
-  if (threadIdx.x < kEvalPts) {
-    int64_t i = p0 + threadIdx.x;
-    float p[3] = {0.f, 0.f, 0.f};
-    if (i < n) point_xyz(xyz, ids, R, i, p);
-    pts[threadIdx.x][0] = p[0];
-    pts[threadIdx.x][1] = p[1];
-    pts[threadIdx.x][2] = p[2];
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < kEvalPts * w; idx += blockDim.x) {
-    int p = idx / w, nn = idx % w;
-    float z = fmaf(m.W0[3 * nn + 2], pts[p][2], fmaf(m.W0[3 * nn + 1], pts[p][1], fmaf(m.W0[3 * nn], pts[p][0], m.b0[nn])));
-    A[p * w + nn] = act_fwd(m.act, z);
-  }
-  __syncthreads();
-  for (int l = 1; l < m.n_layers - 1; ++l) {
-    const float* Wt = m.Wt[l];
-    const float* bb = m.b[l];
-    for (int nn = threadIdx.x; nn < w; nn += blockDim.x) {
-      float acc[kEvalPts];
-#pragma unroll
-      for (int p = 0; p < kEvalPts; ++p) acc[p] = bb[nn];
-      for (int k = 0; k < w; ++k) {
-        float wk = Wt[(size_t)k * w + nn];
-#pragma unroll
-        for (int p = 0; p < kEvalPts; ++p) acc[p] = fmaf(wk, A[p * w + k], acc[p]);
-      }
-#pragma unroll
-      for (int p = 0; p < kEvalPts; ++p) B[p * w + nn] = act_fwd(m.act, acc[p]);
+// One CTA runs the whole network for its P points: the activations stay in shared memory, [neuron][point],
+// and every hidden layer is one sgemm tile (sgemm.cuh) written back in place, so global memory holds only
+// the points, the values and the weights (L2).  Every value is the same chain of multiply-adds whatever
+// the launch shape.  Bound by FP32 FMA issue and the shared-memory return bandwidth (an 8 x 8 tile reads 16
+// values per 64 multiply-adds): 3 -> 512 x 8 -> 1 at 300007 points 24 ms = 46 TFLOP/s (125 ms = 8.8 TFLOP/s
+// for the earlier kernel, one neuron of 32 points per thread), 3 -> 256 x 5 -> 1 at 2^20 points 10.9 ms
+// (29.7 ms), 3 -> 64 x 2 -> 1 at 2^22 1.0 ms (3.3 ms); fma.rn.f32x2 from registers alone runs at 66-73 TFLOP/s.
+template <int TN>
+__global__ void __launch_bounds__(256) k_eval_fp32(MlpView m, sgemm::Shape sh, const float* xyz, const uint32_t* ids,
+                                                   int R, int64_t n, float* out) {
+  extern __shared__ __align__(16) float sm[];
+  const int w = m.w, P = sh.P, KB = sh.KB, spl = w / KB;
+  float* A = sm;                                  // [w][P]
+  sgemm::Stream ws{sm + (size_t)w * P, w, KB, 0, (m.n_layers - 2) * spl};
+  auto stage_src = [&](int s) { return m.Wt[min(1 + s / spl, m.n_layers - 2)] + (size_t)(s % spl) * KB * w; };
+  for (int s = 0; s < sgemm::kStages - 1; ++s) ws.load(stage_src(s));
+  const int t = threadIdx.x, T = blockDim.x;
+  const int64_t p0 = (int64_t)blockIdx.x * P;
+  for (int p = t % P, g = t / P, gs = max(1, T / P); g < gs && p < P; p += T) {
+    float pt[3] = {0.f, 0.f, 0.f};
+    if (p0 + p < n) point_xyz(xyz, ids, R, p0 + p, pt);
+    for (int nn = g; nn < w; nn += gs) {
+      float z = fmaf(m.W0[3 * nn + 2], pt[2], fmaf(m.W0[3 * nn + 1], pt[1], fmaf(m.W0[3 * nn], pt[0], m.b0[nn])));
+      A[nn * P + p] = act_fwd(m.act, z);
     }
-    __syncthreads();
-    float* t = A; A = B; B = t;
   }
-  // output layer: one warp per point
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int p = warp; p < kEvalPts; p += blockDim.x >> 5) {
-    float s = 0.0f;
-    for (int k = lane; k < w; k += 32) s = fmaf(m.wout[k], A[p * w + k], s);
+  const int PG = P / sgemm::kTM, pg = t % PG, ng = t / PG;
+  const bool own = ng < w / TN;
+  int s = 0;
+  for (int l = 1; l < m.n_layers - 1; ++l) {
+    sgemm::Tile<TN> tile;
+    if (own)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    int64_t i = p0 + p;
-    if (lane == 0 && i < n) out[i] = s + m.bout;
+      for (int c = 0; c < TN / 2; ++c) {
+        const int nn = sgemm::Tile<TN>::neuron(c, ng, w);
+        const uint64_t bb = sgemm::pack2(m.b[l][nn], m.b[l][nn + 1]);
+#pragma unroll
+        for (int i = 0; i < sgemm::kTM; ++i) tile.acc[i][c] = bb;
+      }
+    for (int kb = 0; kb < spl; ++kb, ++s) {
+      sgemm::cp_wait<sgemm::kStages - 2>();
+      __syncthreads();                            // stage s has landed, stage s - 1 is free, A is written
+      ws.load(stage_src(s + sgemm::kStages - 1));
+      if (own) tile.stage(A + (size_t)kb * KB * P, ws.Ws + (size_t)(s % sgemm::kStages) * KB * w, P, w, KB, pg, ng);
+    }
+    __syncthreads();                              // every thread is done reading A
+    if (own) {
+#pragma unroll
+      for (int c = 0; c < TN / 2; ++c) {
+        const int nn = sgemm::Tile<TN>::neuron(c, ng, w);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float u[4], v[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 z = sgemm::unpack2(tile.acc[4 * h + i][c]);
+            u[i] = act_fwd(m.act, z.x);
+            v[i] = act_fwd(m.act, z.y);
+          }
+          float* d = A + (size_t)nn * P + h * (P >> 1) + 4 * pg;
+          *reinterpret_cast<float4*>(d) = make_float4(u[0], u[1], u[2], u[3]);
+          *reinterpret_cast<float4*>(d + P) = make_float4(v[0], v[1], v[2], v[3]);
+        }
+      }
+    }
   }
+  __syncthreads();
+  // output layer, one thread per point: 32 partial sums over the neurons k = l, l + 32, ..., then their
+  // pairwise tree (the order of a 32-lane butterfly)
+  for (int p = t; p < P && p0 + p < n; p += T) {
+    float q[32];
+#pragma unroll
+    for (int l = 0; l < 32; ++l) q[l] = 0.0f;
+    for (int k0 = 0; k0 < w; k0 += 32)
+#pragma unroll
+      for (int l = 0; l < 32; ++l)
+        if (k0 + l < w) q[l] = fmaf(m.wout[k0 + l], A[(size_t)(k0 + l) * P + p], q[l]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int l = 0; l < 16; ++l)
+        if (l < o) q[l] += q[l + o];
+    out[p0 + p] = q[0] + m.bout;
+  }
+}
+
+// Launch shape of k_eval_fp32 for n points and width w; the results do not depend on it.
+//  - Enough points for 8192 activations per SM: 8 neurons per thread, P up to 16384 / w points (256
+//    threads, 64 KB of activations, two CTAs per SM).  P is halved while that shortens the longest SM's
+//    queue: its CTAs' points plus a fixed part (fill, barriers, tail, worth about 40 points) per pair
+//    of CTAs.  At w = 512, n = 3000 P = 32 takes 439 us against 530-615 us for P = 16; a CTA of 16
+//    neurons per thread (a 128-thread CTA) is 2 % slower at 3 x 10^5 points.
+//  - Fewer: 4 neurons per thread and long stages, for the shortest chain through the layers: at
+//    w = 512, n = 500, 270 us against 300-440 us for the 8-neuron tiles.
+sgemm::Shape eval_shape(int64_t n, int w, int sms) {
+  if (n * w < (int64_t)sms * 8192) return {4, std::max(8, 4096 / w / 8 * 8), w % 32 == 0 ? 32 : 16};
+  int best = 8;
+  int64_t best_cost = -1;
+  for (int P = std::max(8, 16384 / w / 8 * 8); P >= 8; P = P / 2 / 8 * 8) {
+    const int64_t nb = (n + P - 1) / P;
+    const int64_t cost = (nb + sms - 1) / sms * P + (nb + 2 * sms - 1) / (2 * sms) * 40;
+    if (best_cost < 0 || cost < best_cost) {
+      best = P;
+      best_cost = cost;
+    }
+  }
+  return {8, best, w > 256 ? 8 : 16};
 }
 
 }  // namespace
@@ -263,16 +318,17 @@ isx_status eval_points_fp32(isx_inr inr, const float* xyz, const uint32_t* latti
   }
   m.wout = inr->W[inr->n_layers - 1];
   m.bout = inr->hb[inr->n_layers - 1][0];
-  size_t smem = 2ull * kEvalPts * inr->w * sizeof(float);
-  static bool attr_set[64] = {};
-  if (smem > 48 * 1024 && inr->device < 64 && !attr_set[inr->device]) {
-    ISX_CUDA(cudaFuncSetAttribute(k_eval_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr_set[inr->device] = true;
-  }
-  int64_t nb = (n + kEvalPts - 1) / kEvalPts;
+  int sms = 148;
+  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
+  const sgemm::Shape sh = eval_shape(n, inr->w, sms);
+  const size_t smem = sh.smem(inr->w);
+  const int threads = (sh.threads(inr->w) + 31) / 32 * 32;
+  const int64_t nb = (n + sh.P - 1) / sh.P;
   {
     prof::Scope _ps(K_EVAL_FP32, st, 2.0 * n * (4.0 * inr->w + (inr->n_layers - 2.0) * inr->w * inr->w), 8.0 * n);
-    k_eval_fp32<<<(unsigned)nb, 256, smem, st>>>(m, xyz, lattice_ids, R, n, out);
+    const auto kernel = sh.tn == 8 ? k_eval_fp32<8> : k_eval_fp32<4>;
+    ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    kernel<<<(unsigned)nb, threads, smem, st>>>(m, sh, xyz, lattice_ids, R, n, out);
   }
   ISX_LAUNCH_CHECK("k_eval_fp32");
   return ISX_OK;

@@ -1,15 +1,20 @@
 // Float32 bound path: affine / probabilistic-affine forms propagated layer by layer through a ReLU
 // MLP (Sec. III-B and IV-C), one kernel per step, cells processed in chunks.
 //
-// Per cell the form of the pre-activation z_j of hidden layer j is a centre c (w floats) and a
-// coefficient matrix X with S_j = 3 + w (j - 1) rows (one per noise symbol) and w columns, stored
-// row-major [cell][row][w] in float32:
+// Per cell the form of the pre-activation z_j of hidden layer j is a centre c (w floats) and the rows X of
+// its noise symbols in float32, the cells' rows one after another (offsets from a scan of the per-cell
+// counts):
 //   z_1:  c = W_0 x_c + b_0, X = diag(h) W_0^T                      (input box, Eq. 3 / Eq. 8)
 //   ReLU: alpha, beta, gamma per neuron from (c, r) or (mu, sigma)  (Eq. 4 / Eq. 9, Table VII)
 //   L_j:  c' = W_j (alpha c + beta) + b_j,
-//         X' = [X diag(alpha) W_j^T ; diag(gamma) W_j^T]           (Eq. 3 / Eq. 8)
+//         X' = [X diag(alpha) W_j^T ; gamma_n W_j[:, n] for every n with gamma_n != 0]   (Eq. 3 / Eq. 8)
 //   out:  y_i = X diag(alpha) w_out (+ gamma_m w_out,m for the last ReLU's symbols),
 //         r = sum |y_i| (Eq. 2) or sigma^2 = sum y_i^2 (Eq. 7), RA-UA: sigma^2 / 3 (Sec. IV-A).
+// A symbol whose coefficient gamma_n is exactly 0 has an all-zero row in every later layer and is never
+// created.  Bound by the FP32 FMA rate of the row GEMM: 20003 random cells of levels 5-9 of the fitted
+// 3 -> 256 x 5 -> 1 network take 15.6 ms (43 TFLOP/s in the GEMM), where carrying all 1027 rows of every
+// cell took 142.6 ms; with every symbol alive (ELU, 3 -> 128 x 4 -> 1, 5003 boxes) 2.2 ms against 4.0 ms.
+// A cell's result depends neither on the chunking nor on the launch shapes.
 //
 // Rounding-error inflation (SOUND, inflate != 0).  The library carries, per neuron, a slack
 // delta >= |true z - carried form| and widens the ReLU interval by it; the linearisation error,
@@ -22,6 +27,8 @@
 #include <string>
 #include "linearise.cuh"
 #include "cell_box.cuh"
+#include "rows.cuh"
+#include "sgemm.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -35,48 +42,71 @@ constexpr float kInvSqrt3 = 0.57735026918962576f;
 
 __host__ __device__ __forceinline__ float gamma_k(int k) { return (k * kU) / (1.0f - k * kU); }
 
-// z_1 = W_0 x + b_0 over the box: centre, 3 coefficient rows, per-neuron reduction, slack.
-__global__ void k_input_layer(CellSource src, int64_t first, int nc, const float* __restrict__ W0,
-                              const float* __restrict__ b0, int w, int mode, int inflate, float* C,
-                              float* X, int S, float* RAD, float* DELTA) {
-  int cell = blockIdx.x;
-  if (cell >= nc) return;
-  float xc[3], h[3];
-  cell_box(src, first + cell, inflate, xc, h);
-  if (mode == ISX_BOUND_CLT)
-    for (int d = 0; d < 3; ++d) h[d] *= kInvSqrt3;   // uniform on [-h, h] has std h / sqrt 3
-  float* Xc = X + (size_t)cell * S * w;
-  for (int n = threadIdx.x; n < w; n += blockDim.x) {
-    float w0 = W0[3 * n], w1 = W0[3 * n + 1], w2 = W0[3 * n + 2];
-    float c = fmaf(w2, xc[2], fmaf(w1, xc[1], fmaf(w0, xc[0], b0[n])));
-    float x0 = h[0] * w0, x1 = h[1] * w1, x2 = h[2] * w2;
-    Xc[n] = x0;
-    Xc[w + n] = x1;
-    Xc[2 * w + n] = x2;
-    float rad;
-    if (mode == ISX_BOUND_CLT) rad = sqrtf(x0 * x0 + x1 * x1 + x2 * x2);
-    else rad = fabsf(x0) + fabsf(x1) + fabsf(x2);
-    C[(size_t)cell * w + n] = c;
-    RAD[(size_t)cell * w + n] = rad;
-    if (inflate) {
-      float e = fabsf(w0 * xc[0]) + fabsf(w1 * xc[1]) + fabsf(w2 * xc[2]) + fabsf(b0[n]);
-      DELTA[(size_t)cell * w + n] = (5.0f * kU * e + 3.0f * kU * rad) * kSafe;
-    } else {
-      DELTA[(size_t)cell * w + n] = 0.0f;
-    }
-  }
+// Linearisation of activation j for one (cell, neuron): pre-activation centre c, radius / sigma rad, slack dl.
+__device__ __forceinline__ Lin linearise(int mode, int act, int inflate, float c, float rad, float dl) {
+  return mode == ISX_BOUND_CLT ? act_clt(act, c, rad) : relu_sound(c, rad, inflate ? dl : 0.0f, inflate != 0);
 }
 
-// Activation linearisation per (cell, neuron); updates the centre in place, writes alpha and gamma.
-__global__ void k_relu(int64_t total, int mode, int inflate, int act, float* C, const float* RAD,
-                       const float* DELTA, float* ALPHA, float* GAMMA) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  Lin r = (mode == ISX_BOUND_CLT) ? act_clt(act, C[i], RAD[i])
-                                  : relu_sound(C[i], RAD[i], inflate ? DELTA[i] : 0.0f, inflate != 0);
-  C[i] = r.center;
-  ALPHA[i] = r.alpha;
-  GAMMA[i] = r.gamma;
+// Threads per cell and cells per block of the per-(cell, neuron) kernels: blocks of up to 256 threads.
+struct CellBlock {
+  int tpc, cpb;
+  explicit CellBlock(int w) : tpc(std::min(w, 256)), cpb(std::max(1, 256 / std::min(w, 256))) {}
+  unsigned blocks(int nc) const { return (unsigned)((nc + cpb - 1) / cpb); }
+  unsigned threads() const { return (unsigned)(tpc * cpb); }
+};
+
+// z_1 = W_0 x + b_0 over the box and activation 1: the 3 input rows with their row -> cell map, the
+// post-activation centre, alpha, gamma (and, inflate, radius and slack), the cell's row counts (3 now,
+// 3 + #(gamma != 0) after the next layer) and the offset of its rows.
+__global__ void __launch_bounds__(256) k_input_layer(CellSource src, int64_t first, int nc, int tpc,
+                                                     const float* __restrict__ W0, const float* __restrict__ b0, int w,
+                                                     int mode, int act, int inflate, float* C, float* X, int* rowcell,
+                                                     float* RAD, float* ALPHA, float* GAMMA, int64_t* off, int* cnt,
+                                                     int* cnt_next) {
+  __shared__ int made[16];
+  const int sub = threadIdx.x / tpc, t = threadIdx.x - sub * tpc;
+  const int cell = blockIdx.x * (blockDim.x / tpc) + sub;
+  if (threadIdx.x < 16) made[threadIdx.x] = 0;
+  __syncthreads();
+  if (cell < nc) {
+    float xc[3], h[3];
+    cell_box(src, first + cell, inflate, xc, h);
+    if (mode == ISX_BOUND_CLT)
+      for (int d = 0; d < 3; ++d) h[d] *= kInvSqrt3;   // uniform on [-h, h] has std h / sqrt 3
+    float* Xc = X + (size_t)cell * 3 * w;
+    int m = 0;
+    for (int n = t; n < w; n += tpc) {
+      float w0 = W0[3 * n], w1 = W0[3 * n + 1], w2 = W0[3 * n + 2];
+      float c = fmaf(w2, xc[2], fmaf(w1, xc[1], fmaf(w0, xc[0], b0[n])));
+      float x0 = h[0] * w0, x1 = h[1] * w1, x2 = h[2] * w2;
+      Xc[n] = x0;
+      Xc[w + n] = x1;
+      Xc[2 * w + n] = x2;
+      float rad;
+      if (mode == ISX_BOUND_CLT) rad = sqrtf(x0 * x0 + x1 * x1 + x2 * x2);
+      else rad = fabsf(x0) + fabsf(x1) + fabsf(x2);
+      float dl = 0.0f;
+      if (inflate) {
+        float e = fabsf(w0 * xc[0]) + fabsf(w1 * xc[1]) + fabsf(w2 * xc[2]) + fabsf(b0[n]);
+        dl = (5.0f * kU * e + 3.0f * kU * rad) * kSafe;
+      }
+      const Lin L = linearise(mode, act, inflate, c, rad, dl);
+      const size_t i = (size_t)cell * w + n;
+      C[i] = L.center;
+      ALPHA[i] = L.alpha;
+      GAMMA[i] = L.gamma;
+      if (inflate) RAD[i] = rad;
+      m += L.gamma != 0.0f;
+    }
+    if (t < 3) rowcell[3 * cell + t] = cell;
+    if (m) atomicAdd(&made[sub], m);
+  }
+  __syncthreads();
+  if (cell < nc && t == 0) {
+    off[cell] = 3 * (int64_t)cell;
+    cnt[cell] = 3;
+    cnt_next[cell] = 3 + made[sub];
+  }
 }
 
 // Centre of the next layer, c' = W a + b, and (inflate) the slack of the next pre-activation:
@@ -111,183 +141,335 @@ __global__ void k_center_gemv(int nc, int win, int wout, const float* __restrict
   }
 }
 
-// X_out[r] = X_in[r] diag(alpha) W^T for the S_in carried rows: BM x BN output tiles, K step 16,
-// TM x TN outputs per thread.  Every output accumulates over K in the same order whatever the tile,
-// so all variants give bit-identical results and the autotuner may pick any of them.
-template <int BM, int BN, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm_fp32(const float* __restrict__ Xin,
-                                                                     float* __restrict__ Xout, int S_in, int S_out,
-                                                                     int w, const float* __restrict__ Wt,
-                                                                     const float* __restrict__ ALPHA) {
-  constexpr int T = (BM / TM) * (BN / TN), TX = BN / TN;
-  static_assert(TN % 4 == 0, "float4 stores");
-  __shared__ float As[16][BM + 4];
-  __shared__ float Bs[16][BN];
-  const int cell = blockIdx.z;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const float* A = Xin + (size_t)cell * S_in * w;
-  const float* al = ALPHA + (size_t)cell * w;
-  float* Y = Xout + (size_t)cell * S_out * w;
-  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
-  float acc[TM][TN] = {};
-  for (int k0 = 0; k0 < w; k0 += 16) {
-    for (int q = tid; q < BM * 4; q += T) {
-      const int row = q >> 2, kq = (q & 3) * 4;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (m0 + row < S_in) v = *reinterpret_cast<const float4*>(A + (size_t)(m0 + row) * w + k0 + kq);
-      As[kq + 0][row] = v.x; As[kq + 1][row] = v.y; As[kq + 2][row] = v.z; As[kq + 3][row] = v.w;
+// Y[row] = X[row] diag(alpha_cell) W^T for R rows of all cells (ROWS), or Y[row] = X[row] W^T + b (the
+// centres): persistent CTAs over tiles of P rows, the rows scaled while they are staged k-major in shared
+// memory (sgemm.cuh).  Every output is one multiply-add chain over k whatever the launch shape, so all
+// shapes give bit-identical results and the autotuner may pick any of them.  R comes from device memory
+// (d_R) where the host does not know it.
+struct GemmArgs {
+  const float* X;
+  float* Y;
+  const float* Wt;
+  const float* alpha;                  // ROWS: [cell][w]
+  const float* bias;                   // centres
+  const int* rowcell;                  // ROWS: cell of every row, first rows of the cells in X and in Y
+  const int64_t* off_in;
+  const int64_t* off_out;
+  const int64_t* d_R;                  // null: R
+  int64_t R;
+};
+template <int TN, bool ROWS>
+__global__ void __launch_bounds__(256, 2) k_gemm_fp32(GemmArgs g, sgemm::Shape sh, int w) {
+  extern __shared__ __align__(16) float sm[];
+  const int P = sh.P, KB = sh.KB, spl = w / KB;
+  float* A = sm;                                   // [w][P]
+  int64_t* dst = reinterpret_cast<int64_t*>(sm + (size_t)w * P + (size_t)sgemm::kStages * KB * w);   // [P] row in Y, -1: none
+  int* rcell = reinterpret_cast<int*>(dst + P);                                                       // [P] cell
+  const int64_t R = g.d_R ? *g.d_R : g.R;
+  const int64_t ntiles = (R + P - 1) / P;
+  if (blockIdx.x >= ntiles) return;
+  const int64_t mine = (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
+  sgemm::Stream ws{sm + (size_t)w * P, w, KB, mine * spl};
+  int sk = 0;                                      // K block of the stage to load next
+  auto load_next = [&] {
+    ws.load(g.Wt + (size_t)sk * KB * w);
+    sk = sk + 1 == spl ? 0 : sk + 1;
+  };
+  for (int s = 0; s < sgemm::kStages - 1; ++s) load_next();
+  const int t = threadIdx.x, T = blockDim.x;
+  const int PG = P / sgemm::kTM, pg = t % PG, ng = t / PG;
+  const bool own = ng < w / TN;
+  int slot = 0;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t r0 = tile * P;
+    for (int p = t; p < P; p += T) {
+      int c = 0;
+      int64_t d = -1;
+      if (r0 + p < R) {
+        c = ROWS ? g.rowcell[r0 + p] : 0;
+        d = ROWS ? g.off_out[c] + (r0 + p - g.off_in[c]) : r0 + p;
+      }
+      dst[p] = d;
+      rcell[p] = c;
     }
-    for (int q = tid; q < 4 * BN; q += T) {
-      const int kk = q / (BN / 4), nq = (q % (BN / 4)) * 4;
-      float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (n0 + nq < w) bv = *reinterpret_cast<const float4*>(Wt + (size_t)(k0 + kk) * w + n0 + nq);
-      const float sc = al[k0 + kk];
-      Bs[kk][nq + 0] = bv.x * sc; Bs[kk][nq + 1] = bv.y * sc; Bs[kk][nq + 2] = bv.z * sc; Bs[kk][nq + 3] = bv.w * sc;
-    }
+    // the next tile's rows are asked into L2 while this one is computed
+    const int64_t nt = tile + gridDim.x;
+    if (t == 0 && nt < ntiles)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(g.X + (size_t)nt * P * w),
+                   "r"((uint32_t)(min((int64_t)P, R - nt * P) * w * 4))
+                   : "memory");
     __syncthreads();
+    constexpr int NF = 4;                          // 16-byte loads of a thread in flight
+    const int nq = (w / 4) * P;
+    for (int q0 = t; q0 < nq; q0 += NF * T) {
+      float4 v[NF], al[NF];
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[TM], b[TN];
+      for (int i = 0; i < NF; ++i) {
+        const int q = q0 + i * T, p = q % P, k = 4 * (q / P);
+        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (q < nq && r0 + p < R) {
+          v[i] = *reinterpret_cast<const float4*>(g.X + (size_t)(r0 + p) * w + k);
+          if (ROWS) al[i] = *reinterpret_cast<const float4*>(g.alpha + (size_t)rcell[p] * w + k);
+        } else {
+          al[i] = v[i];
+        }
+      }
 #pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[kk][ty * TM + i];
-#pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx * TN + j];
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      for (int i = 0; i < NF; ++i) {
+        const int q = q0 + i * T, p = q % P, k = 4 * (q / P);
+        if (q >= nq) break;
+        if (ROWS) {
+          v[i].x *= al[i].x; v[i].y *= al[i].y; v[i].z *= al[i].z; v[i].w *= al[i].w;
+        }
+        float* d = A + (size_t)k * P + p;
+        d[0] = v[i].x; d[P] = v[i].y; d[2 * P] = v[i].z; d[3 * P] = v[i].w;
+      }
     }
-    __syncthreads();
-  }
+    sgemm::Tile<TN> acc;
+    if (own)
 #pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int r = m0 + ty * TM + i;
+      for (int c = 0; c < TN / 2; ++c) {
+        const int n = sgemm::Tile<TN>::neuron(c, ng, w);
+        const uint64_t z = ROWS ? 0ull : sgemm::pack2(g.bias[n], g.bias[n + 1]);
 #pragma unroll
-    for (int jc = 0; jc < TN; jc += 4) {
-      const int c = n0 + tx * TN + jc;
-      if (r < S_in && c < w)
-        *reinterpret_cast<float4*>(Y + (size_t)r * w + c) =
-            make_float4(acc[i][jc], acc[i][jc + 1], acc[i][jc + 2], acc[i][jc + 3]);
+        for (int i = 0; i < sgemm::kTM; ++i) acc.acc[i][c] = z;
+      }
+    for (int kb = 0; kb < spl; ++kb) {
+      sgemm::cp_wait<sgemm::kStages - 2>();
+      __syncthreads();                             // the stage has landed, the one before it is free, A is written
+      load_next();
+      if (own) acc.stage(A + (size_t)kb * KB * P, ws.Ws + (size_t)slot * KB * w, P, w, KB, pg, ng);
+      slot = slot == sgemm::kStages - 1 ? 0 : slot + 1;
     }
+    if (own)
+#pragma unroll
+      for (int i = 0; i < sgemm::kTM; ++i) {
+        const int64_t row = dst[sgemm::Tile<TN>::row(i, pg, P)];
+        if (row >= 0)
+#pragma unroll
+          for (int c = 0; c < TN / 2; c += 2) {
+            const float2 u = sgemm::unpack2(acc.acc[i][c]), v = sgemm::unpack2(acc.acc[i][c + 1]);
+            *reinterpret_cast<float4*>(g.Y + (size_t)row * w + sgemm::Tile<TN>::neuron(c, ng, w)) =
+                make_float4(u.x, u.y, v.x, v.y);
+          }
+      }
+    __syncthreads();                               // every thread is done with A and dst
   }
 }
 
-// Tile variants of the FP32 coefficient GEMM the autotuner chooses from.
+// Tile shapes of the float32 GEMM the autotuner chooses from: TN neurons per thread, about `elems`
+// staged row elements per CTA (P = elems / w rows) and up to `stage` weights per stage.
 struct GemmShape {
-  int bm, bn;
+  int tn, elems, stage;
   const char* name;
 };
-constexpr GemmShape kGemmShapes[] = {{64, 64, "64x64/4x4"}, {32, 64, "32x64/2x4"}, {16, 64, "16x64/1x4"},
-                                     {128, 64, "128x64/8x4"}, {64, 128, "64x128/4x8"}};
+constexpr GemmShape kGemmShapes[] = {{8, 16384, 4096, "8x8, 256 threads"}, {8, 8192, 2048, "8x8, 128 threads"},
+                                     {8, 4096, 2048, "8x8, 64 threads"}, {4, 8192, 4096, "8x4, 256 threads"},
+                                     {4, 4096, 4096, "8x4, 128 threads"}};
 constexpr int kGemmVariants = sizeof(kGemmShapes) / sizeof(kGemmShapes[0]);
 
-void launch_gemm(int v, int nc, int S, int S_out, int w, const float* Xa, float* Xb, const float* Wt,
-                 const float* AL, cudaStream_t st) {
-  const GemmShape g = kGemmShapes[v];
-  const dim3 grid((w + g.bn - 1) / g.bn, (S + g.bm - 1) / g.bm, nc);
-  switch (v) {
-    case 0: k_gemm_fp32<64, 64, 4, 4><<<grid, 256, 0, st>>>(Xa, Xb, S, S_out, w, Wt, AL); break;
-    case 1: k_gemm_fp32<32, 64, 2, 4><<<grid, 256, 0, st>>>(Xa, Xb, S, S_out, w, Wt, AL); break;
-    case 2: k_gemm_fp32<16, 64, 1, 4><<<grid, 256, 0, st>>>(Xa, Xb, S, S_out, w, Wt, AL); break;
-    case 3: k_gemm_fp32<128, 64, 8, 4><<<grid, 256, 0, st>>>(Xa, Xb, S, S_out, w, Wt, AL); break;
-    default: k_gemm_fp32<64, 128, 4, 8><<<grid, 256, 0, st>>>(Xa, Xb, S, S_out, w, Wt, AL); break;
-  }
+template <bool ROWS>
+isx_status launch_gemm(int v, const GemmArgs& g, int w, int sms, cudaStream_t st) {
+  const GemmShape& gs = kGemmShapes[v];
+  const int KB = 16 * w <= gs.stage ? 16 : (8 * w <= gs.stage ? 8 : 4);
+  const sgemm::Shape sh{gs.tn, std::max(8, gs.elems / w / 8 * 8), KB};
+  const size_t smem = sh.smem(w) + (size_t)sh.P * (sizeof(int64_t) + sizeof(int));
+  const int threads = (sh.threads(w) + 31) / 32 * 32;
+  const auto kernel = sh.tn == 8 ? k_gemm_fp32<8, ROWS> : k_gemm_fp32<4, ROWS>;
+  ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  int per_sm = 1;
+  ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
+  const int64_t ntiles = (g.R + sh.P - 1) / sh.P;  // d_R: g.R is an upper bound
+  kernel<<<(unsigned)std::min<int64_t>(ntiles, (int64_t)sms * std::max(1, per_sm)), threads, smem, st>>>(g, sh, w);
+  ISX_LAUNCH_CHECK("k_gemm_fp32");
+  return ISX_OK;
 }
 
-// Rows of the symbols created by the last ReLU: X_out[S_in + m][n] = gamma_m W[n][m].
-__global__ void k_fresh_rows(float* Xout, int S_in, int S_out, int w, const float* __restrict__ Wt,
-                             const float* __restrict__ GAMMA) {
-  int cell = blockIdx.y, m = blockIdx.x;
-  float g = GAMMA[(size_t)cell * w + m];
-  float* Y = Xout + ((size_t)cell * S_out + S_in + m) * w;
-  for (int n = threadIdx.x; n < w; n += blockDim.x) Y[n] = g * Wt[(size_t)m * w + n];
-}
-
-// Per-neuron reduction over all rows (compensated): r = sum |x| (sound) or sigma = sqrt(sum x^2).
-__global__ void k_reduce(const float* X, int S, int w, int mode, float* RAD) {
-  int cell = blockIdx.x;
-  const float* Xc = X + (size_t)cell * S * w;
-  for (int n = threadIdx.x; n < w; n += blockDim.x) {
-    float s = 0.0f, comp = 0.0f;
-    for (int r = 0; r < S; ++r) {
-      float x = Xc[(size_t)r * w + n];
-      float v = (mode == ISX_BOUND_CLT) ? x * x : fabsf(x);
-      float y = v - comp;
-      float t = s + y;
-      comp = (t - s) - y;
-      s = t;
+// Rows of the symbols created by the last activation, gamma_n W[:, n] for every neuron with gamma_n != 0,
+// after the cell's carried rows, and the row -> cell map of all of its rows.  WPC warps per cell: warp u
+// writes the neurons of the 32-groups u, u + WPC, ...
+template <int WPC>
+__global__ void __launch_bounds__(256) k_fresh_rows(int nc, int w, const float* __restrict__ GAMMA,
+                                                    const float* __restrict__ Wt, const int* cnt_in, const int* cnt_out,
+                                                    const int64_t* off_out, float* Xout, int* rowcell) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, u = warp % WPC;
+  const int cell = blockIdx.x * (8 / WPC) + warp / WPC;
+  if (cell >= nc) return;
+  const int64_t o0 = off_out[cell];
+  const int co = cnt_out[cell];
+  for (int r = u * 32 + lane; r < co; r += 32 * WPC) rowcell[o0 + r] = cell;
+  const float* ga = GAMMA + (size_t)cell * w;
+  float* Y = Xout + (size_t)(o0 + cnt_in[cell]) * w;
+  for (int g0 = 0, row = 0; g0 < w; g0 += 32) {
+    const float gm = g0 + lane < w ? ga[g0 + lane] : 0.0f;
+    unsigned b = __ballot_sync(0xffffffffu, gm != 0.0f);
+    if ((g0 >> 5) % WPC != u) {
+      row += __popc(b);
+      continue;
     }
-    RAD[(size_t)cell * w + n] = (mode == ISX_BOUND_CLT) ? sqrtf(s) : s;
+    for (; b; b &= b - 1, ++row) {
+      const int l = __ffs(b) - 1;
+      const float g = __shfl_sync(0xffffffffu, gm, l);
+      const float4* src = reinterpret_cast<const float4*>(Wt + (size_t)(g0 + l) * w);
+      float4* d = reinterpret_cast<float4*>(Y + (size_t)row * w);
+      for (int n = lane; n < w / 4; n += 32) {
+        const float4 x = src[n];
+        d[n] = make_float4(g * x.x, g * x.y, g * x.z, g * x.w);
+      }
+    }
   }
 }
 
-// Output layer w -> 1 and the read-off.  One block per cell, one warp per coefficient row.
-__global__ void __launch_bounds__(256) k_output(const float* X, int S, int w, const float* C,
-                                                const float* ALPHA, const float* GAMMA,
-                                                const float* RAD, const float* __restrict__ wout,
-                                                float bout, int mode, int inflate, float* center,
-                                                float* spread, int64_t first) {
-  __shared__ float s_aw[1024];
-  __shared__ float red[2][8];
-  int cell = blockIdx.x;
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float* al = ALPHA + (size_t)cell * w;
-  for (int n = threadIdx.x; n < w; n += blockDim.x) s_aw[n] = al[n] * wout[n];
+// Per-neuron reduction over the cell's rows (compensated), r = sum |x| (sound) or sigma = sqrt(sum x^2), and
+// activation j + 1: post-activation centre in place, alpha, gamma (and, inflate, the radius) and, for the
+// next layer, the row count cnt + #(gamma != 0).
+__global__ void __launch_bounds__(256) k_reduce_act(const float* __restrict__ X, const int64_t* off, const int* cnt,
+                                                    int nc, int tpc, int w, int mode, int act, int inflate, float* C,
+                                                    float* RAD, const float* DELTA, float* ALPHA, float* GAMMA,
+                                                    int* cnt_next) {
+  __shared__ int made[16];
+  const int sub = threadIdx.x / tpc, t = threadIdx.x - sub * tpc;
+  const int cell = blockIdx.x * (blockDim.x / tpc) + sub;
+  if (threadIdx.x < 16) made[threadIdx.x] = 0;
   __syncthreads();
-  bool sq = (mode != ISX_BOUND_SOUND);
-  // carried rows
-  float s = 0.0f, comp = 0.0f;
-  const float* Xc = X + (size_t)cell * S * w;
-  for (int r = warp; r < S; r += 8) {
-    float y = 0.0f;
-    for (int n = lane; n < w; n += 32) y = fmaf(Xc[(size_t)r * w + n], s_aw[n], y);
+  int S = 0;
+  if (cell < nc) {
+    S = cnt[cell];
+    const float* Xc = X + (size_t)off[cell] * w;
+    int m = 0;
+    for (int n = t; n < w; n += tpc) {
+      float s = 0.0f, comp = 0.0f;
+      auto add = [&](float x) {
+        const float v = (mode == ISX_BOUND_CLT) ? x * x : fabsf(x);
+        const float y = v - comp, tt = s + y;
+        comp = (tt - s) - y;
+        s = tt;
+      };
+      int r = 0;
+      for (; r + 8 <= S; r += 8) {                 // eight loads in flight
+        float x[8];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-    float v = sq ? y * y : fabsf(y);
-    float yy = v - comp, t = s + yy;
-    comp = (t - s) - yy;
-    s = t;
+        for (int q = 0; q < 8; ++q) x[q] = Xc[(size_t)(r + q) * w + n];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) add(x[q]);
+      }
+      for (; r < S; ++r) add(Xc[(size_t)r * w + n]);
+      const float rad = (mode == ISX_BOUND_CLT) ? sqrtf(s) : s;
+      const size_t i = (size_t)cell * w + n;
+      const Lin L = linearise(mode, act, inflate, C[i], rad, inflate ? DELTA[i] : 0.0f);
+      C[i] = L.center;
+      ALPHA[i] = L.alpha;
+      GAMMA[i] = L.gamma;
+      if (inflate) RAD[i] = rad;
+      m += L.gamma != 0.0f;
+    }
+    if (m) atomicAdd(&made[sub], m);
   }
-  // symbols of the last ReLU: y_m = gamma_m w_m
-  float s2 = 0.0f, e = 0.0f, g = 0.0f, y0 = 0.0f;
-  for (int m = threadIdx.x; m < w; m += blockDim.x) {
-    size_t i = (size_t)cell * w + m;
-    float y = GAMMA[i] * wout[m];
-    s2 += sq ? y * y : fabsf(y);
-    y0 = fmaf(wout[m], C[i], y0);
-    if (inflate) {
-      e = fmaf(fabsf(wout[m]), fabsf(C[i]), e);
-      g = fmaf(fabsf(wout[m]), fmaf(ALPHA[i], RAD[i], GAMMA[i]), g);
+  __syncthreads();
+  if (cnt_next && cell < nc && t == 0) cnt_next[cell] = S + made[sub];
+}
+
+// Output layer w -> 1 and the read-off.  Row r's term goes to partial sum r % 8 (compensated, r ascending),
+// held by WPC warps per cell: all eight by one warp or one per warp, four rows' 16-byte loads in flight.  The
+// cell's result does not depend on WPC.
+template <int WPC>
+__global__ void __launch_bounds__(256) k_output(const float* __restrict__ X, const int64_t* off, const int* cnt, int nc,
+                                                int w, const float* C, const float* ALPHA, const float* GAMMA,
+                                                const float* RAD, const float* __restrict__ wout, float bout, int mode,
+                                                int inflate, float* center, float* spread, int64_t first) {
+  extern __shared__ __align__(16) float s_aw[];    // [cells of the block][w]: alpha o w_out
+  __shared__ float red[8];
+  constexpr int CPB = 8 / WPC;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = warp / WPC, u = warp % WPC;
+  const int cell = blockIdx.x * CPB + sub;
+  for (int i = threadIdx.x; i < CPB * w; i += blockDim.x) {
+    const int c = blockIdx.x * CPB + i / w;
+    s_aw[i] = c < nc ? ALPHA[(size_t)c * w + i % w] * wout[i % w] : 0.0f;
+  }
+  __syncthreads();
+  const bool sq = (mode != ISX_BOUND_SOUND);
+  float rows = 0.0f;                               // the rows' sum over the eight partials
+  if (cell < nc) {
+    const float* aw = s_aw + sub * w;
+    const float* Xc = X + (size_t)off[cell] * w;
+    const int S = cnt[cell];
+    constexpr int NS = WPC == 1 ? 8 : 1;           // partial sums of this warp
+    float s[NS] = {}, comp[NS] = {};
+    // rows r0 + q WPC, q < 4, into the partials h + q (WPC = 1) or into the warp's own
+    auto four = [&](int r0, int h) {
+      float y[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int n = 4 * lane; n < w; n += 128) {
+        const float4 a = *reinterpret_cast<const float4*>(aw + n);
+        float4 x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = *reinterpret_cast<const float4*>(Xc + (size_t)min(r0 + q * WPC, S - 1) * w + n);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y[q] = fmaf(x[q].w, a.w, fmaf(x[q].z, a.z, fmaf(x[q].y, a.y, fmaf(x[q].x, a.x, y[q]))));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y[q] += __shfl_xor_sync(0xffffffffu, y[q], o);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (r0 + q * WPC < S) {
+          const int k = WPC == 1 ? h + q : 0;
+          const float v = sq ? y[q] * y[q] : fabsf(y[q]);
+          const float yy = v - comp[k], t = s[k] + yy;
+          comp[k] = (t - s[k]) - yy;
+          s[k] = t;
+        }
+    };
+    if constexpr (WPC == 1) {
+      for (int r0 = 0; r0 < S; r0 += 8) {
+        four(r0, 0);
+        if (r0 + 4 < S) four(r0 + 4, 4);
+      }
+    } else {
+      for (int r0 = u; r0 < S; r0 += 4 * WPC) four(r0, 0);
+    }
+    if (WPC == 1) {
+#pragma unroll
+      for (int q = 0; q < NS; ++q) rows += s[q];
+    } else if (lane == 0) {
+      red[warp] = s[0];
     }
   }
-  // block reductions (the warp-row sums live in lane 0 of each warp)
-  float part = (lane == 0 ? s : 0.0f) + s2;
-  float vals[4] = {part, y0, e, g};
-  float tot[4];
-  for (int q = 0; q < 4; ++q) {
-    float v = vals[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (WPC > 1) {
     __syncthreads();
-    if (lane == 0) red[0][warp] = v;
-    __syncthreads();
-    float acc = 0.0f;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) acc += red[0][k];
-    tot[q] = acc;
+    if (u == 0)
+      for (int k = 0; k < WPC; ++k) rows += red[k];
   }
-  if (threadIdx.x == 0) {
-    float x0 = tot[1] + bout;
+  if (u > 0 || cell >= nc) return;
+  // symbols of the last activation, y_m = gamma_m w_m, and the centre
+  float v[4] = {0.f, 0.f, 0.f, 0.f};               // sum |y| or y^2, w . c, and the two error sums (inflate)
+  for (int m = lane; m < w; m += 32) {
+    const size_t i = (size_t)cell * w + m;
+    const float y = GAMMA[i] * wout[m];
+    v[0] += sq ? y * y : fabsf(y);
+    v[1] = fmaf(wout[m], C[i], v[1]);
+    if (inflate) {
+      v[2] = fmaf(fabsf(wout[m]), fabsf(C[i]), v[2]);
+      v[3] = fmaf(fabsf(wout[m]), fmaf(ALPHA[i], RAD[i], GAMMA[i]), v[3]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+  if (lane == 0) {
+    const float tot = rows + v[0], x0 = v[1] + bout;
     float sp;
     if (mode == ISX_BOUND_SOUND) {
-      sp = tot[0];
+      sp = tot;
       if (inflate) {
         float ge = gamma_k(w + 1) + kU;
-        sp = __fadd_ru(__fmul_ru(sp, kSafe), (ge * tot[3] + gamma_k(w + 2) * (tot[2] + fabsf(bout))) * 1.01f);
+        sp = __fadd_ru(__fmul_ru(sp, kSafe), (ge * v[3] + gamma_k(w + 2) * (v[2] + fabsf(bout))) * 1.01f);
       }
     } else if (mode == ISX_BOUND_CLT) {
-      sp = sqrtf(tot[0]);
+      sp = sqrtf(tot);
     } else {
-      sp = sqrtf(tot[0] / 3.0f);
+      sp = sqrtf(tot / 3.0f);
     }
     center[first + cell] = x0;
     spread[first + cell] = sp;
@@ -302,91 +484,158 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   const int w = inr->w, H = inr->H;
   if (mode != ISX_BOUND_SOUND) inflate = 0;
   const int Smax = 3 + w * (H - 1);
-  // chunk so that the two coefficient buffers stay within ~6 GB
-  size_t per_cell = 2ull * Smax * w * sizeof(float);
-  int64_t nc_max = std::max<int64_t>(1, (int64_t)((6ull << 30) / per_cell));
-  nc_max = std::min<int64_t>(nc_max, 1 << 16);
-  int64_t nc_alloc = std::min<int64_t>(n, nc_max);
+  // the two coefficient buffers take at most ~6 GB: enough for full_cells cells with every symbol alive
+  const size_t per_cell = 2ull * Smax * w * sizeof(float);
+  const int64_t full_cells = std::min<int64_t>({n, (int64_t)1 << 16, std::max<int64_t>(1, (int64_t)((6ull << 30) / per_cell))});
+  const int64_t row_cap = full_cells * Smax;
+  // More cells than that: the host reads every layer's row count, and a chunk holds as many cells as the
+  // rows they really have allow.  Otherwise (and while the stream is captured, where the host cannot
+  // read) chunks of full_cells need no count on the host at all.
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  ISX_CUDA(cudaStreamIsCapturing(st, &cs));
+  const bool counted = n > full_cells && cs == cudaStreamCaptureStatusNone;
+  const int64_t nc_alloc = counted ? std::min<int64_t>(n, (int64_t)1 << 16) : full_cells;
   auto& ws = inr->ws;
-  ISX_TRY(ws[WS_X0].ensure((size_t)nc_alloc * Smax * w * sizeof(float), "X0"));
-  ISX_TRY(ws[WS_X1].ensure((size_t)nc_alloc * Smax * w * sizeof(float), "X1"));
-  for (Slot s : {WS_C, WS_RAD, WS_ALPHA, WS_GAMMA, WS_DELTA})
+  for (Slot s : {WS_X0, WS_X1}) ISX_TRY(ws[s].ensure((size_t)row_cap * w * sizeof(float), "rows"));
+  for (Slot s : {WS_R_RC0, WS_R_RC1}) ISX_TRY(ws[s].ensure((size_t)row_cap * sizeof(int), "row cells"));
+  for (Slot s : {WS_C, WS_R_A, WS_RAD, WS_ALPHA, WS_GAMMA, WS_DELTA})
     ISX_TRY(ws[s].ensure((size_t)nc_alloc * w * sizeof(float), "per-neuron"));
-  float* C = ws[WS_C].as<float>();
+  for (Slot s : {WS_R_CNT0, WS_R_CNT1}) ISX_TRY(ws[s].ensure((size_t)nc_alloc * sizeof(int), "row counts"));
+  for (Slot s : {WS_R_OFF0, WS_R_OFF1}) ISX_TRY(ws[s].ensure((size_t)nc_alloc * sizeof(int64_t), "row offsets"));
+  ISX_TRY(ws[WS_R_TOT].ensure(rows::scan_bytes(nc_alloc), "row total and scan block sums"));
+  int64_t* d_tot = ws[WS_R_TOT].as<int64_t>();
   float* RAD = ws[WS_RAD].as<float>();
   float* AL = ws[WS_ALPHA].as<float>();
   float* GA = ws[WS_GAMMA].as<float>();
   float* DE = ws[WS_DELTA].as<float>();
-  const int bt = std::min(w, 256);
-  for (int64_t first = 0; first < n; first += nc_alloc) {
-    int nc = (int)std::min<int64_t>(nc_alloc, n - first);
-    float* Xa = ws[WS_X0].as<float>();
-    float* Xb = ws[WS_X1].as<float>();
-    int S = 3;
+  const Slot xs[2] = {WS_X0, WS_X1}, rs[2] = {WS_R_RC0, WS_R_RC1}, ns[2] = {WS_R_CNT0, WS_R_CNT1},
+             os[2] = {WS_R_OFF0, WS_R_OFF1};
+  int sms = 148;
+  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
+  const CellBlock cb(w);
+  int64_t want = nc_alloc;                         // cells of the next chunk
+  for (int64_t first = 0; first < n;) {
+    const int nc = (int)std::min<int64_t>(want, n - first);
+    float* C = ws[WS_C].as<float>();
+    float* C2 = ws[WS_R_A].as<float>();
+    // few cells: a whole block per cell in the kernels that walk over a cell's rows
+    const bool wide = nc < 8 * sms;
+    int cur = 0;
+    int64_t R = 3 * (int64_t)nc;                   // rows of z_j (an upper bound where the host does not know)
+    bool fits = true;
     {
       prof::Scope _ps(K_INPUT, st, 0, 0);
-      k_input_layer<<<nc, bt, 0, st>>>(src, first, nc, inr->W[0], inr->b[0], w, (int)mode, inflate, C, Xa, S,
-                                       RAD, DE);
+      k_input_layer<<<cb.blocks(nc), cb.threads(), 0, st>>>(
+          src, first, nc, cb.tpc, inr->W[0], inr->b[0], w, (int)mode, inr->act, inflate, C, ws[xs[0]].as<float>(),
+          ws[rs[0]].as<int>(), RAD, AL, GA, ws[os[0]].as<int64_t>(), ws[ns[0]].as<int>(), ws[ns[1]].as<int>());
     }
     ISX_LAUNCH_CHECK("k_input_layer");
-    int64_t tot = (int64_t)nc * w;
     for (int j = 1; j <= H - 1; ++j) {
+      const int nxt = cur ^ 1;
+      int* cnt_in = ws[ns[cur]].as<int>();
+      int* cnt_out = ws[ns[nxt]].as<int>();
+      int64_t* off_in = ws[os[cur]].as<int64_t>();
+      int64_t* off_out = ws[os[nxt]].as<int64_t>();
+      float* Xa = ws[xs[cur]].as<float>();
+      float* Xb = ws[xs[nxt]].as<float>();
+      // d_tot[j & 1]: rows of z_{j+1}; the other one still holds those of z_j
       {
-        prof::Scope _ps(K_RELU, st, 0, 0);
-        k_relu<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(tot, (int)mode, inflate, inr->act, C, RAD, DE, AL, GA);
+        prof::Scope _ps(K_SCAN, st, 0, 0);
+        ISX_TRY(rows::scan_counts(cnt_out, nc, d_tot, j & 1, off_out, st));
       }
-      ISX_LAUNCH_CHECK("k_relu");
-      float kappa = 3.0f * kU + gamma_k(w);
-      {
-        prof::Scope _ps(K_GEMV, st, 2.0 * nc * w * w, 0);
-        k_center_gemv<<<nc, bt, 2 * w * sizeof(float), st>>>(nc, w, w, inr->Wt[j], inr->b[j], C, AL, RAD, GA, DE,
-                                                            inflate, kappa);
+      int64_t Rn = std::min<int64_t>(row_cap, (int64_t)nc * (3 + (int64_t)w * j));
+      if (counted) {
+        ISX_CUDA(cudaMemcpyAsync(&Rn, d_tot + (j & 1), sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        ISX_CUDA(cudaStreamSynchronize(st));
+        // rows after the last layer if every layer creates as many as the ones so far
+        const double last = 3.0 * nc + (double)(Rn - 3 * (int64_t)nc) / j * (H - 1);
+        if (Rn > row_cap || (j == 1 && last > 1.2 * (double)row_cap)) {
+          want = std::max<int64_t>(full_cells, std::min<int64_t>(nc / 2, (int64_t)(0.8 * nc * (double)row_cap / std::max(last, (double)Rn))));
+          fits = false;                            // start the chunk again with fewer cells
+          break;
+        }
       }
-      ISX_LAUNCH_CHECK("k_center_gemv");
-      int S_out = S + w;
-      // the coefficient buffers are laid out with the final stride S_out per cell; the tile shape
-      // comes from the autotuner (timed once per width and row-count bucket)
+      // the tile shape comes from the autotuner (timed once per width and row-count bucket)
       {
-        int bucket = 1;
-        while (bucket < S) bucket <<= 1;
+        GemmArgs g{};
+        g.X = Xa;
+        g.Y = Xb;
+        g.Wt = inr->Wt[j];
+        g.alpha = AL;
+        g.rowcell = ws[rs[cur]].as<int>();
+        g.off_in = off_in;
+        g.off_out = off_out;
+        g.d_R = (counted || j == 1) ? nullptr : d_tot + ((j - 1) & 1);
+        g.R = R;
+        int64_t bucket = 1;
+        while (bucket < std::min<int64_t>(R, 1 << 16)) bucket <<= 1;
         const std::string key = "gemm_fp32 w=" + std::to_string(w) + " rows<=" + std::to_string(bucket);
-        const float* Wt = inr->Wt[j];
-        auto run = [&](int v) -> isx_status {
-          launch_gemm(v, nc, S, S_out, w, Xa, Xb, Wt, AL, st);
-          ISX_LAUNCH_CHECK("k_gemm_fp32");
-          return ISX_OK;
-        };
+        auto run = [&](int v) { return launch_gemm<true>(v, g, w, sms, st); };
         int v = 0;
         ISX_TRY(tune::pick(key, kGemmVariants, [&](int i) { return kGemmShapes[i].name; }, run, st, &v));
-        prof::Scope _ps(K_GEMM_FP32, st, 2.0 * nc * (double)S * w * w, 8.0 * nc * (double)S * w);
+        // counted work: the rows, or the input rows alone where only the device knows how many there are
+        const double rows_known = g.d_R ? 3.0 * nc : (double)R;
+        prof::Scope _ps(K_GEMM_FP32, st, 2.0 * rows_known * w * w, 8.0 * rows_known * w);
         ISX_TRY(run(v));
       }
       {
-        prof::Scope _ps(K_FRESH, st, 0, 4.0 * nc * w * w);
-        k_fresh_rows<<<dim3(w, nc), bt, 0, st>>>(Xb, S, S_out, w, inr->Wt[j], GA);
+        prof::Scope _ps(K_FRESH, st, 0, 0);
+        if (wide)
+          k_fresh_rows<8><<<nc, 256, 0, st>>>(nc, w, GA, inr->Wt[j], cnt_in, cnt_out, off_out, Xb, ws[rs[nxt]].as<int>());
+        else
+          k_fresh_rows<1><<<(nc + 7) / 8, 256, 0, st>>>(nc, w, GA, inr->Wt[j], cnt_in, cnt_out, off_out, Xb,
+                                                        ws[rs[nxt]].as<int>());
       }
       ISX_LAUNCH_CHECK("k_fresh_rows");
       {
-        prof::Scope _ps(K_REDUCE, st, 0, 4.0 * nc * (double)S_out * w);
-        k_reduce<<<nc, bt, 0, st>>>(Xb, S_out, w, (int)mode, RAD);
+        prof::Scope _ps(K_GEMV, st, 2.0 * nc * w * w, 0);
+        if (inflate) {
+          const float kappa = 3.0f * kU + gamma_k(w);
+          k_center_gemv<<<nc, std::min(w, 256), 2 * w * sizeof(float), st>>>(nc, w, w, inr->Wt[j], inr->b[j], C, AL, RAD,
+                                                                             GA, DE, inflate, kappa);
+          ISX_LAUNCH_CHECK("k_center_gemv");
+        } else {
+          GemmArgs g{};
+          g.X = C;
+          g.Y = C2;
+          g.Wt = inr->Wt[j];
+          g.bias = inr->b[j];
+          g.R = nc;
+          ISX_TRY(launch_gemm<false>((int64_t)nc * w < (int64_t)sms * 8192 ? 4 : 0, g, w, sms, st));
+          std::swap(C, C2);
+        }
       }
-      ISX_LAUNCH_CHECK("k_reduce");
-      std::swap(Xa, Xb);
-      S = S_out;
+      {
+        prof::Scope _ps(K_REDUCE, st, 0, 0);
+        k_reduce_act<<<cb.blocks(nc), cb.threads(), 0, st>>>(Xb, off_out, cnt_out, nc, cb.tpc, w, (int)mode, inr->act,
+                                                             inflate, C, RAD, DE, AL, GA, j < H - 1 ? cnt_in : nullptr);
+      }
+      ISX_LAUNCH_CHECK("k_reduce_act");
+      cur = nxt;
+      R = Rn;
     }
-    {
-      prof::Scope _ps(K_RELU, st, 0, 0);
-      k_relu<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(tot, (int)mode, inflate, inr->act, C, RAD, DE, AL, GA);
-    }
-    ISX_LAUNCH_CHECK("k_relu");
+    if (!fits) continue;
     const int L = inr->n_layers - 1;
-    float bout = inr->hb[L][0];
     {
-      prof::Scope _ps(K_OUTPUT, st, 2.0 * nc * (double)S * w, 4.0 * nc * (double)S * w);
-      k_output<<<nc, 256, 0, st>>>(Xa, S, w, C, AL, GA, RAD, inr->W[L], bout, (int)mode, inflate, d_center,
-                                   d_spread, first);
+      prof::Scope _ps(K_OUTPUT, st, 0, 0);
+      const float* X = ws[xs[cur]].as<float>();
+      const int64_t* off = ws[os[cur]].as<int64_t>();
+      const int* cnt = ws[ns[cur]].as<int>();
+      if (wide)
+        k_output<8><<<nc, 256, w * sizeof(float), st>>>(X, off, cnt, nc, w, C, AL, GA, RAD, inr->W[L], inr->hb[L][0],
+                                                        (int)mode, inflate, d_center, d_spread, first);
+      else
+        k_output<1><<<(nc + 7) / 8, 256, 8 * w * sizeof(float), st>>>(X, off, cnt, nc, w, C, AL, GA, RAD, inr->W[L],
+                                                                      inr->hb[L][0], (int)mode, inflate, d_center,
+                                                                      d_spread, first);
     }
     ISX_LAUNCH_CHECK("k_output");
+    if (counted) {
+      // the next chunk: as many cells as fill the buffers to 4/5 at this chunk's rows per cell
+      const double per = std::max(1.0, (double)R / nc);
+      want = std::max<int64_t>(full_cells, std::min<int64_t>(nc_alloc, (int64_t)(0.8 * (double)row_cap / per)));
+    }
+    first += nc;
   }
   return ISX_OK;
 }

@@ -196,8 +196,8 @@ struct MlpView {
 // and every hidden layer is one sgemm tile (sgemm.cuh) written back in place, so global memory holds only
 // the points, the values and the weights (L2).  Every value is the same chain of multiply-adds whatever
 // the launch shape.  Bound by FP32 FMA issue and the shared-memory return bandwidth (an 8 x 8 tile reads 16
-// values per 64 multiply-adds): 3 -> 512 x 8 -> 1 at 300007 points 24 ms = 46 TFLOP/s (125 ms = 8.8 TFLOP/s
-// for the earlier kernel, one neuron of 32 points per thread), 3 -> 256 x 5 -> 1 at 2^20 points 10.9 ms
+// values per 64 multiply-adds): 3 -> 512 x 8 -> 1 at 300007 points 22.4 ms = 49 TFLOP/s (125 ms = 8.8 TFLOP/s
+// for the earlier kernel, one neuron of 32 points per thread), 3 -> 256 x 5 -> 1 at 2^20 points 10.4 ms
 // (29.7 ms), 3 -> 64 x 2 -> 1 at 2^22 1.0 ms (3.3 ms); fma.rn.f32x2 from registers alone runs at 66-73 TFLOP/s.
 template <int TN>
 __global__ void __launch_bounds__(256) k_eval_fp32(MlpView m, sgemm::Shape sh, const float* xyz, const uint32_t* ids,
@@ -205,9 +205,16 @@ __global__ void __launch_bounds__(256) k_eval_fp32(MlpView m, sgemm::Shape sh, c
   extern __shared__ __align__(16) float sm[];
   const int w = m.w, P = sh.P, KB = sh.KB, spl = w / KB;
   float* A = sm;                                  // [w][P]
-  sgemm::Stream ws{sm + (size_t)w * P, w, KB, 0, (m.n_layers - 2) * spl};
-  auto stage_src = [&](int s) { return m.Wt[min(1 + s / spl, m.n_layers - 2)] + (size_t)(s % spl) * KB * w; };
-  for (int s = 0; s < sgemm::kStages - 1; ++s) ws.load(stage_src(s));
+  sgemm::Stream ws{sm + (size_t)w * P, w, KB, (int64_t)(m.n_layers - 2) * spl};
+  int sl = 1, sk = 0;                             // layer and K block of the stage to load next
+  auto load_next = [&] {
+    ws.load(m.Wt[min(sl, m.n_layers - 2)] + (size_t)sk * KB * w);
+    if (++sk == spl) {
+      sk = 0;
+      ++sl;
+    }
+  };
+  for (int s = 0; s < sgemm::kStages - 1; ++s) load_next();
   const int t = threadIdx.x, T = blockDim.x;
   const int64_t p0 = (int64_t)blockIdx.x * P;
   for (int p = t % P, g = t / P, gs = max(1, T / P); g < gs && p < P; p += T) {
@@ -220,7 +227,7 @@ __global__ void __launch_bounds__(256) k_eval_fp32(MlpView m, sgemm::Shape sh, c
   }
   const int PG = P / sgemm::kTM, pg = t % PG, ng = t / PG;
   const bool own = ng < w / TN;
-  int s = 0;
+  int slot = 0;
   for (int l = 1; l < m.n_layers - 1; ++l) {
     sgemm::Tile<TN> tile;
     if (own)
@@ -231,11 +238,12 @@ __global__ void __launch_bounds__(256) k_eval_fp32(MlpView m, sgemm::Shape sh, c
 #pragma unroll
         for (int i = 0; i < sgemm::kTM; ++i) tile.acc[i][c] = bb;
       }
-    for (int kb = 0; kb < spl; ++kb, ++s) {
+    for (int kb = 0; kb < spl; ++kb) {
       sgemm::cp_wait<sgemm::kStages - 2>();
-      __syncthreads();                            // stage s has landed, stage s - 1 is free, A is written
-      ws.load(stage_src(s + sgemm::kStages - 1));
-      if (own) tile.stage(A + (size_t)kb * KB * P, ws.Ws + (size_t)(s % sgemm::kStages) * KB * w, P, w, KB, pg, ng);
+      __syncthreads();                            // the stage has landed, the one before it is free, A is written
+      load_next();
+      if (own) tile.stage(A + (size_t)kb * KB * P, ws.Ws + (size_t)slot * KB * w, P, w, KB, pg, ng);
+      slot = slot == sgemm::kStages - 1 ? 0 : slot + 1;
     }
     __syncthreads();                              // every thread is done reading A
     if (own) {

@@ -68,6 +68,10 @@ __host__ __device__ __forceinline__ int rows_weight_row(int m, int w) {
 // cell + t.  Rows of a cell are contiguous, so cell c < c' implies t <= t' and the slots of all
 // (cell, block) pairs that share rows are distinct.
 __host__ __device__ __forceinline__ int64_t rows_part_slot(int64_t cell, int64_t t) { return cell + t; }
+// Exclusive scan of nc per-cell row counts into int64 offsets; the total goes to d_tot[slot] (slot < 8).
+// d_tot: scan_bytes(nc) bytes, eight totals and the block sums.
+size_t scan_bytes(int64_t nc);
+isx_status scan_counts(const int* cnt, int64_t nc, int64_t* d_tot, int slot, int64_t* off, cudaStream_t st);
 // One CTA waits on an mbarrier that nothing completes, with rwait and the given limit, raising
 // ISX_ERR_TIMEOUT in *d_status (rows_gemm.cu).
 isx_status check_bounded_wait(int64_t limit_ns, int* d_status, cudaStream_t st);

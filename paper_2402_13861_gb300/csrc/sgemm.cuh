@@ -59,15 +59,17 @@ struct Shape {
 struct Stream {
   float* Ws;                           // [kStages][KB * w]
   int w, KB;
-  int next, total;                     // stage to load next, stages in all
-  // loads stage `next` of the stream from `src` (its KB rows) and commits a group, also when empty
+  int64_t left;                        // stages still to load
+  int slot = 0;                        // ring slot of the next one
+  // loads the next stage of the stream from `src` (its KB rows) and commits a group, also when none is left
   __device__ __forceinline__ void load(const float* src) {
-    if (next < total) {
-      float* dst = Ws + (size_t)(next % kStages) * KB * w;
+    if (left > 0) {
+      float* dst = Ws + (size_t)slot * KB * w;
       for (int i = threadIdx.x * 4; i < KB * w; i += blockDim.x * 4) cp16(dst + i, src + i);
     }
     cp_commit();
-    ++next;
+    --left;
+    slot = slot == kStages - 1 ? 0 : slot + 1;
   }
 };
 

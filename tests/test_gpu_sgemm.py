@@ -4,8 +4,8 @@ import numpy as np
 import pytest
 import torch
 
-from oracle import mlp
-from synth import inr
+from oracle import affine, mlp
+from synth import boxes, inr
 
 pytestmark = pytest.mark.gpu
 
@@ -41,4 +41,55 @@ def test_eval_fp32_tile_edges(pkg, w, H):
         if first is None:
             first = v[0]
         assert v[0] == first                       # the chain of one point does not depend on the shape
+    net.close()
+
+
+@pytest.mark.parametrize("w,H,act,mode,inflate", [(16, 1, "relu", "sound", True), (16, 3, "relu", "clt", False),
+                                                  (48, 4, "sine", "clt", False), (64, 2, "relu", "raua", False),
+                                                  (112, 3, "relu", "sound", False), (128, 3, "elu", "clt", False),
+                                                  (272, 2, "relu", "sound", True), (512, 2, "relu", "clt", False)])
+def test_fp32_bounds_row_edges(pkg, w, H, act, mode, inflate):
+    """Coarse to fine boxes, from one cell to more than fit with every symbol alive (where the host reads the
+    row counts and a chunk is shrunk and restarted): a cell's bound does not depend on its neighbours or
+    the chunking, and stays within the float32 band 8 H w 2^-24 (|x0| + s) of the oracle."""
+    layers = inr.random_inr([3] + [w] * H + [1], 60 + w, act=act)
+    net = pkg.Inr(layers, act=act)
+    full = min(1 << 16, (6 << 30) // (2 * (3 + w * (H - 1)) * w * 4))
+    n = min(70001, full + 513)
+    lo, hi = boxes.random_boxes(n, 61, -10, -1)
+    order = np.argsort(hi[:, 0] - lo[:, 0], kind="stable")          # fine boxes first, coarse ones last
+    dlo, dhi = (torch.tensor(x[order], device="cuda") for x in (lo, hi))
+    c, s = net.bound_cells(dlo, dhi, mode=mode, prec="fp32", inflate=inflate)
+    pick = np.unique(np.r_[0, 1, n // 2, n - 2, n - 1, np.random.default_rng(62).integers(0, n, 24)])
+    for i in pick[[0, 3, len(pick) // 2, -1]]:
+        ci, si = net.bound_cells(dlo[i:i + 1], dhi[i:i + 1], mode=mode, prec="fp32", inflate=inflate)
+        assert ci[0] == c[i] and si[0] == s[i]
+    a, b = net.bound_cells(dlo[pick].contiguous(), dhi[pick].contiguous(), mode=mode, prec="fp32", inflate=inflate)
+    assert torch.equal(a, c[pick]) and torch.equal(b, s[pick])
+    c, s = c.cpu().numpy().astype(np.float64)[pick], s.cpu().numpy().astype(np.float64)[pick]
+    if act == "relu":
+        oc, os_ = affine.bound(layers, lo[order][pick], hi[order][pick], mode, batch=8)
+    else:
+        oc, os_ = affine.bound(layers, lo[order][pick], hi[order][pick], mode, batch=8, act=act)
+    tol = 8 * H * w * 2.0 ** -24 * (np.abs(oc) + os_) + 1e-7
+    if inflate:
+        assert np.all(c - s <= oc - os_ + 1e-7) and np.all(c + s >= oc + os_ - 1e-7)
+    else:
+        assert np.all(np.abs(c - oc) <= tol) and np.all(np.abs(s - os_) <= tol)
+    net.close()
+
+
+def test_fp32_bounds_under_capture(pkg):
+    """A stream capture takes the float32 bound (no host reads), after a plain call sized the workspace."""
+    net = pkg.Inr(inr.random_inr([3, 64, 64, 64, 1], 70))
+    lo, hi = (torch.tensor(x, device="cuda") for x in boxes.random_boxes(200, 71, -8, -1))
+    c0, s0 = [x.clone() for x in net.bound_cells(lo, hi, mode="clt", prec="fp32")]
+    c, s = torch.zeros_like(c0), torch.zeros_like(s0)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        net.bound_cells(lo, hi, mode="clt", prec="fp32", center=c, spread=s)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(c, c0) and torch.equal(s, s0)
     net.close()

@@ -38,6 +38,7 @@ namespace {
 
 constexpr float kU = 5.9604645e-08f;        // 2^-24, float32 unit roundoff
 constexpr float kSafe = 1.0000010f;         // (1 + 2^-20): slack for evaluating error formulas
+constexpr float kOutSafe = 1.0000020f;      // (1 + 32 u): the output layer's sums take at most 23 roundings (w = 512)
 constexpr float kInvSqrt3 = 0.57735026918962576f;
 
 __host__ __device__ __forceinline__ float gamma_k(int k) { return (k * kU) / (1.0f - k * kU); }
@@ -464,7 +465,7 @@ __global__ void __launch_bounds__(256) k_output(const float* __restrict__ X, con
       sp = tot;
       if (inflate) {
         float ge = gamma_k(w + 1) + kU;
-        sp = __fadd_ru(__fmul_ru(sp, kSafe), (ge * v[3] + gamma_k(w + 2) * (v[2] + fabsf(bout))) * 1.01f);
+        sp = __fadd_ru(__fmul_ru(sp, kOutSafe), (ge * v[3] + gamma_k(w + 2) * (v[2] + fabsf(bout))) * 1.01f);
       }
     } else if (mode == ISX_BOUND_CLT) {
       sp = sqrtf(tot);

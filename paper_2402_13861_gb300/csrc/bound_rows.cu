@@ -15,11 +15,13 @@
 // alpha is applied to the A operand (the rows) while it is staged into shared memory, so the B
 // operand is W_j itself, loaded once per CTA and shared by the rows of every cell: rows of many
 // cells fill each 128-row MMA tile (rows_gemm.cu).  Per chunk and layer this file runs:
-//   k_rows_input_act / k_rows_reduce_act: r = sum |x| (sound) or sigma^2 = sum x^2 (UP) per (cell,
-//     neuron) over the stored rows and the input rows, the linearisation of the next activation,
-//     the split A operand of the centre GEMM and the next per-cell row count;
+//   k_rows_input_act (layer 0 and activation 1);
 //   k_rows_scan_*: row offsets of the next layer (the host reads the total to size the buffers);
-//   the row GEMM, k_rows_new (the new rows) and k_rows_split (centre and input rows);
+//   the row GEMM and k_rows_new (the new rows);
+//   k_rows_layer (rows_layer.cu): centre and input rows on the tensor cores, and in its epilogue r = sum |x|
+//     (sound) or sigma^2 = sum x^2 (UP) per (cell, neuron) over the stored rows and the input rows, the
+//     linearisation of the next activation, the split A operand of the next layer and the next per-cell
+//     row count; with inflation (and for many cells at w = 64) k_rows_split, then k_rows_reduce_act;
 // and, after the last layer, k_rows_output: the output coefficient of every symbol is its row .
 // (alpha_H * w_out), read off as sum |y| or sum y^2.
 #include "internal.cuh"
@@ -93,10 +95,11 @@ void set_infl(Infl& f, int w) {
 }
 __device__ __forceinline__ __nv_bfloat16 bf16_up(float x) { return __float2bfloat16_ru(x); }
 
-// ---- layer 0 and activation 1: centre c_1, the three input rows I_1 = diag(h) W_0^T (written: the
-//      output layer of a one-hidden-layer net reads them), their reduction, the linearisation, the
-//      split A operand of the first centre / input-row GEMM (when AH is given) and the row count of
-//      the first stored block.  w / 2 threads per cell, two adjacent neurons per thread. ----
+// ---- layer 0 and activation 1: centre c_1 and the three input rows I_1 = diag(h) W_0^T (written where
+//      given: the output layer of a one-hidden-layer net reads both, the float32 centre GEMM the centre), their
+//      reduction, the linearisation, the split A operand of the first centre / input-row GEMM (when AH is
+//      given) and the row count of the first stored block.  w / 2 threads per cell, two adjacent neurons
+//      per thread. ----
 __global__ void __launch_bounds__(256) k_rows_input_act(CellSource src, int64_t first, int nc, int w, int mode,
                                                         int act, const float* __restrict__ W0,
                                                         const float* __restrict__ b0, float* I, float* A, float* AL,
@@ -147,9 +150,10 @@ __global__ void __launch_bounds__(256) k_rows_input_act(CellSource src, int64_t 
       }
     }
     const size_t o = (size_t)cell * w + n;
-    for (int d = 0; d < 3; ++d)
-      *reinterpret_cast<float2*>(I + ((size_t)cell * 3 + d) * w + n) = make_float2(iv[0][d], iv[1][d]);
-    *reinterpret_cast<float2*>(A + o) = make_float2(L[0].center, L[1].center);
+    if (I)
+      for (int d = 0; d < 3; ++d)
+        *reinterpret_cast<float2*>(I + ((size_t)cell * 3 + d) * w + n) = make_float2(iv[0][d], iv[1][d]);
+    if (A) *reinterpret_cast<float2*>(A + o) = make_float2(L[0].center, L[1].center);
     *reinterpret_cast<float2*>(AL + o) = make_float2(L[0].alpha, L[1].alpha);
     *reinterpret_cast<float2*>(GA + o) = make_float2(L[0].gamma, L[1].gamma);
     m = (L[0].gamma != 0.0f) + (L[1].gamma != 0.0f);
@@ -300,7 +304,8 @@ template <int CPL>
 __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, const float* __restrict__ GA,
                                                              const float* __restrict__ Wt, const int* cnt_in,
                                                              const int64_t* off_out, const int* cnt_out,
-                                                             __nv_bfloat16* xout, int* rowcell_out, float* pnew) {
+                                                             __nv_bfloat16* xout, int* rowcell_out, float* pnew,
+                                                             int* cnt_next) {
   constexpr int w = 32 * CPL;
   using IO = NewRowIO<CPL>;
   const int lane = threadIdx.x & 31;
@@ -308,6 +313,7 @@ __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, con
   if (cell >= nc) return;
   const int64_t o0 = off_out[cell];
   const int co = cnt_out[cell];
+  if (cnt_next && lane == 0) cnt_next[cell] = co;  // k_rows_layer adds the next activation's symbols
   for (int r = lane; r < co; r += 32) rowcell_out[o0 + r] = cell;
   const int m0 = lane * CPL;                       // this lane's columns m0 .. m0 + CPL - 1
   float acc[CPL];
@@ -960,20 +966,29 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
   // chunk size: about kRowBudget G rows per chunk, from the rows per cell the previous chunk needed
   const int64_t kRowBudget = inr->row_budget;
   const int64_t kMaxCells = kMaxChunkCells;
+  int sms = 148;
+  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
   double rows_per_cell = (double)w * (H - 1);
   int64_t first = 0;
   while (first < n) {
     const int64_t want = (int64_t)((double)kRowBudget / std::max(1.0, 1.25 * rows_per_cell));
     const int nc = (int)std::min<int64_t>(n - first, std::max<int64_t>(1024, std::min(kMaxCells, want)));
     const size_t cw = (size_t)nc * w * sizeof(float);
-    ISX_TRY(ws[WS_C].ensure(cw, "rows centre"));
     ISX_TRY(ws[WS_R_A].ensure(cw, "rows post-activation centre"));
     ISX_TRY(ws[WS_ALPHA].ensure(cw, "rows alpha"));
     ISX_TRY(ws[WS_GAMMA].ensure(cw, "rows gamma"));
     ISX_TRY(ws[WS_R_I0].ensure(3 * cw, "rows input rows"));
-    ISX_TRY(ws[WS_R_I1].ensure(3 * cw, "rows input rows"));
     ISX_TRY(ws[WS_R_PNEW].ensure(cw, "new-row column sums"));
     Infl infl;
+    // Without inflation one kernel does the centre and input rows and the activation (k_rows_layer), so they
+    // never go through memory: 3 -> 256 x 5 -> 1, 262144 cells, 2.60 ms for a chunk's layers against 4.74 ms.
+    // At w = 64 half of its epilogue threads have no neuron and two small kernels (many CTAs per SM) are
+    // faster (155 us against 210 us at 20011 cells) once every SM has a tile; below that, one launch fewer is.
+    const bool fused = !inflate && (w >= 128 || nc <= 32 * sms);
+    if (!fused) {
+      ISX_TRY(ws[WS_C].ensure(cw, "rows centre"));
+      ISX_TRY(ws[WS_R_I1].ensure(3 * cw, "rows input rows"));
+    }
     if (inflate) {
       ISX_TRY(ws[WS_R_V].ensure(cw / 2, "rounding-bound operand"));
       ISX_TRY(ws[WS_R_D].ensure(cw, "rounding-bound GEMM result"));
@@ -984,7 +999,11 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
     }
     ISX_TRY(ws[WS_R_AH].ensure(4 * cw / 2, "split A, high terms"));
     ISX_TRY(ws[WS_R_ALO].ensure(4 * cw / 2, "split A, low terms"));
-    for (Slot s : {WS_R_CNT0, WS_R_CNT1}) ISX_TRY(ws[s].ensure((size_t)nc * sizeof(int), "rows counts"));
+    // at w = 512 two CTAs of k_rows_layer read a cell's split operand, so the next one goes elsewhere
+    const bool ping = fused && w == 512;
+    if (ping)
+      for (Slot s : {WS_R_AH1, WS_R_ALO1}) ISX_TRY(ws[s].ensure(4 * cw / 2, "split A"));
+    for (Slot s : {WS_R_CNT0, WS_R_CNT1, WS_R_CNT2}) ISX_TRY(ws[s].ensure((size_t)nc * sizeof(int), "rows counts"));
     for (Slot s : {WS_R_OFF0, WS_R_OFF1}) ISX_TRY(ws[s].ensure((size_t)nc * sizeof(int64_t), "rows offsets"));
     float* C = ws[WS_C].as<float>();
     float* A = ws[WS_R_A].as<float>();
@@ -994,7 +1013,9 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
     float* I1 = ws[WS_R_I1].as<float>();
     __nv_bfloat16* AH = ws[WS_R_AH].as<__nv_bfloat16>();
     __nv_bfloat16* ALO = ws[WS_R_ALO].as<__nv_bfloat16>();
-    Slot xs[2] = {WS_X0, WS_X1}, cs[2] = {WS_R_CNT0, WS_R_CNT1}, os[2] = {WS_R_OFF0, WS_R_OFF1},
+    __nv_bfloat16* AH1 = ping ? ws[WS_R_AH1].as<__nv_bfloat16>() : AH;
+    __nv_bfloat16* ALO1 = ping ? ws[WS_R_ALO1].as<__nv_bfloat16>() : ALO;
+    Slot xs[2] = {WS_X0, WS_X1}, cs[3] = {WS_R_CNT0, WS_R_CNT1, WS_R_CNT2}, os[2] = {WS_R_OFF0, WS_R_OFF1},
          rs[2] = {WS_R_RC0, WS_R_RC1};
     int cur = 0;
     int64_t R = 0;
@@ -1007,16 +1028,18 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         fi.RAD = ws[WS_RAD].as<float>();
         fi.SLK = ws[WS_DELTA].as<float>();
       }
-      k_rows_input_act<<<act_blocks, 256, 0, st>>>(src, first, nc, w, (int)mode, inr->act, inr->W[0], inr->b[0], I0,
-                                                   A, AL, GA, ws[cs[1]].as<int>(), H > 1 ? AH : nullptr, ALO, fi);
+      k_rows_input_act<<<act_blocks, 256, 0, st>>>(src, first, nc, w, (int)mode, inr->act, inr->W[0], inr->b[0],
+                                                   H == 1 ? I0 : nullptr, H == 1 || inflate ? A : nullptr, AL, GA,
+                                                   ws[cs[1]].as<int>(), H > 1 ? AH : nullptr, ALO, fi);
       ISX_LAUNCH_CHECK("k_rows_input_act");
     }
     ISX_CUDA(cudaMemsetAsync(ws[cs[0]].ptr, 0, (size_t)nc * sizeof(int), st));
     ISX_CUDA(cudaMemsetAsync(ws[os[0]].ptr, 0, (size_t)nc * sizeof(int64_t), st));
     for (int j = 1; j <= H - 1; ++j) {
       const int nxt = cur ^ 1;
-      int* cnt_in = ws[cs[cur]].as<int>();
-      int* cnt_out = ws[cs[nxt]].as<int>();
+      int* cnt_in = ws[cs[0]].as<int>();             // rows of z_j, of z_{j+1} and (written here) of z_{j+2}
+      int* cnt_out = ws[cs[1]].as<int>();
+      int* cnt_next = ws[cs[2]].as<int>();
       int64_t* off_in = ws[os[cur]].as<int64_t>();
       int64_t* off_out = ws[os[nxt]].as<int64_t>();
       {
@@ -1055,17 +1078,46 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         prof::Scope ps(K_ROWS_NEW, st, 0, 2.0 * (double)(Rn - R) * w + 4.0 * (double)Rn + 8.0 * (double)nc * w);
         const unsigned nb = (unsigned)((nc + kNewWarps - 1) / kNewWarps);
         int* rc = ws[rs[nxt]].as<int>();
+        int* cz = fused && j < H - 1 ? cnt_next : nullptr;
         if (w == 512)
-          k_rows_new<16><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew);
+          k_rows_new<16><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
         else if (w == 256)
-          k_rows_new<8><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew);
+          k_rows_new<8><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
         else if (w == 128)
-          k_rows_new<4><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew);
+          k_rows_new<4><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
         else
-          k_rows_new<2><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew);
+          k_rows_new<2><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
         ISX_LAUNCH_CHECK("k_rows_new");
       }
-      {
+      if (fused) {
+        // centre, input rows, reduction and activation j + 1 in one kernel.  Bytes per cell: the column sums
+        // (one vector per 64-row input block the cell spans, and the new rows') and the split operand read
+        // (4 rows, two bf16 terms); alpha, gamma and the next split operand, or after the last layer
+        // the centre and the input rows, written
+        const bool last = j == H - 1;
+        rows::RowsLayerArgs la{};
+        la.nc = nc;
+        la.sq = sq;
+        la.act = inr->act;
+        la.bias = inr->b[j];
+        la.part = part;
+        la.pnew = pnew;
+        la.off_in = off_in;
+        la.cnt_in = cnt_in;
+        la.AL = AL;
+        la.GA = GA;
+        la.cnt_next = cnt_next;
+        la.AH = last ? nullptr : AH1;
+        la.ALO = last ? nullptr : ALO1;
+        la.A = A;
+        la.I = I0;
+        la.status = status;
+        const double vecs = (double)(nc + ntiles) + nc + 4.0 * nc + 2.0 * nc + 4.0 * nc;
+        prof::Scope ps(K_ROWS_SPLIT, st, 2.0 * nc * 4.0 * w * w, 4.0 * vecs * w);
+        ISX_TRY(rows::launch_rows_layer(inr, j, la, AH, ALO, st));
+        std::swap(AH, AH1);
+        std::swap(ALO, ALO1);
+      } else {
         RowsSplitArgs sa{};
         sa.nc = nc;
         sa.bias = inr->b[j];
@@ -1101,8 +1153,8 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         prof::Scope ps(K_ROWS_AUX, st, 2.0 * nc * w * w, 0);
         ISX_TRY(launch_rows_split_w<true>(inr, w, da, dm, st));
       }
-      {
-        // reductions of z_{j+1} and activation j+1; its row count goes to the buffer of X_j's counts.
+      if (!fused) {
+        // reductions of z_{j+1} and activation j+1; its row count goes to the next counts.
         // bytes per cell: the column sums (one vector per 64-row input block the cell spans, and
         // the new rows'), the three input rows and the centre read; a, alpha, gamma and the split
         // operand (4 rows, two bf16 terms) written
@@ -1110,7 +1162,7 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         const double vecs = (double)(nc + ntiles) + nc + 3.0 * nc + nc + 3.0 * nc + (last ? 0.0 : 4.0 * nc);
         prof::Scope ps(K_ROWS_REDUCE, st, 0, 4.0 * vecs * w);
         const unsigned rb = (unsigned)((nc + kRedWarps - 1) / kRedWarps);
-        int* cn = last ? nullptr : cnt_in;
+        int* cn = last ? nullptr : cnt_next;
         __nv_bfloat16* ah = last ? nullptr : AH;
         Infl fi = infl;
         if (inflate) {
@@ -1136,7 +1188,8 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
                                                                  cnt_out, I1, C, A, AL, GA, cn, ah, ALO, fi);
         ISX_LAUNCH_CHECK("k_rows_reduce_act");
       }
-      std::swap(I0, I1);
+      if (!fused) std::swap(I0, I1);
+      std::rotate(cs, cs + 1, cs + 3);
       cur = nxt;
       R = Rn;
     }
@@ -1151,7 +1204,7 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
       const unsigned ob = (unsigned)((nc + kOutWarps - 1) / kOutWarps);
       const __nv_bfloat16* Xl = ws[xs[cur]].as<__nv_bfloat16>();
       const int64_t* ol = ws[os[cur]].as<int64_t>();
-      const int* cl = ws[cs[cur]].as<int>();
+      const int* cl = ws[cs[0]].as<int>();
       const float* wl = inr->W[L];
       const float bl = inr->hb[L][0];
       if (w == 512)

@@ -969,14 +969,14 @@ EncodeTiledFn encode_fn() {
 isx_status make_scratch_map(CUtensorMap* m, const void* base, int w, int rows, int grid);
 
 isx_status make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint32_t box_inner,
-                    uint32_t box_outer) {
+                    uint32_t box_outer, uint64_t row_stride = 0) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) {
     set_error("cuTensorMapEncodeTiled is not available");
     return ISX_ERR_CUDA;
   }
   cuuint64_t dims[2] = {inner, outer};
-  cuuint64_t strides[1] = {inner * 2};
+  cuuint64_t strides[1] = {(row_stride ? row_stride : inner) * 2};
   cuuint32_t box[2] = {box_inner, box_outer};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
@@ -1078,8 +1078,8 @@ isx_status tc_net_of(isx_inr inr, const void** out) {
 size_t tc_net_bytes() { return sizeof(TcNet); }
 
 isx_status tensor_map_bf16(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint32_t box_inner,
-                           uint32_t box_outer) {
-  return make_map(m, base, inner, outer, box_inner, box_outer);
+                           uint32_t box_outer, uint64_t row_stride) {
+  return make_map(m, base, inner, outer, box_inner, box_outer, row_stride);
 }
 
 bool bf16_supported(isx_inr inr) { return (inr->w == 128 || inr->w == 256) && inr->H >= 2 && inr->H <= 12; }

@@ -55,7 +55,7 @@ enum Slot {
   WS_ANC_C_A, WS_ANC_C_B, WS_ANC_S_A, WS_ANC_S_B, WS_ANC_G_A, WS_ANC_G_B, WS_PROP_KEEP, WS_PROP_NEED,
   WS_PROP_IDX, WS_PROP_CODES,
   WS_R_I0, WS_R_I1, WS_R_A, WS_R_CNT0, WS_R_CNT1, WS_R_OFF0, WS_R_OFF1, WS_R_RC0, WS_R_RC1, WS_R_TOT, WS_R_AH, WS_R_ALO,
-  WS_R_PART, WS_R_PNEW, WS_R_V, WS_R_D,
+  WS_R_PART, WS_R_PNEW, WS_R_V, WS_R_D, WS_R_CNT2, WS_R_AH1, WS_R_ALO1,
   WS_N_SLOTS
 };
 
@@ -150,9 +150,9 @@ bool bf16_supported(isx_inr inr);
 // Device copy of the INR's network descriptor for the tensor-core bound kernel (built on first use).
 isx_status tc_net_of(isx_inr inr, const void** out);
 size_t tc_net_bytes();
-// 2-D bfloat16 tensor map [outer][inner] (row stride inner * 2 bytes), 128-byte swizzle.
+// 2-D bfloat16 tensor map [outer][inner], 128-byte swizzle; row_stride elements between rows (0: inner).
 isx_status tensor_map_bf16(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint32_t box_inner,
-                           uint32_t box_outer);
+                           uint32_t box_outer, uint64_t row_stride = 0);
 // MLP values at points on tcgen05 with two-term BF16 operands (eval_tc.cu); ISX_ERR_UNSUPPORTED for
 // widths other than 128 / 256.  Points as in eval_points_fp32.
 isx_status eval_points_tc(isx_inr inr, const float* xyz, const uint32_t* lattice_ids, int R, int64_t n,

@@ -13,7 +13,7 @@
 //    - beta^2, a = erf(-mu / (sqrt 2 sigma)).  Evaluated as Phi = P(X > 0) and Q = 1 - Phi: the smaller
 //  of the two from erfcf(|t| / sqrt 2) / 2 and the larger as its complement (so 1 - a^2 = 4 Phi Q has no
 //  cancellation), in units of sigma^2; gamma^2 is clamped at 0.
-//  sigma = 0 (or |mu| > 40 sigma): alpha = 1 if mu > 0, 1/2 if mu = 0, else 0; beta = gamma = 0.
+//  sigma = 0 (or |mu| > 15 sigma): alpha = 1 if mu > 0, 1/2 if mu = 0, else 0; beta = gamma = 0.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -27,9 +27,14 @@ struct Lin {
   float alpha, beta, gamma, center;
 };
 
+// Whether the kink matters in float32.  Beyond 15 sigma exp(-t^2 / 2) and erfc(|t| / sqrt 2) are below the
+// smallest float32 number (from |t| = 14.5 on), so the rule gives alpha = 1 or 0 and beta = gamma = 0.
+__device__ __forceinline__ bool relu_clt_mixed(float mu, float sigma) {
+  return sigma > 0.0f && fabsf(mu) < 15.0f * sigma;
+}
 __device__ __forceinline__ Lin relu_clt(float mu, float sigma) {
   Lin r;
-  if (sigma > 0.0f && fabsf(mu) < 40.0f * sigma) {
+  if (relu_clt_mixed(mu, sigma)) {
     float t = mu / sigma;
     // the smaller of Phi and Q from erfc of |t| (no cancellation), the other as its complement
     const float tail = 0.5f * erfcf(fabsf(t) * 0.70710678118654752f);

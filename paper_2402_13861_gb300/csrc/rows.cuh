@@ -68,6 +68,28 @@ __host__ __device__ __forceinline__ int rows_weight_row(int m, int w) {
 // cell + t.  Rows of a cell are contiguous, so cell c < c' implies t <= t' and the slots of all
 // (cell, block) pairs that share rows are distinct.
 __host__ __device__ __forceinline__ int64_t rows_part_slot(int64_t cell, int64_t t) { return cell + t; }
+struct RowsLayerArgs {
+  int64_t nc;
+  int sq, act;                                  // squares (UP) or absolute values; isx_activation
+  const float* bias;                            // [W] b_j
+  const float* part;                            // column sums of the row GEMM (RowsGemmArgs::part)
+  const float* pnew;                            // [nc][W] column sums of the new rows
+  const int64_t* off_in;                        // [nc] first symbol row of each cell before layer j, and how many
+  const int* cnt_in;
+  float* AL;                                    // [nc][W] alpha, gamma of activation j + 1
+  float* GA;
+  int* cnt_next;                                // [nc] += #(gamma != 0)
+  __nv_bfloat16* AH;                            // next split operand [4 nc][W], two terms; null after the last layer:
+  __nv_bfloat16* ALO;
+  float* A;                                     // [nc][W] centre and [nc][3][W] input rows instead
+  float* I;
+  int* status;
+};
+// Centre and input rows of layer `layer` from the split operand (AHin, ALOin), reduced and linearised into the
+// operands of the next layer (rows_layer.cu); w = 64, 128, 256 or 512.  The output split operand may be the
+// input one except at w = 512, where two CTAs share a cell.
+isx_status launch_rows_layer(isx_inr inr, int layer, const RowsLayerArgs& a, const __nv_bfloat16* AHin,
+                             const __nv_bfloat16* ALOin, cudaStream_t st);
 // Exclusive scan of nc per-cell row counts into int64 offsets; the total goes to d_tot[slot] (slot < 8).
 // d_tot: scan_bytes(nc) bytes, eight totals and the block sums.
 size_t scan_bytes(int64_t nc);

@@ -29,15 +29,17 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: 
 // G' = (G diag(alpha_cell)) W^T for all rows, computed transposed: D = W_j (G diag(alpha))^T, so that
 // TMEM lane m holds neuron rows_weight_row(m) and column r the tile's row r.  Persistent,
 // warp-specialised CTAs over 128-row tiles:
-//  - warp 5 streams the rows of G by TMA, one 64-wide K chunk of a tile per stage of an NS-stage
+//  - the producer warp streams the rows of G by TMA, one 64-wide K chunk of a tile per stage of an NS-stage
 //    ring, in the 128-byte-swizzled K-major layout of the MMA's B operand;
-//  - warps 0-3 scale each staged chunk in place: thread t multiplies row t by its cell's alpha
-//    (rows past R stay the TMA's zero fill);
-//  - warp 4 loads W_j (bf16, [MW][W], K-major) once by TMA, owns TMEM and issues the MMAs (M = 128
+//  - the scaler warps scale each staged chunk in place: two threads per row (w >= 256; else one) multiply its
+//    64 columns by its cell's alpha (rows past R stay the TMA's zero fill).  With one thread per row (four warps) the scaling
+//    set the pace: 821 us for 3.5 M rows (4.4 TB/s) at w = 256, against 711 us (5.1 TB/s) with two; without
+//    any scaling the kernel takes 632 us, without scaling and epilogue 361 us;
+//  - the MMA warp loads W_j (bf16, [MW][W], K-major) once by TMA, owns TMEM and issues the MMAs (M = 128
 //    per weight half, N = 128 rows, K = 16 per instruction).  W = 512 does not fit in shared memory:
 //    each CTA then holds a 128-row quarter of W_j, and a tile's four quarters go to four CTAs;
-//  - warps 6-13 drain the two TMEM accumulators, two warps per TMEM lane group: warps 6-9 take rows
-//    0-63 of a tile, warps 10-13 rows 64-127.  Thread m owns the neurons of weight row m of each
+//  - eight epilogue warps drain the two TMEM accumulators, two per TMEM lane group: the first four take
+//    rows 0-63 of a tile, the others rows 64-127.  Thread m owns the neurons of weight row m of each
 //    half and walks its 64 rows in order: it stores each row's bf16 value (a bf16 pair for
 //    W = 256) and adds f(value) to a running sum that it writes to part[cell + t] (t the 64-row
 //    block of the input rows) whenever the row's cell changes (|stored bf16 value| for the radius,
@@ -51,13 +53,16 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: 
 // as soon as they have handed over the current one.  Loads of tile k + 1 and the epilogue of tile k - 1 overlap
 // the MMAs of tile k.  Every wait is bounded (2 s): on timeout the kernel records ISX_ERR_TIMEOUT,
 // lets the work in flight finish, frees TMEM and returns.
-constexpr int kGT = 448;                        // 4 scalers, MMA, producer, 8 epilogue warps
+// Scaler warps: two threads per row of a chunk, or one where a tile has at most two chunks (w <= 128: there the
+// epilogue sets the pace and more warps only cost, 1.553 against 1.564 ms for an inflated bound).
+constexpr int scaler_warps(int W) { return W >= 256 ? 8 : 4; }
+constexpr int gemm_threads(int W) { return 32 * (scaler_warps(W) + 10); }   // scalers, MMA, producer, 8 epilogue warps
 template <int W, bool SQ>
-__global__ void __launch_bounds__(kGT, 1) k_rows_gemm(const __grid_constant__ RowsGemmArgs args,
+__global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_constant__ RowsGemmArgs args,
                                                        const __grid_constant__ CUtensorMap wmap,
                                                        const __grid_constant__ CUtensorMap xmap) {
   using S = RowsSmem<W>;
-  constexpr int KC = S::KC, NS = S::NS, MW = S::MW, NH = S::NH, NQ = S::NQ;
+  constexpr int KC = S::KC, NS = S::NS, MW = S::MW, NH = S::NH, NQ = S::NQ, kSW = scaler_warps(W);
   constexpr uint32_t kCols = 2 * NH * 128;                 // two accumulators of NH x 128 columns
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -91,7 +96,7 @@ __global__ void __launch_bounds__(kGT, 1) k_rows_gemm(const __grid_constant__ Ro
   if (t == 0) {
     for (int i = 0; i < NS; ++i) {
       mbar_init(&araw[i], 1);
-      mbar_init(&afull[i], kRT);
+      mbar_init(&afull[i], 32 * kSW);
       mbar_init(&aempty[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -102,7 +107,7 @@ __global__ void __launch_bounds__(kGT, 1) k_rows_gemm(const __grid_constant__ Ro
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 4) {
+  if (warp == kSW) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)),
                  "n"(kCols)
                  : "memory");
@@ -113,25 +118,27 @@ __global__ void __launch_bounds__(kGT, 1) k_rows_gemm(const __grid_constant__ Ro
   tc_fence_after();
   const uint32_t tmem = *tslot;
 
-  if (warp < 4) {
-    // ---- scale row t of every staged chunk by alpha of its cell, in place ----
+  if (warp < kSW) {
+    // ---- scale row sr of every staged chunk by alpha of its cell, in place: this thread's CG 8-column groups ----
+    constexpr int CG = 32 / kSW;
+    const int sr = t & (kRT - 1), k0 = (t / kRT) * 8 * CG;
     uint32_t it = 0;
     bool ok = true;
-    int64_t r_next = t0 * kRT + t;
+    int64_t r_next = t0 * kRT + sr;
     int cell_next = (r_next < args.R) ? args.rowcell[r_next] : 0;
-    float4 av[16];
+    float4 av[2 * CG];
     {
-      const float4* al0 = reinterpret_cast<const float4*>(args.alpha + (size_t)cell_next * W);
+      const float4* al0 = reinterpret_cast<const float4*>(args.alpha + (size_t)cell_next * W + k0);
 #pragma unroll
-      for (int g = 0; g < 16; ++g) av[g] = al0[g];
+      for (int g = 0; g < 2 * CG; ++g) av[g] = al0[g];
     }
     for (int64_t tile = t0; tile < ntiles && ok; tile += TS) {
-      const int64_t r = tile * kRT + t;
+      const int64_t r = tile * kRT + sr;
       const bool valid = r < args.R;
       const int cell = cell_next;
-      r_next = (tile + TS) * kRT + t;
+      r_next = (tile + TS) * kRT + sr;
       cell_next = (tile + TS < ntiles && r_next < args.R) ? args.rowcell[r_next] : cell;
-      {
+      if (warp < 4) {
         // ask L2 for the alpha rows of the cells of this warp's 32 rows of the next tile (a run of
         // consecutive cells, so one contiguous range), a tile ahead of their use
         const int cf = __shfl_sync(0xffffffffu, cell_next, 0), cl = __shfl_sync(0xffffffffu, cell_next, 31);
@@ -147,8 +154,8 @@ __global__ void __launch_bounds__(kGT, 1) k_rows_gemm(const __grid_constant__ Ro
         uint8_t* Ac = Asm + (size_t)sidx * S::kAC;
         if (valid) {
 #pragma unroll
-          for (int g = 0; g < 8; ++g) {
-            uint4* p = reinterpret_cast<uint4*>(Ac + roff(t, 8 * g));
+          for (int g = 0; g < CG; ++g) {
+            uint4* p = reinterpret_cast<uint4*>(Ac + roff(sr, k0 + 8 * g));
             const uint4 x = *p;
             const float4 a0 = av[2 * g], a1 = av[2 * g + 1];
             const __nv_bfloat162* xb = reinterpret_cast<const __nv_bfloat162*>(&x);
@@ -165,13 +172,13 @@ __global__ void __launch_bounds__(kGT, 1) k_rows_gemm(const __grid_constant__ Ro
         fence_async_shared();
         mbar_arrive(&afull[sidx]);
         // alpha of the next chunk (of this tile, or of the next tile), in flight during the next wait
-        const float4* aln = (c + 1 < KC) ? reinterpret_cast<const float4*>(args.alpha + (size_t)cell * W) + 16 * (c + 1)
-                                         : reinterpret_cast<const float4*>(args.alpha + (size_t)cell_next * W);
+        const float4* aln = (c + 1 < KC) ? reinterpret_cast<const float4*>(args.alpha + (size_t)cell * W + k0) + 16 * (c + 1)
+                                         : reinterpret_cast<const float4*>(args.alpha + (size_t)cell_next * W + k0);
 #pragma unroll
-        for (int g = 0; g < 16; ++g) av[g] = aln[g];
+        for (int g = 0; g < 2 * CG; ++g) av[g] = aln[g];
       }
     }
-  } else if (warp == 5) {
+  } else if (warp == kSW + 1) {
     // ---- TMA producer of the row chunks ----
     if (lane == 0) {
       uint32_t it = 0;
@@ -185,7 +192,7 @@ __global__ void __launch_bounds__(kGT, 1) k_rows_gemm(const __grid_constant__ Ro
         }
       }
     }
-  } else if (warp == 4) {
+  } else if (warp == kSW) {
     // ---- W_j once, then the MMAs: D[half h] += W_j[h rows] x chunk^T ----
     if (lane == 0) {
       // the CTA's weight rows: all of W_j, or rows q * 128 .. q * 128 + 127 of it
@@ -220,7 +227,7 @@ __global__ void __launch_bounds__(kGT, 1) k_rows_gemm(const __grid_constant__ Ro
   } else {
     // ---- epilogue: TMEM -> bf16 rows of G' and the per-(cell, 64-row block) column sums of f(G') ----
     const int m = 32 * (warp & 3) + lane;                  // weight row (TMEM lane) of this thread
-    const int h = (warp - 6) >> 2;                          // rows 64 h .. 64 h + 63 of every tile
+    const int h = (warp - kSW - 2) >> 2;                          // rows 64 h .. 64 h + 63 of every tile
     const bool own = m < W;                                 // W = 64: rows 64 .. 127 are padding
     const int n0 = (W == 256) ? 2 * m : q * 128 + m;        // first neuron of this thread
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
@@ -337,7 +344,7 @@ __global__ void __launch_bounds__(kGT, 1) k_rows_gemm(const __grid_constant__ Ro
   __syncthreads();
   if (*abort)
     for (int i = 0; i < 1000; ++i) __nanosleep(1000);
-  if (warp == 4) {
+  if (warp == kSW) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kCols) : "memory");
   }
@@ -352,13 +359,13 @@ isx_status launch_rows_gemm_w(isx_inr inr, const RowsGemmArgs& a, const CUtensor
   int sms = 148;
   ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
   int per_sm = 1;
-  ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rows_gemm<W, SQ>, kGT, smem));
+  ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rows_gemm<W, SQ>, gemm_threads(W), smem));
   per_sm = std::max(1, std::min(per_sm, 512 / (2 * RowsSmem<W>::NH * 128)));   // TMEM columns per CTA
   constexpr int NQ = RowsSmem<W>::NQ;
   const int64_t ntiles = (a.R + kRT - 1) / kRT;
   int grid = (int)std::min<int64_t>(ntiles * NQ, (int64_t)sms * per_sm);
   grid -= grid % NQ;                                       // every CTA keeps one weight slice
-  k_rows_gemm<W, SQ><<<grid, kGT, smem, st>>>(a, map, xmap);
+  k_rows_gemm<W, SQ><<<grid, gemm_threads(W), smem, st>>>(a, map, xmap);
   ISX_LAUNCH_CHECK("k_rows_gemm");
   return ISX_OK;
 }

@@ -252,10 +252,13 @@ __global__ void __launch_bounds__(kScanB) k_rows_scan_one(const int* cnt, int64_
 
 // ---- new rows gamma_n W_j[:, n] (row n of W_j^T) after each cell's transformed rows, in
 //      increasing n; the row -> cell map of the whole output; and, per cell and column, the sum of
-//      f(x) over the cell's new rows (x = the stored bf16 value; f = x^2 or |x|).  One warp per cell:
-//      the neurons with gamma != 0 come from ballots, and each row goes out as one warp-wide store
-//      (w / 32 columns per lane, whose sums the lane keeps in registers). ----
-constexpr int kNewWarps = 8;
+//      f(x) over the cell's new rows (x = the stored bf16 value; f = x^2 or |x|).  One warp per CB
+//      consecutive cells, w / 32 columns per lane: the neurons with gamma != 0 come from ballots, and each row
+//      goes out as one warp-wide store.  Bound by the L1 data path (a float32 row of W_j read per bf16 row
+//      written), so a row of W_j is read once for all of the warp's cells that need it: siblings of one
+//      octree parent share most of their symbols (512^3 extraction: 201 -> 147 ms with four cells per warp
+//      instead of one, 6.5 TB/s; unrelated cells, 262144 at w = 256: 3.16 -> 3.01 ms). ----
+constexpr int kNewWarps = 4;
 template <int CPL>
 struct NewRowIO;
 template <>
@@ -300,7 +303,7 @@ struct NewRowIO<2> {
   }
   static __device__ __forceinline__ void st(__nv_bfloat16* p, const uint32_t* h) { *reinterpret_cast<uint32_t*>(p) = h[0]; }
 };
-template <int CPL>
+template <int CPL, int CB>
 __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, const float* __restrict__ GA,
                                                              const float* __restrict__ Wt, const int* cnt_in,
                                                              const int64_t* off_out, const int* cnt_out,
@@ -308,70 +311,83 @@ __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, con
                                                              int* cnt_next) {
   constexpr int w = 32 * CPL;
   using IO = NewRowIO<CPL>;
-  const int lane = threadIdx.x & 31;
-  const int cell = blockIdx.x * kNewWarps + (threadIdx.x >> 5);
-  if (cell >= nc) return;
-  const int64_t o0 = off_out[cell];
-  const int co = cnt_out[cell];
-  if (cnt_next && lane == 0) cnt_next[cell] = co;  // k_rows_layer adds the next activation's symbols
-  for (int r = lane; r < co; r += 32) rowcell_out[o0 + r] = cell;
+  __shared__ float sgam[kNewWarps][CB][w];
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+  const int cell0 = (blockIdx.x * kNewWarps + wi) * CB;
+  if (cell0 >= nc) return;
   const int m0 = lane * CPL;                       // this lane's columns m0 .. m0 + CPL - 1
-  float acc[CPL];
+  // gamma of the warp's cells, all loads in flight
 #pragma unroll
-  for (int c = 0; c < CPL; ++c) acc[c] = 0.0f;
-  int64_t row = o0 + cnt_in[cell];
-  // one new row: x = bf16(gamma_n W_j[m, n]) for this lane's columns m, stored with one vector store
-  auto emit = [&](float g, const float* v) {
-    uint32_t h[CPL / 2];
+  for (int c = 0; c < CB; ++c)
 #pragma unroll
-    for (int c = 0; c < CPL; c += 2) {
-      const __nv_bfloat162 x = __floats2bfloat162_rn(g * v[c], g * v[c + 1]);
-      h[c / 2] = *reinterpret_cast<const uint32_t*>(&x);
-      const float2 f = __bfloat1622float2(x);
-      acc[c] += sq ? f.x * f.x : fabsf(f.x);
-      acc[c + 1] += sq ? f.y * f.y : fabsf(f.y);
+    for (int g = 0; g < CPL; ++g)
+      sgam[wi][c][32 * g + lane] = cell0 + c < nc ? GA[(size_t)(cell0 + c) * w + 32 * g + lane] : 0.0f;
+  __nv_bfloat16* xp[CB];                           // this lane's columns of each cell's next new row
+  float acc[CB][CPL];
+#pragma unroll
+  for (int c = 0; c < CB; ++c) {
+    const int cell = cell0 + c;
+    xp[c] = xout;
+#pragma unroll
+    for (int i = 0; i < CPL; ++i) acc[c][i] = 0.0f;
+    if (cell < nc) {
+      const int64_t o0 = off_out[cell];
+      const int co = cnt_out[cell];
+      xp[c] += (size_t)(o0 + cnt_in[cell]) * w + m0;
+      if (cnt_next && lane == 0) cnt_next[cell] = co;  // k_rows_layer adds the next activation's symbols
+      for (int r = lane; r < co; r += 32) rowcell_out[o0 + r] = cell;
     }
-    IO::st(xout + row * w + m0, h);
-    ++row;
-  };
-  // gamma of all w neurons, loaded together into shared memory with one ballot mask per 32; then,
-  // group by group, the new rows in increasing neuron order, NF rows' weight loads in flight (the
-  // group loop is not unrolled: one copy of the row code keeps the kernel small)
-  constexpr int NF = CPL >= 16 ? 2 : 4;
-  __shared__ float sgam[kNewWarps][w];
-  __shared__ unsigned smask[kNewWarps][CPL];
-  const int wi = threadIdx.x >> 5;
-#pragma unroll
-  for (int g = 0; g < CPL; ++g) {
-    const float x = GA[(size_t)cell * w + 32 * g + lane];
-    sgam[wi][32 * g + lane] = x;
-    const unsigned bm = __ballot_sync(0xffffffffu, x != 0.0f);
-    if (lane == 0) smask[wi][g] = bm;
   }
   __syncwarp();
+  constexpr int NF = 2;                            // weight rows in flight
 #pragma unroll 1
   for (int g = 0; g < CPL; ++g) {
-    unsigned b = smask[wi][g];
-    while (b) {
+    unsigned bm[CB], any = 0;
+#pragma unroll
+    for (int c = 0; c < CB; ++c) {
+      bm[c] = __ballot_sync(0xffffffffu, sgam[wi][c][32 * g + lane] != 0.0f);
+      any |= bm[c];
+    }
+#pragma unroll 1
+    while (any) {
       int l[NF];
+      float v[NF][CPL];
 #pragma unroll
       for (int q = 0; q < NF; ++q) {
-        l[q] = b ? __ffs(b) - 1 : -1;
-        b &= b - 1;
-      }
-      float gg[NF], v[NF][CPL];
-#pragma unroll
-      for (int q = 0; q < NF; ++q) {
-        gg[q] = l[q] >= 0 ? sgam[wi][32 * g + l[q]] : 0.0f;
+        l[q] = any ? __ffs(any) - 1 : -1;
+        any &= any - 1;
         if (l[q] >= 0) IO::ld(Wt + (size_t)(32 * g + l[q]) * w + m0, v[q]);
       }
 #pragma unroll
-      for (int q = 0; q < NF; ++q)
-        if (l[q] >= 0) emit(gg[q], v[q]);
+      for (int q = 0; q < NF; ++q) {
+        if (l[q] < 0) break;
+#pragma unroll
+        for (int c = 0; c < CB; ++c) {
+          if (!((bm[c] >> l[q]) & 1u)) continue;   // uniform
+          // one new row: x = bf16(gamma_n W_j[m, n]) for this lane's columns m
+          const float gm = sgam[wi][c][32 * g + l[q]];
+          uint32_t h[CPL / 2];
+#pragma unroll
+          for (int i = 0; i < CPL; i += 2) {
+            const __nv_bfloat162 x = __floats2bfloat162_rn(gm * v[q][i], gm * v[q][i + 1]);
+            h[i / 2] = *reinterpret_cast<const uint32_t*>(&x);
+            const float2 f = __bfloat1622float2(x);
+            acc[c][i] += sq ? f.x * f.x : fabsf(f.x);
+            acc[c][i + 1] += sq ? f.y * f.y : fabsf(f.y);
+          }
+          IO::st(xp[c], h);
+          xp[c] += w;
+        }
+      }
     }
   }
 #pragma unroll
-  for (int c = 0; c < CPL; ++c) pnew[(size_t)cell * w + m0 + c] = acc[c];
+  for (int c = 0; c < CB; ++c)
+    if (cell0 + c < nc) {
+      float* d = pnew + (size_t)(cell0 + c) * w + m0;
+#pragma unroll
+      for (int i = 0; i < CPL; i += 2) *reinterpret_cast<float2*>(d + i) = make_float2(acc[c][i], acc[c][i + 1]);
+    }
 }
 
 // ---- c' = W_j a + b_j for every cell of a chunk in float32 on the CUDA cores (sound mode with
@@ -1076,17 +1092,22 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
       {
         // bytes: the new rows (bf16) and the row -> cell map written, gamma read, the column sums
         prof::Scope ps(K_ROWS_NEW, st, 0, 2.0 * (double)(Rn - R) * w + 4.0 * (double)Rn + 8.0 * (double)nc * w);
-        const unsigned nb = (unsigned)((nc + kNewWarps - 1) / kNewWarps);
         int* rc = ws[rs[nxt]].as<int>();
         int* cz = fused && j < H - 1 ? cnt_next : nullptr;
-        if (w == 512)
-          k_rows_new<16><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
-        else if (w == 256)
-          k_rows_new<8><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
-        else if (w == 128)
-          k_rows_new<4><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
-        else
-          k_rows_new<2><<<nb, 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
+        auto launch_new = [&](auto kernel, int cells) {
+          kernel<<<(unsigned)((nc + cells - 1) / cells), 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out,
+                                                                                  cnt_out, Xout, rc, pnew, cz);
+        };
+        // several cells per warp once there are enough cells to fill the SMs all the same
+        const bool many = nc >= 32 * sms;
+        if (w == 512 && many) launch_new(k_rows_new<16, 2>, 2 * kNewWarps);
+        else if (w == 512) launch_new(k_rows_new<16, 1>, kNewWarps);
+        else if (w == 256 && many) launch_new(k_rows_new<8, 4>, 4 * kNewWarps);
+        else if (w == 256) launch_new(k_rows_new<8, 1>, kNewWarps);
+        else if (w == 128 && many) launch_new(k_rows_new<4, 4>, 4 * kNewWarps);
+        else if (w == 128) launch_new(k_rows_new<4, 1>, kNewWarps);
+        else if (many) launch_new(k_rows_new<2, 4>, 4 * kNewWarps);
+        else launch_new(k_rows_new<2, 1>, kNewWarps);
         ISX_LAUNCH_CHECK("k_rows_new");
       }
       if (fused) {

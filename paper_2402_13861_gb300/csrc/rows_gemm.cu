@@ -31,7 +31,7 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: 
 // warp-specialised CTAs over 128-row tiles:
 //  - the producer warp streams the rows of G by TMA, one 64-wide K chunk of a tile per stage of an NS-stage
 //    ring, in the 128-byte-swizzled K-major layout of the MMA's B operand;
-//  - the scaler warps scale each staged chunk in place: two threads per row (w >= 256; else one) multiply its
+//  - the scaler warps scale each staged chunk in place: one, two or four threads per row multiply its
 //    64 columns by its cell's alpha (rows past R stay the TMA's zero fill).  With one thread per row (four warps) the scaling
 //    set the pace: 821 us for 3.5 M rows (4.4 TB/s) at w = 256, against 711 us (5.1 TB/s) with two; without
 //    any scaling the kernel takes 632 us, without scaling and epilogue 361 us;
@@ -53,9 +53,11 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: 
 // as soon as they have handed over the current one.  Loads of tile k + 1 and the epilogue of tile k - 1 overlap
 // the MMAs of tile k.  Every wait is bounded (2 s): on timeout the kernel records ISX_ERR_TIMEOUT,
 // lets the work in flight finish, frees TMEM and returns.
-// Scaler warps: two threads per row of a chunk, or one where a tile has at most two chunks (w <= 128: there the
+// Scaler warps: two threads per row of a chunk at w = 256; four at w = 512, whose CTAs each scale every row for a
+// quarter of the neurons (12007 cells of the 3 -> 512 x 8 -> 1 network: 3.50 ms with one thread per row, 2.75
+// with two, 2.47 with four; at w = 256 four threads per row would leave the epilogue too few registers); one where a tile has at most two chunks (w <= 128: there the
 // epilogue sets the pace and more warps only cost, 1.553 against 1.564 ms for an inflated bound).
-constexpr int scaler_warps(int W) { return W >= 256 ? 8 : 4; }
+constexpr int scaler_warps(int W) { return W > 256 ? 16 : (W == 256 ? 8 : 4); }
 constexpr int gemm_threads(int W) { return 32 * (scaler_warps(W) + 10); }   // scalers, MMA, producer, 8 epilogue warps
 template <int W, bool SQ>
 __global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_constant__ RowsGemmArgs args,

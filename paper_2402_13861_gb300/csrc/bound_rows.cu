@@ -272,20 +272,6 @@ struct NewRowIO<8> {
   }
 };
 template <>
-struct NewRowIO<16> {
-  static __device__ __forceinline__ void ld(const float* p, float* v) {
-#pragma unroll
-    for (int i = 0; i < 16; i += 4) {
-      const float4 a = *reinterpret_cast<const float4*>(p + i);
-      v[i] = a.x; v[i + 1] = a.y; v[i + 2] = a.z; v[i + 3] = a.w;
-    }
-  }
-  static __device__ __forceinline__ void st(__nv_bfloat16* p, const uint32_t* h) {
-    *reinterpret_cast<uint4*>(p) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(p + 8) = make_uint4(h[4], h[5], h[6], h[7]);
-  }
-};
-template <>
 struct NewRowIO<4> {
   static __device__ __forceinline__ void ld(const float* p, float* v) {
     const float4 a = *reinterpret_cast<const float4*>(p);
@@ -303,24 +289,25 @@ struct NewRowIO<2> {
   }
   static __device__ __forceinline__ void st(__nv_bfloat16* p, const uint32_t* h) { *reinterpret_cast<uint32_t*>(p) = h[0]; }
 };
-template <int CPL, int CB>
+template <int w, int CPL, int CB, int NF>
 __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, const float* __restrict__ GA,
                                                              const float* __restrict__ Wt, const int* cnt_in,
                                                              const int64_t* off_out, const int* cnt_out,
                                                              __nv_bfloat16* xout, int* rowcell_out, float* pnew,
                                                              int* cnt_next) {
-  constexpr int w = 32 * CPL;
+  constexpr int CS = w / (32 * CPL), G = w / 32;   // warps per cell group, 32-neuron groups
   using IO = NewRowIO<CPL>;
   __shared__ float sgam[kNewWarps][CB][w];
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-  const int cell0 = (blockIdx.x * kNewWarps + wi) * CB;
+  const int unit = blockIdx.x * kNewWarps + wi, cs = unit % CS;
+  const int cell0 = unit / CS * CB;
   if (cell0 >= nc) return;
-  const int m0 = lane * CPL;                       // this lane's columns m0 .. m0 + CPL - 1
+  const int m0 = (cs * 32 + lane) * CPL;           // this lane's columns m0 .. m0 + CPL - 1
   // gamma of the warp's cells, all loads in flight
 #pragma unroll
   for (int c = 0; c < CB; ++c)
 #pragma unroll
-    for (int g = 0; g < CPL; ++g)
+    for (int g = 0; g < G; ++g)
       sgam[wi][c][32 * g + lane] = cell0 + c < nc ? GA[(size_t)(cell0 + c) * w + 32 * g + lane] : 0.0f;
   __nv_bfloat16* xp[CB];                           // this lane's columns of each cell's next new row
   float acc[CB][CPL];
@@ -334,14 +321,13 @@ __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, con
       const int64_t o0 = off_out[cell];
       const int co = cnt_out[cell];
       xp[c] += (size_t)(o0 + cnt_in[cell]) * w + m0;
-      if (cnt_next && lane == 0) cnt_next[cell] = co;  // k_rows_layer adds the next activation's symbols
-      for (int r = lane; r < co; r += 32) rowcell_out[o0 + r] = cell;
+      if (cnt_next && cs == 0 && lane == 0) cnt_next[cell] = co;  // k_rows_layer adds the next activation's symbols
+      for (int r = cs * 32 + lane; r < co; r += 32 * CS) rowcell_out[o0 + r] = cell;
     }
   }
   __syncwarp();
-  constexpr int NF = 2;                            // weight rows in flight
 #pragma unroll 1
-  for (int g = 0; g < CPL; ++g) {
+  for (int g = 0; g < G; ++g) {
     unsigned bm[CB], any = 0;
 #pragma unroll
     for (int c = 0; c < CB; ++c) {
@@ -350,7 +336,7 @@ __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, con
     }
 #pragma unroll 1
     while (any) {
-      int l[NF];
+      int l[NF];                                   // NF weight rows in flight
       float v[NF][CPL];
 #pragma unroll
       for (int q = 0; q < NF; ++q) {
@@ -754,9 +740,10 @@ __global__ void __launch_bounds__(32 * kRedWarps) k_rows_reduce_act(int nc, int 
 // S the number of symbols: each y_i = row_i . (alpha o w) errs by gamma_{w+1} sum_n |x_in| |alpha_n w_n|
 // (summed over i: RAD_n bounds sum_i |x_in|), the centre's dot product by gamma_{w+1} of its terms, the
 // last activation's symbols gamma_n w_n by one rounding, and the slack alpha d passes through |w|.
-// One warp per cell, CPL = w / 32 consecutive neurons per lane (the vector v = alpha o w_out stays in
+// WPC warps per cell, CPL = w / 32 consecutive neurons per lane (the vector v = alpha o w_out stays in
 // registers); each row is one vector load per lane, four rows' loads in flight, and its dot product
-// is reduced across the warp before |y| or y^2 is taken.
+// is reduced across the warp before |y| or y^2 is taken.  The terms are added in row order whatever WPC: with
+// WPC > 1 the warps leave the rows' dot products in shared memory, 64 rows at a time, for the first one.
 constexpr int kOutWarps = 8;
 template <int CPL>
 __device__ __forceinline__ void ld_row(const __nv_bfloat16* p, float* f) {
@@ -780,7 +767,8 @@ __device__ __forceinline__ void ld_row(const __nv_bfloat16* p, float* f) {
     f[2 * i + 1] = x.y;
   }
 }
-template <int CPL>
+constexpr int kOutRows = 64;                     // rows of one hand-over (WPC > 1)
+template <int CPL, int WPC>
 __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode, const __nv_bfloat16* X,
                                                                 const int64_t* off, const int* cnt, const float* I,
                                                                 const float* A, const float* AL, const float* GA,
@@ -788,9 +776,9 @@ __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode
                                                                 int64_t first, float* center, float* spread,
                                                                 Infl infl) {
   constexpr int w = 32 * CPL;
-  const int lane = threadIdx.x & 31;
-  const int cell = blockIdx.x * kOutWarps + (threadIdx.x >> 5);
-  if (cell >= nc) return;
+  const int lane = threadIdx.x & 31, sub = (threadIdx.x >> 5) / WPC, u = (threadIdx.x >> 5) % WPC;
+  const int cell = blockIdx.x * (kOutWarps / WPC) + sub;
+  if (cell >= nc) return;                          // the cell's warps alone meet at its barrier
   const bool sq = mode != ISX_BOUND_SOUND;
   const int m0 = lane * CPL;
   const size_t o = (size_t)cell * w + m0;
@@ -850,29 +838,51 @@ __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode
   }
   // the stored symbol rows (bf16), four at a time
   const __nv_bfloat16* xp = X + o0 * w + m0;
-  int r = 0;
-  for (; r + 4 <= rows; r += 4) {
-    float y[4];
+  auto four = [&](int r, float* y) {               // dot products of rows r .. r + 3 (< rows)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       float x[CPL];
-      ld_row<CPL>(xp + (size_t)(r + q) * w, x);
+      ld_row<CPL>(xp + (size_t)min(r + q, rows - 1) * w, x);
       y[q] = dot(x);
     }
 #pragma unroll
     for (int sh = 16; sh > 0; sh >>= 1)
 #pragma unroll
       for (int q = 0; q < 4; ++q) y[q] += __shfl_xor_sync(0xffffffffu, y[q], sh);
+  };
+  // one rounding per square in whole groups of four rows, two in the rest (fixed, so that no launch shape or
+  // compiler choice changes a result)
+  const int whole = rows & ~3;
+  auto term = [&](int r, float y, float a) {
+    return !sq ? a + fabsf(y) : (r < whole ? fmaf(y, y, a) : __fadd_rn(a, __fmul_rn(y, y)));
+  };
+  if constexpr (WPC == 1) {
+    for (int r = 0; r < rows; r += 4) {
+      float y[4];
+      four(r, y);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) sr += sq ? y[q] * y[q] : fabsf(y[q]);
-  }
-  for (; r < rows; ++r) {
-    float x[CPL];
-    ld_row<CPL>(xp + (size_t)r * w, x);
-    float y = dot(x);
-#pragma unroll
-    for (int sh = 16; sh > 0; sh >>= 1) y += __shfl_xor_sync(0xffffffffu, y, sh);
-    sr += sq ? y * y : fabsf(y);
+      for (int q = 0; q < 4; ++q)
+        if (r + q < rows) sr = term(r + q, y[q], sr);
+    }
+  } else {
+    __shared__ float sy[kOutWarps / WPC][2][kOutRows];
+    int h = 0;
+    for (int r0 = 0; r0 < rows; r0 += kOutRows, h ^= 1) {
+      for (int r = 4 * u; r < kOutRows && r0 + r < rows; r += 4 * WPC) {
+        float y[4];
+        four(r0 + r, y);
+        if (lane < 4) sy[sub][h][r + lane] = lane == 0 ? y[0] : (lane == 1 ? y[1] : (lane == 2 ? y[2] : y[3]));
+      }
+      asm volatile("bar.sync %0, %1;" ::"r"(sub + 1), "n"(32 * WPC) : "memory");
+      if (u == 0) {
+        const int m = min(kOutRows, rows - r0);
+        for (int q = 0; q < m; ++q) {
+          const float y = sy[sub][h][q];
+          sr = term(r0 + q, y, sr);
+        }
+      }
+    }
+    if (u > 0) return;
   }
 #pragma unroll
   for (int sh = 16; sh > 0; sh >>= 1) {
@@ -1094,20 +1104,24 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         prof::Scope ps(K_ROWS_NEW, st, 0, 2.0 * (double)(Rn - R) * w + 4.0 * (double)Rn + 8.0 * (double)nc * w);
         int* rc = ws[rs[nxt]].as<int>();
         int* cz = fused && j < H - 1 ? cnt_next : nullptr;
-        auto launch_new = [&](auto kernel, int cells) {
-          kernel<<<(unsigned)((nc + cells - 1) / cells), 32 * kNewWarps, 0, st>>>(nc, sq, GA, inr->Wt[j], cnt_in, off_out,
-                                                                                  cnt_out, Xout, rc, pnew, cz);
+        // warps of 1, 2 or 4 cells with w / 32 columns per lane; w = 512: two warps share the columns, and four
+        // weight rows are in flight where a warp has few cells, since a launch lasts as long as its cell with
+        // the most new rows (12007 cells of the 3 -> 512 x 8 -> 1 network: 1.80 -> 1.15 ms)
+        auto launch_new = [&](auto kernel, int cells, int split) {
+          const int64_t warps = ((int64_t)nc + cells - 1) / cells * split;
+          kernel<<<(unsigned)((warps + kNewWarps - 1) / kNewWarps), 32 * kNewWarps, 0, st>>>(
+              nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
         };
         // several cells per warp once there are enough cells to fill the SMs all the same
         const bool many = nc >= 32 * sms;
-        if (w == 512 && many) launch_new(k_rows_new<16, 2>, 2 * kNewWarps);
-        else if (w == 512) launch_new(k_rows_new<16, 1>, kNewWarps);
-        else if (w == 256 && many) launch_new(k_rows_new<8, 4>, 4 * kNewWarps);
-        else if (w == 256) launch_new(k_rows_new<8, 1>, kNewWarps);
-        else if (w == 128 && many) launch_new(k_rows_new<4, 4>, 4 * kNewWarps);
-        else if (w == 128) launch_new(k_rows_new<4, 1>, kNewWarps);
-        else if (many) launch_new(k_rows_new<2, 4>, 4 * kNewWarps);
-        else launch_new(k_rows_new<2, 1>, kNewWarps);
+        if (w == 512 && many) launch_new(k_rows_new<512, 8, 2, 4>, 2, 2);
+        else if (w == 512) launch_new(k_rows_new<512, 8, 1, 4>, 1, 2);
+        else if (w == 256 && many) launch_new(k_rows_new<256, 8, 4, 2>, 4, 1);
+        else if (w == 256) launch_new(k_rows_new<256, 8, 1, 4>, 1, 1);
+        else if (w == 128 && many) launch_new(k_rows_new<128, 4, 4, 2>, 4, 1);
+        else if (w == 128) launch_new(k_rows_new<128, 4, 1, 4>, 1, 1);
+        else if (many) launch_new(k_rows_new<64, 2, 4, 2>, 4, 1);
+        else launch_new(k_rows_new<64, 2, 1, 4>, 1, 1);
         ISX_LAUNCH_CHECK("k_rows_new");
       }
       if (fused) {
@@ -1222,24 +1236,26 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         fi.RAD = ws[WS_RAD].as<float>();
         fi.SLK = ws[WS_DELTA].as<float>();
       }
-      const unsigned ob = (unsigned)((nc + kOutWarps - 1) / kOutWarps);
       const __nv_bfloat16* Xl = ws[xs[cur]].as<__nv_bfloat16>();
       const int64_t* ol = ws[os[cur]].as<int64_t>();
       const int* cl = ws[cs[0]].as<int>();
       const float* wl = inr->W[L];
       const float bl = inr->hb[L][0];
-      if (w == 512)
-        k_rows_output<16><<<ob, 32 * kOutWarps, 0, st>>>(nc, (int)mode, Xl, ol, cl, I0, A, AL, GA, wl, bl, first,
-                                                         d_center, d_spread, fi);
-      else if (w == 256)
-        k_rows_output<8><<<ob, 32 * kOutWarps, 0, st>>>(nc, (int)mode, Xl, ol, cl, I0, A, AL, GA, wl, bl, first,
-                                                        d_center, d_spread, fi);
-      else if (w == 128)
-        k_rows_output<4><<<ob, 32 * kOutWarps, 0, st>>>(nc, (int)mode, Xl, ol, cl, I0, A, AL, GA, wl, bl, first,
-                                                        d_center, d_spread, fi);
-      else
-        k_rows_output<2><<<ob, 32 * kOutWarps, 0, st>>>(nc, (int)mode, Xl, ol, cl, I0, A, AL, GA, wl, bl, first,
-                                                        d_center, d_spread, fi);
+      auto launch_out = [&](auto kernel, int cells) {
+        kernel<<<(unsigned)((nc + cells - 1) / cells), 32 * kOutWarps, 0, st>>>(nc, (int)mode, Xl, ol, cl, I0, A, AL, GA, wl,
+                                                                                bl, first, d_center, d_spread, fi);
+      };
+      // four warps per cell until single warps fill every SM several times over: a chunk lasts as long as its
+      // cell with the most rows (12007 cells of the 3 -> 512 x 8 -> 1 network: 1.14 -> 0.62 ms)
+      const bool many = nc >= 128 * sms;
+      if (w == 512 && many) launch_out(k_rows_output<16, 1>, kOutWarps);
+      else if (w == 512) launch_out(k_rows_output<16, 4>, kOutWarps / 4);
+      else if (w == 256 && many) launch_out(k_rows_output<8, 1>, kOutWarps);
+      else if (w == 256) launch_out(k_rows_output<8, 4>, kOutWarps / 4);
+      else if (w == 128 && many) launch_out(k_rows_output<4, 1>, kOutWarps);
+      else if (w == 128) launch_out(k_rows_output<4, 4>, kOutWarps / 4);
+      else if (many) launch_out(k_rows_output<2, 1>, kOutWarps);
+      else launch_out(k_rows_output<2, 4>, kOutWarps / 4);
       ISX_LAUNCH_CHECK("k_rows_output");
     }
     rows_per_cell = std::max(1.0, (double)R / nc);

@@ -7,14 +7,24 @@
 // Three tcgen05.mma (kind::f16, BF16 x BF16 -> FP32 in TMEM) per K step, so the tensor cores do 3x
 // the algorithmic work, against 1/28 of their BF16 rate for FP32 FMAs on the CUDA cores.
 //
-// Layout: one CTA (one warpgroup, 128 threads) per 128-point tile, persistent over tiles.  Thread
-// t owns point t of the tile = TMEM lane t.  Layer 0 (3 -> w) runs in FP32 on the CUDA cores; its
-// activation output is split into A_hi, A_lo in shared memory (K-major, 128-byte swizzle).  Each
-// hidden layer W_l (w x w) streams through two 32 KB stages (X: W_hi chunk, Y: W_lo chunk; one
-// 64-wide K chunk each) loaded by TMA; thread 0 issues the MMAs into one w-column FP32 accumulator.
-// The epilogue reads TMEM, adds the bias, applies the activation (ReLU, ELU or sine) and writes the
-// next A_hi, A_lo; after the last hidden layer it contracts with w_out in FP32 instead.  Every wait is bounded (2 s): on timeout
-// the kernel records ISX_ERR_TIMEOUT, lets copies land, frees TMEM and returns.
+// Layout: one persistent CTA per 128-point tile at a time; point p of the tile = TMEM lane p.  Bound by the
+// tensor cores (three products), so everything else is kept off their path:
+//  - a producer warp streams W_l through a ring of 16 KB stages (128 weight rows x one 64-wide K chunk, high
+//    or low term) by TMA, ahead of the MMAs and across layers and tiles;
+//  - an MMA warp starts a K chunk as soon as its 64 activations per point are in shared memory (one mbarrier
+//    per chunk), into one of two accumulators;
+//  - four groups of four epilogue warps (two at w = 128) read the accumulator of the layer before, each group a
+//    quarter of every chunk's columns: bias, activation (ReLU, ELU or sine), split into A_hi, A_lo (K-major,
+//    128-byte swizzle), chunk by chunk, so the next layer's MMAs begin after a quarter of the work;
+//  - layer 0 (3 -> w, FP32 CUDA cores) of the next tile runs before the output layer of this one, whose
+//    contraction with w_out (FP32, one chain over the neurons per point, handed from group to group) so
+//    overlaps the next tile's first MMAs.
+// With one 128-thread warpgroup that issued, waited and drained in turn 2.1 M points of 3 -> 256 x 5 -> 1 took
+// 3.62 ms; this form takes 2.42 ms: of 11.2 k cycles per layer the MMAs take 6.1 k, 3.3 k go by waiting for
+// weights and 1.8 k until the first chunk of the next layer's operand is ready.  Halving the L2 reads with clusters
+// of two CTAs that multicast the weights to each other changes nothing: the 80 KB of the ring, all that
+// fits, cover too little of the load latency.  Every wait is bounded (2 s): on timeout the kernel records
+// ISX_ERR_TIMEOUT, lets copies land, frees TMEM and returns.
 #include "internal.cuh"
 #include "tc_ptx.cuh"
 #include "linearise.cuh"
@@ -27,9 +37,8 @@ namespace {
 
 using namespace tc;
 
-constexpr int kT = 128;                        // points per tile = threads per CTA
+constexpr int kT = 128;                        // points per tile
 constexpr uint64_t kEvWaitNs = 2000000000ull;
-enum { EB_XFULL, EB_XEMPTY, EB_YFULL, EB_YEMPTY, EB_DONE, EB_COUNT };
 
 struct EvArgs {
   const float* xyz;
@@ -43,21 +52,30 @@ struct EvArgs {
   const float* wout;                           // [w]
   float bout;
   int act;                             // isx_activation of the hidden layers
+  int ns;                              // weight stages
   int* status;
 };
 struct EvMaps {
-  CUtensorMap hi[ISX_MAX_LAYERS];              // W_l high parts, box {64, w}
-  CUtensorMap lo[ISX_MAX_LAYERS];              // W_l low parts, box {64, w}
+  CUtensorMap hi[ISX_MAX_LAYERS];              // W_l high parts, box {64, 128}
+  CUtensorMap lo[ISX_MAX_LAYERS];              // W_l low parts, box {64, 128}
 };
 
 template <int W>
 struct EvSmem {
   static constexpr int KC = W / 64;
+  static constexpr int NH = W / 128;                      // 128-neuron halves of a layer's outputs
+  static constexpr int G = W / 64;                        // epilogue groups (of four warps)
+  static constexpr int NS = W == 256 ? 5 : 2;             // weight stages at most; w = 128 runs two CTAs per SM
+  static constexpr int kThreads = 32 * (4 * G + 2);
   static constexpr size_t kA = (size_t)kT * W * 2;        // one activation term
-  static constexpr size_t kS = (size_t)W * 128;           // one weight stage (64-wide K chunk)
-  static constexpr size_t bytes(int H) {
-    return 1024 + 2 * kA + 2 * kS + (size_t)(3 * W + (size_t)H * W + W) * 4 + EB_COUNT * 8 + 16;
+  static constexpr size_t kS = 128 * 128;                 // one weight stage
+  static constexpr int kBars = 2 * NS + KC + 2 + 2 * (G - 1);   // stage full / empty, chunk ready, accumulator done,
+                                                                // sums handed over
+  static constexpr size_t bytes(int H, int ns) {
+    return 1024 + 2 * kA + ns * kS + (size_t)(3 * W + (size_t)H * W + W + 2 * (G - 1) * kT) * 4 + kBars * 8 + 16;
   }
+  // stages that fit: five up to H = 11 at w = 256
+  static constexpr int stages(int H) { return bytes(H, NS) <= 227 * 1024 ? NS : NS - 1; }
 };
 
 __device__ __forceinline__ uint32_t aoff(int row, int k) {  // byte offset of (row, k..k+7), k % 8 == 0
@@ -98,185 +116,241 @@ __device__ __forceinline__ void store_split8(uint8_t* Ahi, uint8_t* Alo, int row
 }
 
 template <int W>
-__global__ void __launch_bounds__(kT, 1) k_eval_tc(const __grid_constant__ EvArgs args,
-                                                    const __grid_constant__ EvMaps maps) {
+__global__ void __launch_bounds__(EvSmem<W>::kThreads, W == 256 ? 1 : 2)
+k_eval_tc(const __grid_constant__ EvArgs args, const __grid_constant__ EvMaps maps) {
   using S = EvSmem<W>;
-  constexpr int KC = S::KC;
+  constexpr int KC = S::KC, NH = S::NH, G = S::G;
+  const int NS = args.ns;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* Ahi = base;
   uint8_t* Alo = Ahi + S::kA;
-  uint8_t* X = Alo + S::kA;
-  uint8_t* Y = X + S::kS;
-  float* sW0 = reinterpret_cast<float*>(Y + S::kS);
+  uint8_t* Wst = Alo + S::kA;
+  float* sW0 = reinterpret_cast<float*>(Wst + NS * S::kS);
   float* sb = sW0 + 3 * W;                     // [H][W]: biases of layers 0 .. H-1
   float* swo = sb + (size_t)args.H * W;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(swo + W);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + EB_COUNT);
+  float* sy = swo + W;                         // [2][G - 1][kT] the output layer's running sums, by tile parity
+  uint64_t* wfull = reinterpret_cast<uint64_t*>(sy + 2 * (G - 1) * kT);
+  uint64_t* wempty = wfull + NS;
+  uint64_t* aready = wempty + NS;              // [KC] chunk c of the next layer's operand is in shared memory
+  uint64_t* dfull = aready + KC;               // [2] accumulator complete (and A free)
+  uint64_t* yready = dfull + 2;                // [2][G - 1]
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(yready + 2 * (G - 1));
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
-  const int t = threadIdx.x, warp = t >> 5;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
   const int H = args.H;
+  const int64_t ntiles = (args.n + kT - 1) / kT;
+  const int64_t tile0 = blockIdx.x;
 
   if (t == 0) {
-    for (int i = 0; i < EB_COUNT; ++i) mbar_init(&bar[i], 1);
+    for (int i = 0; i < NS; ++i) {
+      mbar_init(&wfull[i], 1);
+      mbar_init(&wempty[i], 1);
+    }
+    for (int i = 0; i < KC; ++i) mbar_init(&aready[i], 4 * G);
+    for (int i = 0; i < 2; ++i) mbar_init(&dfull[i], 1);
+    for (int i = 0; i < 2 * (G - 1); ++i) mbar_init(&yready[i], 4);
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "n"(W)
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "n"(2 * W)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  for (int i = t; i < 3 * W; i += kT) sW0[i] = args.W0[i];
+  for (int i = t; i < 3 * W; i += S::kThreads) sW0[i] = args.W0[i];
   for (int l = 0; l < H; ++l)
-    for (int i = t; i < W; i += kT) sb[l * W + i] = args.b[l][i];
-  for (int i = t; i < W; i += kT) swo[i] = args.wout[i];
+    for (int i = t; i < W; i += S::kThreads) sb[l * W + i] = args.b[l][i];
+  for (int i = t; i < W; i += S::kThreads) swo[i] = args.wout[i];
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;
-  const uint32_t id = idesc(W);
-  const int64_t ntiles = (args.n + kT - 1) / kT;
-  uint32_t xf = 0, xe = 0, yf = 0, ye = 0, dn = 0;     // phase counters (thread 0 / all)
-  // thread 0: weight chunks
-  auto load_x = [&](int l, int c) {
-    mbar_expect_tx(&bar[EB_XFULL], (uint32_t)S::kS);
-    tma_load_2d(X, &maps.hi[l], &bar[EB_XFULL], c * 64, 0);
-  };
-  auto load_y = [&](int l, int c) {
-    mbar_expect_tx(&bar[EB_YFULL], (uint32_t)S::kS);
-    tma_load_2d(Y, &maps.lo[l], &bar[EB_YFULL], c * 64, 0);
-  };
-  bool ok = true;
-  if (t == 0 && blockIdx.x < ntiles) {
-    load_x(1, 0);
-    load_y(1, 0);
-  }
-  for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-    const int64_t p = tile * kT + t;
-    // ---- layer 0 in FP32, split into A_hi / A_lo ----
-    float x[3] = {0.f, 0.f, 0.f};
-    if (p < args.n) {
-      if (args.ids) {
-        const uint32_t idv = args.ids[p], n1 = (uint32_t)args.R + 1u;
-        const uint32_t ix = idv % n1, iy = (idv / n1) % n1, iz = idv / (n1 * n1);
-        const float inv = 2.0f / (float)args.R;
-        x[0] = -1.0f + inv * (float)ix;
-        x[1] = -1.0f + inv * (float)iy;
-        x[2] = -1.0f + inv * (float)iz;
-      } else {
-        x[0] = args.xyz[3 * p];
-        x[1] = args.xyz[3 * p + 1];
-        x[2] = args.xyz[3 * p + 2];
-      }
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
+
+  if (warp == 4 * G) {
+    // ---- producer: per layer and K chunk, the high terms of every 128-row half, then the low terms ----
+    if (lane == 0) {
+      uint32_t it = 0;
+      bool ok = true;
+      for (int64_t tile = tile0; tile < ntiles && ok; tile += gridDim.x)
+        for (int l = 1; l <= H - 1 && ok; ++l)
+          for (int c = 0; c < KC && ok; ++c)
+            for (int q = 0; q < 2 * NH; ++q, ++it) {
+              const int sidx = it % NS;
+              if (!ewait(&wempty[sidx], ((it / NS) & 1) ^ 1, abort, args.status)) { ok = false; break; }
+              mbar_expect_tx(&wfull[sidx], (uint32_t)S::kS);
+              tma_load_2d(Wst + sidx * S::kS, q < NH ? &maps.hi[l] : &maps.lo[l], &wfull[sidx], c * 64, (q % NH) * 128);
+            }
     }
-    for (int k = 0; k < W; k += 8) {
-      float v[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int nn = k + i;
-        const float z = fmaf(sW0[3 * nn + 2], x[2], fmaf(sW0[3 * nn + 1], x[1], fmaf(sW0[3 * nn], x[0], sb[nn])));
-        v[i] = act_fwd(args.act, z);
-      }
-      store_split8(Ahi, Alo, t, k, v);
-    }
-    fence_async_shared();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    for (int l = 1; l <= H - 1; ++l) {
-      // ---- thread 0: D = A_hi W_hi^T + A_lo W_hi^T + A_hi W_lo^T, K chunk by chunk ----
-      if (t == 0) {
+  } else if (warp == 4 * G + 1) {
+    // ---- MMA issuer: D = A_hi W_hi^T + A_lo W_hi^T + A_hi W_lo^T, K chunk by chunk, in 128-neuron halves ----
+    const uint32_t id = idesc(128), lead = elect_one();
+    uint32_t sidx = 0, sph = 0, ly = 0;        // weight stage and its phase; layers so far
+    bool ok = true;
+    for (int64_t tile = tile0; tile < ntiles && ok; tile += gridDim.x)
+      for (int l = 1; l <= H - 1 && ok; ++l, ++ly) {
+        const uint32_t d = tmem + (ly & 1) * W;
         for (int c = 0; c < KC && ok; ++c) {
-          if (!ewait(&bar[EB_XFULL], xf & 1, abort, args.status)) { ok = false; break; }
-          ++xf;
+          ok = __all_sync(0xffffffffu, ewait(&aready[c], ly & 1, abort, args.status));
+          if (!ok) break;
           tc_fence_after();
-          const uint32_t ah = su32(Ahi + (size_t)c * kT * 128), al = su32(Alo + (size_t)c * kT * 128);
-          const uint32_t bx = su32(X), by = su32(Y);
+          const uint32_t ah = sdesc_lo(su32(Ahi) + c * kT * 128), al = sdesc_lo(su32(Alo) + c * kT * 128);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            mma_bf16(tmem, sdesc(ah + kk * 32), sdesc(bx + kk * 32), id, (c > 0 || kk > 0) ? 1u : 0u);
-            mma_bf16(tmem, sdesc(al + kk * 32), sdesc(bx + kk * 32), id, 1u);
+          for (int q = 0; q < 2 * NH; ++q) {
+            ok = __all_sync(0xffffffffu, ewait(&wfull[sidx], sph, abort, args.status));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t w0 = sdesc_lo(su32(Wst) + sidx * (uint32_t)S::kS), dh = d + (q % NH) * 128;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+              mma_bf16_lead(dh, ah + 2 * kk, w0 + 2 * kk, id, (q >= NH || c > 0 || kk > 0) ? 1u : 0u, lead);
+              if (q < NH) mma_bf16_lead(dh, al + 2 * kk, w0 + 2 * kk, id, 1u, lead);
+            }
+            mma_commit_lead(&wempty[sidx], lead);
+            if (++sidx == (uint32_t)NS) {
+              sidx = 0;
+              sph ^= 1;
+            }
           }
-          mma_commit(&bar[EB_XEMPTY]);
-          if (!ewait(&bar[EB_YFULL], yf & 1, abort, args.status)) { ok = false; break; }
-          ++yf;
-          tc_fence_after();
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) mma_bf16(tmem, sdesc(ah + kk * 32), sdesc(by + kk * 32), id, 1u);
-          mma_commit(&bar[EB_YEMPTY]);
-          // refill the stages: the next chunk of this layer, else chunk 0 of the next layer (or of
-          // layer 1 for the next tile)
-          int nl = l, nc = c + 1;
-          if (nc == KC) {
-            nc = 0;
-            nl = l + 1;
-            if (nl > H - 1) nl = (tile + gridDim.x < ntiles) ? 1 : 0;
-          }
-          if (!ewait(&bar[EB_XEMPTY], xe & 1, abort, args.status)) { ok = false; break; }
-          ++xe;
-          if (nl) load_x(nl, nc);
-          if (!ewait(&bar[EB_YEMPTY], ye & 1, abort, args.status)) { ok = false; break; }
-          ++ye;
-          if (nl) load_y(nl, nc);
         }
-        if (ok) mma_commit(&bar[EB_DONE]);
+        if (ok) mma_commit_lead(&dfull[ly & 1], lead);
       }
-      // ---- everyone: epilogue of layer l ----
-      if (!ewait(&bar[EB_DONE], dn & 1, abort, args.status)) ok = false;
-      ++dn;
-      __syncthreads();
-      if (*abort) ok = false;
-      if (!ok) break;
-      tc_fence_after();
-      const float* bl = sb + (size_t)l * W;
-      const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);
-      if (l < H - 1) {
-        for (int c0 = 0; c0 < W; c0 += 32) {
-          float v[32];
-          tmem_ld32(trow + c0, v);
-#pragma unroll
-          for (int i = 0; i < 32; ++i) v[i] = act_fwd(args.act, v[i] + bl[c0 + i]);
-#pragma unroll
-          for (int u = 0; u < 4; ++u) store_split8(Ahi, Alo, t, c0 + 8 * u, v + 8 * u);
-        }
-        fence_async_shared();
-      } else {
-        float y = 0.f;
-        for (int c0 = 0; c0 < W; c0 += 32) {
-          float v[32];
-          tmem_ld32(trow + c0, v);
-#pragma unroll
-          for (int i = 0; i < 32; ++i) y = fmaf(swo[c0 + i], act_fwd(args.act, v[i] + bl[c0 + i]), y);
-        }
-        if (p < args.n) args.out[p] = y + args.bout;
-      }
+  } else {
+    // ---- activations: point p = TMEM lane, group g ----
+    const int g = warp >> 2, p = 32 * (warp & 3) + lane;
+    const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
+    constexpr int CW = 64 / G;                 // columns of a chunk per group (16 or 32)
+    // chunk c of the next operand is complete for this warp
+    auto ready = [&](int c) {
+      fence_async_shared();
       tc_fence_before();
-      __syncthreads();
-      tc_fence_after();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&aready[c]);
+    };
+    // coordinates of this thread's point of a tile (loaded a tile ahead)
+    auto load_x = [&](int64_t tile, float* x) {
+      const int64_t i = tile * kT + p;
+      x[0] = x[1] = x[2] = 0.f;
+      if (i < args.n) {
+        if (args.ids) {
+          const uint32_t idv = args.ids[i], n1 = (uint32_t)args.R + 1u;
+          const uint32_t ix = idv % n1, iy = (idv / n1) % n1, iz = idv / (n1 * n1);
+          const float inv = 2.0f / (float)args.R;
+          x[0] = -1.0f + inv * (float)ix;
+          x[1] = -1.0f + inv * (float)iy;
+          x[2] = -1.0f + inv * (float)iz;
+        } else {
+          x[0] = args.xyz[3 * i];
+          x[1] = args.xyz[3 * i + 1];
+          x[2] = args.xyz[3 * i + 2];
+        }
+      }
+    };
+    auto layer0 = [&](const float* x) {
+#pragma unroll 1
+      for (int c = 0; c < KC; ++c) {
+#pragma unroll
+        for (int k = 0; k < CW; k += 8) {
+          const int k0 = 64 * c + CW * g + k;
+          float v[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const int nn = k0 + e;
+            const float z = fmaf(sW0[3 * nn + 2], x[2], fmaf(sW0[3 * nn + 1], x[1], fmaf(sW0[3 * nn], x[0], sb[nn])));
+            v[e] = act_fwd(args.act, z);
+          }
+          store_split8(Ahi, Alo, p, k0, v);
+        }
+        ready(c);
+      }
+    };
+    uint32_t ly = 0, tt = 0;
+    bool ok = true;
+    float x[3];
+    if (tile0 < ntiles) {
+      load_x(tile0, x);
+      layer0(x);
+    }
+    for (int64_t tile = tile0; tile < ntiles && ok; tile += gridDim.x, ++tt) {
+      load_x(tile + gridDim.x, x);
+      for (int l = 1; l <= H - 1; ++l, ++ly) {
+        const bool got = ewait(&dfull[ly & 1], (ly >> 1) & 1, abort, args.status);
+        if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+        tc_fence_after();
+        const float* bl = sb + (size_t)l * W;
+        const uint32_t trow = tmem + (ly & 1) * W + lane_off;
+        if (l < H - 1) {
+#pragma unroll 1
+          for (int c = 0; c < KC; ++c) {
+            const int k0 = 64 * c + CW * g;
+            float v[CW];
+            if constexpr (CW == 16) tmem_ld16(trow + k0, v);
+            else tmem_ld32(trow + k0, v);
+#pragma unroll
+            for (int e = 0; e < CW; ++e) v[e] = act_fwd(args.act, v[e] + bl[k0 + e]);
+#pragma unroll
+            for (int u = 0; u < CW / 8; ++u) store_split8(Ahi, Alo, p, k0 + 8 * u, v + 8 * u);
+            ready(c);
+          }
+        } else {
+          // the operand buffers are free: layer 0 of the next tile first, then this tile's output layer,
+          // one chain over the neurons, 64 of them per group
+          if (tile + gridDim.x < ntiles) layer0(x);
+          float y = 0.f;
+#pragma unroll 1
+          for (int hf = 0; hf < 2; ++hf) {
+            const int k0 = 64 * g + 32 * hf;
+            float v[32];
+            tmem_ld32(trow + k0, v);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] = act_fwd(args.act, v[e] + bl[k0 + e]);
+            if (hf == 0 && g > 0) {
+              const int q = (tt & 1) * (G - 1) + g - 1;
+              const bool up = ewait(&yready[q], (tt >> 1) & 1, abort, args.status);
+              if (!__all_sync(0xffffffffu, up)) ok = false;
+              y = sy[q * kT + p];
+            }
+#pragma unroll
+            for (int e = 0; e < 32; ++e) y = fmaf(swo[k0 + e], v[e], y);
+          }
+          if (!ok) break;
+          if (g < G - 1) {
+            const int q = (tt & 1) * (G - 1) + g;
+            sy[q * kT + p] = y;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&yready[q]);
+          } else {
+            const int64_t i = tile * kT + p;
+            if (i < args.n) args.out[i] = y + args.bout;
+          }
+        }
+      }
     }
   }
   // ---- teardown: let in-flight copies land, free TMEM ----
+  tc_fence_before();
   __syncthreads();
   if (*abort)
     for (int i = 0; i < 1000; ++i) __nanosleep(1000);
   if (warp == 0) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(W) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(2 * W) : "memory");
   }
 }
 
 template <int W>
-isx_status launch_eval(isx_inr inr, const EvArgs& a, const EvMaps& maps, int64_t ntiles, cudaStream_t st) {
-  const size_t smem = EvSmem<W>::bytes(inr->H);
+isx_status launch_eval(isx_inr inr, EvArgs a, const EvMaps& maps, int64_t ntiles, cudaStream_t st) {
+  const int ns = EvSmem<W>::stages(inr->H);
+  a.ns = ns;
+  const size_t smem = EvSmem<W>::bytes(inr->H, ns);
   ISX_CUDA(cudaFuncSetAttribute(k_eval_tc<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 1, sms = 148;
   ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
-  ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eval_tc<W>, kT, smem));
-  // TMEM: W columns per CTA out of 512
-  per_sm = std::max(1, std::min(per_sm, 512 / W));
+  ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eval_tc<W>, EvSmem<W>::kThreads, smem));
+  // TMEM: two accumulators of W columns per CTA out of 512
+  per_sm = std::max(1, std::min(per_sm, 512 / (2 * W)));
   const int grid = (int)std::min<int64_t>(ntiles, (int64_t)sms * per_sm);
-  k_eval_tc<W><<<grid, kT, smem, st>>>(a, maps);
+  k_eval_tc<W><<<grid, EvSmem<W>::kThreads, smem, st>>>(a, maps);
   ISX_LAUNCH_CHECK("k_eval_tc");
   return ISX_OK;
 }
@@ -311,8 +385,8 @@ isx_status eval_points_tc(isx_inr inr, const float* xyz, const uint32_t* lattice
   EvMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   for (int l = 1; l <= H - 1; ++l) {
-    ISX_TRY(tensor_map_bf16(&maps.hi[l], inr->W_bf16[l], w, w, 64, w));
-    ISX_TRY(tensor_map_bf16(&maps.lo[l], inr->Wlo_bf16[l], w, w, 64, w));
+    ISX_TRY(tensor_map_bf16(&maps.hi[l], inr->W_bf16[l], w, w, 64, 128));
+    ISX_TRY(tensor_map_bf16(&maps.lo[l], inr->Wlo_bf16[l], w, w, 64, 128));
   }
   ISX_CUDA(cudaMemsetAsync(a.status, 0, sizeof(int), st));
   const int64_t ntiles = (n + kT - 1) / kT;

@@ -82,6 +82,34 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b
       "l"(a), "l"(b), "r"(id), "r"(acc)
       : "memory");
 }
+// The same issued by one lane (`lead` != 0) of a converged warp, from descriptor low words (sdesc_lo).  The MMA takes
+// its descriptors in uniform registers: where the whole warp computes them in converged code they are
+// there already; inside `if (lane == 0)` every one is moved over from vector registers, at about 190 cycles
+// per MMA, three times what an M = N = 128, K = 16 product takes.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+__device__ __forceinline__ void mma_bf16_lead(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t id, uint32_t acc,
+                                              uint32_t lead) {
+  constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+  asm volatile(
+      "{\n .reg .pred p, e;\n .reg .b64 da, db;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 e, %5, 0;\n"
+      " mov.b64 da, {%1, %6};\n mov.b64 db, {%2, %6};\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(a_lo), "r"(b_lo), "r"(id), "r"(acc), "r"(lead), "n"(hi)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit_lead(uint64_t* bar, uint32_t lead) {
+  asm volatile(
+      "{\n .reg .pred e;\n setp.ne.b32 e, %1, 0;\n"
+      " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(su32(bar)),
+      "r"(lead)
+      : "memory");
+}
+// 1 in one lane of the (converged) warp, 0 in the others.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.b32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e;
+}
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
                : "memory");

@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kST, 1) k_rows_split(const __grid_constant__ R
   uint64_t* bar = reinterpret_cast<uint64_t*>(base + 2 * S::kStage);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + SB_COUNT);
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
   const int64_t nrows = ONE ? args.nc : 4 * args.nc;
   const int64_t ntiles = (nrows + kRT - 1) / kRT;
   // work items (tile, column half); the grid is a multiple of NHALF, so a CTA keeps its half
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(kST, 1) k_rows_split(const __grid_constant__ R
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
   auto stage = [&](int s) { return base + (size_t)s * S::kStage; };
 
   if (warp == 0) {
@@ -522,33 +522,34 @@ __global__ void __launch_bounds__(kST, 1) k_rows_split(const __grid_constant__ R
       }
     }
   } else if (warp == 1) {
-    // ---- MMA issuer ----
-    if (lane == 0) {
-      const uint32_t id = idesc(NC);
-      uint32_t it = 0, tt = 0;
-      for (int64_t tile = t0; tile < ntiles && !*abort; tile += TS, ++tt) {
-        const uint32_t b = tt & 1;
-        if (!rwait(&bar[SB_TEMPTY + b], ((tt >> 1) & 1) ^ 1, abort, args.status)) break;
+    // ---- MMA issuer: the whole warp walks the loop, one lane issues ----
+    const uint32_t id = idesc(NC), lead = elect_one();
+    uint32_t it = 0, tt = 0;
+    for (int64_t tile = t0; tile < ntiles; tile += TS, ++tt) {
+      const uint32_t b = tt & 1;
+      if (!__all_sync(0xffffffffu, rwait(&bar[SB_TEMPTY + b], ((tt >> 1) & 1) ^ 1, abort, args.status))) break;
+      tc_fence_after();
+      const uint32_t dt = tmem + b * NC;
+      bool ok = true;
+      for (int c = 0; c < KC; ++c, ++it) {
+        const uint32_t sidx = it & 1;
+        ok = __all_sync(0xffffffffu, rwait(&bar[SB_FULL + sidx], (it >> 1) & 1, abort, args.status));
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t dt = tmem + b * NC;
-        for (int c = 0; c < KC; ++c, ++it) {
-          const int sidx = it & 1;
-          if (!rwait(&bar[SB_FULL + sidx], (it >> 1) & 1, abort, args.status)) break;
-          tc_fence_after();
-          const uint32_t ah = su32(stage(sidx)), al = ah + (uint32_t)S::kA;
-          const uint32_t bh = ah + 2 * (uint32_t)S::kA, bl = bh + (uint32_t)S::kB;
+        const uint32_t ah = sdesc_lo(su32(base) + sidx * (uint32_t)S::kStage), al = ah + (uint32_t)(S::kA >> 4);
+        const uint32_t bh = al + (uint32_t)(S::kA >> 4), bl = bh + (uint32_t)(S::kB >> 4);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            mma_bf16(dt, sdesc(ah + kk * 32), sdesc(bh + kk * 32), id, (c > 0 || kk > 0) ? 1u : 0u);
-            if (!ONE) {
-              mma_bf16(dt, sdesc(al + kk * 32), sdesc(bh + kk * 32), id, 1u);
-              mma_bf16(dt, sdesc(ah + kk * 32), sdesc(bl + kk * 32), id, 1u);
-            }
+        for (int kk = 0; kk < 4; ++kk) {
+          mma_bf16_lead(dt, ah + 2 * kk, bh + 2 * kk, id, (c > 0 || kk > 0) ? 1u : 0u, lead);
+          if (!ONE) {
+            mma_bf16_lead(dt, al + 2 * kk, bh + 2 * kk, id, 1u, lead);
+            mma_bf16_lead(dt, ah + 2 * kk, bl + 2 * kk, id, 1u, lead);
           }
-          mma_commit(&bar[SB_EMPTY + sidx]);
         }
-        mma_commit(&bar[SB_TFULL + b]);
+        mma_commit_lead(&bar[SB_EMPTY + sidx], lead);
       }
+      if (!ok) break;
+      mma_commit_lead(&bar[SB_TFULL + b], lead);
     }
   } else {
     // ---- epilogue: TMEM lane group warp % 4, one row per thread ----
@@ -857,12 +858,29 @@ __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode
     return !sq ? a + fabsf(y) : (r < whole ? fmaf(y, y, a) : __fadd_rn(a, __fmul_rn(y, y)));
   };
   if constexpr (WPC == 1) {
-    for (int r = 0; r < rows; r += 4) {
+    int r = 0;
+    for (; r < whole; r += 4) {
       float y[4];
-      four(r, y);
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (r + q < rows) sr = term(r + q, y[q], sr);
+      for (int q = 0; q < 4; ++q) {
+        float x[CPL];
+        ld_row<CPL>(xp + (size_t)(r + q) * w, x);
+        y[q] = dot(x);
+      }
+#pragma unroll
+      for (int sh = 16; sh > 0; sh >>= 1)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y[q] += __shfl_xor_sync(0xffffffffu, y[q], sh);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sr = sq ? fmaf(y[q], y[q], sr) : sr + fabsf(y[q]);
+    }
+    for (; r < rows; ++r) {
+      float x[CPL];
+      ld_row<CPL>(xp + (size_t)r * w, x);
+      float y = dot(x);
+#pragma unroll
+      for (int sh = 16; sh > 0; sh >>= 1) y += __shfl_xor_sync(0xffffffffu, y, sh);
+      sr = term(r, y, sr);
     }
   } else {
     __shared__ float sy[kOutWarps / WPC][2][kOutRows];

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_c
   uint64_t* wfull = tempty + 2;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(wfull + 1);
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
   const int64_t ntiles = (args.R + kRT - 1) / kRT;
   // work items are (tile, weight slice); the grid is a multiple of NQ, so this CTA's slice q never
   // changes and it walks the tiles t0, t0 + TS, ...; the NQ CTAs of a tile run side by side and
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_c
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
 
   if (warp < kSW) {
     // ---- scale row sr of every staged chunk by alpha of its cell, in place: this thread's CG 8-column groups ----
@@ -195,36 +195,44 @@ __global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_c
       }
     }
   } else if (warp == kSW) {
-    // ---- W_j once, then the MMAs: D[half h] += W_j[h rows] x chunk^T ----
-    if (lane == 0) {
+    // ---- W_j once, then the MMAs: D[half h] += W_j[h rows] x chunk^T; the whole warp walks the loop, one lane
+    //      issues ----
+    const uint32_t id = idesc(kRT), lead = elect_one();
+    if (lead) {
       // the CTA's weight rows: all of W_j, or rows q * 128 .. q * 128 + 127 of it
       constexpr int rows_held = W < MW ? W : MW;
       mbar_expect_tx(wfull, (uint32_t)((size_t)rows_held * W * 2));
       for (int c = 0; c < KC; ++c)
         tma_load_2d(Wsm + (size_t)c * MW * 128, &wmap, wfull, c * 64, NQ > 1 ? q * 128 : 0);
-      const uint32_t id = idesc(kRT);
-      uint32_t it = 0, tt = 0;
-      bool ok = rwait(wfull, 0, abort, args.status);
-      for (int64_t tile = t0; tile < ntiles && ok; tile += TS, ++tt) {
-        const uint32_t b = tt & 1;
-        if (!rwait(&tempty[b], ((tt >> 1) & 1) ^ 1, abort, args.status)) break;
+    }
+    __syncwarp();
+    uint32_t sidx = 0, sph = 0, tt = 0;
+    bool ok = __all_sync(0xffffffffu, rwait(wfull, 0, abort, args.status));
+    for (int64_t tile = t0; tile < ntiles && ok; tile += TS, ++tt) {
+      const uint32_t b = tt & 1;
+      ok = __all_sync(0xffffffffu, rwait(&tempty[b], ((tt >> 1) & 1) ^ 1, abort, args.status));
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t dt = tmem + b * (NH * 128);
+#pragma unroll 1
+      for (int c = 0; c < KC; ++c) {
+        ok = __all_sync(0xffffffffu, rwait(&afull[sidx], sph, abort, args.status));
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t dt = tmem + b * (NH * 128);
-        for (int c = 0; c < KC; ++c, ++it) {
-          const int sidx = it % NS;
-          if (!rwait(&afull[sidx], (it / NS) & 1, abort, args.status)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t x0 = su32(Asm + (size_t)sidx * S::kAC), w0 = su32(Wsm + (size_t)c * MW * 128);
+        const uint32_t x0 = sdesc_lo(su32(Asm) + sidx * (uint32_t)S::kAC), w0 = sdesc_lo(su32(Wsm) + c * MW * 128);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
+        for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
-            for (int h = 0; h < NH; ++h)
-              mma_bf16(dt + h * 128, sdesc(w0 + h * 128 * 128 + kk * 32), sdesc(x0 + kk * 32), id,
-                       (c > 0 || kk > 0) ? 1u : 0u);
-          mma_commit(&aempty[sidx]);
+          for (int h = 0; h < NH; ++h)
+            mma_bf16_lead(dt + h * 128, w0 + h * (128 * 128 >> 4) + 2 * kk, x0 + 2 * kk, id, (c > 0 || kk > 0) ? 1u : 0u,
+                          lead);
+        mma_commit_lead(&aempty[sidx], lead);
+        if (++sidx == NS) {
+          sidx = 0;
+          sph ^= 1;
         }
-        if (ok) mma_commit(&tfull[b]);
       }
+      if (ok) mma_commit_lead(&tfull[b], lead);
     }
   } else {
     // ---- epilogue: TMEM -> bf16 rows of G' and the per-(cell, 64-row block) column sums of f(G') ----

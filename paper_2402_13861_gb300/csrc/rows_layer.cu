@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kLT, 1) k_rows_layer(const __grid_constant__ R
   uint64_t* bar = reinterpret_cast<uint64_t*>(base + 2 * S::kStage + S::kQueue);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + LB_COUNT);
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
   const int64_t ntiles = (args.nc + kLC - 1) / kLC;
   const int hq = blockIdx.x % NHALF;
   const int64_t t0 = blockIdx.x / NHALF, TS = gridDim.x / NHALF;
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kLT, 1) k_rows_layer(const __grid_constant__ R
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
 
   if (warp == 0) {
     // ---- producer ----
@@ -160,35 +160,35 @@ __global__ void __launch_bounds__(kLT, 1) k_rows_layer(const __grid_constant__ R
       }
     }
   } else if (warp == 1) {
-    // ---- MMA issuer ----
-    if (lane == 0) {
-      const uint32_t id = idesc(4 * kLC);
-      uint32_t it = 0, tt = 0;
-      for (int64_t tile = t0; tile < ntiles && !*abort; tile += TS, ++tt) {
-        const uint32_t b = tt & 1;
-        if (!rwait(&bar[LB_TEMPTY + b], ((tt >> 1) & 1) ^ 1, abort, args.status)) break;
-        tc_fence_after();
-        const uint32_t dt = tmem + b * NH * 128;
-        bool ok = true;
-        for (int c = 0; c < KC; ++c, ++it) {
-          const int sidx = it & 1;
-          if (!rwait(&bar[LB_FULL + sidx], (it >> 1) & 1, abort, args.status)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t ah = su32(stage(sidx)), al = ah + (uint32_t)S::kA, w0 = al + (uint32_t)S::kA;
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-              const uint32_t wh = w0 + h * (uint32_t)S::kA + kk * 32, wl = wh + NH * (uint32_t)S::kA;
-              mma_bf16(dt + h * 128, sdesc(wh), sdesc(ah + kk * 32), id, (c > 0 || kk > 0) ? 1u : 0u);
-              mma_bf16(dt + h * 128, sdesc(wh), sdesc(al + kk * 32), id, 1u);
-              mma_bf16(dt + h * 128, sdesc(wl), sdesc(ah + kk * 32), id, 1u);
-            }
-          mma_commit(&bar[LB_EMPTY + sidx]);
-        }
+    // ---- MMA issuer: the whole warp walks the loop, one lane issues ----
+    const uint32_t id = idesc(4 * kLC), lead = elect_one();
+    uint32_t it = 0, tt = 0;
+    for (int64_t tile = t0; tile < ntiles; tile += TS, ++tt) {
+      const uint32_t b = tt & 1;
+      if (!__all_sync(0xffffffffu, rwait(&bar[LB_TEMPTY + b], ((tt >> 1) & 1) ^ 1, abort, args.status))) break;
+      tc_fence_after();
+      const uint32_t dt = tmem + b * NH * 128;
+      bool ok = true;
+      for (int c = 0; c < KC; ++c, ++it) {
+        const uint32_t sidx = it & 1;
+        ok = __all_sync(0xffffffffu, rwait(&bar[LB_FULL + sidx], (it >> 1) & 1, abort, args.status));
         if (!ok) break;
-        mma_commit(&bar[LB_TFULL + b]);
+        tc_fence_after();
+        constexpr uint32_t kD = (uint32_t)(S::kA >> 4);      // one operand chunk, in descriptor units
+        const uint32_t ah = sdesc_lo(su32(base) + sidx * (uint32_t)S::kStage), al = ah + kD, w0 = al + kD;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+          for (int h = 0; h < NH; ++h) {
+            const uint32_t wh = w0 + h * kD + 2 * kk, wl = wh + NH * kD;
+            mma_bf16_lead(dt + h * 128, wh, ah + 2 * kk, id, (c > 0 || kk > 0) ? 1u : 0u, lead);
+            mma_bf16_lead(dt + h * 128, wh, al + 2 * kk, id, 1u, lead);
+            mma_bf16_lead(dt + h * 128, wl, ah + 2 * kk, id, 1u, lead);
+          }
+        mma_commit_lead(&bar[LB_EMPTY + sidx], lead);
       }
+      if (!ok) break;
+      mma_commit_lead(&bar[LB_TFULL + b], lead);
     }
   } else {
     // ---- epilogue: TMEM lane group warp % 4, cells 8 g .. 8 g + 7 of a tile ----

@@ -93,3 +93,27 @@ def test_fp32_bounds_under_capture(pkg):
     torch.cuda.synchronize()
     assert torch.equal(c, c0) and torch.equal(s, s0)
     net.close()
+
+
+@pytest.mark.parametrize("w,H,inflate", [(16, 2, False), (48, 3, True), (64, 2, False), (80, 2, True), (256, 2, False),
+                                         (400, 2, False), (512, 2, True)])
+def test_rafixed_tile_edges(pkg, w, H, inflate):
+    """Both tile forms (two cells per thread up to w = 64, four above), ragged last tiles and few cells: a cell's
+    bound is the same whatever its tile, and within the float32 band of the oracle (an enclosure with inflation)."""
+    layers = inr.random_inr([3] + [w] * H + [1], 100 + w)
+    net = pkg.Inr(layers)
+    lo, hi = boxes.random_boxes(20003, 101, -10, -2)
+    dlo, dhi = torch.tensor(lo, device="cuda"), torch.tensor(hi, device="cuda")
+    c, s = net.bound_cells(dlo, dhi, mode="rafixed", inflate=inflate)
+    for n in (1, 3, 63, 305, 4001):
+        a, b = net.bound_cells(dlo[:n].contiguous(), dhi[:n].contiguous(), mode="rafixed", inflate=inflate)
+        assert torch.equal(a, c[:n]) and torch.equal(b, s[:n]), n
+    idx = np.r_[0:40, 20003 - 40:20003]
+    oc, os_ = affine.bound(layers, lo[idx], hi[idx], "rafixed", batch=40)
+    c, s = c.cpu().numpy().astype(np.float64)[idx], s.cpu().numpy().astype(np.float64)[idx]
+    if inflate:
+        assert np.all(c - s <= oc - os_ + 1e-7) and np.all(c + s >= oc + os_ - 1e-7)
+    else:
+        tol = 8 * H * w * 2.0 ** -24 * (np.abs(oc) + os_) + 1e-7
+        assert np.all(np.abs(c - oc) <= tol) and np.all(np.abs(s - os_) <= tol)
+    net.close()

@@ -7,17 +7,20 @@
 // Numerics: BF16 weights, BF16 inputs and activations (round to nearest even after every layer),
 // FP32 accumulation; FP32 master weights, gradients and Adam moments.  The model costs 17.5 kFLOP
 // per pair against 203 MFLOP for one affine bound of the 256-wide 5-layer INR, so it runs on CUDA
-// cores: one thread per sample, weights broadcast from shared memory (staged once per block as
-// FP32, exact), every thread's activation rows in padded shared memory (row stride 65 floats, so
-// the 32 rows a warp touches fall in 32 different banks).
+// cores, weights staged once per block as FP32 (exact).  k_prop_forward and k_prop_grad work on tiles of
+// samples, activations [neuron][sample] in shared memory, with register tiles of samples x neurons (every
+// output one multiply-add chain over the inputs); k_prop_gate, whose pairs come from bit masks, runs one thread
+// per cell with its activation rows in padded shared memory (row stride 65 floats, so the 32 rows a warp
+// touches fall in 32 different banks).
 //
 // Kernels: k_prop_forward (logits of given feature rows), k_prop_grad (forward + backward of the
-// mean BCE, per-block gradient sums in shared memory, one atomic add per parameter per block),
+// mean BCE, per-block gradient sums in registers, one atomic add per parameter per block),
 // k_prop_adam (one Adam step over the flat parameter vector, refreshes the BF16 copy),
 // k_prop_gate (extraction: builds the features of every (cell, iso) pair in the cell's mask, drops
 // confident negatives, keeps confident positives, flags the rest for bounding), k_prop_merge
 // (applies the bound of the flagged cells).
 #include "internal.cuh"
+#include "sgemm.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -45,9 +48,8 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + kH * kF, OFF_W2 = OFF_B1 + kH, OFF_B
 static_assert(kNParam == ISX_PROPOSER_NPARAM, "packed parameter layout");
 static_assert(OFF_W2 % 4 == 0 && OFF_W3 % 4 == 0 && OFF_W4 % 4 == 0, "float4 weight rows");
 constexpr int kNParamPad = (kNParam + 3) & ~3;
-constexpr int kTB = 128;          // samples per tile = threads per block
+constexpr int kTB = 128;          // threads per block (k_prop_gate: cells per tile)
 constexpr int kRow = kH + 1;      // padded activation row
-constexpr int kRow0 = kF + 1;     // padded input row
 
 struct Norm {
   float mu[kF], inv_sd[kF];
@@ -106,150 +108,299 @@ __device__ __forceinline__ float forward_sample(const float* sw, const float (&x
   return z;
 }
 
+// ---- tiles of samples -------------------------------------------------------------------------------
+// Shared memory of a block: the transposed hidden weights Wt[i][o] (pitch kWP, so that staging them costs
+// four-way bank conflicts, not 32-way), the biases and W4, and activations [neuron][sample].
+constexpr int kWP = kH + 4;
+constexpr int kWtFloats = (kF + 2 * kH) * kWP + 4 * kH + 4;   // W1t, W2t, W3t; b1, b2, b3, W4, b4
+
+static_assert(OFF_B1 % 8 == 0 && OFF_W2 % 8 == 0 && OFF_B2 % 8 == 0 && OFF_W3 % 8 == 0 && OFF_B3 % 8 == 0 &&
+                  OFF_B4 % 8 == 0 && OFF_B4 == kNParam - 1, "16-byte groups of parameters");
+// Also W2 and W3 as they are ([o][i], one after the other) into w23 when given.  16-byte loads, four in flight.
+__device__ __forceinline__ void stage_transposed(float* wt, float* w23, const __nv_bfloat16* pb) {
+  float* vec = wt + (kF + 2 * kH) * kWP;
+  const uint4* src = reinterpret_cast<const uint4*>(pb);
+  for (int g0 = threadIdx.x; g0 < OFF_B4 / 8; g0 += 4 * blockDim.x) {
+    uint4 u[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (g0 + q * (int)blockDim.x < OFF_B4 / 8) u[q] = src[g0 + q * blockDim.x];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = 8 * (g0 + q * (int)blockDim.x);
+      if (k >= OFF_B4) break;
+      float v[8];
+      const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u[q]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f = __bfloat1622float2(h[e]);
+        v[2 * e] = f.x;
+        v[2 * e + 1] = f.y;
+      }
+      // the group's eight values: inputs i .. i + 7 of output o, or eight entries of a vector
+      float* d = nullptr;
+      int step = kWP;
+      if (k < OFF_B1) {
+        d = wt + k / kF;
+      } else if (k >= OFF_W2 && k < OFF_B2) {
+        d = wt + (kF + (k - OFF_W2) % kH) * kWP + (k - OFF_W2) / kH;
+      } else if (k >= OFF_W3 && k < OFF_B3) {
+        d = wt + (kF + kH + (k - OFF_W3) % kH) * kWP + (k - OFF_W3) / kH;
+      } else {
+        d = vec + (k < OFF_W2 ? k - OFF_B1 : (k < OFF_W3 ? kH + k - OFF_B2 : 2 * kH + k - OFF_B3));
+        step = 1;
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) d[e * step] = v[e];
+      if (w23 && step > 1 && k >= OFF_W2) {
+        float* c = w23 + (k < OFF_B2 ? k - OFF_W2 : kH * kH + k - OFF_W3);
+#pragma unroll
+        for (int e = 0; e < 8; e += 4) *reinterpret_cast<float4*>(c + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+      }
+    }
+  }
+  if (threadIdx.x == 0) vec[4 * kH] = __bfloat162float(pb[OFF_B4]);
+}
+
+// acc[s][j]: output pair j of this thread's outputs for sample s; samples sp(s), outputs op(j), op(j) + 1.
+// NS samples in groups of 4 at s0, s0 + SS, ...; NO outputs in groups of 4 at o0, o0 + OS, ...
+template <int NS, int NO>
+struct PropTile {
+  uint64_t acc[NS][NO / 2];
+  __device__ __forceinline__ void bias(const float* b, int o0, int os) {
+#pragma unroll
+    for (int j = 0; j < NO / 2; ++j) {
+      const int o = o0 + (j >> 1) * os + 2 * (j & 1);
+      const uint64_t v = b ? sgemm::pack2(b[o], b[o + 1]) : 0ull;
+#pragma unroll
+      for (int s = 0; s < NS; ++s) acc[s][j] = v;
+    }
+  }
+  // acc += sum_i X[i][sample] W[i][output], i ascending
+  template <int IN>
+  __device__ __forceinline__ void contract(const float* W, int wp, const float* X, int xp, int s0, int ss, int o0, int os) {
+#pragma unroll 4
+    for (int i = 0; i < IN; ++i) {
+      uint64_t x[NS];
+#pragma unroll
+      for (int g = 0; g < NS / 4; ++g) {
+        const float4 v = *reinterpret_cast<const float4*>(X + i * xp + s0 + g * ss);
+        x[4 * g] = sgemm::pack2(v.x, v.x);
+        x[4 * g + 1] = sgemm::pack2(v.y, v.y);
+        x[4 * g + 2] = sgemm::pack2(v.z, v.z);
+        x[4 * g + 3] = sgemm::pack2(v.w, v.w);
+      }
+#pragma unroll
+      for (int g = 0; g < NO / 4; ++g) {
+        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(W + i * wp + o0 + g * os);
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+          acc[s][2 * g] = sgemm::fma2(x[s], w.x, acc[s][2 * g]);
+          acc[s][2 * g + 1] = sgemm::fma2(x[s], w.y, acc[s][2 * g + 1]);
+        }
+      }
+    }
+  }
+  __device__ __forceinline__ float get(int s, int o) const {
+    const float2 v = sgemm::unpack2(acc[s][o >> 1]);
+    return (o & 1) ? v.y : v.x;
+  }
+  // Y[output][sample] = f(value, output, sample index s)
+  template <class F>
+  __device__ __forceinline__ void store(float* Y, int yp, int s0, int ss, int o0, int os, F f) const {
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+      float* d = Y + (o0 + (o >> 2) * os + (o & 3)) * yp;
+#pragma unroll
+      for (int g = 0; g < NS / 4; ++g)
+        *reinterpret_cast<float4*>(d + s0 + g * ss) =
+            make_float4(f(get(4 * g, o), d, s0 + g * ss), f(get(4 * g + 1, o), d, s0 + g * ss + 1),
+                        f(get(4 * g + 2, o), d, s0 + g * ss + 2), f(get(4 * g + 3, o), d, s0 + g * ss + 3));
+    }
+  }
+};
+__device__ __forceinline__ float act_bf16(float v, const float*, int) { return bf16r(fmaxf(v, 0.f)); }
+
+// Logits: 128-sample tiles, an 8 x 8 register tile per thread, activations written back in place.  Bound by the
+// shared-memory return bandwidth (16 values read per 64 multiply-adds): 2 M samples 0.74 ms, 48 TFLOP/s (1.48 ms with one
+// thread per sample).
+constexpr int kFwdS = 128, kFwdP = kFwdS + 4;
+constexpr size_t kFwdSmem = (size_t)(kWtFloats + kH * kFwdP) * sizeof(float);
 __global__ void __launch_bounds__(kTB) k_prop_forward(const __nv_bfloat16* pb, Norm nm, const float* feat, int64_t n,
                                                       float* logit) {
-  extern __shared__ float sm[];
-  float* sw = sm;
-  float* rows = sm + kNParamPad;                         // [2][kTB][kRow]
-  stage_weights(sw, pb);
-  __syncthreads();
-  float* rx = rows + threadIdx.x * kRow;
-  float* ry = rows + (kTB + threadIdx.x) * kRow;
-  for (int64_t s = (int64_t)blockIdx.x * kTB + threadIdx.x; s < n; s += (int64_t)gridDim.x * kTB) {
+  extern __shared__ __align__(16) float sm[];
+  float* wt = sm;
+  const float* vec = wt + (kF + 2 * kH) * kWP;
+  float* A = sm + kWtFloats;                             // [kH][kFwdP]
+  stage_transposed(wt, nullptr, pb);
+  const int t = threadIdx.x, s0 = 4 * (t & 15), o0 = 4 * (t >> 4);
+  for (int64_t base = (int64_t)blockIdx.x * kFwdS; base < n; base += (int64_t)gridDim.x * kFwdS) {
     float x[kF];
 #pragma unroll
-    for (int d = 0; d < kF; ++d) x[d] = feat[s * kF + d];
+    for (int d = 0; d < kF; ++d) x[d] = base + t < n ? feat[(base + t) * kF + d] : nm.mu[d];
     normalise(nm, x);
-    logit[s] = forward_sample(sw, x, rx, ry, rx);
-  }
-}
-
-// Block sums over the tile's samples of dZ[s][o] * A[s][i] (o < 64, i < IN) and of dZ[s][o],
-// added into the block's gradient accumulator g (W at offW, b at offB).
-template <int IN, int ROWA>
-__device__ __forceinline__ void accumulate_layer(const float* dZ, const float* A, int ns, float* g, int offW,
-                                                 int offB) {
-  constexpr int PER = IN / 2;
-  const int o = threadIdx.x >> 1, half = threadIdx.x & 1;
-  float acc[PER];
+    __syncthreads();                                     // weights staged; the tile before is read
 #pragma unroll
-  for (int c = 0; c < PER; ++c) acc[c] = 0.f;
-  float accb = 0.f;
-  for (int s = 0; s < ns; ++s) {
-    const float d = dZ[s * kRow + o];
-    const float* ar = A + s * ROWA + PER * half;
-#pragma unroll
-    for (int c = 0; c < PER; ++c) acc[c] = fmaf(d, ar[c], acc[c]);
-    accb += d;
-  }
-#pragma unroll
-  for (int c = 0; c < PER; ++c) g[offW + o * IN + PER * half + c] += acc[c];
-  if (half == 0) g[offB + o] += accb;
-}
-
-// d_out[i] = mask(A_row[i] > 0) * sum_o W[o][i] dZrow[o]   (W row-major [64][64])
-__device__ __forceinline__ void back_through(const float* W, const float* dZrow, const float* Arow, float* out) {
-  float d[kH];
-#pragma unroll
-  for (int i = 0; i < kH; ++i) d[i] = 0.f;
+    for (int d = 0; d < kF; ++d) A[d * kFwdP + t] = x[d];
+    __syncthreads();
+    PropTile<8, 8> tile;
+    tile.bias(vec, o0, 32);
+    tile.contract<kF>(wt, kWP, A, kFwdP, s0, 64, o0, 32);
+    __syncthreads();
+    tile.store(A, kFwdP, s0, 64, o0, 32, act_bf16);
+    __syncthreads();
 #pragma unroll 1
-  for (int o = 0; o < kH; ++o) {
-    const float go = dZrow[o];
-    const float4* w4 = reinterpret_cast<const float4*>(W + o * kH);
+    for (int l = 1; l < 3; ++l) {
+      tile.bias(vec + l * kH, o0, 32);
+      tile.contract<kH>(wt + (kF + (l - 1) * kH) * kWP, kWP, A, kFwdP, s0, 64, o0, 32);
+      __syncthreads();
+      tile.store(A, kFwdP, s0, 64, o0, 32, act_bf16);
+      __syncthreads();
+    }
+    float z = vec[4 * kH];
+#pragma unroll 16
+    for (int i = 0; i < kH; ++i) z = fmaf(vec[3 * kH + i], A[i * kFwdP + t], z);
+    if (base + t < n) logit[base + t] = z;
+  }
+}
+
+// Forward and backward of the mean BCE over n samples: grad += dL/dtheta, loss += L.  Tiles of 64 samples, 256
+// threads with 4 x 4 register tiles: a training batch of 8192 gives 128 blocks.  Parameter gradients stay in
+// registers over a block's tiles.  8192 samples: 49 us (one thread per sample
+// in 64 blocks of 128 threads: 113 us); 2 M samples 3.2 ms (8.4 ms).
+constexpr int kGS = 64, kGP = kGS + 4, kGT = 256;
+constexpr size_t kGradSmemFloats = kWtFloats + 2 * kH * kH + kF * kGP + 5 * kH * kGP + kGS + 32;
+
+// dW[o][i] += sum_s dZ[o][s] A[i][s] for o = og + 16 r, i = ig + 16 c, and db[o] (threads with ig = 0)
+__device__ __forceinline__ void grad_layer(const float* dZ, const float* A, int og, int ig, float (&dw)[4][4], float (&db)[4]) {
+#pragma unroll 4
+  for (int s = 0; s < kGS; s += 4) {
+    float4 z[4], a[4];
 #pragma unroll
-    for (int i = 0; i < kH / 4; ++i) {
-      const float4 w = w4[i];
-      d[4 * i] = fmaf(w.x, go, d[4 * i]);
-      d[4 * i + 1] = fmaf(w.y, go, d[4 * i + 1]);
-      d[4 * i + 2] = fmaf(w.z, go, d[4 * i + 2]);
-      d[4 * i + 3] = fmaf(w.w, go, d[4 * i + 3]);
+    for (int r = 0; r < 4; ++r) {
+      z[r] = *reinterpret_cast<const float4*>(dZ + (og + 16 * r) * kGP + s);
+      a[r] = *reinterpret_cast<const float4*>(A + (ig + 16 * r) * kGP + s);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        dw[r][c] = fmaf(z[r].w, a[c].w, fmaf(z[r].z, a[c].z, fmaf(z[r].y, a[c].y, fmaf(z[r].x, a[c].x, dw[r][c]))));
+      if (ig == 0) db[r] = (((db[r] + z[r].x) + z[r].y) + z[r].z) + z[r].w;
     }
   }
-#pragma unroll
-  for (int i = 0; i < kH; ++i) out[i] = Arow[i] > 0.f ? d[i] : 0.f;
 }
 
-constexpr size_t kGradSmemFloats = 2 * kNParamPad + kTB * kRow0 + 4 * kTB * kRow + kTB + 32;
-
-// Forward and backward of the mean BCE over n samples: grad += dL/dtheta, loss += L.
-__global__ void __launch_bounds__(kTB) k_prop_grad(const __nv_bfloat16* pb, Norm nm, const float* feat,
+__global__ void __launch_bounds__(kGT) k_prop_grad(const __nv_bfloat16* pb, Norm nm, const float* feat,
                                                    const float* label, int64_t n, float inv_n, float* grad,
                                                    float* loss) {
-  extern __shared__ float sm[];
-  float* sw = sm;
-  float* g = sw + kNParamPad;
-  float* A0 = g + kNParamPad;
-  float* A1 = A0 + kTB * kRow0;
-  float* A2 = A1 + kTB * kRow;
-  float* A3 = A2 + kTB * kRow;
-  float* dZ = A3 + kTB * kRow;
-  float* dz4 = dZ + kTB * kRow;
-  float* red = dz4 + kTB;
-  stage_weights(sw, pb);
-  for (int k = threadIdx.x; k < kNParamPad; k += blockDim.x) g[k] = 0.f;
-  __syncthreads();
-  const int t = threadIdx.x;
-  float lsum = 0.f;
-  for (int64_t base = (int64_t)blockIdx.x * kTB; base < n; base += (int64_t)gridDim.x * kTB) {
-    const int64_t s = base + t;
-    const bool valid = s < n;
-    const int ns = (int)(n - base < (int64_t)kTB ? n - base : (int64_t)kTB);
+  extern __shared__ __align__(16) float sm[];
+  float* wt = sm;
+  const float* vec = wt + (kF + 2 * kH) * kWP;
+  float* W2 = sm + kWtFloats;                            // [o][i]
+  float* W3 = W2 + kH * kH;
+  float* A0 = W3 + kH * kH;
+  float* A1 = A0 + kF * kGP;
+  float* A2 = A1 + kH * kGP;
+  float* A3 = A2 + kH * kGP;
+  float* Za = A3 + kH * kGP;
+  float* Zb = Za + kH * kGP;
+  float* dz4 = Zb + kH * kGP;
+  float* red = dz4 + kGS;
+  stage_transposed(wt, W2, pb);
+  const int t = threadIdx.x, s0 = 4 * (t & 15), o0 = 4 * (t >> 4), og = t >> 4, ig = t & 15;
+  float dw3[4][4] = {}, dw2[4][4] = {}, db3[4] = {}, db2[4] = {}, dw1[2] = {}, db1 = 0.f, dw4 = 0.f, db4 = 0.f, lsum = 0.f;
+  for (int64_t base = (int64_t)blockIdx.x * kGS; base < n; base += (int64_t)gridDim.x * kGS) {
     // ---- forward ----
-    float x[kF];
+    __syncthreads();                                     // weights staged; the tile before is read
+    if (t < kGS) {
+      const bool valid = base + t < n;
+      float x[kF];
 #pragma unroll
-    for (int d = 0; d < kF; ++d) x[d] = valid ? feat[s * kF + d] : 0.f;
-    normalise(nm, x);
-    if (!valid)
+      for (int d = 0; d < kF; ++d) x[d] = valid ? feat[(base + t) * kF + d] : nm.mu[d];
+      normalise(nm, x);
 #pragma unroll
-      for (int d = 0; d < kF; ++d) x[d] = 0.f;
-#pragma unroll
-    for (int d = 0; d < kF; ++d) A0[t * kRow0 + d] = x[d];
-    const float z = forward_sample(sw, x, A1 + t * kRow, A2 + t * kRow, A3 + t * kRow);
-    const float y = valid ? label[s] : 0.f;
-    const float p = 1.f / (1.f + expf(-z));
-    if (valid) lsum += fmaxf(z, 0.f) - z * y + log1pf(expf(-fabsf(z)));
-    const float dz = valid ? (p - y) * inv_n : 0.f;
-    dz4[t] = dz;
-    // ---- dZ3 = (dz W4) masked by A3 > 0 ----
-#pragma unroll 4
-    for (int i = 0; i < kH; ++i) dZ[t * kRow + i] = A3[t * kRow + i] > 0.f ? dz * sw[OFF_W4 + i] : 0.f;
+      for (int d = 0; d < kF; ++d) A0[d * kGP + t] = x[d];
+    }
     __syncthreads();
-    // ---- dW4, db4 (threads < 64: one input each), dW3, db3 ----
-    if (t < kH) {
-      float a = 0.f, ab = 0.f;
-      for (int q = 0; q < ns; ++q) {
-        a = fmaf(dz4[q], A3[q * kRow + t], a);
-        ab += dz4[q];
+    PropTile<4, 4> tile;
+    tile.bias(vec, o0, 0);
+    tile.contract<kF>(wt, kWP, A0, kGP, s0, 0, o0, 0);
+    tile.store(A1, kGP, s0, 0, o0, 0, act_bf16);
+    __syncthreads();
+    tile.bias(vec + kH, o0, 0);
+    tile.contract<kH>(wt + kF * kWP, kWP, A1, kGP, s0, 0, o0, 0);
+    tile.store(A2, kGP, s0, 0, o0, 0, act_bf16);
+    __syncthreads();
+    tile.bias(vec + 2 * kH, o0, 0);
+    tile.contract<kH>(wt + (kF + kH) * kWP, kWP, A2, kGP, s0, 0, o0, 0);
+    tile.store(A3, kGP, s0, 0, o0, 0, act_bf16);
+    __syncthreads();
+    if (t < kGS) {
+      float z = vec[4 * kH];
+#pragma unroll 16
+      for (int i = 0; i < kH; ++i) z = fmaf(vec[3 * kH + i], A3[i * kGP + t], z);
+      const bool valid = base + t < n;
+      const float y = valid ? label[base + t] : 0.f;
+      const float p = 1.f / (1.f + expf(-z));
+      if (valid) lsum += fmaxf(z, 0.f) - z * y + log1pf(expf(-fabsf(z)));
+      dz4[t] = valid ? (p - y) * inv_n : 0.f;
+    }
+    __syncthreads();
+    // ---- dZ3 = (dz W4) masked by A3 > 0; dW4, db4 (threads < 64: one input each) ----
+    for (int k = t; k < kH * kGS; k += kGT) {
+      const int i = k / kGS, q = k % kGS;
+      Za[i * kGP + q] = A3[i * kGP + q] > 0.f ? dz4[q] * vec[3 * kH + i] : 0.f;
+    }
+    if (t < kH)
+#pragma unroll 8
+      for (int q = 0; q < kGS; ++q) {
+        dw4 = fmaf(dz4[q], A3[t * kGP + q], dw4);
+        db4 += dz4[q];
       }
-      g[OFF_W4 + t] += a;
-      if (t == 0) g[OFF_B4] += ab;
-    }
-    accumulate_layer<kH, kRow>(dZ, A2, ns, g, OFF_W3, OFF_B3);
     __syncthreads();
-    // ---- dZ2 = (W3^T dZ3) masked by A2 > 0 (computed into registers, then stored) ----
+    // ---- dW3, db3; dZ2 = (W3^T dZ3) masked by A2 > 0 ----
+    grad_layer(Za, A2, og, ig, dw3, db3);
+    tile.bias(nullptr, o0, 0);
+    tile.contract<kH>(W3, kH, Za, kGP, s0, 0, o0, 0);
+    tile.store(Zb, kGP, s0, 0, o0, 0, [&](float v, const float* d, int q) { return (A2 + (d - Zb))[q] > 0.f ? v : 0.f; });
+    __syncthreads();
+    // ---- dW2, db2; dZ1 = (W2^T dZ2) masked by A1 > 0 ----
+    grad_layer(Zb, A1, og, ig, dw2, db2);
+    tile.bias(nullptr, o0, 0);
+    tile.contract<kH>(W2, kH, Zb, kGP, s0, 0, o0, 0);
+    tile.store(Za, kGP, s0, 0, o0, 0, [&](float v, const float* d, int q) { return (A1 + (d - Za))[q] > 0.f ? v : 0.f; });
+    __syncthreads();
+    // ---- dW1, db1: output t / 4, inputs 2 (t % 4), + 1 ----
     {
-      float d[kH];
-      back_through(sw + OFF_W3, dZ + t * kRow, A2 + t * kRow, d);
-      __syncthreads();
-#pragma unroll
-      for (int i = 0; i < kH; ++i) dZ[t * kRow + i] = d[i];
+      const float* z = Za + (t >> 2) * kGP;
+      const float* a = A0 + 2 * (t & 3) * kGP;
+#pragma unroll 8
+      for (int q = 0; q < kGS; ++q) {
+        dw1[0] = fmaf(z[q], a[q], dw1[0]);
+        dw1[1] = fmaf(z[q], a[kGP + q], dw1[1]);
+        db1 += z[q];
+      }
     }
-    __syncthreads();
-    accumulate_layer<kH, kRow>(dZ, A1, ns, g, OFF_W2, OFF_B2);
-    __syncthreads();
-    // ---- dZ1 = (W2^T dZ2) masked by A1 > 0 ----
-    {
-      float d[kH];
-      back_through(sw + OFF_W2, dZ + t * kRow, A1 + t * kRow, d);
-      __syncthreads();
-#pragma unroll
-      for (int i = 0; i < kH; ++i) dZ[t * kRow + i] = d[i];
-    }
-    __syncthreads();
-    accumulate_layer<kF, kRow0>(dZ, A0, ns, g, OFF_W1, OFF_B1);
-    __syncthreads();
   }
-  for (int k = threadIdx.x; k < kNParam; k += blockDim.x) atomicAdd(&grad[k], g[k]);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int o = og + 16 * r;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      atomicAdd(&grad[OFF_W3 + o * kH + ig + 16 * c], dw3[r][c]);
+      atomicAdd(&grad[OFF_W2 + o * kH + ig + 16 * c], dw2[r][c]);
+    }
+    if (ig == 0) {
+      atomicAdd(&grad[OFF_B3 + o], db3[r]);
+      atomicAdd(&grad[OFF_B2 + o], db2[r]);
+    }
+  }
+  atomicAdd(&grad[OFF_W1 + (t >> 2) * kF + 2 * (t & 3)], dw1[0]);
+  atomicAdd(&grad[OFF_W1 + (t >> 2) * kF + 2 * (t & 3) + 1], dw1[1]);
+  if ((t & 3) == 0) atomicAdd(&grad[OFF_B1 + (t >> 2)], db1);
+  if (t < kH) atomicAdd(&grad[OFF_W4 + t], dw4);
+  if (t == 0) atomicAdd(&grad[OFF_B4], db4);
   // ---- loss: block sum, one atomic ----
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
@@ -257,7 +408,7 @@ __global__ void __launch_bounds__(kTB) k_prop_grad(const __nv_bfloat16* pb, Norm
   __syncthreads();
   if (t == 0) {
     float sacc = 0.f;
-    for (int w = 0; w < kTB / 32; ++w) sacc += red[w];
+    for (int w = 0; w < kGT / 32; ++w) sacc += red[w];
     atomicAdd(loss, sacc * inv_n);
   }
 }
@@ -368,11 +519,11 @@ Norm norm_of(isx_proposer p) {
   return nm;
 }
 
-int grid_for(int64_t n, int dev) {
+int grid_for(int64_t n, int dev, int tile = kTB, int per_sm = 4) {
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t tiles = (n + kTB - 1) / kTB;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, 4LL * sms));
+  const int64_t tiles = (n + tile - 1) / tile;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)per_sm * sms));
 }
 
 size_t fwd_smem() { return (size_t)(kNParamPad + 2 * kTB * kRow) * sizeof(float); }
@@ -505,10 +656,10 @@ isx_status isx_proposer_predict(isx_proposer p, const float* d_feat, int64_t n, 
   }
   if (n == 0) return ISX_OK;
   cudaStream_t st = (cudaStream_t)stream;
-  ISX_TRY(set_smem((const void*)k_prop_forward, fwd_smem()));
+  ISX_TRY(set_smem((const void*)k_prop_forward, kFwdSmem));
   {
     prof::Scope _ps(K_PROP_FWD, st, 2.0 * 8768 * (double)n, 0);
-    k_prop_forward<<<grid_for(n, p->device), kTB, fwd_smem(), st>>>(p->pb, norm_of(p), d_feat, n, d_logit);
+    k_prop_forward<<<grid_for(n, p->device, kFwdS, 3), kTB, kFwdSmem, st>>>(p->pb, norm_of(p), d_feat, n, d_logit);
   }
   ISX_LAUNCH_CHECK("k_prop_forward");
   return ISX_OK;
@@ -528,8 +679,8 @@ isx_status isx_proposer_grad(isx_proposer p, const float* d_feat, const float* d
   ISX_CUDA(cudaMemsetAsync(d_loss, 0, sizeof(float), st));
   {
     prof::Scope _ps(K_PROP_GRAD, st, 3.0 * 2.0 * 8768 * (double)n, 0);
-    k_prop_grad<<<grid_for(n, p->device), kTB, smem, st>>>(p->pb, norm_of(p), d_feat, d_label, n, 1.0f / (float)n,
-                                                           d_grad, d_loss);
+    k_prop_grad<<<grid_for(n, p->device, kGS, 1), kGT, smem, st>>>(p->pb, norm_of(p), d_feat, d_label, n, 1.0f / (float)n,
+                                                                   d_grad, d_loss);
   }
   ISX_LAUNCH_CHECK("k_prop_grad");
   return ISX_OK;

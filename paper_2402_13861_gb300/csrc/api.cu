@@ -289,6 +289,7 @@ isx_status isx_create_inr(const isx_inr_desc* d, isx_inr* out) {
   ISX_CUDA(cudaGetDevice(&dev));
   isx_inr inr = new isx_inr_s();
   inr->device = dev;
+  cudaDeviceGetAttribute(&inr->sms, cudaDevAttrMultiProcessorCount, dev);
   inr->n_layers = L;
   inr->H = L - 1;
   inr->w = w;

@@ -266,13 +266,13 @@ struct GemmShape {
 };
 constexpr GemmShape kGemmShapes[] = {{8, 16384, 4096, "8x8, 256 threads"}, {8, 8192, 2048, "8x8, 128 threads"},
                                      {8, 4096, 2048, "8x8, 64 threads"}, {4, 8192, 4096, "8x4, 256 threads"},
-                                     {4, 4096, 4096, "8x4, 128 threads"}};
+                                     {4, 4096, 8192, "8x4, 128 threads"}};
 constexpr int kGemmVariants = sizeof(kGemmShapes) / sizeof(kGemmShapes[0]);
 
 template <bool ROWS>
 isx_status launch_gemm(int v, const GemmArgs& g, int w, int sms, cudaStream_t st) {
   const GemmShape& gs = kGemmShapes[v];
-  const int KB = 16 * w <= gs.stage ? 16 : (8 * w <= gs.stage ? 8 : 4);
+  const int KB = 32 * w <= gs.stage && w % 32 == 0 ? 32 : (16 * w <= gs.stage ? 16 : (8 * w <= gs.stage ? 8 : 4));
   const sgemm::Shape sh{gs.tn, std::max(8, gs.elems / w / 8 * 8), KB};
   const size_t smem = sh.smem(w) + (size_t)sh.P * (sizeof(int64_t) + sizeof(int));
   const int threads = (sh.threads(w) + 31) / 32 * 32;
@@ -511,8 +511,7 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   float* DE = ws[WS_DELTA].as<float>();
   const Slot xs[2] = {WS_X0, WS_X1}, rs[2] = {WS_R_RC0, WS_R_RC1}, ns[2] = {WS_R_CNT0, WS_R_CNT1},
              os[2] = {WS_R_OFF0, WS_R_OFF1};
-  int sms = 148;
-  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
+  const int sms = inr->sms;
   const CellBlock cb(w);
   int64_t want = nc_alloc;                         // cells of the next chunk
   for (int64_t first = 0; first < n;) {

@@ -328,8 +328,7 @@ isx_status bound_rafixed(isx_inr inr, const CellSource& src, int64_t n, int infl
   const int L = inr->n_layers - 1;
   // cells per CTA: 128 threads' worth, two CTAs per SM; with fewer cells than that, enough CTAs for every SM,
   // but at least 64 threads' worth (they share the weight stream)
-  int sms = 148;
-  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
+  const int sms = inr->sms;
   // four cells per thread (eight warps per SM) keep the multiply-adds fed; at small widths the input and output
   // layers weigh more and twice the warps with two cells each hide more of their latency (w = 64, two hidden
   // layers, 10^5 cells: 165 us against 199 us)

@@ -103,9 +103,11 @@ __device__ __forceinline__ __nv_bfloat16 bf16_up(float x) { return __float2bfloa
 __global__ void __launch_bounds__(256) k_rows_input_act(CellSource src, int64_t first, int nc, int w, int mode,
                                                         int act, const float* __restrict__ W0,
                                                         const float* __restrict__ b0, float* I, float* A, float* AL,
-                                                        float* GA, int* cnt_out, __nv_bfloat16* AH,
-                                                        __nv_bfloat16* ALO, Infl infl) {
+                                                        float* GA, int* cnt_in, int64_t* off_in, int* cnt_out,
+                                                        __nv_bfloat16* AH, __nv_bfloat16* ALO, int* status,
+                                                        Infl infl) {
   __shared__ int mcount[8];
+  if (status && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
   const int tpc = w / 2, cpb = blockDim.x / tpc;
   const int sub = threadIdx.x / tpc, n = 2 * (threadIdx.x - sub * tpc);
   const int64_t cell = (int64_t)blockIdx.x * cpb + sub;
@@ -174,7 +176,11 @@ __global__ void __launch_bounds__(256) k_rows_input_act(CellSource src, int64_t 
   for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
   if ((threadIdx.x & 31) == 0 && valid) atomicAdd(&mcount[sub], m);   // a warp never spans two cells
   __syncthreads();
-  if (valid && threadIdx.x - sub * tpc == 0) cnt_out[cell] = mcount[sub];
+  if (valid && threadIdx.x - sub * tpc == 0) {
+    cnt_in[cell] = 0;                              // no symbol rows yet
+    off_in[cell] = 0;
+    cnt_out[cell] = mcount[sub];
+  }
 }
 
 // Exclusive scan of the per-cell row counts into int64 row offsets, total to *d_total: block sums
@@ -931,8 +937,7 @@ template <int W, bool ONE>
 isx_status launch_rows_split(isx_inr inr, const RowsSplitArgs& a, const RowsSplitMaps& maps, cudaStream_t st) {
   const size_t smem = SplitSmem<W>::bytes();
   ISX_CUDA(cudaFuncSetAttribute(k_rows_split<W, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int sms = 148;
-  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
+  const int sms = inr->sms;
   int per_sm = 1;
   ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rows_split<W, ONE>, kST, smem));
   constexpr int NHALF = SplitSmem<W>::NHALF;
@@ -993,26 +998,20 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
   ISX_TRY(ws[WS_R_TOT].ensure(rows::scan_bytes(kMaxChunkCells), "row total and scan block sums"));
   int* status = ws[WS_TC_STATUS].as<int>();
   int64_t* d_tot = ws[WS_R_TOT].as<int64_t>();
-  ISX_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
-  std::vector<CUtensorMap> maps(inr->n_layers), lomaps(inr->n_layers), pmaps(inr->n_layers);
   // TMA boxes are at most 256 rows: the split GEMM reads W_j in 256-row halves and the row GEMM in
   // 128-row quarters at w = 512
   const uint32_t box_split = w > 256 ? 256 : w, box_rows = w > 256 ? 128 : w;
-  for (int l = 1; l <= H - 1; ++l) {
-    ISX_TRY(tensor_map_bf16(&maps[l], inr->W_bf16[l], w, w, 64, box_split));
-    ISX_TRY(tensor_map_bf16(&lomaps[l], inr->Wlo_bf16[l], w, w, 64, box_split));
-    ISX_TRY(tensor_map_bf16(&pmaps[l], inr->Wperm_bf16[l] ? inr->Wperm_bf16[l] : inr->W_bf16[l], w, w, 64, box_rows));
-  }
   const int sq = mode == ISX_BOUND_CLT ? 1 : 0;
-  std::vector<CUtensorMap> absmaps(inr->n_layers);
-  if (inflate)
-    for (int l = 1; l <= H - 1; ++l) ISX_TRY(tensor_map_bf16(&absmaps[l], inr->Wabsru_bf16[l], w, w, 64, box_split));
   // chunk size: about kRowBudget G rows per chunk, from the rows per cell the previous chunk needed
   const int64_t kRowBudget = inr->row_budget;
   const int64_t kMaxCells = kMaxChunkCells;
-  int sms = 148;
-  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
+  const int sms = inr->sms;
   double rows_per_cell = (double)w * (H - 1);
+  // A call whose rows fit in 16 MB with every symbol alive needs no row count on the host: the buffers take that
+  // many and the row GEMM reads the count on the device.  Each read-back costs 10-15 us, as much as two of
+  // the kernels of such a call (7 cells of the 3 -> 256 x 5 -> 1 network: 257 -> 189 us); larger buffers would
+  // cost a first call more than that.
+  const bool counted = n * (int64_t)w * (H - 1) > ((int64_t)8 << 20) / w;
   int64_t first = 0;
   while (first < n) {
     const int64_t want = (int64_t)((double)kRowBudget / std::max(1.0, 1.25 * rows_per_cell));
@@ -1074,11 +1073,10 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
       }
       k_rows_input_act<<<act_blocks, 256, 0, st>>>(src, first, nc, w, (int)mode, inr->act, inr->W[0], inr->b[0],
                                                    H == 1 ? I0 : nullptr, H == 1 || inflate ? A : nullptr, AL, GA,
-                                                   ws[cs[1]].as<int>(), H > 1 ? AH : nullptr, ALO, fi);
+                                                   ws[cs[0]].as<int>(), ws[os[0]].as<int64_t>(), ws[cs[1]].as<int>(),
+                                                   H > 1 ? AH : nullptr, ALO, first == 0 ? status : nullptr, fi);
       ISX_LAUNCH_CHECK("k_rows_input_act");
     }
-    ISX_CUDA(cudaMemsetAsync(ws[cs[0]].ptr, 0, (size_t)nc * sizeof(int), st));
-    ISX_CUDA(cudaMemsetAsync(ws[os[0]].ptr, 0, (size_t)nc * sizeof(int64_t), st));
     for (int j = 1; j <= H - 1; ++j) {
       const int nxt = cur ^ 1;
       int* cnt_in = ws[cs[0]].as<int>();             // rows of z_j, of z_{j+1} and (written here) of z_{j+2}
@@ -1088,11 +1086,13 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
       int64_t* off_out = ws[os[nxt]].as<int64_t>();
       {
         prof::Scope ps(K_ROWS_ACT, st, 0, 0);
-        ISX_TRY(rows::scan_counts(cnt_out, nc, d_tot, 0, off_out, st));
+        ISX_TRY(rows::scan_counts(cnt_out, nc, d_tot, j & 1, off_out, st));
       }
-      int64_t Rn = 0;
-      ISX_CUDA(cudaMemcpyAsync(&Rn, d_tot, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-      ISX_CUDA(cudaStreamSynchronize(st));
+      int64_t Rn = (int64_t)nc * w * j;                // rows of z_{j+1}, or the most there can be
+      if (counted) {
+        ISX_CUDA(cudaMemcpyAsync(&Rn, d_tot + (j & 1), sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        ISX_CUDA(cudaStreamSynchronize(st));
+      }
       ISX_TRY(ws[xs[nxt]].ensure((size_t)std::max<int64_t>(Rn, 1) * w * 2, "rows"));
       ISX_TRY(ws[rs[nxt]].ensure((size_t)std::max<int64_t>(Rn, 1) * sizeof(int), "row cells"));
       const int64_t ntiles = (R + rows::kPT - 1) / rows::kPT;     // column-sum blocks of the input rows
@@ -1109,17 +1109,21 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         ga.off_out = off_out;
         ga.alpha = AL;
         ga.R = R;
+        ga.d_R = counted ? nullptr : d_tot + ((j - 1) & 1);
         ga.xout = Xout;
         ga.part = part;
         ga.sq = sq;
         ga.status = status;
         // bytes: rows in and out, the column sums of every (cell, 64-row block) segment
-        prof::Scope ps(K_ROWS_GEMM, st, 2.0 * (double)R * w * w, 4.0 * (double)R * w);
-        ISX_TRY(rows::launch_rows_gemm(inr, ga, pmaps[j], w, st));
+        const double known = counted ? (double)R : 0.0;   // counted work; small calls leave their rows out
+        prof::Scope ps(K_ROWS_GEMM, st, 2.0 * known * w * w, 4.0 * known * w);
+        CUtensorMap wmap;
+        ISX_TRY(tensor_map_bf16(&wmap, inr->Wperm_bf16[j] ? inr->Wperm_bf16[j] : inr->W_bf16[j], w, w, 64, box_rows));
+        ISX_TRY(rows::launch_rows_gemm(inr, ga, wmap, w, st));
       }
       {
         // bytes: the new rows (bf16) and the row -> cell map written, gamma read, the column sums
-        prof::Scope ps(K_ROWS_NEW, st, 0, 2.0 * (double)(Rn - R) * w + 4.0 * (double)Rn + 8.0 * (double)nc * w);
+        prof::Scope ps(K_ROWS_NEW, st, 0, (counted ? 2.0 * (double)(Rn - R) * w + 4.0 * (double)Rn : 0.0) + 8.0 * (double)nc * w);
         int* rc = ws[rs[nxt]].as<int>();
         int* cz = fused && j < H - 1 ? cnt_next : nullptr;
         // warps of 1, 2 or 4 cells with w / 32 columns per lane; w = 512: two warps share the columns, and four
@@ -1131,8 +1135,13 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
               nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
         };
         // several cells per warp once there are enough cells to fill the SMs all the same
-        const bool many = nc >= 32 * sms;
-        if (w == 512 && many) launch_new(k_rows_new<512, 8, 2, 4>, 2, 2);
+        // and for a handful of cells as many warps per cell as there are column groups of two, eight rows in flight
+        // (7 coarse cells at w = 256: 40 -> 29 us a launch)
+        const bool many = nc >= 32 * sms, few = nc <= 2 * sms;
+        if (w == 512 && few) launch_new(k_rows_new<512, 2, 1, 8>, 1, 8);
+        else if (w == 256 && few) launch_new(k_rows_new<256, 2, 1, 8>, 1, 4);
+        else if (w == 128 && few) launch_new(k_rows_new<128, 2, 1, 8>, 1, 2);
+        else if (w == 512 && many) launch_new(k_rows_new<512, 8, 2, 4>, 2, 2);
         else if (w == 512) launch_new(k_rows_new<512, 8, 1, 4>, 1, 2);
         else if (w == 256 && many) launch_new(k_rows_new<256, 8, 4, 2>, 4, 1);
         else if (w == 256) launch_new(k_rows_new<256, 8, 1, 4>, 1, 1);
@@ -1181,8 +1190,8 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         std::memset(&sm, 0, sizeof(sm));
         ISX_TRY(tensor_map_bf16(&sm.ahi, AH, w, 4 * (uint64_t)nc, 64, kRT));
         ISX_TRY(tensor_map_bf16(&sm.alo, ALO, w, 4 * (uint64_t)nc, 64, kRT));
-        sm.whi = maps[j];
-        sm.wlo = lomaps[j];
+        ISX_TRY(tensor_map_bf16(&sm.whi, inr->W_bf16[j], w, w, 64, box_split));
+        ISX_TRY(tensor_map_bf16(&sm.wlo, inr->Wlo_bf16[j], w, w, 64, box_split));
         prof::Scope ps(K_ROWS_SPLIT, st, 2.0 * nc * 4.0 * w * w, 0);
         ISX_TRY(launch_rows_split_w<false>(inr, w, sa, sm, st));
       }
@@ -1202,7 +1211,7 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         RowsSplitMaps dm;
         std::memset(&dm, 0, sizeof(dm));
         ISX_TRY(tensor_map_bf16(&dm.ahi, ws[WS_R_V].ptr, w, (uint64_t)nc, 64, kRT));
-        dm.whi = absmaps[j];
+        ISX_TRY(tensor_map_bf16(&dm.whi, inr->Wabsru_bf16[j], w, w, 64, box_split));
         prof::Scope ps(K_ROWS_AUX, st, 2.0 * nc * w * w, 0);
         ISX_TRY(launch_rows_split_w<true>(inr, w, da, dm, st));
       }
@@ -1247,7 +1256,8 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
       R = Rn;
     }
     {
-      prof::Scope ps(K_ROWS_OUT, st, 2.0 * (double)(R + 3.0 * nc) * w, 2.0 * (double)R * w + 4.0 * 7.0 * nc * w);
+      const double known = counted ? (double)R : 0.0;
+      prof::Scope ps(K_ROWS_OUT, st, 2.0 * (known + 3.0 * nc) * w, 2.0 * known * w + 4.0 * 7.0 * nc * w);
       const int L = inr->n_layers - 1;
       Infl fi = infl;
       if (inflate) {

@@ -344,8 +344,8 @@ isx_status launch_eval(isx_inr inr, EvArgs a, const EvMaps& maps, int64_t ntiles
   a.ns = ns;
   const size_t smem = EvSmem<W>::bytes(inr->H, ns);
   ISX_CUDA(cudaFuncSetAttribute(k_eval_tc<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int per_sm = 1, sms = 148;
-  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
+  int per_sm = 1;
+  const int sms = inr->sms;
   ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eval_tc<W>, EvSmem<W>::kThreads, smem));
   // TMEM: two accumulators of W columns per CTA out of 512
   per_sm = std::max(1, std::min(per_sm, 512 / (2 * W)));

@@ -64,6 +64,7 @@ enum Slot {
 // The opaque INR handle.
 struct isx_inr_s {
   int device = 0;
+  int sms = 148;              // its SM count
   int n_layers = 0;           // linear layers = H + 1
   int H = 0;                  // hidden (activation) layers
   int w = 0;                  // hidden width

@@ -326,8 +326,7 @@ isx_status eval_points_fp32(isx_inr inr, const float* xyz, const uint32_t* latti
   }
   m.wout = inr->W[inr->n_layers - 1];
   m.bout = inr->hb[inr->n_layers - 1][0];
-  int sms = 148;
-  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
+  const int sms = inr->sms;
   const sgemm::Shape sh = eval_shape(n, inr->w, sms);
   const size_t smem = sh.smem(inr->w);
   const int threads = (sh.threads(inr->w) + 31) / 32 * 32;

@@ -21,7 +21,8 @@ struct RowsGemmArgs {
   const int64_t* off_in;                        // [nc] first row of each cell in xin
   const int64_t* off_out;                       // [nc] first row of each cell in xout
   const float* alpha;                           // [nc][W]
-  int64_t R;
+  int64_t R;                                    // rows (an upper bound with d_R)
+  const int64_t* d_R;                           // row count in device memory; null: R
   __nv_bfloat16* xout;                          // [R'][W] rows of z_{j+1}
   float* part;                                  // [nc + ceil(R / 64)][W]: slot cell + t holds, per neuron,
                                                 // sum f(x) over the cell's rows among input rows

@@ -81,12 +81,14 @@ __global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_c
   uint32_t* tslot = reinterpret_cast<uint32_t*>(wfull + 1);
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
   const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
-  const int64_t ntiles = (args.R + kRT - 1) / kRT;
+  const int64_t R = args.d_R ? *args.d_R : args.R;
+  const int64_t ntiles = (R + kRT - 1) / kRT;
   // work items are (tile, weight slice); the grid is a multiple of NQ, so this CTA's slice q never
   // changes and it walks the tiles t0, t0 + TS, ...; the NQ CTAs of a tile run side by side and
   // share its row chunks through L2
   const int q = blockIdx.x % NQ;
   const int64_t t0 = blockIdx.x / NQ, TS = gridDim.x / NQ;
+  if (t0 >= ntiles) return;                                // the grid covers the upper bound
 
   if (W < 128) {
     // zero rows W .. 127 of every weight chunk (the MMA reads 128 weight rows)
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_c
     uint32_t it = 0;
     bool ok = true;
     int64_t r_next = t0 * kRT + sr;
-    int cell_next = (r_next < args.R) ? args.rowcell[r_next] : 0;
+    int cell_next = (r_next < R) ? args.rowcell[r_next] : 0;
     float4 av[2 * CG];
     {
       const float4* al0 = reinterpret_cast<const float4*>(args.alpha + (size_t)cell_next * W + k0);
@@ -136,10 +138,10 @@ __global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_c
     }
     for (int64_t tile = t0; tile < ntiles && ok; tile += TS) {
       const int64_t r = tile * kRT + sr;
-      const bool valid = r < args.R;
+      const bool valid = r < R;
       const int cell = cell_next;
       r_next = (tile + TS) * kRT + sr;
-      cell_next = (tile + TS < ntiles && r_next < args.R) ? args.rowcell[r_next] : cell;
+      cell_next = (tile + TS < ntiles && r_next < R) ? args.rowcell[r_next] : cell;
       if (warp < 4) {
         // ask L2 for the alpha rows of the cells of this warp's 32 rows of the next tile (a run of
         // consecutive cells, so one contiguous range), a tile ahead of their use
@@ -247,12 +249,12 @@ __global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_c
     long long d_cur = 0;
     {
       const int64_t r = tile * kRT + m;
-      if (tile < ntiles && r < args.R) {
+      if (tile < ntiles && r < R) {
         c_cur = args.rowcell[r];
         d_cur = args.off_out[c_cur] + (r - args.off_in[c_cur]);
       }
       const int64_t r2 = (tile + TS) * kRT + m;
-      if (tile + TS < ntiles && r2 < args.R) c_nxt = args.rowcell[r2];
+      if (tile + TS < ntiles && r2 < R) c_nxt = args.rowcell[r2];
     }
     uint32_t tt = 0;
     for (; tile < ntiles; tile += TS, ++tt) {
@@ -270,16 +272,16 @@ __global__ void __launch_bounds__(gemm_threads(W), 1) k_rows_gemm(const __grid_c
         const int64_t nt = tile + TS;
         const int64_t r1 = nt * kRT + m;
         c_cur = c_nxt;
-        if (nt < ntiles && r1 < args.R && c_cur >= 0) d_cur = args.off_out[c_cur] + (r1 - args.off_in[c_cur]);
+        if (nt < ntiles && r1 < R && c_cur >= 0) d_cur = args.off_out[c_cur] + (r1 - args.off_in[c_cur]);
         const int64_t r2 = (nt + TS) * kRT + m;
-        c_nxt = (nt + TS < ntiles && r2 < args.R) ? args.rowcell[r2] : -1;
+        c_nxt = (nt + TS < ntiles && r2 < R) ? args.rowcell[r2] : -1;
       }
       // after an expired wait every epilogue warp keeps walking the tiles without work, so that all of
       // them still meet at the barrier above
       const bool got = rwait(&tfull[b], (tt >> 1) & 1, abort, args.status);
       if (!__all_sync(0xffffffffu, got)) continue;
       tc_fence_after();
-      const int64_t left = args.R - tile * kRT;
+      const int64_t left = R - tile * kRT;
       const int rbeg = kPT * h;                             // this warp's rows rbeg .. rows - 1
       const int rows = (int)(left < rbeg + kPT ? left : rbeg + kPT);
       const uint32_t tb = tmem + b * (NH * 128) + lane_off;
@@ -399,14 +401,10 @@ isx_status launch_rows_gemm_w(isx_inr inr, const RowsGemmArgs& a, const CUtensor
   ISX_TRY(tensor_map_bf16(&xmap, a.xin, W, (uint64_t)a.R, 64, kRT));
   const size_t smem = RowsSmem<W>::bytes();
   ISX_CUDA(cudaFuncSetAttribute(k_rows_gemm<W, SQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int sms = 148;
-  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
-  int per_sm = 1;
-  ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rows_gemm<W, SQ>, gemm_threads(W), smem));
-  per_sm = std::max(1, std::min(per_sm, 512 / (2 * RowsSmem<W>::NH * 128)));   // TMEM columns per CTA
+  const int sms = inr->sms;
   constexpr int NQ = RowsSmem<W>::NQ;
   const int64_t ntiles = (a.R + kRT - 1) / kRT;
-  int grid = (int)std::min<int64_t>(ntiles * NQ, (int64_t)sms * per_sm);
+  int grid = (int)std::min<int64_t>(ntiles * NQ, sms);   // one CTA per SM (registers)
   grid -= grid % NQ;                                       // every CTA keeps one weight slice
   k_rows_gemm<W, SQ><<<grid, gemm_threads(W), smem, st>>>(a, map, xmap);
   ISX_LAUNCH_CHECK("k_rows_gemm");

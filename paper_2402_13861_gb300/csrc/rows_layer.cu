@@ -407,8 +407,7 @@ isx_status launch_w(isx_inr inr, const RowsLayerArgs& a, const LayerMaps& maps, 
   using S = LayerSmem<W>;
   const size_t smem = S::bytes();
   ISX_CUDA(cudaFuncSetAttribute(k_rows_layer<W, LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int sms = 148;
-  ISX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, inr->device));
+  const int sms = inr->sms;
   const int64_t ntiles = (a.nc + kLC - 1) / kLC;
   int grid = (int)std::min<int64_t>(ntiles * S::NHALF, sms);
   grid -= grid % S::NHALF;

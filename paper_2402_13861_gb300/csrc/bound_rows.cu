@@ -183,6 +183,110 @@ __global__ void __launch_bounds__(256) k_rows_input_act(CellSource src, int64_t 
   }
 }
 
+// The same for UP with ReLU, four cells per warp and turn.  erfc and exp for every (cell, neuron) bounded
+// k_rows_input_act there, although most neurons are far from the kink: here a warp keeps mu and sigma of its 4 x 64
+// (cell, neuron) pairs in shared memory, lists those near the kink and evaluates them 32 at a time.
+// 512^3 extraction: 78 -> 58 ms (row scans included), 262144 cells at w = 256 0.72 -> 0.59 ms.
+constexpr int kActC = 4;
+__global__ void __launch_bounds__(256, 4) k_rows_input_relu(CellSource src, int64_t first, int nc, int w,
+                                                            const float* __restrict__ W0, const float* __restrict__ b0,
+                                                            float* I, float* A, float* AL, float* GA, int* cnt_in,
+                                                            int64_t* off_in, int* cnt_out, __nv_bfloat16* AH,
+                                                            __nv_bfloat16* ALO, int* status) {
+  struct Warp {
+    float mu[kActC][64], al[kActC][64], be[kActC][64], ga[kActC][64];   // al holds sigma until the pair is evaluated
+    uint8_t list[kActC * 64];
+  };
+  __shared__ Warp warps[8];
+  __shared__ int mcount[8][kActC];
+  if (status && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+  const int tpc = w / 2, cpb = blockDim.x / tpc;
+  const int sub = threadIdx.x / tpc, u = threadIdx.x - sub * tpc, n = 2 * u, lane = threadIdx.x & 31;
+  const int64_t cell0 = ((int64_t)blockIdx.x * cpb + sub) * kActC;
+  if (threadIdx.x < 8 * kActC) mcount[threadIdx.x / kActC][threadIdx.x % kActC] = 0;
+  __syncthreads();
+  Warp& s = warps[threadIdx.x >> 5];
+  if (sub < cpb && cell0 < nc) {
+    const int cells = (int)min((int64_t)kActC, nc - cell0);
+    float wv[2][3], bv[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      bv[e] = b0[n + e];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) wv[e][d] = W0[3 * (n + e) + d];
+    }
+    auto box = [&](int c, float* xc, float* h) {
+      cell_box(src, first + cell0 + c, 0, xc, h);
+      for (int d = 0; d < 3; ++d) h[d] *= 0.57735026918962576f;   // uniform on [-h, h] has std h / sqrt 3
+    };
+    int nq = 0;
+#pragma unroll 1
+    for (int c = 0; c < cells; ++c) {
+      float xc[3], h[3], mu[2], al[2];
+      box(c, xc, h);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        mu[e] = fmaf(wv[e][2], xc[2], fmaf(wv[e][1], xc[1], fmaf(wv[e][0], xc[0], bv[e])));
+        const float i0 = h[0] * wv[e][0], i1 = h[1] * wv[e][1], i2 = h[2] * wv[e][2];
+        const float sg = sqrtf(fmaf(i2, i2, fmaf(i0, i0, i1 * i1)));
+        const bool need = relu_clt_mixed(mu[e], sg);
+        const unsigned bm = __ballot_sync(0xffffffffu, need);
+        if (need) s.list[nq + __popc(bm & ((1u << lane) - 1u))] = (uint8_t)(64 * c + 2 * lane + e);
+        nq += __popc(bm);
+        al[e] = need ? sg : (mu[e] > 0.0f ? 1.0f : (mu[e] == 0.0f ? 0.5f : 0.0f));
+      }
+      *reinterpret_cast<float2*>(&s.mu[c][2 * lane]) = make_float2(mu[0], mu[1]);
+      *reinterpret_cast<float2*>(&s.al[c][2 * lane]) = make_float2(al[0], al[1]);
+      *reinterpret_cast<float2*>(&s.be[c][2 * lane]) = make_float2(0.0f, 0.0f);
+      *reinterpret_cast<float2*>(&s.ga[c][2 * lane]) = make_float2(0.0f, 0.0f);
+    }
+    __syncwarp();
+    for (int i = lane; i < nq; i += 32) {
+      const int k = s.list[i];
+      const Lin r = relu_clt((&s.mu[0][0])[k], (&s.al[0][0])[k]);
+      (&s.al[0][0])[k] = r.alpha;
+      (&s.be[0][0])[k] = r.beta;
+      (&s.ga[0][0])[k] = r.gamma;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int c = 0; c < cells; ++c) {
+      float xc[3], h[3];
+      box(c, xc, h);
+      const float2 mu = *reinterpret_cast<const float2*>(&s.mu[c][2 * lane]), al = *reinterpret_cast<const float2*>(&s.al[c][2 * lane]);
+      const float2 be = *reinterpret_cast<const float2*>(&s.be[c][2 * lane]), ga = *reinterpret_cast<const float2*>(&s.ga[c][2 * lane]);
+      const float2 ce = make_float2(fmaf(al.x, mu.x, be.x), fmaf(al.y, mu.y, be.y));
+      const int64_t cell = cell0 + c;
+      const size_t o = (size_t)cell * w + n;
+      *reinterpret_cast<float2*>(AL + o) = al;
+      *reinterpret_cast<float2*>(GA + o) = ga;
+      if (A) *reinterpret_cast<float2*>(A + o) = ce;
+      auto put = [&](size_t i, float v0, float v1) {
+        const __nv_bfloat162 hh = __floats2bfloat162_rn(v0, v1);
+        const float2 hf = __bfloat1622float2(hh);
+        *reinterpret_cast<__nv_bfloat162*>(AH + i) = hh;
+        *reinterpret_cast<__nv_bfloat162*>(ALO + i) = __floats2bfloat162_rn(v0 - hf.x, v1 - hf.y);
+      };
+      const size_t r0 = (size_t)cell * 4 * w + n;
+      if (AH) put(r0, ce.x, ce.y);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const float x = h[d] * wv[0][d], y = h[d] * wv[1][d];
+        if (I) *reinterpret_cast<float2*>(I + ((size_t)cell * 3 + d) * w + n) = make_float2(x, y);
+        if (AH) put(r0 + (size_t)(d + 1) * w, al.x * x, al.y * y);
+      }
+      const int m = __popc(__ballot_sync(0xffffffffu, ga.x != 0.0f)) + __popc(__ballot_sync(0xffffffffu, ga.y != 0.0f));
+      if (lane == 0) atomicAdd(&mcount[sub][c], m);  // a warp never spans two cells
+    }
+  }
+  __syncthreads();
+  if (sub < cpb && u < kActC && cell0 + u < nc) {
+    cnt_in[cell0 + u] = 0;                         // no symbol rows yet
+    off_in[cell0 + u] = 0;
+    cnt_out[cell0 + u] = mcount[sub][u];
+  }
+}
+
 // Exclusive scan of the per-cell row counts into int64 row offsets, total to *d_total: block sums
 // of 1024 counts, one block scanning the sums, then every block's scan plus its offset.
 constexpr int kScanB = 1024;
@@ -1071,7 +1175,13 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         fi.RAD = ws[WS_RAD].as<float>();
         fi.SLK = ws[WS_DELTA].as<float>();
       }
-      k_rows_input_act<<<act_blocks, 256, 0, st>>>(src, first, nc, w, (int)mode, inr->act, inr->W[0], inr->b[0],
+      const bool relu = sq && inr->act == ISX_ACT_RELU && nc >= 16 * sms;   // enough cells to group them
+      if (relu)
+        k_rows_input_relu<<<(act_blocks + kActC - 1) / kActC, 256, 0, st>>>(
+            src, first, nc, w, inr->W[0], inr->b[0], H == 1 ? I0 : nullptr, H == 1 ? A : nullptr, AL, GA, ws[cs[0]].as<int>(),
+            ws[os[0]].as<int64_t>(), ws[cs[1]].as<int>(), H > 1 ? AH : nullptr, ALO, first == 0 ? status : nullptr);
+      else
+        k_rows_input_act<<<act_blocks, 256, 0, st>>>(src, first, nc, w, (int)mode, inr->act, inr->W[0], inr->b[0],
                                                    H == 1 ? I0 : nullptr, H == 1 || inflate ? A : nullptr, AL, GA,
                                                    ws[cs[0]].as<int>(), ws[os[0]].as<int64_t>(), ws[cs[1]].as<int>(),
                                                    H > 1 ? AH : nullptr, ALO, first == 0 ? status : nullptr, fi);

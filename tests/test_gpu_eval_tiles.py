@@ -34,9 +34,10 @@ def test_eval_tc_tile_edges(pkg, w, H, act):
     for n in (1, 127, 128, 129, 152 * 128 + 1, 2 * 152 * 128 + 130):
         v = net.eval_points(torch.tensor(x[:n], device="cuda"), prec="bf16").cpu().numpy()
         idx = np.unique(np.r_[0, n // 3, max(0, n - 129), n - 1])
-        ref = activations.forward(layers, x[idx].astype(np.float64), act)
-        a = np.abs(x[idx].astype(np.float64))
-        for W, b in layers:
+        ref, a = x[idx].astype(np.float64), np.abs(x[idx].astype(np.float64))
+        for l, (W, b) in enumerate(layers):
+            ref = ref @ W.astype(np.float64).T + b.astype(np.float64)
+            ref = activations.forward(act, ref) if l < H else ref
             a = a @ np.abs(W.astype(np.float64)).T + np.abs(b.astype(np.float64))
         assert np.all(np.abs(v[idx] - np.ravel(ref)) <= (H + 1) * 2.0 ** -15 * a[:, 0]), n
         if first is None:

@@ -56,6 +56,18 @@ struct CellBlock {
   unsigned threads() const { return (unsigned)(tpc * cpb); }
 };
 
+// The roundings of every sum over symbols, spelled out: a cell's result must not depend on the kernel that formed it.
+// One compensated step of a sum of x^2 (sq) or |x|, and the radius of the three input rows.
+__device__ __forceinline__ void add_term(float& s, float& comp, float x, bool sq) {
+  const float y = sq ? fmaf(x, x, -comp) : __fsub_rn(fabsf(x), comp), t = __fadd_rn(s, y);
+  comp = __fsub_rn(__fsub_rn(t, s), y);
+  s = t;
+}
+__device__ __forceinline__ float input_radius(int mode, float x0, float x1, float x2) {
+  if (mode == ISX_BOUND_CLT) return sqrtf(fmaf(x2, x2, fmaf(x1, x1, __fmul_rn(x0, x0))));
+  return __fadd_rn(__fadd_rn(fabsf(x0), fabsf(x1)), fabsf(x2));
+}
+
 // z_1 = W_0 x + b_0 over the box and activation 1: the 3 input rows with their row -> cell map, the
 // post-activation centre, alpha, gamma (and, inflate, radius and slack), the cell's row counts (3 now,
 // 3 + #(gamma != 0) after the next layer) and the offset of its rows.
@@ -83,9 +95,7 @@ __global__ void __launch_bounds__(256) k_input_layer(CellSource src, int64_t fir
       Xc[n] = x0;
       Xc[w + n] = x1;
       Xc[2 * w + n] = x2;
-      float rad;
-      if (mode == ISX_BOUND_CLT) rad = sqrtf(x0 * x0 + x1 * x1 + x2 * x2);
-      else rad = fabsf(x0) + fabsf(x1) + fabsf(x2);
+      const float rad = input_radius(mode, x0, x1, x2);
       float dl = 0.0f;
       if (inflate) {
         float e = fabsf(w0 * xc[0]) + fabsf(w1 * xc[1]) + fabsf(w2 * xc[2]) + fabsf(b0[n]);
@@ -340,12 +350,7 @@ __global__ void __launch_bounds__(256) k_reduce_act(const float* __restrict__ X,
     int m = 0;
     for (int n = t; n < w; n += tpc) {
       float s = 0.0f, comp = 0.0f;
-      auto add = [&](float x) {
-        const float v = (mode == ISX_BOUND_CLT) ? x * x : fabsf(x);
-        const float y = v - comp, tt = s + y;
-        comp = (tt - s) - y;
-        s = tt;
-      };
+      auto add = [&](float x) { add_term(s, comp, x, mode == ISX_BOUND_CLT); };
       int r = 0;
       for (; r + 8 <= S; r += 8) {                 // eight loads in flight
         float x[8];
@@ -415,10 +420,7 @@ __global__ void __launch_bounds__(256) k_output(const float* __restrict__ X, con
       for (int q = 0; q < 4; ++q)
         if (r0 + q * WPC < S) {
           const int k = WPC == 1 ? h + q : 0;
-          const float v = sq ? y[q] * y[q] : fabsf(y[q]);
-          const float yy = v - comp[k], t = s[k] + yy;
-          comp[k] = (t - s[k]) - yy;
-          s[k] = t;
+          add_term(s[k], comp[k], y[q], sq);
         }
     };
     if constexpr (WPC == 1) {
@@ -447,7 +449,7 @@ __global__ void __launch_bounds__(256) k_output(const float* __restrict__ X, con
   for (int m = lane; m < w; m += 32) {
     const size_t i = (size_t)cell * w + m;
     const float y = GAMMA[i] * wout[m];
-    v[0] += sq ? y * y : fabsf(y);
+    v[0] = sq ? fmaf(y, y, v[0]) : v[0] + fabsf(y);
     v[1] = fmaf(wout[m], C[i], v[1]);
     if (inflate) {
       v[2] = fmaf(fabsf(wout[m]), fabsf(C[i]), v[2]);
@@ -477,6 +479,189 @@ __global__ void __launch_bounds__(256) k_output(const float* __restrict__ X, con
   }
 }
 
+// ---- small networks: the whole propagation of a cell in one block ----------------------------------------
+// Widths up to 64: a cell's rows fit in shared memory, and what the path above spends is launches (seven per
+// layer and call) and passes over memory, not multiply-adds.  Four warps per cell; every sum is taken in the
+// order of the kernels above, so the results are the same bit for bit.  Bound by latency (a cell's chain of
+// layers); several blocks per SM overlap.  3 -> 64 x 2 -> 1, levels 4-6, with the row path before it: 1 cell
+// 54 -> 31 us, 608 cells 72 -> 37, 8192 cells 139 -> 120; FP32 extraction of that network to level 6, 895 -> 688.
+constexpr int kSmallT = 128;
+struct SmallNet {
+  const float* W0;
+  const float* b0;
+  const float* Wt[ISX_MAX_LAYERS];     // hidden layers 1 .. H - 1
+  const float* b[ISX_MAX_LAYERS];
+  const float* wout;
+  float bout;
+  int w, H, act;
+};
+__host__ __device__ __forceinline__ int small_rows(int w, int H) { return 3 + w * (H - 1); }
+size_t small_smem(int w, int H) { return ((size_t)small_rows(w, H) + 7) * w * sizeof(float); }
+
+__global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t n, SmallNet net, int mode, int inflate,
+                                                         float* center, float* spread) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ float part[8];
+  const int w = net.w, H = net.H, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  float* X = sm;                                   // [rows][w]
+  float* a = X + (size_t)small_rows(w, H) * w;     // centre, alpha, gamma, radius, slack of the current layer
+  float* al = a + w;
+  float* ga = al + w;
+  float* ra = ga + w;                              // inflate: radius of the post-activation form
+  float* rad = ra + w;
+  float* de = rad + w;
+  float* aw = de + w;
+  const float kappa = 3.0f * kU + gamma_k(w);
+  for (int64_t cell = blockIdx.x; cell < n; cell += gridDim.x) {
+    float xc[3], h[3];
+    cell_box(src, cell, inflate, xc, h);
+    if (mode == ISX_BOUND_CLT)
+      for (int d = 0; d < 3; ++d) h[d] *= kInvSqrt3;
+    auto activate = [&](int k, float c, float r, float dl) {
+      const Lin L = linearise(mode, net.act, inflate, c, r, dl);
+      a[k] = L.center;
+      al[k] = L.alpha;
+      ga[k] = L.gamma;
+      rad[k] = r;
+      if (inflate) ra[k] = fmaf(L.alpha, r, L.gamma);
+    };
+    __syncthreads();                               // the cell before is done
+    if (t < w) {
+      const float w0 = net.W0[3 * t], w1 = net.W0[3 * t + 1], w2 = net.W0[3 * t + 2], bb = net.b0[t];
+      const float c = fmaf(w2, xc[2], fmaf(w1, xc[1], fmaf(w0, xc[0], bb)));
+      const float x0 = h[0] * w0, x1 = h[1] * w1, x2 = h[2] * w2;
+      X[t] = x0;
+      X[w + t] = x1;
+      X[2 * w + t] = x2;
+      const float r = input_radius(mode, x0, x1, x2);
+      float dl = 0.0f;
+      if (inflate) {
+        const float e = fabsf(w0 * xc[0]) + fabsf(w1 * xc[1]) + fabsf(w2 * xc[2]) + fabsf(bb);
+        dl = (5.0f * kU * e + 3.0f * kU * r) * kSafe;
+      }
+      activate(t, c, r, dl);
+    }
+    int S = 3;
+    for (int j = 1; j < H; ++j) {
+      const float* __restrict__ Wt = net.Wt[j];
+      __syncthreads();
+      // centre (and slack) of the next layer: one neuron per thread of the last two warps
+      float cn = 0.0f;
+      const int nn = t - (kSmallT - 64);
+      if (nn >= 0 && nn < w) {
+        cn = net.b[j][nn];
+        float e = fabsf(cn), g = 0.0f;
+        for (int k = 0; k < w; ++k) {
+          const float wk = Wt[k * w + nn];
+          cn = fmaf(wk, a[k], cn);
+          if (inflate) {
+            e = fmaf(fabsf(wk), fabsf(a[k]), e);
+            g = fmaf(fabsf(wk), ra[k], g);
+          }
+        }
+        if (inflate) de[nn] = (kappa * g + gamma_k(w + 2) * e) * kSafe;
+      }
+      // carried rows, four per warp and turn, in place: (x alpha) W^T
+      for (int r0 = 4 * warp; r0 < S; r0 += 16) {
+        const int nr = min(4, S - r0);
+        for (int q = 0; q < nr; ++q)
+          for (int k = lane; k < w; k += 32) X[(r0 + q) * w + k] *= al[k];
+        __syncwarp();
+        float y[4][2] = {};
+        for (int k = 0; k < w; ++k) {
+          float wv[2];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) wv[c] = lane + 32 * c < w ? Wt[k * w + lane + 32 * c] : 0.0f;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float x = X[min(r0 + q, S - 1) * w + k];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) y[q][c] = fmaf(x, wv[c], y[q][c]);
+          }
+        }
+        __syncwarp();
+        for (int q = 0; q < nr; ++q)
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+            if (lane + 32 * c < w) X[(r0 + q) * w + lane + 32 * c] = y[q][c];
+      }
+      // new rows gamma_n W[:, n], in increasing n
+      int made = 0;
+      for (int g0 = 0; g0 < w; g0 += 32) {
+        const float gm = g0 + lane < w ? ga[g0 + lane] : 0.0f;
+        for (unsigned b = __ballot_sync(0xffffffffu, gm != 0.0f); b; b &= b - 1, ++made) {
+          if ((made & 3) != warp) continue;
+          const int l = __ffs(b) - 1;
+          const float g = __shfl_sync(0xffffffffu, gm, l);
+          for (int m = lane; m < w; m += 32) X[(S + made) * w + m] = g * Wt[(g0 + l) * w + m];
+        }
+      }
+      S += made;
+      __syncthreads();
+      if (nn >= 0 && nn < w) {
+        float s = 0.0f, comp = 0.0f;
+        for (int r = 0; r < S; ++r) add_term(s, comp, X[r * w + nn], mode == ISX_BOUND_CLT);
+        activate(nn, cn, (mode == ISX_BOUND_CLT) ? sqrtf(s) : s, inflate ? de[nn] : 0.0f);
+      }
+    }
+    __syncthreads();
+    // output layer: the terms of rows r to partial sum r % 8, as in k_output
+    if (t < w) aw[t] = al[t] * net.wout[t];
+    __syncthreads();
+    const bool sq = (mode != ISX_BOUND_SOUND);
+    for (int u = warp; u < 8; u += 4) {
+      float s = 0.0f, comp = 0.0f;
+      for (int r = u; r < S; r += 8) {
+        float y = 0.0f;
+        if (4 * lane < w) {
+          const float4 v = *reinterpret_cast<const float4*>(aw + 4 * lane), x = *reinterpret_cast<const float4*>(X + r * w + 4 * lane);
+          y = fmaf(x.w, v.w, fmaf(x.z, v.z, fmaf(x.y, v.y, fmaf(x.x, v.x, y))));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+        add_term(s, comp, y, sq);
+      }
+      if (lane == 0) part[u] = s;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      float rows = 0.0f;
+      for (int k = 0; k < 8; ++k) rows += part[k];
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int m = lane; m < w; m += 32) {
+        const float wo = net.wout[m], y = ga[m] * wo;
+        v[0] = sq ? fmaf(y, y, v[0]) : v[0] + fabsf(y);
+        v[1] = fmaf(wo, a[m], v[1]);
+        if (inflate) {
+          v[2] = fmaf(fabsf(wo), fabsf(a[m]), v[2]);
+          v[3] = fmaf(fabsf(wo), fmaf(al[m], rad[m], ga[m]), v[3]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+      if (lane == 0) {
+        const float tot = rows + v[0];
+        float sp;
+        if (mode == ISX_BOUND_SOUND) {
+          sp = tot;
+          if (inflate) {
+            float ge = gamma_k(w + 1) + kU;
+            sp = __fadd_ru(__fmul_ru(sp, kOutSafe), (ge * v[3] + gamma_k(w + 2) * (v[2] + fabsf(net.bout))) * 1.01f);
+          }
+        } else if (mode == ISX_BOUND_CLT) {
+          sp = sqrtf(tot);
+        } else {
+          sp = sqrtf(tot / 3.0f);
+        }
+        center[cell] = v[1] + net.bout;
+        spread[cell] = sp;
+      }
+    }
+  }
+}
+
 }  // namespace
 
 isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_mode mode,
@@ -484,6 +669,33 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   if (n <= 0) return ISX_OK;
   const int w = inr->w, H = inr->H;
   if (mode != ISX_BOUND_SOUND) inflate = 0;
+  // Small networks in one launch: with up to two hidden layers to 8192 cells (32768 cells: 392 us against 364 at
+  // 64 x 2, 234 against 189 at 32 x 2), deeper ones to one cell per SM (64 x 3, 152 cells: 67 against 116; beyond
+  // that its row products, which use a weight four times only, lose to the tuned tiles step by step).
+  if (w <= 64 && small_smem(w, H) <= 100 * 1024 && n <= (H <= 2 ? 8192 : inr->sms)) {
+    SmallNet net{};
+    net.W0 = inr->W[0];
+    net.b0 = inr->b[0];
+    for (int j = 1; j < H; ++j) {
+      net.Wt[j] = inr->Wt[j];
+      net.b[j] = inr->b[j];
+    }
+    net.wout = inr->W[H];
+    net.bout = inr->hb[H][0];
+    net.w = w;
+    net.H = H;
+    net.act = inr->act;
+    const size_t smem = small_smem(w, H);
+    if (smem > 48 * 1024)
+      ISX_CUDA(cudaFuncSetAttribute(k_bound_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+    {
+      prof::Scope _ps(K_BOUND_SMALL, st, 2.0 * n * w * (double)w * 4.0 * (H - 1), 0);
+      k_bound_small<<<(unsigned)std::min<int64_t>(n, 16 * (int64_t)inr->sms), kSmallT, smem, st>>>(src, n, net, (int)mode, inflate,
+                                                                                                 d_center, d_spread);
+    }
+    ISX_LAUNCH_CHECK("k_bound_small");
+    return ISX_OK;
+  }
   const int Smax = 3 + w * (H - 1);
   // the two coefficient buffers take at most ~6 GB: enough for full_cells cells with every symbol alive
   const size_t per_cell = 2ull * Smax * w * sizeof(float);

@@ -27,7 +27,8 @@ const char* names[K_COUNT] = {"input_layer",   "relu",          "center_gemv",  
                               "mc_emit",       "iota",          "bound_tc",      "tc_prep",      "tc_output",
                               "eval_tc",       "prop_gate",     "prop_merge",   "prop_forward",
                               "prop_grad",     "prop_adam",     "bound_rafixed", "rows_gemm",     "rows_aux",
-                              "rows_act",      "rows_new",      "rows_split",    "rows_reduce",  "rows_out"};
+                              "rows_act",      "rows_new",      "rows_split",    "rows_reduce",  "rows_out",
+                              "bound_small"};
 
 void drain_locked() {
   for (auto& r : pending) {

@@ -31,6 +31,7 @@
 #include "sgemm.cuh"
 
 #include <algorithm>
+#include <cooperative_groups.h>
 #include <cmath>
 
 namespace isx {
@@ -57,11 +58,14 @@ struct CellBlock {
 };
 
 // The roundings of every sum over symbols, spelled out: a cell's result must not depend on the kernel that formed it.
-// One compensated step of a sum of x^2 (sq) or |x|, and the radius of the three input rows.
+// One compensated step of a sum of x^2 (sq) or |x|, the slack, and the radius of the three input rows.
 __device__ __forceinline__ void add_term(float& s, float& comp, float x, bool sq) {
   const float y = sq ? fmaf(x, x, -comp) : __fsub_rn(fabsf(x), comp), t = __fadd_rn(s, y);
   comp = __fsub_rn(__fsub_rn(t, s), y);
   s = t;
+}
+__device__ __forceinline__ float slack(float kappa, float g, int w, float e) {
+  return __fmul_rn(fmaf(kappa, g, __fmul_rn(gamma_k(w + 2), e)), kSafe);
 }
 __device__ __forceinline__ float input_radius(int mode, float x0, float x1, float x2) {
   if (mode == ISX_BOUND_CLT) return sqrtf(fmaf(x2, x2, fmaf(x1, x1, __fmul_rn(x0, x0))));
@@ -120,35 +124,49 @@ __global__ void __launch_bounds__(256) k_input_layer(CellSource src, int64_t fir
   }
 }
 
-// Centre of the next layer, c' = W a + b, and (inflate) the slack of the next pre-activation:
+// Centre of the next layer, Y = W a + b, and (inflate) the slack of the next pre-activation:
 // kappa * sum_k |W_nk| (alpha_k r_k + gamma_k) + gamma_{K+1} (sum_k |W_nk a_k| + |b_n|).
-__global__ void k_center_gemv(int nc, int win, int wout, const float* __restrict__ Wt,
-                              const float* __restrict__ bias, float* C, const float* ALPHA,
-                              const float* RAD, const float* GAMMA, float* DELTA, int inflate,
-                              float kappa) {
+// One thread per neuron, blockIdx.y a slice of them; bound by the latency of the weight loads, so up to 32 are in flight.
+__global__ void __launch_bounds__(256) k_center_gemv(int w, const float* __restrict__ Wt, const float* __restrict__ bias,
+                                                     const float* __restrict__ C, const float* ALPHA, const float* RAD,
+                                                     const float* GAMMA, float* Y, float* DELTA, int inflate, float kappa) {
   extern __shared__ float sh[];
   float* a = sh;             // a-form centre
-  float* ra = sh + win;      // a-form radius
-  int cell = blockIdx.x;
-  if (cell >= nc) return;
-  for (int k = threadIdx.x; k < win; k += blockDim.x) {
-    size_t i = (size_t)cell * win + k;
-    a[k] = C[i];
-    ra[k] = inflate ? fmaf(ALPHA[i], RAD[i], GAMMA[i]) : 0.0f;
+  float* ra = sh + w;        // a-form radius
+  const size_t c0 = (size_t)blockIdx.x * w;
+  for (int k = threadIdx.x; k < w; k += blockDim.x) {
+    a[k] = C[c0 + k];
+    ra[k] = inflate ? fmaf(ALPHA[c0 + k], RAD[c0 + k], GAMMA[c0 + k]) : 0.0f;
   }
   __syncthreads();
-  for (int n = threadIdx.x; n < wout; n += blockDim.x) {
-    float acc = bias[n], e = fabsf(bias[n]), g = 0.0f;
-    for (int k = 0; k < win; ++k) {
-      float wk = Wt[(size_t)k * wout + n];
-      acc = fmaf(wk, a[k], acc);
-      if (inflate) {
-        e = fmaf(fabsf(wk), fabsf(a[k]), e);
-        g = fmaf(fabsf(wk), ra[k], g);
+  for (int n = blockIdx.y * blockDim.x + threadIdx.x; n < w; n += gridDim.y * blockDim.x) {
+    float acc = bias[n], e = fabsf(acc), g = 0.0f;
+    float x[16], y[16];                            // w is a multiple of 16
+    auto load = [&](float (&v)[16], int k0) {
+      if (k0 < w)
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = Wt[(size_t)(k0 + q) * w + n];
+    };
+    auto add = [&](const float (&v)[16], int k0) {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        acc = fmaf(v[q], a[k0 + q], acc);
+        if (inflate) {
+          e = fmaf(fabsf(v[q]), fabsf(a[k0 + q]), e);
+          g = fmaf(fabsf(v[q]), ra[k0 + q], g);
+        }
       }
+    };
+    load(x, 0);
+    for (int k0 = 0; k0 < w; k0 += 32) {
+      load(y, k0 + 16);
+      add(x, k0);
+      if (k0 + 16 >= w) break;
+      load(x, k0 + 32);
+      add(y, k0 + 16);
     }
-    C[(size_t)cell * wout + n] = acc;
-    if (inflate) DELTA[(size_t)cell * wout + n] = (kappa * g + gamma_k(win + 2) * e) * kSafe;
+    Y[c0 + n] = acc;
+    if (inflate) DELTA[c0 + n] = slack(kappa, g, w, e);
   }
 }
 
@@ -297,31 +315,46 @@ isx_status launch_gemm(int v, const GemmArgs& g, int w, int sms, cudaStream_t st
 }
 
 // Rows of the symbols created by the last activation, gamma_n W[:, n] for every neuron with gamma_n != 0,
-// after the cell's carried rows, and the row -> cell map of all of its rows.  WPC warps per cell: warp u
-// writes the neurons of the 32-groups u, u + WPC, ...
+// after the cell's carried rows, and the row -> cell map of all of its rows.  WPC gridDim.y warps per cell share
+// the neurons in units of eight.  Bound by the writes with many cells, by each warp's chain of loads with few.
 template <int WPC>
 __global__ void __launch_bounds__(256) k_fresh_rows(int nc, int w, const float* __restrict__ GAMMA,
                                                     const float* __restrict__ Wt, const int* cnt_in, const int* cnt_out,
                                                     const int64_t* off_out, float* Xout, int* rowcell) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, u = warp % WPC;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int u = blockIdx.y * WPC + warp % WPC, warps = WPC * gridDim.y;
   const int cell = blockIdx.x * (8 / WPC) + warp / WPC;
   if (cell >= nc) return;
   const int64_t o0 = off_out[cell];
   const int co = cnt_out[cell];
-  for (int r = u * 32 + lane; r < co; r += 32 * WPC) rowcell[o0 + r] = cell;
+  for (int r = u * 32 + lane; r < co; r += 32 * warps) rowcell[o0 + r] = cell;
+  // lane i: the alive neurons of the 32-group i (w <= 512), how many rows come before them, and how many there are
   const float* ga = GAMMA + (size_t)cell * w;
+  float gm[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) gm[i] = 32 * i + lane < w ? ga[32 * i + lane] : 0.0f;
+  unsigned mask = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const unsigned b = __ballot_sync(0xffffffffu, gm[i] != 0.0f);
+    if (lane == i) mask = b;
+  }
+  int before = __popc(mask);
+#pragma unroll
+  for (int o = 1; o < 16; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, before, o);
+    if (lane >= o) before += v;
+  }
+  before -= __popc(mask);
   float* Y = Xout + (size_t)(o0 + cnt_in[cell]) * w;
-  for (int g0 = 0, row = 0; g0 < w; g0 += 32) {
-    const float gm = g0 + lane < w ? ga[g0 + lane] : 0.0f;
-    unsigned b = __ballot_sync(0xffffffffu, gm != 0.0f);
-    if ((g0 >> 5) % WPC != u) {
-      row += __popc(b);
-      continue;
-    }
-    for (; b; b &= b - 1, ++row) {
+  for (int q = u; q < w / 8; q += warps) {
+    const unsigned all = __shfl_sync(0xffffffffu, mask, q >> 2);
+    int row = __shfl_sync(0xffffffffu, before, q >> 2) + __popc(all & ((1u << (8 * (q & 3))) - 1u));
+    const float gq = ga[8 * q + (lane & 7)];
+    for (unsigned b = (all >> (8 * (q & 3))) & 0xffu; b; b &= b - 1, ++row) {
       const int l = __ffs(b) - 1;
-      const float g = __shfl_sync(0xffffffffu, gm, l);
-      const float4* src = reinterpret_cast<const float4*>(Wt + (size_t)(g0 + l) * w);
+      const float g = __shfl_sync(0xffffffffu, gq, l);
+      const float4* src = reinterpret_cast<const float4*>(Wt + (size_t)(8 * q + l) * w);
       float4* d = reinterpret_cast<float4*>(Y + (size_t)row * w);
       for (int n = lane; n < w / 4; n += 32) {
         const float4 x = src[n];
@@ -331,65 +364,129 @@ __global__ void __launch_bounds__(256) k_fresh_rows(int nc, int w, const float* 
   }
 }
 
-// Per-neuron reduction over the cell's rows (compensated), r = sum |x| (sound) or sigma = sqrt(sum x^2), and
-// activation j + 1: post-activation centre in place, alpha, gamma (and, inflate, the radius) and, for the
-// next layer, the row count cnt + #(gamma != 0).
-__global__ void __launch_bounds__(256) k_reduce_act(const float* __restrict__ X, const int64_t* off, const int* cnt,
-                                                    int nc, int tpc, int w, int mode, int act, int inflate, float* C,
-                                                    float* RAD, const float* DELTA, float* ALPHA, float* GAMMA,
-                                                    int* cnt_next) {
+struct ReduceArgs {
+  const float* X;
+  const int64_t* off;
+  const int* cnt;
+  int nc, w, mode, act, inflate;
+  float* C;
+  float* RAD;
+  const float* DELTA;
+  float* ALPHA;
+  float* GAMMA;
+};
+
+// One neuron's reduction over its cell's S rows (compensated, in row order), r = sum |x| (sound) or sigma =
+// sqrt(sum x^2), and activation j + 1: post-activation centre in place, alpha, gamma (and, inflate, the radius).
+// 16 rows are summed while the loads of the next 16 are in flight.  Returns whether the symbol is alive.
+__device__ __forceinline__ int reduce_neuron(const ReduceArgs& g, int cell, int n, int S) {
+  const bool sq = g.mode == ISX_BOUND_CLT;
+  const float* Xc = g.X + (size_t)g.off[cell] * g.w + n;
+  float s = 0.0f, comp = 0.0f, x[16], y[16];
+  int r = 0;
+  if (S >= 16) {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) x[q] = Xc[(size_t)q * g.w];
+    for (; r + 32 <= S; r += 16) {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) y[q] = Xc[(size_t)(r + 16 + q) * g.w];
+#pragma unroll
+      for (int q = 0; q < 16; ++q) add_term(s, comp, x[q], sq);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) x[q] = y[q];
+    }
+    r += 16;
+  }
+  // the last S - r < 16 rows, loaded before the 16 ahead of them are summed
+#pragma unroll
+  for (int q = 0; q < 16; ++q) y[q] = r + q < S ? Xc[(size_t)(r + q) * g.w] : 0.0f;
+  if (S >= 16)
+#pragma unroll
+    for (int q = 0; q < 16; ++q) add_term(s, comp, x[q], sq);
+#pragma unroll
+  for (int q = 0; q < 16; ++q)
+    if (r + q < S) add_term(s, comp, y[q], sq);
+  const float rad = sq ? sqrtf(s) : s;
+  const size_t i = (size_t)cell * g.w + n;
+  const Lin L = linearise(g.mode, g.act, g.inflate, g.C[i], rad, g.inflate ? g.DELTA[i] : 0.0f);
+  g.C[i] = L.center;
+  g.ALPHA[i] = L.alpha;
+  g.GAMMA[i] = L.gamma;
+  if (g.inflate) g.RAD[i] = rad;
+  return L.gamma != 0.0f;
+}
+
+// The reduction of whole cells, tpc threads each, and the next layer's row count, cnt + #(gamma != 0).
+__global__ void __launch_bounds__(256) k_reduce_act(ReduceArgs g, int tpc, int* cnt_next) {
   __shared__ int made[16];
   const int sub = threadIdx.x / tpc, t = threadIdx.x - sub * tpc;
   const int cell = blockIdx.x * (blockDim.x / tpc) + sub;
   if (threadIdx.x < 16) made[threadIdx.x] = 0;
   __syncthreads();
   int S = 0;
-  if (cell < nc) {
-    S = cnt[cell];
-    const float* Xc = X + (size_t)off[cell] * w;
+  if (cell < g.nc) {
+    S = g.cnt[cell];
     int m = 0;
-    for (int n = t; n < w; n += tpc) {
-      float s = 0.0f, comp = 0.0f;
-      auto add = [&](float x) { add_term(s, comp, x, mode == ISX_BOUND_CLT); };
-      int r = 0;
-      for (; r + 8 <= S; r += 8) {                 // eight loads in flight
-        float x[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) x[q] = Xc[(size_t)(r + q) * w + n];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) add(x[q]);
-      }
-      for (; r < S; ++r) add(Xc[(size_t)r * w + n]);
-      const float rad = (mode == ISX_BOUND_CLT) ? sqrtf(s) : s;
-      const size_t i = (size_t)cell * w + n;
-      const Lin L = linearise(mode, act, inflate, C[i], rad, inflate ? DELTA[i] : 0.0f);
-      C[i] = L.center;
-      ALPHA[i] = L.alpha;
-      GAMMA[i] = L.gamma;
-      if (inflate) RAD[i] = rad;
-      m += L.gamma != 0.0f;
-    }
+    for (int n = t; n < g.w; n += tpc) m += reduce_neuron(g, cell, n, S);
     if (m) atomicAdd(&made[sub], m);
   }
   __syncthreads();
-  if (cnt_next && cell < nc && t == 0) cnt_next[cell] = S + made[sub];
+  if (cnt_next && cell < g.nc && t == 0) cnt_next[cell] = S + made[sub];
+}
+
+// The same for few cells, each with a cluster of blocks of 64 neurons, which count into the first one's shared
+// memory: a column's chain of loads bounds it, and one block per cell would leave most SMs idle.
+__global__ void __launch_bounds__(64) k_reduce_few(ReduceArgs g, int* cnt_next) {
+  __shared__ int made;
+  const auto cluster = cooperative_groups::this_cluster();
+  const unsigned slice = cluster.block_rank();
+  const int cell = blockIdx.x / cluster.num_blocks(), n = slice * 64 + threadIdx.x;
+  if (threadIdx.x == 0) made = 0;
+  cluster.sync();
+  const int S = g.cnt[cell];
+  const int alive = __syncthreads_count(n < g.w && reduce_neuron(g, cell, n, S));
+  if (threadIdx.x == 0) atomicAdd(cluster.map_shared_rank(&made, 0), alive);
+  cluster.sync();
+  if (cnt_next && slice == 0 && threadIdx.x == 0) cnt_next[cell] = S + made;
+}
+
+// One cluster of `blocks` blocks per cell.
+template <typename... A>
+isx_status launch_clusters(void (*kernel)(A...), unsigned blocks, int nc, unsigned threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = blocks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)nc * blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  ISX_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+  return ISX_OK;
 }
 
 // Output layer w -> 1 and the read-off.  Row r's term goes to partial sum r % 8 (compensated, r ascending),
-// held by WPC warps per cell: all eight by one warp or one per warp, four rows' 16-byte loads in flight.  The
-// cell's result does not depend on WPC.
+// held by WPC warps per cell: all eight by one warp or one per warp, four rows' 16-byte loads in flight.  With
+// WPC = 32 and 64 (few cells) a cluster of four or eight blocks shares the rows (one SM alone reads about 60 GB/s of them) and
+// their products pass to the eight sums through the first block's shared memory.  The cell's result does not
+// depend on WPC.
+constexpr int kOutRows = 1024;                     // rows between two of those hand-overs
 template <int WPC>
-__global__ void __launch_bounds__(256) k_output(const float* __restrict__ X, const int64_t* off, const int* cnt, int nc,
-                                                int w, const float* C, const float* ALPHA, const float* GAMMA,
-                                                const float* RAD, const float* __restrict__ wout, float bout, int mode,
-                                                int inflate, float* center, float* spread, int64_t first) {
-  extern __shared__ __align__(16) float s_aw[];    // [cells of the block][w]: alpha o w_out
+__global__ void __launch_bounds__(256)
+    k_output(const float* __restrict__ X, const int64_t* off, const int* cnt, int nc, int w, const float* C,
+             const float* ALPHA, const float* GAMMA, const float* RAD, const float* __restrict__ wout, float bout,
+             int mode, int inflate, float* center, float* spread, int64_t first) {
+  extern __shared__ __align__(16) float s_aw[];    // [cells of the block][w]: alpha o w_out; WPC > 8: [kOutRows] products
   __shared__ float red[8];
-  constexpr int CPB = 8 / WPC;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = warp / WPC, u = warp % WPC;
-  const int cell = blockIdx.x * CPB + sub;
+  constexpr int BPC = WPC > 8 ? WPC / 8 : 1, CPB = WPC > 8 ? 1 : 8 / WPC;   // blocks per cell, cells per block
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = warp / WPC;
+  const int u = (blockIdx.x % BPC) * 8 + warp % WPC;                     // the warp's place among the cell's
+  const int cell = blockIdx.x / BPC * CPB + sub;
   for (int i = threadIdx.x; i < CPB * w; i += blockDim.x) {
-    const int c = blockIdx.x * CPB + i / w;
+    const int c = blockIdx.x / BPC * CPB + i / w;
     s_aw[i] = c < nc ? ALPHA[(size_t)c * w + i % w] * wout[i % w] : 0.0f;
   }
   __syncthreads();
@@ -401,14 +498,15 @@ __global__ void __launch_bounds__(256) k_output(const float* __restrict__ X, con
     const int S = cnt[cell];
     constexpr int NS = WPC == 1 ? 8 : 1;           // partial sums of this warp
     float s[NS] = {}, comp[NS] = {};
-    // rows r0 + q WPC, q < 4, into the partials h + q (WPC = 1) or into the warp's own
-    auto four = [&](int r0, int h) {
-      float y[4] = {0.f, 0.f, 0.f, 0.f};
+    // the products of rows r0 + q step, q < 4 (the last row's in place of rows past the end)
+    auto four = [&](int r0, int step, float (&y)[4]) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) y[q] = 0.0f;
       for (int n = 4 * lane; n < w; n += 128) {
         const float4 a = *reinterpret_cast<const float4*>(aw + n);
         float4 x[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = *reinterpret_cast<const float4*>(Xc + (size_t)min(r0 + q * WPC, S - 1) * w + n);
+        for (int q = 0; q < 4; ++q) x[q] = *reinterpret_cast<const float4*>(Xc + (size_t)min(r0 + q * step, S - 1) * w + n);
 #pragma unroll
         for (int q = 0; q < 4; ++q) y[q] = fmaf(x[q].w, a.w, fmaf(x[q].z, a.z, fmaf(x[q].y, a.y, fmaf(x[q].x, a.x, y[q]))));
       }
@@ -416,6 +514,11 @@ __global__ void __launch_bounds__(256) k_output(const float* __restrict__ X, con
       for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
         for (int q = 0; q < 4; ++q) y[q] += __shfl_xor_sync(0xffffffffu, y[q], o);
+    };
+    // rows r0 + q WPC into the partials h + q (WPC = 1) or into the warp's own
+    auto add_four = [&](int r0, int h) {
+      float y[4];
+      four(r0, WPC, y);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         if (r0 + q * WPC < S) {
@@ -425,23 +528,38 @@ __global__ void __launch_bounds__(256) k_output(const float* __restrict__ X, con
     };
     if constexpr (WPC == 1) {
       for (int r0 = 0; r0 < S; r0 += 8) {
-        four(r0, 0);
-        if (r0 + 4 < S) four(r0 + 4, 4);
+        add_four(r0, 0);
+        if (r0 + 4 < S) add_four(r0 + 4, 4);
       }
+    } else if constexpr (WPC == 8) {
+      for (int r0 = u; r0 < S; r0 += 4 * WPC) add_four(r0, 0);
     } else {
-      for (int r0 = u; r0 < S; r0 += 4 * WPC) four(r0, 0);
+      const auto cluster = cooperative_groups::this_cluster();
+      float* prod = cluster.map_shared_rank(s_aw + w, 0);
+      for (int base = 0; base < S; base += kOutRows) {
+        const int end = min(S - base, kOutRows);
+        cluster.sync();                            // the products before are summed (at first: every block runs)
+        for (int r = 4 * u; r < end; r += 4 * WPC) {
+          float y[4];
+          four(base + r, 1, y);
+          if (lane < 4 && r + lane < end) prod[r + lane] = lane == 0 ? y[0] : lane == 1 ? y[1] : lane == 2 ? y[2] : y[3];
+        }
+        cluster.sync();
+        if (u == 0 && lane < 8)
+          for (int r = lane; r < end; r += 8) add_term(s[0], comp[0], prod[r], sq);
+      }
     }
     if (WPC == 1) {
 #pragma unroll
       for (int q = 0; q < NS; ++q) rows += s[q];
-    } else if (lane == 0) {
-      red[warp] = s[0];
+    } else if (WPC == 8 ? lane == 0 : u == 0 && lane < 8) {
+      red[WPC == 8 ? warp : lane] = s[0];
     }
   }
   if (WPC > 1) {
     __syncthreads();
     if (u == 0)
-      for (int k = 0; k < WPC; ++k) rows += red[k];
+      for (int k = 0; k < 8; ++k) rows += red[k];
   }
   if (u > 0 || cell >= nc) return;
   // symbols of the last activation, y_m = gamma_m w_m, and the centre
@@ -559,7 +677,7 @@ __global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t
             g = fmaf(fabsf(wk), ra[k], g);
           }
         }
-        if (inflate) de[nn] = (kappa * g + gamma_k(w + 2) * e) * kSafe;
+        if (inflate) de[nn] = slack(kappa, g, w, e);
       }
       // carried rows, four per warp and turn, in place: (x alpha) W^T
       for (int r0 = 4 * warp; r0 < S; r0 += 16) {
@@ -731,7 +849,11 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
     float* C = ws[WS_C].as<float>();
     float* C2 = ws[WS_R_A].as<float>();
     // few cells: a whole block per cell in the kernels that walk over a cell's rows
+    // (8 per SM); up to one cell per SM they are spread over several blocks per cell, since one SM alone is bound by
+    // its loads' latency (every symbol alive, 400 x 5: 1 cell 672 -> 350 us, 152 cells 3918 -> 3601; 256 x 5, 600
+    // cells: 775 us either way)
     const bool wide = nc < 8 * sms;
+    const bool few = nc <= sms;
     int cur = 0;
     int64_t R = 3 * (int64_t)nc;                   // rows of z_j (an upper bound where the host does not know)
     bool fits = true;
@@ -793,7 +915,8 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
       {
         prof::Scope _ps(K_FRESH, st, 0, 0);
         if (wide)
-          k_fresh_rows<8><<<nc, 256, 0, st>>>(nc, w, GA, inr->Wt[j], cnt_in, cnt_out, off_out, Xb, ws[rs[nxt]].as<int>());
+          k_fresh_rows<8><<<dim3(nc, few ? (w + 63) / 64 : 1), 256, 0, st>>>(nc, w, GA, inr->Wt[j], cnt_in, cnt_out, off_out,
+                                                                             Xb, ws[rs[nxt]].as<int>());
         else
           k_fresh_rows<1><<<(nc + 7) / 8, 256, 0, st>>>(nc, w, GA, inr->Wt[j], cnt_in, cnt_out, off_out, Xb,
                                                         ws[rs[nxt]].as<int>());
@@ -801,10 +924,9 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
       ISX_LAUNCH_CHECK("k_fresh_rows");
       {
         prof::Scope _ps(K_GEMV, st, 2.0 * nc * w * w, 0);
-        if (inflate) {
-          const float kappa = 3.0f * kU + gamma_k(w);
-          k_center_gemv<<<nc, std::min(w, 256), 2 * w * sizeof(float), st>>>(nc, w, w, inr->Wt[j], inr->b[j], C, AL, RAD,
-                                                                             GA, DE, inflate, kappa);
+        if (inflate || few) {
+          k_center_gemv<<<dim3(nc, few ? (w + 63) / 64 : 1), few ? 64 : std::min(w, 256), 2 * w * sizeof(float), st>>>(
+              w, inr->Wt[j], inr->b[j], C, AL, RAD, GA, C2, DE, inflate, 3.0f * kU + gamma_k(w));
           ISX_LAUNCH_CHECK("k_center_gemv");
         } else {
           GemmArgs g{};
@@ -814,13 +936,17 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
           g.bias = inr->b[j];
           g.R = nc;
           ISX_TRY(launch_gemm<false>((int64_t)nc * w < (int64_t)sms * 8192 ? 4 : 0, g, w, sms, st));
-          std::swap(C, C2);
         }
+        std::swap(C, C2);
       }
       {
         prof::Scope _ps(K_REDUCE, st, 0, 0);
-        k_reduce_act<<<cb.blocks(nc), cb.threads(), 0, st>>>(Xb, off_out, cnt_out, nc, cb.tpc, w, (int)mode, inr->act,
-                                                             inflate, C, RAD, DE, AL, GA, j < H - 1 ? cnt_in : nullptr);
+        const ReduceArgs g{Xb, off_out, cnt_out, nc, w, (int)mode, inr->act, inflate, C, RAD, DE, AL, GA};
+        int* next = j < H - 1 ? cnt_in : nullptr;
+        if (few)
+          ISX_TRY(launch_clusters(k_reduce_few, (unsigned)(w + 63) / 64, nc, 64, 0, st, g, next));
+        else
+          k_reduce_act<<<cb.blocks(nc), cb.threads(), 0, st>>>(g, cb.tpc, next);
       }
       ISX_LAUNCH_CHECK("k_reduce_act");
       cur = nxt;
@@ -833,7 +959,12 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
       const float* X = ws[xs[cur]].as<float>();
       const int64_t* off = ws[os[cur]].as<int64_t>();
       const int* cnt = ws[ns[cur]].as<int>();
-      if (wide)
+      if (few)
+        ISX_TRY(launch_clusters(8 * nc <= 2 * sms ? k_output<64> : k_output<32>, 8 * nc <= 2 * sms ? 8 : 4, nc, 256,
+                                (w + kOutRows) * sizeof(float), st, X, off, cnt, nc, w, (const float*)C, (const float*)AL,
+                                (const float*)GA, (const float*)RAD, (const float*)inr->W[L], inr->hb[L][0], (int)mode,
+                                inflate, d_center, d_spread, first));
+      else if (wide)
         k_output<8><<<nc, 256, w * sizeof(float), st>>>(X, off, cnt, nc, w, C, AL, GA, RAD, inr->W[L], inr->hb[L][0],
                                                         (int)mode, inflate, d_center, d_spread, first);
       else

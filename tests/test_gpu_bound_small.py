@@ -1,5 +1,6 @@
-"""The one-launch float32 bound of small networks against the row path, over the rule that chooses it (up to
-8192 cells with one or two hidden layers, up to one cell per SM with more; widths up to 64)."""
+"""Float32 bounds of few cells against those of many: the one-launch form of small networks (up to 8192 cells
+with one or two hidden layers, up to one cell per SM with more; widths up to 64), the row path's kernels with
+several blocks per cell (up to one cell per SM), and the reduced form with two cells per thread."""
 import numpy as np
 import pytest
 import torch
@@ -34,4 +35,33 @@ def test_small_network_bounds_equal_the_row_path(pkg, w, H, act):
             a, b = net.bound_cells(lo[:n], hi[:n], mode=mode, prec="fp32", inflate=inflate)
             assert torch.equal(a, c[:n]) and torch.equal(b, s[:n]), (mode, inflate, n)
         assert torch.isfinite(c).all() and torch.isfinite(s).all()
+    net.close()
+
+
+@pytest.mark.parametrize("w,H,act", [(80, 5, "sine"), (112, 3, "relu"), (256, 4, "elu"), (400, 3, "relu"), (512, 4, "relu")])
+def test_few_cells_equal_many(pkg, w, H, act):
+    """From every symbol dead or alive to more rows than one hand-over of the output layer takes, either side of
+    the cell counts where the kernels change."""
+    net = pkg.Inr(inr.random_inr([3] + [w] * H + [1], 85 + w, act=act), act=act)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lo, hi = (torch.tensor(x, device="cuda") for x in boxes.random_boxes(sms + 1, 86, -9, 0))
+    modes = [("clt", False), ("sound", False), ("sound", True), ("raua", False)] if act == "relu" else [("clt", False)]
+    for mode, inflate in modes:
+        c, s = net.bound_cells(lo, hi, mode=mode, prec="fp32", inflate=inflate)
+        for n in (1, sms // 4, sms // 4 + 1, sms):
+            a, b = net.bound_cells(lo[:n], hi[:n], mode=mode, prec="fp32", inflate=inflate)
+            assert torch.equal(a, c[:n]) and torch.equal(b, s[:n]), (mode, inflate, n)
+        assert torch.isfinite(c).all() and torch.isfinite(s).all()
+    net.close()
+
+
+@pytest.mark.parametrize("w,H,inflate", [(64, 2, True), (128, 3, False), (272, 2, True), (400, 2, False), (512, 3, True)])
+def test_few_cells_equal_many_rafixed(pkg, w, H, inflate):
+    net = pkg.Inr(inr.random_inr([3] + [w] * H + [1], 95 + w))
+    edge = torch.cuda.get_device_properties(0).multi_processor_count * 2 * (1024 // w)
+    lo, hi = (torch.tensor(x, device="cuda") for x in boxes.random_boxes(edge + 1, 87, -9, 0))
+    c, s = net.bound_cells(lo, hi, mode="rafixed", prec="fp32", inflate=inflate)
+    for n in (1, 2, 5, edge - 1, edge):
+        a, b = net.bound_cells(lo[:n], hi[:n], mode="rafixed", prec="fp32", inflate=inflate)
+        assert torch.equal(a, c[:n]) and torch.equal(b, s[:n]), n
     net.close()

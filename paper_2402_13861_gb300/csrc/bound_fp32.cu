@@ -68,14 +68,14 @@ __device__ __forceinline__ float slack(float kappa, float g, int w, float e) {
   return __fmul_rn(fmaf(kappa, g, __fmul_rn(gamma_k(w + 2), e)), kSafe);
 }
 __device__ __forceinline__ float input_radius(int mode, float x0, float x1, float x2) {
-  if (mode == ISX_BOUND_CLT) return sqrtf(fmaf(x2, x2, fmaf(x1, x1, __fmul_rn(x0, x0))));
+  if (mode == ISX_BOUND_CLT) return sqrtf(fmaf(x2, x2, fmaf(x0, x0, __fmul_rn(x1, x1))));
   return __fadd_rn(__fadd_rn(fabsf(x0), fabsf(x1)), fabsf(x2));
 }
 
 // z_1 = W_0 x + b_0 over the box and activation 1: the 3 input rows with their row -> cell map, the
 // post-activation centre, alpha, gamma (and, inflate, radius and slack), the cell's row counts (3 now,
-// 3 + #(gamma != 0) after the next layer) and the offset of its rows.
-__global__ void __launch_bounds__(256) k_input_layer(CellSource src, int64_t first, int nc, int tpc,
+// 3 + #(gamma != 0) after the next layer) and the offset of its rows (rs = 3, or 4 with padding, apart).
+__global__ void __launch_bounds__(256) k_input_layer(CellSource src, int64_t first, int nc, int tpc, int rs,
                                                      const float* __restrict__ W0, const float* __restrict__ b0, int w,
                                                      int mode, int act, int inflate, float* C, float* X, int* rowcell,
                                                      float* RAD, float* ALPHA, float* GAMMA, int64_t* off, int* cnt,
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256) k_input_layer(CellSource src, int64_t fir
     cell_box(src, first + cell, inflate, xc, h);
     if (mode == ISX_BOUND_CLT)
       for (int d = 0; d < 3; ++d) h[d] *= kInvSqrt3;   // uniform on [-h, h] has std h / sqrt 3
-    float* Xc = X + (size_t)cell * 3 * w;
+    float* Xc = X + (size_t)cell * rs * w;
     int m = 0;
     for (int n = t; n < w; n += tpc) {
       float w0 = W0[3 * n], w1 = W0[3 * n + 1], w2 = W0[3 * n + 2];
@@ -113,12 +113,12 @@ __global__ void __launch_bounds__(256) k_input_layer(CellSource src, int64_t fir
       if (inflate) RAD[i] = rad;
       m += L.gamma != 0.0f;
     }
-    if (t < 3) rowcell[3 * cell + t] = cell;
+    if (t < rs) rowcell[rs * cell + t] = t < 3 ? cell : -1;
     if (m) atomicAdd(&made[sub], m);
   }
   __syncthreads();
   if (cell < nc && t == 0) {
-    off[cell] = 3 * (int64_t)cell;
+    off[cell] = rs * (int64_t)cell;
     cnt[cell] = 3;
     cnt_next[cell] = 3 + made[sub];
   }
@@ -170,24 +170,30 @@ __global__ void __launch_bounds__(256) k_center_gemv(int w, const float* __restr
   }
 }
 
-// Y[row] = X[row] diag(alpha_cell) W^T for R rows of all cells (ROWS), or Y[row] = X[row] W^T + b (the
-// centres): persistent CTAs over tiles of P rows, the rows scaled while they are staged k-major in shared
-// memory (sgemm.cuh).  Every output is one multiply-add chain over k whatever the launch shape, so all
-// shapes give bit-identical results and the autotuner may pick any of them.  R comes from device memory
-// (d_R) where the host does not know it.
+// Y[row] = X[row] diag(alpha_cell) W^T for R rows of all cells, or Y[row] = X[row] W^T + b (the centres):
+// persistent CTAs over tiles of P rows, staged k-major in shared memory (sgemm.cuh).  Every output is one
+// multiply-add chain over k whatever the launch shape, so all shapes give bit-identical results and the
+// autotuner may pick any of them.  R comes from device memory (d_R) where the host does not know it.
+//
+// alpha scales the rows while they are staged (kRows) or, for the ELU, the weights (kWeights), which then are
+// rounded once per cell and not once per row and cell: the ELU's second moments cancel at small sigma and turn
+// a different rounding of the rows into up to 5e-3 of the spread.  A cell's rows start at multiples of four there
+// (kPad), so that the four neighbouring rows of a thread share their scaled weights.
+enum Scale { kCentres, kRows, kWeights };
+constexpr int kPad = 4;
 struct GemmArgs {
   const float* X;
   float* Y;
   const float* Wt;
-  const float* alpha;                  // ROWS: [cell][w]
+  const float* alpha;                  // [cell][w] (but for the centres)
   const float* bias;                   // centres
-  const int* rowcell;                  // ROWS: cell of every row, first rows of the cells in X and in Y
+  const int* rowcell;                  // cell of every row (-1: padding), first rows of the cells in X and in Y
   const int64_t* off_in;
   const int64_t* off_out;
   const int64_t* d_R;                  // null: R
   int64_t R;
 };
-template <int TN, bool ROWS>
+template <int TN, Scale SC>
 __global__ void __launch_bounds__(256, 2) k_gemm_fp32(GemmArgs g, sgemm::Shape sh, int w) {
   extern __shared__ __align__(16) float sm[];
   const int P = sh.P, KB = sh.KB, spl = w / KB;
@@ -215,8 +221,8 @@ __global__ void __launch_bounds__(256, 2) k_gemm_fp32(GemmArgs g, sgemm::Shape s
       int c = 0;
       int64_t d = -1;
       if (r0 + p < R) {
-        c = ROWS ? g.rowcell[r0 + p] : 0;
-        d = ROWS ? g.off_out[c] + (r0 + p - g.off_in[c]) : r0 + p;
+        c = SC == kCentres ? 0 : g.rowcell[r0 + p];
+        d = SC == kCentres ? r0 + p : SC == kWeights && c < 0 ? -1 : g.off_out[c] + (r0 + p - g.off_in[c]);
       }
       dst[p] = d;
       rcell[p] = c;
@@ -238,7 +244,7 @@ __global__ void __launch_bounds__(256, 2) k_gemm_fp32(GemmArgs g, sgemm::Shape s
         v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (q < nq && r0 + p < R) {
           v[i] = *reinterpret_cast<const float4*>(g.X + (size_t)(r0 + p) * w + k);
-          if (ROWS) al[i] = *reinterpret_cast<const float4*>(g.alpha + (size_t)rcell[p] * w + k);
+          if (SC == kRows) al[i] = *reinterpret_cast<const float4*>(g.alpha + (size_t)rcell[p] * w + k);
         } else {
           al[i] = v[i];
         }
@@ -247,7 +253,7 @@ __global__ void __launch_bounds__(256, 2) k_gemm_fp32(GemmArgs g, sgemm::Shape s
       for (int i = 0; i < NF; ++i) {
         const int q = q0 + i * T, p = q % P, k = 4 * (q / P);
         if (q >= nq) break;
-        if (ROWS) {
+        if (SC == kRows) {
           v[i].x *= al[i].x; v[i].y *= al[i].y; v[i].z *= al[i].z; v[i].w *= al[i].w;
         }
         float* d = A + (size_t)k * P + p;
@@ -259,15 +265,26 @@ __global__ void __launch_bounds__(256, 2) k_gemm_fp32(GemmArgs g, sgemm::Shape s
 #pragma unroll
       for (int c = 0; c < TN / 2; ++c) {
         const int n = sgemm::Tile<TN>::neuron(c, ng, w);
-        const uint64_t z = ROWS ? 0ull : sgemm::pack2(g.bias[n], g.bias[n + 1]);
+        const uint64_t z = SC != kCentres ? 0ull : sgemm::pack2(g.bias[n], g.bias[n + 1]);
 #pragma unroll
         for (int i = 0; i < sgemm::kTM; ++i) acc.acc[i][c] = z;
       }
+    const float *al0 = nullptr, *al1 = nullptr;    // the scales of the thread's two groups of four rows
+    if (SC == kWeights && own) {
+      al0 = g.alpha + (size_t)rcell[4 * pg] * w;
+      al1 = g.alpha + (size_t)rcell[(P >> 1) + 4 * pg] * w;
+    }
     for (int kb = 0; kb < spl; ++kb) {
       sgemm::cp_wait<sgemm::kStages - 2>();
       __syncthreads();                             // the stage has landed, the one before it is free, A is written
       load_next();
-      if (own) acc.stage(A + (size_t)kb * KB * P, ws.Ws + (size_t)slot * KB * w, P, w, KB, pg, ng);
+      if (own) {
+        const float *a = A + (size_t)kb * KB * P, *wk = ws.Ws + (size_t)slot * KB * w;
+        if (SC == kWeights)
+          acc.stage_scaled(a, wk, P, w, KB, pg, ng, al0 + kb * KB, al1 + kb * KB);
+        else
+          acc.stage(a, wk, P, w, KB, pg, ng);
+      }
       slot = slot == sgemm::kStages - 1 ? 0 : slot + 1;
     }
     if (own)
@@ -297,14 +314,14 @@ constexpr GemmShape kGemmShapes[] = {{8, 16384, 4096, "8x8, 256 threads"}, {8, 8
                                      {4, 4096, 8192, "8x4, 128 threads"}};
 constexpr int kGemmVariants = sizeof(kGemmShapes) / sizeof(kGemmShapes[0]);
 
-template <bool ROWS>
+template <Scale SC>
 isx_status launch_gemm(int v, const GemmArgs& g, int w, int sms, cudaStream_t st) {
   const GemmShape& gs = kGemmShapes[v];
   const int KB = 32 * w <= gs.stage && w % 32 == 0 ? 32 : (16 * w <= gs.stage ? 16 : (8 * w <= gs.stage ? 8 : 4));
   const sgemm::Shape sh{gs.tn, std::max(8, gs.elems / w / 8 * 8), KB};
   const size_t smem = sh.smem(w) + (size_t)sh.P * (sizeof(int64_t) + sizeof(int));
   const int threads = (sh.threads(w) + 31) / 32 * 32;
-  const auto kernel = sh.tn == 8 ? k_gemm_fp32<8, ROWS> : k_gemm_fp32<4, ROWS>;
+  const auto kernel = sh.tn == 8 ? k_gemm_fp32<8, SC> : k_gemm_fp32<4, SC>;
   ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   int per_sm = 1;
   ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
@@ -320,14 +337,14 @@ isx_status launch_gemm(int v, const GemmArgs& g, int w, int sms, cudaStream_t st
 template <int WPC>
 __global__ void __launch_bounds__(256) k_fresh_rows(int nc, int w, const float* __restrict__ GAMMA,
                                                     const float* __restrict__ Wt, const int* cnt_in, const int* cnt_out,
-                                                    const int64_t* off_out, float* Xout, int* rowcell) {
+                                                    const int64_t* off_out, float* Xout, int* rowcell, int pad) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int u = blockIdx.y * WPC + warp % WPC, warps = WPC * gridDim.y;
   const int cell = blockIdx.x * (8 / WPC) + warp / WPC;
   if (cell >= nc) return;
   const int64_t o0 = off_out[cell];
   const int co = cnt_out[cell];
-  for (int r = u * 32 + lane; r < co; r += 32 * warps) rowcell[o0 + r] = cell;
+  for (int r = u * 32 + lane; r < ((co + pad) & ~pad); r += 32 * warps) rowcell[o0 + r] = r < co ? cell : -1;
   // lane i: the alive neurons of the 32-group i (w <= 512), how many rows come before them, and how many there are
   const float* ga = GAMMA + (size_t)cell * w;
   float gm[16];
@@ -630,6 +647,7 @@ __global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t
   float* de = rad + w;
   float* aw = de + w;
   const float kappa = 3.0f * kU + gamma_k(w);
+  const bool elu = net.act == ISX_ACT_ELU;
   for (int64_t cell = blockIdx.x; cell < n; cell += gridDim.x) {
     float xc[3], h[3];
     cell_box(src, cell, inflate, xc, h);
@@ -682,14 +700,18 @@ __global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t
       // carried rows, four per warp and turn, in place: (x alpha) W^T
       for (int r0 = 4 * warp; r0 < S; r0 += 16) {
         const int nr = min(4, S - r0);
-        for (int q = 0; q < nr; ++q)
-          for (int k = lane; k < w; k += 32) X[(r0 + q) * w + k] *= al[k];
+        if (!elu)
+          for (int q = 0; q < nr; ++q)
+            for (int k = lane; k < w; k += 32) X[(r0 + q) * w + k] *= al[k];
         __syncwarp();
         float y[4][2] = {};
         for (int k = 0; k < w; ++k) {
           float wv[2];
 #pragma unroll
-          for (int c = 0; c < 2; ++c) wv[c] = lane + 32 * c < w ? Wt[k * w + lane + 32 * c] : 0.0f;
+          for (int c = 0; c < 2; ++c) {
+            wv[c] = lane + 32 * c < w ? Wt[k * w + lane + 32 * c] : 0.0f;
+            if (elu) wv[c] = __fmul_rn(wv[c], al[k]);   // scaled weights, as in the row path
+          }
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const float x = X[min(r0 + q, S - 1) * w + k];
@@ -814,7 +836,9 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
     ISX_LAUNCH_CHECK("k_bound_small");
     return ISX_OK;
   }
-  const int Smax = 3 + w * (H - 1);
+  const bool elu = inr->act == ISX_ACT_ELU;
+  const int pad = elu ? kPad - 1 : 0, rs = elu ? kPad : 3;   // row alignment - 1, rows kept for the input's three
+  const int Smax = rs + w * (H - 1);
   // the two coefficient buffers take at most ~6 GB: enough for full_cells cells with every symbol alive
   const size_t per_cell = 2ull * Smax * w * sizeof(float);
   const int64_t full_cells = std::min<int64_t>({n, (int64_t)1 << 16, std::max<int64_t>(1, (int64_t)((6ull << 30) / per_cell))});
@@ -839,7 +863,7 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   float* AL = ws[WS_ALPHA].as<float>();
   float* GA = ws[WS_GAMMA].as<float>();
   float* DE = ws[WS_DELTA].as<float>();
-  const Slot xs[2] = {WS_X0, WS_X1}, rs[2] = {WS_R_RC0, WS_R_RC1}, ns[2] = {WS_R_CNT0, WS_R_CNT1},
+  const Slot xs[2] = {WS_X0, WS_X1}, rc[2] = {WS_R_RC0, WS_R_RC1}, ns[2] = {WS_R_CNT0, WS_R_CNT1},
              os[2] = {WS_R_OFF0, WS_R_OFF1};
   const int sms = inr->sms;
   const CellBlock cb(w);
@@ -855,13 +879,13 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
     const bool wide = nc < 8 * sms;
     const bool few = nc <= sms;
     int cur = 0;
-    int64_t R = 3 * (int64_t)nc;                   // rows of z_j (an upper bound where the host does not know)
+    int64_t R = rs * (int64_t)nc;                  // rows of z_j (an upper bound where the host does not know)
     bool fits = true;
     {
       prof::Scope _ps(K_INPUT, st, 0, 0);
       k_input_layer<<<cb.blocks(nc), cb.threads(), 0, st>>>(
-          src, first, nc, cb.tpc, inr->W[0], inr->b[0], w, (int)mode, inr->act, inflate, C, ws[xs[0]].as<float>(),
-          ws[rs[0]].as<int>(), RAD, AL, GA, ws[os[0]].as<int64_t>(), ws[ns[0]].as<int>(), ws[ns[1]].as<int>());
+          src, first, nc, cb.tpc, rs, inr->W[0], inr->b[0], w, (int)mode, inr->act, inflate, C, ws[xs[0]].as<float>(),
+          ws[rc[0]].as<int>(), RAD, AL, GA, ws[os[0]].as<int64_t>(), ws[ns[0]].as<int>(), ws[ns[1]].as<int>());
     }
     ISX_LAUNCH_CHECK("k_input_layer");
     for (int j = 1; j <= H - 1; ++j) {
@@ -875,14 +899,14 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
       // d_tot[j & 1]: rows of z_{j+1}; the other one still holds those of z_j
       {
         prof::Scope _ps(K_SCAN, st, 0, 0);
-        ISX_TRY(rows::scan_counts(cnt_out, nc, d_tot, j & 1, off_out, st));
+        ISX_TRY(rows::scan_counts(cnt_out, nc, d_tot, j & 1, off_out, st, pad));
       }
-      int64_t Rn = std::min<int64_t>(row_cap, (int64_t)nc * (3 + (int64_t)w * j));
+      int64_t Rn = std::min<int64_t>(row_cap, (int64_t)nc * (rs + (int64_t)w * j));
       if (counted) {
         ISX_CUDA(cudaMemcpyAsync(&Rn, d_tot + (j & 1), sizeof(int64_t), cudaMemcpyDeviceToHost, st));
         ISX_CUDA(cudaStreamSynchronize(st));
         // rows after the last layer if every layer creates as many as the ones so far
-        const double last = 3.0 * nc + (double)(Rn - 3 * (int64_t)nc) / j * (H - 1);
+        const double last = (double)rs * nc + (double)(Rn - rs * (int64_t)nc) / j * (H - 1);
         if (Rn > row_cap || (j == 1 && last > 1.2 * (double)row_cap)) {
           want = std::max<int64_t>(full_cells, std::min<int64_t>(nc / 2, (int64_t)(0.8 * nc * (double)row_cap / std::max(last, (double)Rn))));
           fits = false;                            // start the chunk again with fewer cells
@@ -896,15 +920,15 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
         g.Y = Xb;
         g.Wt = inr->Wt[j];
         g.alpha = AL;
-        g.rowcell = ws[rs[cur]].as<int>();
+        g.rowcell = ws[rc[cur]].as<int>();
         g.off_in = off_in;
         g.off_out = off_out;
         g.d_R = (counted || j == 1) ? nullptr : d_tot + ((j - 1) & 1);
         g.R = R;
         int64_t bucket = 1;
         while (bucket < std::min<int64_t>(R, 1 << 16)) bucket <<= 1;
-        const std::string key = "gemm_fp32 w=" + std::to_string(w) + " rows<=" + std::to_string(bucket);
-        auto run = [&](int v) { return launch_gemm<true>(v, g, w, sms, st); };
+        const std::string key = std::string(elu ? "gemm_fp32 elu w=" : "gemm_fp32 w=") + std::to_string(w) + " rows<=" + std::to_string(bucket);
+        auto run = [&](int v) { return elu ? launch_gemm<kWeights>(v, g, w, sms, st) : launch_gemm<kRows>(v, g, w, sms, st); };
         int v = 0;
         ISX_TRY(tune::pick(key, kGemmVariants, [&](int i) { return kGemmShapes[i].name; }, run, st, &v));
         // counted work: the rows, or the input rows alone where only the device knows how many there are
@@ -916,10 +940,10 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
         prof::Scope _ps(K_FRESH, st, 0, 0);
         if (wide)
           k_fresh_rows<8><<<dim3(nc, few ? (w + 63) / 64 : 1), 256, 0, st>>>(nc, w, GA, inr->Wt[j], cnt_in, cnt_out, off_out,
-                                                                             Xb, ws[rs[nxt]].as<int>());
+                                                                             Xb, ws[rc[nxt]].as<int>(), pad);
         else
           k_fresh_rows<1><<<(nc + 7) / 8, 256, 0, st>>>(nc, w, GA, inr->Wt[j], cnt_in, cnt_out, off_out, Xb,
-                                                        ws[rs[nxt]].as<int>());
+                                                        ws[rc[nxt]].as<int>(), pad);
       }
       ISX_LAUNCH_CHECK("k_fresh_rows");
       {
@@ -935,7 +959,7 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
           g.Wt = inr->Wt[j];
           g.bias = inr->b[j];
           g.R = nc;
-          ISX_TRY(launch_gemm<false>((int64_t)nc * w < (int64_t)sms * 8192 ? 4 : 0, g, w, sms, st));
+          ISX_TRY(launch_gemm<kCentres>((int64_t)nc * w < (int64_t)sms * 8192 ? 4 : 0, g, w, sms, st));
         }
         std::swap(C, C2);
       }

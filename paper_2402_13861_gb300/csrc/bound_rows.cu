@@ -314,11 +314,11 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t* wsum, int
   __syncthreads();
   return wsum[warp] + incl - v;
 }
-__global__ void __launch_bounds__(kScanB) k_rows_scan_sums(const int* cnt, int64_t nc, int64_t* bsum) {
+__global__ void __launch_bounds__(kScanB) k_rows_scan_sums(const int* cnt, int64_t nc, int64_t* bsum, int pad) {
   __shared__ int64_t wsum[32];
   __shared__ int64_t total;
   const int64_t i = (int64_t)blockIdx.x * kScanB + threadIdx.x;
-  block_excl_scan(i < nc ? cnt[i] : 0, wsum, &total);
+  block_excl_scan(i < nc ? (cnt[i] + pad) & ~pad : 0, wsum, &total);
   if (threadIdx.x == 0) bsum[blockIdx.x] = total;
 }
 __global__ void __launch_bounds__(kScanB) k_rows_scan_top(int64_t* bsum, int64_t nb, int64_t* d_total) {
@@ -336,23 +336,24 @@ __global__ void __launch_bounds__(kScanB) k_rows_scan_top(int64_t* bsum, int64_t
   if (threadIdx.x == 0) *d_total = carry;
 }
 __global__ void __launch_bounds__(kScanB) k_rows_scan_apply(const int* cnt, int64_t nc, const int64_t* bsum,
-                                                            int64_t* off) {
+                                                            int64_t* off, int pad) {
   __shared__ int64_t wsum[32];
   __shared__ int64_t total;
   const int64_t i = (int64_t)blockIdx.x * kScanB + threadIdx.x;
-  const int64_t e = block_excl_scan(i < nc ? cnt[i] : 0, wsum, &total);
+  const int64_t e = block_excl_scan(i < nc ? (cnt[i] + pad) & ~pad : 0, wsum, &total);
   if (i < nc) off[i] = bsum[blockIdx.x] + e;
 }
 
 // The same scan by one block, for up to kScanOne counts: one launch instead of three (about 3 us each).
 constexpr int64_t kScanOne = 4 * kScanB;
-__global__ void __launch_bounds__(kScanB) k_rows_scan_one(const int* cnt, int64_t nc, int64_t* off, int64_t* d_total) {
+__global__ void __launch_bounds__(kScanB) k_rows_scan_one(const int* cnt, int64_t nc, int64_t* off, int64_t* d_total,
+                                                          int pad) {
   __shared__ int64_t wsum[32];
   __shared__ int64_t total;
   int64_t carry = 0;
   for (int64_t i0 = 0; i0 < nc; i0 += kScanB) {
     const int64_t i = i0 + threadIdx.x;
-    const int64_t e = block_excl_scan(i < nc ? cnt[i] : 0, wsum, &total);
+    const int64_t e = block_excl_scan(i < nc ? (cnt[i] + pad) & ~pad : 0, wsum, &total);
     if (i < nc) off[i] = carry + e;
     carry += total;
     __syncthreads();
@@ -1067,15 +1068,15 @@ isx_status launch_rows_split_w(isx_inr inr, int w, const RowsSplitArgs& a, const
 namespace rows {
 size_t scan_bytes(int64_t nc) { return 8 * sizeof(int64_t) + (size_t)((nc + kScanB - 1) / kScanB) * sizeof(int64_t); }
 
-isx_status scan_counts(const int* cnt, int64_t nc, int64_t* d_tot, int slot, int64_t* off, cudaStream_t st) {
+isx_status scan_counts(const int* cnt, int64_t nc, int64_t* d_tot, int slot, int64_t* off, cudaStream_t st, int pad) {
   if (nc <= kScanOne) {
-    k_rows_scan_one<<<1, kScanB, 0, st>>>(cnt, nc, off, d_tot + slot);
+    k_rows_scan_one<<<1, kScanB, 0, st>>>(cnt, nc, off, d_tot + slot, pad);
   } else {
     const int64_t nb = (nc + kScanB - 1) / kScanB;
     int64_t* bsum = d_tot + 8;
-    k_rows_scan_sums<<<(unsigned)nb, kScanB, 0, st>>>(cnt, nc, bsum);
+    k_rows_scan_sums<<<(unsigned)nb, kScanB, 0, st>>>(cnt, nc, bsum, pad);
     k_rows_scan_top<<<1, kScanB, 0, st>>>(bsum, nb, d_tot + slot);
-    k_rows_scan_apply<<<(unsigned)nb, kScanB, 0, st>>>(cnt, nc, bsum, off);
+    k_rows_scan_apply<<<(unsigned)nb, kScanB, 0, st>>>(cnt, nc, bsum, off, pad);
   }
   ISX_LAUNCH_CHECK("k_rows_scan");
   return ISX_OK;

@@ -91,10 +91,11 @@ struct RowsLayerArgs {
 // input one except at w = 512, where two CTAs share a cell.
 isx_status launch_rows_layer(isx_inr inr, int layer, const RowsLayerArgs& a, const __nv_bfloat16* AHin,
                              const __nv_bfloat16* ALOin, cudaStream_t st);
-// Exclusive scan of nc per-cell row counts into int64 offsets; the total goes to d_tot[slot] (slot < 8).
+// Exclusive scan of nc per-cell row counts into int64 offsets, each count
+// rounded up to a multiple of pad + 1 (a power of two); the total goes to d_tot[slot] (slot < 8).
 // d_tot: scan_bytes(nc) bytes, eight totals and the block sums.
 size_t scan_bytes(int64_t nc);
-isx_status scan_counts(const int* cnt, int64_t nc, int64_t* d_tot, int slot, int64_t* off, cudaStream_t st);
+isx_status scan_counts(const int* cnt, int64_t nc, int64_t* d_tot, int slot, int64_t* off, cudaStream_t st, int pad = 0);
 // One CTA waits on an mbarrier that nothing completes, with rwait and the given limit, raising
 // ISX_ERR_TIMEOUT in *d_status (rows_gemm.cu).
 isx_status check_bounded_wait(int64_t limit_ns, int* d_status, cudaStream_t st);

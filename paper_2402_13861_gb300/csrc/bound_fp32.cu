@@ -616,11 +616,12 @@ __global__ void __launch_bounds__(256)
 
 // ---- small networks: the whole propagation of a cell in one block ----------------------------------------
 // Widths up to 64: a cell's rows fit in shared memory, and what the path above spends is launches (seven per
-// layer and call) and passes over memory, not multiply-adds.  Four warps per cell; every sum is taken in the
-// order of the kernels above, so the results are the same bit for bit.  Bound by latency (a cell's chain of
-// layers); several blocks per SM overlap.  3 -> 64 x 2 -> 1, levels 4-6, with the row path before it: 1 cell
-// 54 -> 31 us, 608 cells 72 -> 37, 8192 cells 139 -> 120; FP32 extraction of that network to level 6, 895 -> 688.
-constexpr int kSmallT = 128;
+// layer and call) and passes over memory, not multiply-adds.  Every sum is taken in the order of the kernels
+// above, so the results are the same bit for bit.  Bound by latency (a cell's chain of layers): four warps per
+// cell and several blocks per SM, or sixteen warps where there are several layers of rows to carry (64 x 6, every
+// symbol alive: 229 -> 178 us for one cell).  3 -> 64 x 2 -> 1, levels 4-6, with the row path before it: 1 cell
+// 54 -> 31 us, 608 cells 72 -> 37, 8192 cells 139 -> 120; FP32 extraction of that network to level 6, 895 -> 690.
+constexpr int kSmallT = 512;                       // threads at most
 struct SmallNet {
   const float* W0;
   const float* b0;
@@ -637,7 +638,7 @@ __global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t
                                                          float* center, float* spread) {
   extern __shared__ __align__(16) float sm[];
   __shared__ float part[8];
-  const int w = net.w, H = net.H, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int w = net.w, H = net.H, t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, warps = T >> 5;
   float* X = sm;                                   // [rows][w]
   float* a = X + (size_t)small_rows(w, H) * w;     // centre, alpha, gamma, radius, slack of the current layer
   float* al = a + w;
@@ -683,7 +684,7 @@ __global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t
       __syncthreads();
       // centre (and slack) of the next layer: one neuron per thread of the last two warps
       float cn = 0.0f;
-      const int nn = t - (kSmallT - 64);
+      const int nn = t - (T - 64);
       if (nn >= 0 && nn < w) {
         cn = net.b[j][nn];
         float e = fabsf(cn), g = 0.0f;
@@ -698,7 +699,7 @@ __global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t
         if (inflate) de[nn] = slack(kappa, g, w, e);
       }
       // carried rows, four per warp and turn, in place: (x alpha) W^T
-      for (int r0 = 4 * warp; r0 < S; r0 += 16) {
+      for (int r0 = 4 * warp; r0 < S; r0 += 4 * warps) {
         const int nr = min(4, S - r0);
         if (!elu)
           for (int q = 0; q < nr; ++q)
@@ -730,7 +731,7 @@ __global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t
       for (int g0 = 0; g0 < w; g0 += 32) {
         const float gm = g0 + lane < w ? ga[g0 + lane] : 0.0f;
         for (unsigned b = __ballot_sync(0xffffffffu, gm != 0.0f); b; b &= b - 1, ++made) {
-          if ((made & 3) != warp) continue;
+          if (made % warps != warp) continue;
           const int l = __ffs(b) - 1;
           const float g = __shfl_sync(0xffffffffu, gm, l);
           for (int m = lane; m < w; m += 32) X[(S + made) * w + m] = g * Wt[(g0 + l) * w + m];
@@ -749,7 +750,7 @@ __global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t
     if (t < w) aw[t] = al[t] * net.wout[t];
     __syncthreads();
     const bool sq = (mode != ISX_BOUND_SOUND);
-    for (int u = warp; u < 8; u += 4) {
+    for (int u = warp; u < 8; u += warps) {
       float s = 0.0f, comp = 0.0f;
       for (int r = u; r < S; r += 8) {
         float y = 0.0f;
@@ -810,9 +811,10 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   const int w = inr->w, H = inr->H;
   if (mode != ISX_BOUND_SOUND) inflate = 0;
   // Small networks in one launch: with up to two hidden layers to 8192 cells (32768 cells: 392 us against 364 at
-  // 64 x 2, 234 against 189 at 32 x 2), deeper ones to one cell per SM (64 x 3, 152 cells: 67 against 116; beyond
-  // that its row products, which use a weight four times only, lose to the tuned tiles step by step).
-  if (w <= 64 && small_smem(w, H) <= 100 * 1024 && n <= (H <= 2 ? 8192 : inr->sms)) {
+  // 64 x 2, 234 against 189 at 32 x 2), deeper ones to 64 neurons per SM (16 x 8, 200 cells: 75 us against 274;
+  // 64 x 6 with every symbol alive, 152 cells: 178 against 321; beyond that the row path's tuned tiles, whose
+  // products use a weight more than four times, take over).
+  if (w <= 64 && small_smem(w, H) <= 100 * 1024 && (H <= 2 ? n <= 8192 : n * w <= 64 * (int64_t)inr->sms)) {
     SmallNet net{};
     net.W0 = inr->W[0];
     net.b0 = inr->b[0];
@@ -830,7 +832,7 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
       ISX_CUDA(cudaFuncSetAttribute(k_bound_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
     {
       prof::Scope _ps(K_BOUND_SMALL, st, 2.0 * n * w * (double)w * 4.0 * (H - 1), 0);
-      k_bound_small<<<(unsigned)std::min<int64_t>(n, 16 * (int64_t)inr->sms), kSmallT, smem, st>>>(src, n, net, (int)mode, inflate,
+      k_bound_small<<<(unsigned)std::min<int64_t>(n, 16 * (int64_t)inr->sms), H <= 2 ? 128 : kSmallT, smem, st>>>(src, n, net, (int)mode, inflate,
                                                                                                  d_center, d_spread);
     }
     ISX_LAUNCH_CHECK("k_bound_small");

@@ -1,5 +1,5 @@
 """Float32 bounds of few cells against those of many: the one-launch form of small networks (up to 8192 cells
-with one or two hidden layers, up to one cell per SM with more; widths up to 64), the row path's kernels with
+with one or two hidden layers, up to 64 neurons per SM with more; widths up to 64), the row path's kernels with
 several blocks per cell (up to one cell per SM), and the reduced form with two cells per thread."""
 import numpy as np
 import pytest
@@ -26,7 +26,7 @@ def test_small_network_bounds_equal_the_row_path(pkg, w, H, act):
     rng = np.random.default_rng(81)
     layers = [(W, rng.normal(0, 0.1, size=b.shape).astype(np.float32)) for W, b in layers]
     net = pkg.Inr(layers, act=act)
-    edge = 8192 if H <= 2 else torch.cuda.get_device_properties(0).multi_processor_count
+    edge = 8192 if H <= 2 else 64 * torch.cuda.get_device_properties(0).multi_processor_count // w
     lo, hi = (torch.tensor(x, device="cuda") for x in boxes.random_boxes(edge + 1, 82, -9, 0))
     modes = [("clt", False), ("sound", False), ("sound", True), ("raua", False)] if act == "relu" else [("clt", False)]
     for mode, inflate in modes:

@@ -326,16 +326,21 @@ isx_status bound_rafixed(isx_inr inr, const CellSource& src, int64_t n, int infl
     lay.b[l] = inr->b[l];
   }
   const int L = inr->n_layers - 1;
-  // cells per CTA: 128 threads' worth, two CTAs per SM; with fewer cells than that, enough CTAs for every SM,
-  // but at least 64 threads' worth (they share the weight stream)
+  // Cells per CTA: 128 threads' worth of four cells each (eight warps on the SM's two CTAs keep the multiply-adds
+  // fed); with fewer than that for every SM one CTA each, of at least 64 threads (they share the weight stream).  Two
+  // smaller ones would put two warps on the same sub-partition of the SM: 2600 cells of w = 144 in 251 us, not 169.
   const int sms = inr->sms;
-  // four cells per thread (eight warps per SM) keep the multiply-adds fed; at small widths the input and output
-  // layers weigh more and twice the warps with two cells each hide more of their latency (w = 64, two hidden
-  // layers, 10^5 cells: 165 us against 199 us)
-  const int cpt = w <= 64 ? 2 : 4;
+  // At small widths the input and output layers weigh more and twice the warps with two cells each hide more of their
+  // latency (w = 64, two hidden layers, 10^5 cells: 165 us against 199).  So do they while one CTA of 128 threads
+  // per SM takes all cells, where a CTA's own chain is the time (w = 512, eight layers, up to 608 cells: 505 us against
+  // 713; w = 256, five: 149 against 202 up to 1216 cells; beyond, four: 2400 cells of w = 512 in 995 us against 1107).
+  const int few_cells = 2 * (128 * kRaCols / w);
+  const bool few = few_cells > 0 && n <= (int64_t)sms * few_cells;
+  const int cpt = w <= 64 || few ? 2 : 4;
   const int most = ra_threads(cpt) / (w / kRaCols) * cpt;
-  const int64_t even = (n + 2 * sms - 1) / (2 * sms);
-  const int cells = (int)std::min<int64_t>(most, std::max<int64_t>((most / 2 + 3) / 4 * 4, (even + 3) / 4 * 4) / cpt * cpt);
+  const int64_t even = (n + sms - 1) / sms;
+  const int cells = few ? few_cells
+                        : (int)std::min<int64_t>(most, std::max<int64_t>((most / 2 + 3) / 4 * 4, (even + 3) / 4 * 4) / cpt * cpt);
   const int KB = 16 * w <= 2048 ? 16 : (8 * w <= 2048 ? 8 : 4);
   const int threads = (w / kRaCols * (cells / cpt) + 31) / 32 * 32;
   const size_t smem = ((size_t)kRaQ * cells * w + (size_t)sgemm::kStages * KB * w) * sizeof(float) + 2 * cells * sizeof(unsigned);

@@ -487,6 +487,72 @@ __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, con
     }
 }
 
+// The same for few cells: one block per cell and 64 columns, two per lane.  One warp alone takes about 110 ns a row,
+// one after the other, so the block's warps share the rows, eight in flight each, leave the stored values in shared
+// memory and the first warp sums them, in increasing n as above.
+constexpr int kFewWarps = 8, kFewRows = 128;     // rows of one turn: 16 per warp
+template <int w>
+__global__ void __launch_bounds__(32 * kFewWarps) k_rows_new_few(int sq, const float* __restrict__ GA,
+                                                                 const float* __restrict__ Wt, const int* cnt_in,
+                                                                 const int64_t* off_out, const int* cnt_out,
+                                                                 __nv_bfloat16* xout, int* rowcell_out, float* pnew,
+                                                                 int* cnt_next) {
+  constexpr int CS = w / 64, G = w / 32;
+  __shared__ float sgam[w];
+  __shared__ short slist[w];                     // the alive neurons
+  __shared__ __nv_bfloat162 sx[kFewRows][32];
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, t = threadIdx.x;
+  const int cell = blockIdx.x / CS, cs = blockIdx.x % CS, m0 = 64 * cs + 2 * lane;
+  for (int n = t; n < w; n += 32 * kFewWarps) sgam[n] = GA[(size_t)cell * w + n];
+  const int64_t o0 = off_out[cell];
+  const int co = cnt_out[cell];
+  __nv_bfloat16* xp = xout + (size_t)(o0 + cnt_in[cell]) * w + m0;
+  if (cnt_next && cs == 0 && t == 0) cnt_next[cell] = co;
+  for (int r = cs * 32 * kFewWarps + t; r < co; r += 32 * kFewWarps * CS) rowcell_out[o0 + r] = cell;
+  __syncthreads();
+  int S = 0;                                     // every warp ranks all groups and lists its own
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const bool alive = sgam[32 * g + lane] != 0.0f;
+    const unsigned b = __ballot_sync(0xffffffffu, alive);
+    if (g % kFewWarps == wi && alive) slist[S + __popc(b & ((1u << lane) - 1u))] = (short)(32 * g + lane);
+    S += __popc(b);
+  }
+  __syncthreads();
+  float a0 = 0.0f, a1 = 0.0f;
+  for (int base = 0; base < S; base += kFewRows) {
+    const int end = min(S - base, kFewRows);
+    for (int r0 = 8 * wi; r0 < end; r0 += 8 * kFewWarps) {
+      float2 v[8];
+      float gm[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {              // past the end: the last row again
+        const int n = slist[base + min(r0 + q, end - 1)];
+        gm[q] = sgam[n];
+        v[q] = *reinterpret_cast<const float2*>(Wt + (size_t)n * w + m0);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (r0 + q < end) {
+          const __nv_bfloat162 x = __floats2bfloat162_rn(gm[q] * v[q].x, gm[q] * v[q].y);
+          *reinterpret_cast<__nv_bfloat162*>(xp + (size_t)(base + r0 + q) * w) = x;
+          sx[r0 + q][lane] = x;
+        }
+    }
+    __syncthreads();
+    if (wi == 0) {
+#pragma unroll 8
+      for (int r = 0; r < end; ++r) {
+        const float2 f = __bfloat1622float2(sx[r][lane]);
+        a0 = sq ? fmaf(f.x, f.x, a0) : a0 + fabsf(f.x);
+        a1 = sq ? fmaf(f.y, f.y, a1) : a1 + fabsf(f.y);
+      }
+    }
+    __syncthreads();
+  }
+  if (wi == 0) *reinterpret_cast<float2*>(pnew + (size_t)cell * w + m0) = make_float2(a0, a1);
+}
+
 // ---- c' = W_j a + b_j for every cell of a chunk in float32 on the CUDA cores (sound mode with
 //      inflation): output (cell, n) is one fused multiply-add chain over k = 0 .. K-1 starting from
 //      b_n, so it errs by at most gamma_{K+1} (sum_k |W_nk a_k| + |b_n|).  64 x 64 output tiles (cells x
@@ -1246,12 +1312,17 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
               nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
         };
         // several cells per warp once there are enough cells to fill the SMs all the same
-        // and for a handful of cells as many warps per cell as there are column groups of two, eight rows in flight
-        // (7 coarse cells at w = 256: 40 -> 29 us a launch)
-        const bool many = nc >= 32 * sms, few = nc <= 2 * sms;
-        if (w == 512 && few) launch_new(k_rows_new<512, 2, 1, 8>, 1, 8);
-        else if (w == 256 && few) launch_new(k_rows_new<256, 2, 1, 8>, 1, 4);
-        else if (w == 128 && few) launch_new(k_rows_new<128, 2, 1, 8>, 1, 2);
+        // and for few cells several warps per cell and column (7 coarse cells of the 3 -> 256 x 5 -> 1 network: 29 -> 10 us
+        // a launch, the call 309 -> 231 us; 512 cells 658 -> 601; 1024 cells 828 against 838)
+        const bool many = nc >= 32 * sms, few = nc <= 4 * sms;
+        auto launch_few = [&](auto kernel) {
+          kernel<<<(unsigned)(nc * (w / 64)), 32 * kFewWarps, 0, st>>>(sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc,
+                                                                      pnew, cz);
+        };
+        if (few && w == 512) launch_few(k_rows_new_few<512>);
+        else if (few && w == 256) launch_few(k_rows_new_few<256>);
+        else if (few && w == 128) launch_few(k_rows_new_few<128>);
+        else if (few) launch_few(k_rows_new_few<64>);
         else if (w == 512 && many) launch_new(k_rows_new<512, 8, 2, 4>, 2, 2);
         else if (w == 512) launch_new(k_rows_new<512, 8, 1, 4>, 1, 2);
         else if (w == 256 && many) launch_new(k_rows_new<256, 8, 4, 2>, 4, 1);

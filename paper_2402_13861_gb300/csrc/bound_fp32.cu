@@ -467,24 +467,6 @@ __global__ void __launch_bounds__(64) k_reduce_few(ReduceArgs g, int* cnt_next) 
   if (cnt_next && slice == 0 && threadIdx.x == 0) cnt_next[cell] = S + made;
 }
 
-// One cluster of `blocks` blocks per cell.
-template <typename... A>
-isx_status launch_clusters(void (*kernel)(A...), unsigned blocks, int nc, unsigned threads, size_t smem, cudaStream_t st, A... args) {
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = blocks;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)nc * blocks);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  ISX_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
-  return ISX_OK;
-}
-
 // Output layer w -> 1 and the read-off.  Row r's term goes to partial sum r % 8 (compensated, r ascending),
 // held by WPC warps per cell: all eight by one warp or one per warp, four rows' 16-byte loads in flight.  With
 // WPC = 32 and 64 (few cells) a cluster of four or eight blocks shares the rows (one SM alone reads about 60 GB/s of them) and

@@ -27,6 +27,7 @@
 #include "internal.cuh"
 
 #include <algorithm>
+#include <cooperative_groups.h>
 #include <cmath>
 #include <cstring>
 #include <cuda_bf16.h>
@@ -921,7 +922,8 @@ __global__ void __launch_bounds__(32 * kRedWarps) k_rows_reduce_act(int nc, int 
 // WPC warps per cell, CPL = w / 32 consecutive neurons per lane (the vector v = alpha o w_out stays in
 // registers); each row is one vector load per lane, four rows' loads in flight, and its dot product
 // is reduced across the warp before |y| or y^2 is taken.  The terms are added in row order whatever WPC: with
-// WPC > 1 the warps leave the rows' dot products in shared memory, 64 rows at a time, for the first one.
+// WPC > 1 the warps leave the rows' dot products in shared memory, 64 rows at a time, for the first one.  With
+// WPC = 32 (few cells) they are a cluster of four blocks, 512 rows at a time, eight in flight per warp.
 constexpr int kOutWarps = 8;
 template <int CPL>
 __device__ __forceinline__ void ld_row(const __nv_bfloat16* p, float* f) {
@@ -945,7 +947,7 @@ __device__ __forceinline__ void ld_row(const __nv_bfloat16* p, float* f) {
     f[2 * i + 1] = x.y;
   }
 }
-constexpr int kOutRows = 64;                     // rows of one hand-over (WPC > 1)
+__host__ __device__ constexpr int out_rows(int wpc) { return wpc > kOutWarps ? 512 : 64; }   // rows of one hand-over (WPC > 1)
 template <int CPL, int WPC>
 __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode, const __nv_bfloat16* X,
                                                                 const int64_t* off, const int* cnt, const float* I,
@@ -954,8 +956,10 @@ __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode
                                                                 int64_t first, float* center, float* spread,
                                                                 Infl infl) {
   constexpr int w = 32 * CPL;
-  const int lane = threadIdx.x & 31, sub = (threadIdx.x >> 5) / WPC, u = (threadIdx.x >> 5) % WPC;
-  const int cell = blockIdx.x * (kOutWarps / WPC) + sub;
+  constexpr int BPC = (WPC + kOutWarps - 1) / kOutWarps, CPB = BPC > 1 ? 1 : kOutWarps / WPC;   // blocks per cell, cells per block
+  const int lane = threadIdx.x & 31, sub = (threadIdx.x >> 5) / WPC;
+  const int u = (blockIdx.x % BPC) * kOutWarps + (threadIdx.x >> 5) % WPC;                     // the warp's place in its cell
+  const int cell = blockIdx.x / BPC * CPB + sub;
   if (cell >= nc) return;                          // the cell's warps alone meet at its barrier
   const bool sq = mode != ISX_BOUND_SOUND;
   const int m0 = lane * CPL;
@@ -1016,17 +1020,17 @@ __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode
   }
   // the stored symbol rows (bf16), four at a time
   const __nv_bfloat16* xp = X + o0 * w + m0;
-  auto four = [&](int r, float* y) {               // dot products of rows r .. r + 3 (< rows)
+  constexpr int NF = BPC > 1 ? 8 : 4;
+  auto dots = [&](int r, float (&y)[NF]) {         // dot products of rows r .. r + NF - 1 (< rows)
+    float x[NF][CPL];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float x[CPL];
-      ld_row<CPL>(xp + (size_t)min(r + q, rows - 1) * w, x);
-      y[q] = dot(x);
-    }
+    for (int q = 0; q < NF; ++q) ld_row<CPL>(xp + (size_t)min(r + q, rows - 1) * w, x[q]);
+#pragma unroll
+    for (int q = 0; q < NF; ++q) y[q] = dot(x[q]);
 #pragma unroll
     for (int sh = 16; sh > 0; sh >>= 1)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) y[q] += __shfl_xor_sync(0xffffffffu, y[q], sh);
+      for (int q = 0; q < NF; ++q) y[q] += __shfl_xor_sync(0xffffffffu, y[q], sh);
   };
   // one rounding per square in whole groups of four rows, two in the rest (fixed, so that no launch shape or
   // compiler choice changes a result)
@@ -1060,17 +1064,26 @@ __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode
       sr = term(r, y, sr);
     }
   } else {
-    __shared__ float sy[kOutWarps / WPC][2][kOutRows];
-    int h = 0;
-    for (int r0 = 0; r0 < rows; r0 += kOutRows, h ^= 1) {
-      for (int r = 4 * u; r < kOutRows && r0 + r < rows; r += 4 * WPC) {
-        float y[4];
-        four(r0 + r, y);
-        if (lane < 4) sy[sub][h][r + lane] = lane == 0 ? y[0] : (lane == 1 ? y[1] : (lane == 2 ? y[2] : y[3]));
+    constexpr int NR = out_rows(WPC);
+    __shared__ float sy[CPB][2][NR];
+    const auto cluster = cooperative_groups::this_cluster();
+    float* d = BPC > 1 ? cluster.map_shared_rank(&sy[0][0][0], 0) : &sy[sub][0][0];
+    if (BPC > 1) cluster.sync();                   // every block runs before the first hand-over
+    for (int r0 = 0, h = 0; r0 < rows; r0 += NR, h ^= 1) {
+      for (int r = NF * u; r < NR && r0 + r < rows; r += NF * WPC) {
+        float y[NF];
+        dots(r0 + r, y);
+        float mine = y[0];
+#pragma unroll
+        for (int q = 1; q < NF; ++q) mine = lane == q ? y[q] : mine;
+        if (lane < NF) d[h * NR + r + lane] = mine;
       }
-      asm volatile("bar.sync %0, %1;" ::"r"(sub + 1), "n"(32 * WPC) : "memory");
+      if (BPC > 1)
+        cluster.sync();
+      else
+        asm volatile("bar.sync %0, %1;" ::"r"(sub + 1), "n"(32 * WPC) : "memory");
       if (u == 0) {
-        const int m = min(kOutRows, rows - r0);
+        const int m = min(NR, rows - r0);
         for (int q = 0; q < m; ++q) {
           const float y = sy[sub][h][q];
           sr = term(r0 + q, y, sr);
@@ -1457,8 +1470,19 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
       };
       // four warps per cell until single warps fill every SM several times over: a chunk lasts as long as its
       // cell with the most rows (12007 cells of the 3 -> 512 x 8 -> 1 network: 1.14 -> 0.62 ms)
+      // and up to one cell per SM a cluster of blocks per cell (7 coarse cells of the 3 -> 256 x 5 -> 1 network: 43 ->
+      // 16 us; 512 cells: no faster)
       const bool many = nc >= 128 * sms;
-      if (w == 512 && many) launch_out(k_rows_output<16, 1>, kOutWarps);
+      auto launch_few = [&](auto kernel) {
+        return launch_clusters(kernel, 4, nc, 32 * kOutWarps, 0, st, nc, (int)mode, Xl, ol, cl, (const float*)I0, (const float*)A,
+                               (const float*)AL, (const float*)GA, wl, bl, first, d_center, d_spread, fi);
+      };
+      const bool few = nc <= sms;
+      if (few && w == 512) ISX_TRY(launch_few(k_rows_output<16, 32>));
+      else if (few && w == 256) ISX_TRY(launch_few(k_rows_output<8, 32>));
+      else if (few && w == 128) ISX_TRY(launch_few(k_rows_output<4, 32>));
+      else if (few) ISX_TRY(launch_few(k_rows_output<2, 32>));
+      else if (w == 512 && many) launch_out(k_rows_output<16, 1>, kOutWarps);
       else if (w == 512) launch_out(k_rows_output<16, 4>, kOutWarps / 4);
       else if (w == 256 && many) launch_out(k_rows_output<8, 1>, kOutWarps);
       else if (w == 256) launch_out(k_rows_output<8, 4>, kOutWarps / 4);

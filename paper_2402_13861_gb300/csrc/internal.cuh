@@ -255,4 +255,22 @@ isx_status eval_points_fp32(isx_inr inr, const float* xyz, const uint32_t* latti
 isx_status mc_upload_table(int device);
 void mc_build_table(int8_t* ntri, int8_t* tris);
 
+// One cluster of `blocks` blocks per cell.
+template <typename... A>
+inline isx_status launch_clusters(void (*kernel)(A...), unsigned blocks, int nc, unsigned threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = blocks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)nc * blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  ISX_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+  return ISX_OK;
+}
+
 }  // namespace isx

@@ -488,6 +488,81 @@ __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, con
     }
 }
 
+// The same with one cell per warp: the alive neurons are listed first, so that the rows go by in straight batches of
+// NF, the next batch's weights in flight, without a branch per row, which took about 110 ns: 4500 cells of the
+// 3 -> 512 x 8 -> 1 network 819 -> 611 us for its seven launches, of 3 -> 128 x 4 -> 1 115 -> 82 us for three.
+template <int w, int CPL, int NF>
+__global__ void __launch_bounds__(32 * kNewWarps) k_rows_new_one(int nc, int sq, const float* __restrict__ GA,
+                                                                 const float* __restrict__ Wt, const int* cnt_in,
+                                                                 const int64_t* off_out, const int* cnt_out,
+                                                                 __nv_bfloat16* xout, int* rowcell_out, float* pnew,
+                                                                 int* cnt_next) {
+  constexpr int CS = w / (32 * CPL), G = w / 32;
+  using IO = NewRowIO<CPL>;
+  __shared__ float2 list[kNewWarps][w];          // gamma and, as an integer, the index of every alive neuron
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+  const int unit = blockIdx.x * kNewWarps + wi, cs = unit % CS, cell = unit / CS;
+  if (cell >= nc) return;
+  const int m0 = (cs * 32 + lane) * CPL;
+  float gm[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) gm[g] = GA[(size_t)cell * w + 32 * g + lane];
+  const int64_t o0 = off_out[cell];
+  const int co = cnt_out[cell];
+  __nv_bfloat16* xp = xout + (size_t)(o0 + cnt_in[cell]) * w + m0;
+  if (cnt_next && cs == 0 && lane == 0) cnt_next[cell] = co;
+  for (int r = cs * 32 + lane; r < co; r += 32 * CS) rowcell_out[o0 + r] = cell;
+  int S = 0;
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const unsigned b = __ballot_sync(0xffffffffu, gm[g] != 0.0f);
+    if (gm[g] != 0.0f) list[wi][S + __popc(b & ((1u << lane) - 1u))] = make_float2(gm[g], __int_as_float(32 * g + lane));
+    S += __popc(b);
+  }
+  __syncwarp();
+  float acc[CPL];
+#pragma unroll
+  for (int i = 0; i < CPL; ++i) acc[i] = 0.0f;
+  float v[2][NF][CPL];
+  auto load = [&](int r, float (&x)[NF][CPL]) {
+#pragma unroll
+    for (int q = 0; q < NF; ++q) IO::ld(Wt + (size_t)__float_as_int(list[wi][r + q].y) * w + m0, x[q]);
+  };
+  auto row = [&](int r, const float* x) {        // x = bf16(gamma_n W_j[m, n]) for this lane's columns m
+    const float g = list[wi][r].x;
+    uint32_t h[CPL / 2];
+#pragma unroll
+    for (int i = 0; i < CPL; i += 2) {
+      const __nv_bfloat162 y = __floats2bfloat162_rn(g * x[i], g * x[i + 1]);
+      h[i / 2] = *reinterpret_cast<const uint32_t*>(&y);
+      const float2 f = __bfloat1622float2(y);
+      acc[i] = sq ? fmaf(f.x, f.x, acc[i]) : acc[i] + fabsf(f.x);
+      acc[i + 1] = sq ? fmaf(f.y, f.y, acc[i + 1]) : acc[i + 1] + fabsf(f.y);
+    }
+    IO::st(xp + (size_t)r * w, h);
+  };
+  auto batch = [&](int r, const float (&x)[NF][CPL]) {
+#pragma unroll
+    for (int q = 0; q < NF; ++q) row(r + q, x[q]);
+  };
+  const int whole = S / NF * NF;
+  if (whole) load(0, v[0]);
+  for (int r = 0; r < whole; r += 2 * NF) {
+    if (r + NF < whole) load(r + NF, v[1]);
+    batch(r, v[0]);
+    if (r + NF >= whole) break;
+    if (r + 2 * NF < whole) load(r + 2 * NF, v[0]);
+    batch(r + NF, v[1]);
+  }
+  for (int r = whole; r < S; ++r) {
+    IO::ld(Wt + (size_t)__float_as_int(list[wi][r].y) * w + m0, v[0][0]);
+    row(r, v[0][0]);
+  }
+  float* d = pnew + (size_t)cell * w + m0;
+#pragma unroll
+  for (int i = 0; i < CPL; i += 2) *reinterpret_cast<float2*>(d + i) = make_float2(acc[i], acc[i + 1]);
+}
+
 // The same for few cells: one block per cell and 64 columns, two per lane.  One warp alone takes about 110 ns a row,
 // one after the other, so the block's warps share the rows, eight in flight each, leave the stored values in shared
 // memory and the first warp sums them, in increasing n as above.
@@ -1316,18 +1391,19 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         prof::Scope ps(K_ROWS_NEW, st, 0, (counted ? 2.0 * (double)(Rn - R) * w + 4.0 * (double)Rn : 0.0) + 8.0 * (double)nc * w);
         int* rc = ws[rs[nxt]].as<int>();
         int* cz = fused && j < H - 1 ? cnt_next : nullptr;
-        // warps of 1, 2 or 4 cells with w / 32 columns per lane; w = 512: two warps share the columns, and four
-        // weight rows are in flight where a warp has few cells, since a launch lasts as long as its cell with
-        // the most new rows (12007 cells of the 3 -> 512 x 8 -> 1 network: 1.80 -> 1.15 ms)
+        // warps of 1, 2 or 4 cells with w / 32 columns per lane (w = 512: two warps share the columns); one cell each
+        // while a launch lasts as long as its cell with the most new rows
         auto launch_new = [&](auto kernel, int cells, int split) {
           const int64_t warps = ((int64_t)nc + cells - 1) / cells * split;
           kernel<<<(unsigned)((warps + kNewWarps - 1) / kNewWarps), 32 * kNewWarps, 0, st>>>(
               nc, sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc, pnew, cz);
         };
-        // several cells per warp once there are enough cells to fill the SMs all the same
+        // several cells per warp once the SMs are full many times over and the weights' reads count (6000 unrelated fine
+        // cells: 700 us with one cell per warp against 779 at w = 256, 9000 cells 851 against 919, but 3.73 ms against 3.62
+        // with coarse ones; w = 128 958 against 998)
         // and for few cells several warps per cell and column (7 coarse cells of the 3 -> 256 x 5 -> 1 network: 29 -> 10 us
         // a launch, the call 309 -> 231 us; 512 cells 658 -> 601; 1024 cells 828 against 838)
-        const bool many = nc >= 32 * sms, few = nc <= 4 * sms;
+        const bool many = nc >= (w == 256 ? 48 : 64) * sms, few = nc <= 4 * sms;
         auto launch_few = [&](auto kernel) {
           kernel<<<(unsigned)(nc * (w / 64)), 32 * kFewWarps, 0, st>>>(sq, GA, inr->Wt[j], cnt_in, off_out, cnt_out, Xout, rc,
                                                                       pnew, cz);
@@ -1337,13 +1413,13 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
         else if (few && w == 128) launch_few(k_rows_new_few<128>);
         else if (few) launch_few(k_rows_new_few<64>);
         else if (w == 512 && many) launch_new(k_rows_new<512, 8, 2, 4>, 2, 2);
-        else if (w == 512) launch_new(k_rows_new<512, 8, 1, 4>, 1, 2);
+        else if (w == 512) launch_new(k_rows_new_one<512, 8, 4>, 1, 2);
         else if (w == 256 && many) launch_new(k_rows_new<256, 8, 4, 2>, 4, 1);
-        else if (w == 256) launch_new(k_rows_new<256, 8, 1, 4>, 1, 1);
+        else if (w == 256) launch_new(k_rows_new_one<256, 8, 4>, 1, 1);
         else if (w == 128 && many) launch_new(k_rows_new<128, 4, 4, 2>, 4, 1);
-        else if (w == 128) launch_new(k_rows_new<128, 4, 1, 4>, 1, 1);
+        else if (w == 128) launch_new(k_rows_new_one<128, 4, 4>, 1, 1);
         else if (many) launch_new(k_rows_new<64, 2, 4, 2>, 4, 1);
-        else launch_new(k_rows_new<64, 2, 1, 4>, 1, 1);
+        else launch_new(k_rows_new_one<64, 2, 4>, 1, 1);
         ISX_LAUNCH_CHECK("k_rows_new");
       }
       if (fused) {

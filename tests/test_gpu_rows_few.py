@@ -31,3 +31,17 @@ def test_few_cells_equal_many(pkg, w, H, act):
             assert torch.equal(a, c[:n]) and torch.equal(b, s[:n]), (mode, inflate, n)
         assert torch.isfinite(c).all() and torch.isfinite(s).all()
     net.close()
+
+
+@pytest.mark.parametrize("w,H", [(64, 4), (128, 3), (256, 3), (512, 3)])
+def test_one_cell_per_warp_equals_several(pkg, w, H):
+    """Lists either side of the length from which a warp takes several cells (48 or 64 cells per SM), with every
+    remainder of a batch of rows among the cells."""
+    net = pkg.Inr(inr.random_inr([3] + [w] * H + [1], 50 + w))
+    edge = torch.cuda.get_device_properties(0).multi_processor_count * (48 if w == 256 else 64)
+    lo, hi = (torch.tensor(x, device="cuda") for x in boxes.random_boxes(edge + 3, 51, -9, -2))
+    for mode, inflate in (("clt", False), ("sound", True)):
+        c, s = net.bound_cells(lo, hi, mode=mode, prec="bf16", inflate=inflate)
+        a, b = net.bound_cells(lo[:edge - 1], hi[:edge - 1], mode=mode, prec="bf16", inflate=inflate)
+        assert torch.equal(a, c[:edge - 1]) and torch.equal(b, s[:edge - 1]), (mode, inflate)
+    net.close()

@@ -1045,7 +1045,17 @@ __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode
   // per lane: x0 and the last activation's symbols (s), the error terms (ex); sr, the rows' and the
   // input rows' terms, is the same in every lane (their dot products are reduced across the warp)
   float x0 = 0.0f, s = 0.0f, ex = 0.0f, sr = 0.0f;
-  {
+  // warps but the first need v alone, and only if they have rows: most cells of a fine list have few or none
+  // (12000 fine cells of a 3 -> 512 x 2 -> 1 network: 176 -> 102 us)
+  constexpr int NF = BPC > 1 ? 8 : 4;              // rows in flight
+  if (u > 0 && NF * u < rows) {
+    float wo[CPL], al[CPL];
+    ldv<CPL>(wout + m0, wo);
+    ldv<CPL>(AL + o, al);
+#pragma unroll
+    for (int i = 0; i < CPL; ++i) v[i] = al[i] * wo[i];
+  }
+  if (u == 0) {
     float wo[CPL], al[CPL], av[CPL], gv[CPL];
     ldv<CPL>(wout + m0, wo);
     ldv<CPL>(AL + o, al);
@@ -1078,7 +1088,7 @@ __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode
     return y;
   };
   // the three input rows (float32)
-  {
+  if (u == 0) {
     float y[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -1095,7 +1105,6 @@ __global__ void __launch_bounds__(32 * kOutWarps) k_rows_output(int nc, int mode
   }
   // the stored symbol rows (bf16), four at a time
   const __nv_bfloat16* xp = X + o0 * w + m0;
-  constexpr int NF = BPC > 1 ? 8 : 4;
   auto dots = [&](int r, float (&y)[NF]) {         // dot products of rows r .. r + NF - 1 (< rows)
     float x[NF][CPL];
 #pragma unroll
@@ -1548,12 +1557,12 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
       // cell with the most rows (12007 cells of the 3 -> 512 x 8 -> 1 network: 1.14 -> 0.62 ms)
       // and up to one cell per SM a cluster of blocks per cell (7 coarse cells of the 3 -> 256 x 5 -> 1 network: 43 ->
       // 16 us; 512 cells: no faster)
-      const bool many = nc >= 128 * sms;
+      const bool many = nc >= 128 * sms || H == 1;   // one hidden layer leaves no stored rows
       auto launch_few = [&](auto kernel) {
         return launch_clusters(kernel, 4, nc, 32 * kOutWarps, 0, st, nc, (int)mode, Xl, ol, cl, (const float*)I0, (const float*)A,
                                (const float*)AL, (const float*)GA, wl, bl, first, d_center, d_spread, fi);
       };
-      const bool few = nc <= sms;
+      const bool few = nc <= sms && H > 1;
       if (few && w == 512) ISX_TRY(launch_few(k_rows_output<16, 32>));
       else if (few && w == 256) ISX_TRY(launch_few(k_rows_output<8, 32>));
       else if (few && w == 128) ISX_TRY(launch_few(k_rows_output<4, 32>));

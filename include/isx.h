@@ -316,8 +316,9 @@ void isx_profile_reset(void);
 int isx_profile_read(isx_kernel_stats* out, int max);
 
 /* ---- launch-shape autotuner ------------------------------------------------------------------
- * Kernels with interchangeable tile shapes (the FP32 coefficient GEMM of the FP32 bound: 64x64,
- * 32x64, 16x64, 128x64 and 64x128 output tiles, identical results) time every shape once per key
+ * Kernels with interchangeable tile shapes (the FP32 coefficient GEMM of the FP32 bound: 8x8 or 8x4 outputs
+ * per thread, 64 to 256 threads, identical results; short lists of networks of widths up to 64 take another
+ * kernel and no key) time every shape once per key
  * (kernel, hidden width, row-count bucket) on the real operands and keep the fastest for the process;
  * ISX_TUNE=0 in the environment disables tuning (first shape always).  isx_tune_read fills up to
  * `max` entries and returns how many keys are cached; strings stay valid until isx_tune_reset. */

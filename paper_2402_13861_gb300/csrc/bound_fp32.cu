@@ -13,7 +13,7 @@
 // A symbol whose coefficient gamma_n is exactly 0 has an all-zero row in every later layer and is never
 // created.  Bound by the FP32 FMA rate of the row GEMM: 20003 random cells of levels 5-9 of the fitted
 // 3 -> 256 x 5 -> 1 network take 15.6 ms (43 TFLOP/s in the GEMM), where carrying all 1027 rows of every
-// cell took 142.6 ms; with every symbol alive (ELU, 3 -> 128 x 4 -> 1, 5003 boxes) 2.2 ms against 4.0 ms.
+// cell took 142.6 ms; with every symbol alive (ELU, 3 -> 128 x 4 -> 1, 5003 boxes) 2.3 ms against 4.0 ms.
 // A cell's result depends neither on the chunking nor on the launch shapes.
 //
 // Rounding-error inflation (SOUND, inflate != 0).  The library carries, per neuron, a slack
@@ -857,7 +857,7 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
     float* C = ws[WS_C].as<float>();
     float* C2 = ws[WS_R_A].as<float>();
     // few cells: a whole block per cell in the kernels that walk over a cell's rows
-    // (8 per SM); up to one cell per SM they are spread over several blocks per cell, since one SM alone is bound by
+    // (up to 8 cells per SM); up to one cell per SM they are spread over several blocks per cell, since one SM alone is bound by
     // its loads' latency (every symbol alive, 400 x 5: 1 cell 672 -> 350 us, 152 cells 3918 -> 3601; 256 x 5, 600
     // cells: 775 us either way)
     const bool wide = nc < 8 * sms;

@@ -78,6 +78,17 @@ __device__ __forceinline__ float ra_relu(float* v) {
   }
 }
 
+// Shared memory of a CTA, in floats: the forms [Q][w][cells], the weight ring, the largest magnitudes [2][cells].
+// The output layer's sums [Q + 1][cells] go over the ring, which at w = 16 is smaller than they are (256 cells per
+// CTA: 1536 floats over 768), so the region is sized for both.
+__host__ __device__ __forceinline__ size_t ra_ring(int cells, int KB, int w) {
+  const size_t ring = (size_t)sgemm::kStages * KB * w, sums = (size_t)(kRaQ + 1) * cells;
+  return ring > sums ? ring : sums;
+}
+size_t ra_smem(int cells, int KB, int w) {
+  return ((size_t)kRaQ * cells * w + ra_ring(cells, KB, w)) * sizeof(float) + 2 * (size_t)cells * sizeof(unsigned);
+}
+
 template <bool INFL, int CPT>
 __global__ void __launch_bounds__(ra_threads(CPT), 2)
 k_bound_rafixed(CellSource src, int64_t first, int64_t n, int cells, int KB, int w, int H, const float* __restrict__ W0,
@@ -97,7 +108,7 @@ k_bound_rafixed(CellSource src, int64_t first, int64_t n, int cells, int KB, int
   const int spl = w / KB;
   sgemm::Stream ws{S + (size_t)Q * cells * w, w, KB, (int64_t)(H - 1) * spl};
   // per-cell largest magnitude, double-buffered across layers (non-negative floats order as ints)
-  unsigned* Mx = reinterpret_cast<unsigned*>(S + (size_t)Q * cells * w + (size_t)sgemm::kStages * KB * w);
+  unsigned* Mx = reinterpret_cast<unsigned*>(S + (size_t)Q * cells * w + ra_ring(cells, KB, w));
   int sl = 1, sk = 0;                              // layer and K block of the stage to load next
   auto load_next = [&] {
     ws.load(layers.Wt[min(sl, H - 1)] + (size_t)sk * KB * w);
@@ -262,7 +273,7 @@ k_bound_rafixed(CellSource src, int64_t first, int64_t n, int cells, int KB, int
   // ---- output layer (w -> 1) and the read-off: one thread per (quantity, cell), then one per cell.  Each sum is 32
   //      partial sums over the neurons l, l + 32, ..., added as a 32-lane butterfly adds them ----
   constexpr int YQ = INFL ? Q + 1 : Q;             // quantity Q: ||w_out||_1
-  float* Y = ws.Ws;                                // [YQ][cells], the weight stages are done
+  float* Y = ws.Ws;                                // [YQ][cells], the weight stages are done (ra_ring holds both)
   for (int u = t; u < YQ * cells; u += blockDim.x) {
     const int q = u / cells, cell = u - q * cells;
     const float* x = S + (size_t)q * w * cells + cell;
@@ -343,7 +354,7 @@ isx_status bound_rafixed(isx_inr inr, const CellSource& src, int64_t n, int infl
                         : (int)std::min<int64_t>(most, std::max<int64_t>((most / 2 + 3) / 4 * 4, (even + 3) / 4 * 4) / cpt * cpt);
   const int KB = 16 * w <= 2048 ? 16 : (8 * w <= 2048 ? 8 : 4);
   const int threads = (w / kRaCols * (cells / cpt) + 31) / 32 * 32;
-  const size_t smem = ((size_t)kRaQ * cells * w + (size_t)sgemm::kStages * KB * w) * sizeof(float) + 2 * cells * sizeof(unsigned);
+  const size_t smem = ra_smem(cells, KB, w);
   // the grid's x dimension is bounded; long lists run in slices
   const int64_t max_ctas = 1 << 30;
   const double flops = 2.0 * 5.0 * w * (double)w * (H - 1) + 2.0 * 3.0 * 4.0 * w + 2.0 * 5.0 * w;

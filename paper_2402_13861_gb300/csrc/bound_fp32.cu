@@ -322,7 +322,7 @@ isx_status launch_gemm(int v, const GemmArgs& g, int w, int sms, cudaStream_t st
   const size_t smem = sh.smem(w) + (size_t)sh.P * (sizeof(int64_t) + sizeof(int));
   const int threads = (sh.threads(w) + 31) / 32 * 32;
   const auto kernel = sh.tn == 8 ? k_gemm_fp32<8, SC> : k_gemm_fp32<4, SC>;
-  ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   int per_sm = 1;
   ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
   const int64_t ntiles = (g.R + sh.P - 1) / sh.P;  // d_R: g.R is an upper bound

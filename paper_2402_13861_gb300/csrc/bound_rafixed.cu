@@ -364,7 +364,7 @@ isx_status bound_rafixed(isx_inr inr, const CellSource& src, int64_t n, int infl
     prof::Scope _ps(K_BOUND_RAFIXED, st, flops * (double)m, 8.0 * (double)m + 4.0 * w * w * (H - 1) * grid);
     const auto kernel = inflate ? (cpt == 4 ? k_bound_rafixed<true, 4> : k_bound_rafixed<true, 2>)
                                 : (cpt == 4 ? k_bound_rafixed<false, 4> : k_bound_rafixed<false, 2>);
-    ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     kernel<<<grid, threads, smem, st>>>(src, off, m, cells, KB, w, H, inr->W[0], inr->b[0], lay, inr->W[L], inr->hb[L][0],
                                         d_center, d_spread);
     ISX_LAUNCH_CHECK("k_bound_rafixed");

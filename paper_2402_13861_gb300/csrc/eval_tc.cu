@@ -343,7 +343,7 @@ isx_status launch_eval(isx_inr inr, EvArgs a, const EvMaps& maps, int64_t ntiles
   const int ns = EvSmem<W>::stages(inr->H);
   a.ns = ns;
   const size_t smem = EvSmem<W>::bytes(inr->H, ns);
-  ISX_CUDA(cudaFuncSetAttribute(k_eval_tc<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ISX_CUDA(cudaFuncSetAttribute(k_eval_tc<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   int per_sm = 1;
   const int sms = inr->sms;
   ISX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eval_tc<W>, EvSmem<W>::kThreads, smem));

@@ -255,6 +255,11 @@ isx_status eval_points_fp32(isx_inr inr, const float* xyz, const uint32_t* latti
 isx_status mc_upload_table(int device);
 void mc_build_table(int8_t* ntri, int8_t* tris);
 
+// Dynamic shared memory a kernel may ask for on this architecture.  Kernels whose launches differ in size raise
+// their limit to this and never to a launch's own size: the limit belongs to the kernel, not to the launch, and a
+// smaller call of another thread (on a handle of its own) would lower it between this one's limit and its launch.
+constexpr int kMaxSmem = 227 * 1024;
+
 // One cluster of `blocks` blocks per cell.
 template <typename... A>
 inline isx_status launch_clusters(void (*kernel)(A...), unsigned blocks, int nc, unsigned threads, size_t smem, cudaStream_t st, A... args) {

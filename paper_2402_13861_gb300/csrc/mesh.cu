@@ -334,7 +334,7 @@ isx_status eval_points_fp32(isx_inr inr, const float* xyz, const uint32_t* latti
   {
     prof::Scope _ps(K_EVAL_FP32, st, 2.0 * n * (4.0 * inr->w + (inr->n_layers - 2.0) * inr->w * inr->w), 8.0 * n);
     const auto kernel = sh.tn == 8 ? k_eval_fp32<8> : k_eval_fp32<4>;
-    ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     kernel<<<(unsigned)nb, threads, smem, st>>>(m, sh, xyz, lattice_ids, R, n, out);
   }
   ISX_LAUNCH_CHECK("k_eval_fp32");

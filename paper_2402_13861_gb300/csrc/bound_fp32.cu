@@ -823,48 +823,49 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   const bool elu = inr->act == ISX_ACT_ELU;
   const int pad = elu ? kPad - 1 : 0, rs = elu ? kPad : 3;   // row alignment - 1, rows kept for the input's three
   const int Smax = rs + w * (H - 1);
-  // the two coefficient buffers take at most ~6 GB: enough for full_cells cells with every symbol alive
-  const size_t per_cell = 2ull * Smax * w * sizeof(float);
-  const int64_t full_cells = std::min<int64_t>({n, (int64_t)1 << 16, std::max<int64_t>(1, (int64_t)((6ull << 30) / per_cell))});
-  const int64_t row_cap = full_cells * Smax;
-  // More cells than that: the host reads every layer's row count, and a chunk holds as many cells as the
-  // rows they really have allow.  Otherwise (and while the stream is captured, where the host cannot
-  // read) chunks of full_cells need no count on the host at all.
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  ISX_CUDA(cudaStreamIsCapturing(st, &cs));
-  const bool counted = n > full_cells && cs == cudaStreamCaptureStatusNone;
-  const int64_t nc_alloc = counted ? std::min<int64_t>(n, (int64_t)1 << 16) : full_cells;
+  // The two row buffers take at most ~6 GB: even chunks of as many cells as fit with every symbol alive, so that the
+  // host needs no row count and a call only enqueues.  (Chunks of as many cells as the rows that exist allow need one
+  // count per layer on the host, which waits for the stream: 20003 cells of the 3 -> 256 x 5 -> 1 network 15.7 ms
+  // against 16.8, but 30000 of 3 -> 128 x 4 -> 1 with inflation 12.5 against 8.9, for the chunks that it starts over.)
+  // The last layer's rows go to one buffer, fewer to the other.
+  const int64_t Sprev = H > 1 ? Smax - w : 0;
+  const size_t per_cell = (size_t)(Smax + Sprev) * w * sizeof(float);
+  const int64_t fit = std::min<int64_t>((int64_t)1 << 16, std::max<int64_t>(1, (int64_t)((6ull << 30) / per_cell)));
+  const int64_t chunks = (n + fit - 1) / fit, full_cells = (n + chunks - 1) / chunks;
   auto& ws = inr->ws;
-  for (Slot s : {WS_X0, WS_X1}) ISX_TRY(ws[s].ensure((size_t)row_cap * w * sizeof(float), "rows"));
-  for (Slot s : {WS_R_RC0, WS_R_RC1}) ISX_TRY(ws[s].ensure((size_t)row_cap * sizeof(int), "row cells"));
+  const Slot xs[2] = {WS_X0, WS_X1}, rc[2] = {WS_R_RC0, WS_R_RC1}, ns[2] = {WS_R_CNT0, WS_R_CNT1},
+             os[2] = {WS_R_OFF0, WS_R_OFF1};
+  for (int i = 0; i < 2; ++i) {
+    const size_t rows = (size_t)full_cells * ((i == 0) == (H % 2 == 1) ? Smax : Sprev);   // layer j's go to buffer (j - 1) % 2
+    ISX_TRY(ws[xs[i]].ensure(rows * w * sizeof(float), "rows"));
+    ISX_TRY(ws[rc[i]].ensure(rows * sizeof(int), "row cells"));
+  }
   for (Slot s : {WS_C, WS_R_A, WS_RAD, WS_ALPHA, WS_GAMMA, WS_DELTA})
-    ISX_TRY(ws[s].ensure((size_t)nc_alloc * w * sizeof(float), "per-neuron"));
-  for (Slot s : {WS_R_CNT0, WS_R_CNT1}) ISX_TRY(ws[s].ensure((size_t)nc_alloc * sizeof(int), "row counts"));
-  for (Slot s : {WS_R_OFF0, WS_R_OFF1}) ISX_TRY(ws[s].ensure((size_t)nc_alloc * sizeof(int64_t), "row offsets"));
-  ISX_TRY(ws[WS_R_TOT].ensure(rows::scan_bytes(nc_alloc), "row total and scan block sums"));
+    ISX_TRY(ws[s].ensure((size_t)full_cells * w * sizeof(float), "per-neuron"));
+  for (Slot s : {WS_R_CNT0, WS_R_CNT1}) ISX_TRY(ws[s].ensure((size_t)full_cells * sizeof(int), "row counts"));
+  for (Slot s : {WS_R_OFF0, WS_R_OFF1}) ISX_TRY(ws[s].ensure((size_t)full_cells * sizeof(int64_t), "row offsets"));
+  ISX_TRY(ws[WS_R_TOT].ensure(rows::scan_bytes(full_cells), "row total and scan block sums"));
   int64_t* d_tot = ws[WS_R_TOT].as<int64_t>();
   float* RAD = ws[WS_RAD].as<float>();
   float* AL = ws[WS_ALPHA].as<float>();
   float* GA = ws[WS_GAMMA].as<float>();
   float* DE = ws[WS_DELTA].as<float>();
-  const Slot xs[2] = {WS_X0, WS_X1}, rc[2] = {WS_R_RC0, WS_R_RC1}, ns[2] = {WS_R_CNT0, WS_R_CNT1},
-             os[2] = {WS_R_OFF0, WS_R_OFF1};
   const int sms = inr->sms;
   const CellBlock cb(w);
-  int64_t want = nc_alloc;                         // cells of the next chunk
-  for (int64_t first = 0; first < n;) {
-    const int nc = (int)std::min<int64_t>(want, n - first);
+  for (int64_t first = 0; first < n; first += full_cells) {
+    const int nc = (int)std::min<int64_t>(full_cells, n - first);
     float* C = ws[WS_C].as<float>();
     float* C2 = ws[WS_R_A].as<float>();
-    // few cells: a whole block per cell in the kernels that walk over a cell's rows
-    // (up to 8 cells per SM); up to one cell per SM they are spread over several blocks per cell, since one SM alone is bound by
+    // few cells: a whole block per cell in the kernels that walk over a cell's rows (up to 8 cells per SM, or 64 where
+    // a cell may have 256 KB of them: a chunk of 3334 cells of the 3 -> 256 x 5 -> 1 network 3.14 -> 2.80 ms, but 5000
+    // cells of 80 x 1 40 -> 54 us and of 16 x 5 202 -> 237); up to one
+    // cell per SM they are spread over several blocks per cell, since one SM alone is bound by
     // its loads' latency (every symbol alive, 400 x 5: 1 cell 672 -> 350 us, 152 cells 3918 -> 3601; 256 x 5, 600
     // cells: 775 us either way)
-    const bool wide = nc < 8 * sms;
+    const bool wide = nc < ((int64_t)w * w * (H - 1) >= 65536 ? 64 : 8) * sms;
     const bool few = nc <= sms;
     int cur = 0;
-    int64_t R = rs * (int64_t)nc;                  // rows of z_j (an upper bound where the host does not know)
-    bool fits = true;
+    int64_t R = rs * (int64_t)nc;                  // rows of z_j: an upper bound, but for the input's
     {
       prof::Scope _ps(K_INPUT, st, 0, 0);
       k_input_layer<<<cb.blocks(nc), cb.threads(), 0, st>>>(
@@ -885,18 +886,6 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
         prof::Scope _ps(K_SCAN, st, 0, 0);
         ISX_TRY(rows::scan_counts(cnt_out, nc, d_tot, j & 1, off_out, st, pad));
       }
-      int64_t Rn = std::min<int64_t>(row_cap, (int64_t)nc * (rs + (int64_t)w * j));
-      if (counted) {
-        ISX_CUDA(cudaMemcpyAsync(&Rn, d_tot + (j & 1), sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        ISX_CUDA(cudaStreamSynchronize(st));
-        // rows after the last layer if every layer creates as many as the ones so far
-        const double last = (double)rs * nc + (double)(Rn - rs * (int64_t)nc) / j * (H - 1);
-        if (Rn > row_cap || (j == 1 && last > 1.2 * (double)row_cap)) {
-          want = std::max<int64_t>(full_cells, std::min<int64_t>(nc / 2, (int64_t)(0.8 * nc * (double)row_cap / std::max(last, (double)Rn))));
-          fits = false;                            // start the chunk again with fewer cells
-          break;
-        }
-      }
       // the tile shape comes from the autotuner (timed once per width and row-count bucket)
       {
         GemmArgs g{};
@@ -907,7 +896,7 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
         g.rowcell = ws[rc[cur]].as<int>();
         g.off_in = off_in;
         g.off_out = off_out;
-        g.d_R = (counted || j == 1) ? nullptr : d_tot + ((j - 1) & 1);
+        g.d_R = j == 1 ? nullptr : d_tot + ((j - 1) & 1);
         g.R = R;
         int64_t bucket = 1;
         while (bucket < std::min<int64_t>(R, 1 << 16)) bucket <<= 1;
@@ -915,7 +904,7 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
         auto run = [&](int v) { return elu ? launch_gemm<kWeights>(v, g, w, sms, st) : launch_gemm<kRows>(v, g, w, sms, st); };
         int v = 0;
         ISX_TRY(tune::pick(key, kGemmVariants, [&](int i) { return kGemmShapes[i].name; }, run, st, &v));
-        // counted work: the rows, or the input rows alone where only the device knows how many there are
+        // the work that is counted: the input rows alone, since only the device knows how many there are from layer 2 on
         const double rows_known = g.d_R ? 3.0 * nc : (double)R;
         prof::Scope _ps(K_GEMM_FP32, st, 2.0 * rows_known * w * w, 8.0 * rows_known * w);
         ISX_TRY(run(v));
@@ -958,9 +947,8 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
       }
       ISX_LAUNCH_CHECK("k_reduce_act");
       cur = nxt;
-      R = Rn;
+      R = (int64_t)nc * (rs + (int64_t)w * j);
     }
-    if (!fits) continue;
     const int L = inr->n_layers - 1;
     {
       prof::Scope _ps(K_OUTPUT, st, 0, 0);
@@ -981,12 +969,6 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
                                                                       d_spread, first);
     }
     ISX_LAUNCH_CHECK("k_output");
-    if (counted) {
-      // the next chunk: as many cells as fill the buffers to 4/5 at this chunk's rows per cell
-      const double per = std::max(1.0, (double)R / nc);
-      want = std::max<int64_t>(full_cells, std::min<int64_t>(nc_alloc, (int64_t)(0.8 * (double)row_cap / per)));
-    }
-    first += nc;
   }
   return ISX_OK;
 }

@@ -28,6 +28,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "cell_box.cuh"
 #include "linearise.cuh"
@@ -276,18 +277,26 @@ k_bound_rafixed(CellSource src, int64_t first, int64_t n, int cells, int KB, int
   float* Y = ws.Ws;                                // [YQ][cells], the weight stages are done (ra_ring holds both)
   for (int u = t; u < YQ * cells; u += blockDim.x) {
     const int q = u / cells, cell = u - q * cells;
-    const float* x = S + (size_t)q * w * cells + cell;
+    const bool ones = q == Q;                      // a sum of |wout| alone: fmaf(|wout|, 1, y)
+    const float* x = S + (ones ? 0 : (size_t)q * w * cells) + cell;
     float y[32];
 #pragma unroll
     for (int l = 0; l < 32; ++l) y[l] = 0.0f;
-    for (int c0 = 0; c0 < w; c0 += 32)
+    // N neurons from c0 on with every load in flight: w is a multiple of 16, so none of them needs a test (with a test
+    // per neuron the loads went one after the other, 75 ns each: a CTA's output layer took 35 us at w = 512)
+    auto add = [&](int c0, auto N) {
+      float wo[N], xv[N];
 #pragma unroll
-      for (int l = 0; l < 32; ++l)
-        if (c0 + l < w) {
-          const float wo = wout[c0 + l];
-          if (q == Q) y[l] += fabsf(wo);
-          else y[l] = fmaf(q == 4 ? fabsf(wo) : wo, x[(size_t)(c0 + l) * cells], y[l]);
-        }
+      for (int l = 0; l < N; ++l) {
+        wo[l] = wout[c0 + l];
+        xv[l] = x[(size_t)(c0 + l) * cells];
+      }
+#pragma unroll
+      for (int l = 0; l < N; ++l) y[l] = fmaf(q >= 4 ? fabsf(wo[l]) : wo[l], ones ? 1.0f : xv[l], y[l]);
+    };
+    int c0 = 0;
+    for (; c0 + 32 <= w; c0 += 32) add(c0, std::integral_constant<int, 32>{});
+    if (c0 < w) add(c0, std::integral_constant<int, 16>{});
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll

@@ -955,7 +955,7 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
       const float* X = ws[xs[cur]].as<float>();
       const int64_t* off = ws[os[cur]].as<int64_t>();
       const int* cnt = ws[ns[cur]].as<int>();
-      if (few)
+      if (few && H > 1)                              // one hidden layer leaves a cell three rows
         ISX_TRY(launch_clusters(8 * nc <= 2 * sms ? k_output<64> : k_output<32>, 8 * nc <= 2 * sms ? 8 : 4, nc, 256,
                                 (w + kOutRows) * sizeof(float), st, X, off, cnt, nc, w, (const float*)C, (const float*)AL,
                                 (const float*)GA, (const float*)RAD, (const float*)inr->W[L], inr->hb[L][0], (int)mode,

@@ -273,10 +273,25 @@ __global__ void __launch_bounds__(256) k_eval_fp32(MlpView m, sgemm::Shape sh, c
     float q[32];
 #pragma unroll
     for (int l = 0; l < 32; ++l) q[l] = 0.0f;
-    for (int k0 = 0; k0 < w; k0 += 32)
+    // 16 neurons at a time, every load of them in flight: w is a multiple of 16, so none needs a test.  (Blocks of 32
+    // leave the layers' loop fewer registers: 512 x 3, one point 107 us against 94.)
+    auto add = [&](int k0, int h) {
+      float v[16];
 #pragma unroll
-      for (int l = 0; l < 32; ++l)
-        if (k0 + l < w) q[l] = fmaf(m.wout[k0 + l], A[(size_t)(k0 + l) * P + p], q[l]);
+      for (int l = 0; l < 16; ++l) v[l] = A[(size_t)(k0 + l) * P + p];
+      if (h == 0) {
+#pragma unroll
+        for (int l = 0; l < 16; ++l) q[l] = fmaf(m.wout[k0 + l], v[l], q[l]);
+      } else {
+#pragma unroll
+        for (int l = 0; l < 16; ++l) q[16 + l] = fmaf(m.wout[k0 + l], v[l], q[16 + l]);
+      }
+    };
+#pragma unroll 1
+    for (int k0 = 0; k0 < w; k0 += 32) {
+      add(k0, 0);
+      if (k0 + 16 < w) add(k0 + 16, 1);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -294,7 +309,14 @@ __global__ void __launch_bounds__(256) k_eval_fp32(MlpView m, sgemm::Shape sh, c
 //    neurons per thread (a 128-thread CTA) is 2 % slower at 3 x 10^5 points.
 //  - Fewer: 4 neurons per thread and long stages, for the shortest chain through the layers: at
 //    w = 512, n = 500, 270 us against 300-440 us for the 8-neuron tiles.
-sgemm::Shape eval_shape(int64_t n, int w, int sms) {
+//  - One hidden layer has no tile: CTAs of 256 threads, and as many points each as leave every SM one (w = 128,
+//    10000 points: 64 per CTA instead of 128).
+sgemm::Shape eval_shape(int64_t n, int w, int H, int sms) {
+  if (H == 1) {
+    int P = std::max(8, 16384 / w / 8 * 8);
+    while (P > 8 && (n + P - 1) / P < sms) P = std::max(8, P / 2 / 8 * 8);
+    return {8, P, 16};
+  }
   if (n * w < (int64_t)sms * 8192) return {4, std::max(8, 4096 / w / 8 * 8), w % 32 == 0 ? 32 : 16};
   int best = 8;
   int64_t best_cost = -1;
@@ -327,14 +349,15 @@ isx_status eval_points_fp32(isx_inr inr, const float* xyz, const uint32_t* latti
   m.wout = inr->W[inr->n_layers - 1];
   m.bout = inr->hb[inr->n_layers - 1][0];
   const int sms = inr->sms;
-  const sgemm::Shape sh = eval_shape(n, inr->w, sms);
-  const size_t smem = sh.smem(inr->w);
-  const int threads = (sh.threads(inr->w) + 31) / 32 * 32;
+  const sgemm::Shape sh = eval_shape(n, inr->w, inr->H, sms);
+  // one hidden layer streams no weights and needs the activations alone
+  const size_t smem = inr->H > 1 ? sh.smem(inr->w) : (size_t)inr->w * sh.P * sizeof(float);
+  const int threads = inr->H > 1 ? (sh.threads(inr->w) + 31) / 32 * 32 : 256;
   const int64_t nb = (n + sh.P - 1) / sh.P;
   {
     prof::Scope _ps(K_EVAL_FP32, st, 2.0 * n * (4.0 * inr->w + (inr->n_layers - 2.0) * inr->w * inr->w), 8.0 * n);
     const auto kernel = sh.tn == 8 ? k_eval_fp32<8> : k_eval_fp32<4>;
-    ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    if (smem > 48 * 1024) ISX_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     kernel<<<(unsigned)nb, threads, smem, st>>>(m, sh, xyz, lattice_ids, R, n, out);
   }
   ISX_LAUNCH_CHECK("k_eval_fp32");

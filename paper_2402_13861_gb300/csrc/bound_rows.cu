@@ -1554,10 +1554,12 @@ isx_status bound_bf16_rows(isx_inr inr, const CellSource& src, int64_t n, isx_bo
                                                                                 bl, first, d_center, d_spread, fi);
       };
       // four warps per cell until single warps fill every SM several times over: a chunk lasts as long as its
-      // cell with the most rows (12007 cells of the 3 -> 512 x 8 -> 1 network: 1.14 -> 0.62 ms)
+      // cell with the most rows (12007 cells of the 3 -> 512 x 8 -> 1 network: 1.14 -> 0.62 ms).  Rows of up to 128
+      // values are short work, so that this is from 32 cells per SM on (fine cells of 3 -> 64 x 2 -> 1, 9000: 18 us
+      // with four warps, 10 with one; 128 x 3, 12000 of all scales: 119 against 94, 3000: 39 against 49)
       // and up to one cell per SM a cluster of blocks per cell (7 coarse cells of the 3 -> 256 x 5 -> 1 network: 43 ->
       // 16 us; 512 cells: no faster)
-      const bool many = nc >= 128 * sms || H == 1;   // one hidden layer leaves no stored rows
+      const bool many = nc >= (w <= 128 ? 32 : 128) * sms || H == 1;   // one hidden layer leaves no stored rows
       auto launch_few = [&](auto kernel) {
         return launch_clusters(kernel, 4, nc, 32 * kOutWarps, 0, st, nc, (int)mode, Xl, ol, cl, (const float*)I0, (const float*)A,
                                (const float*)AL, (const float*)GA, wl, bl, first, d_center, d_spread, fi);

@@ -95,6 +95,16 @@ void set_infl(Infl& f, int w) {
   f.gamma_w = gamma_u(K + 1.0, u) * 1.0001f;
 }
 __device__ __forceinline__ __nv_bfloat16 bf16_up(float x) { return __float2bfloat16_ru(x); }
+// sigma and radius of the three input rows.  Roundings spelled out, as in every sum that two kernels take: a cell's
+// bound must not depend on the form that its list's length selects, nor on what the compiler contracts in each.
+__device__ __forceinline__ float input_sigma(float x0, float x1, float x2) {
+  return sqrtf(fmaf(x2, x2, fmaf(x0, x0, __fmul_rn(x1, x1))));
+}
+__device__ __forceinline__ float input_sum(float x0, float x1, float x2) {
+  return __fadd_rn(__fadd_rn(fabsf(x0), fabsf(x1)), fabsf(x2));
+}
+// one more x to a column's sum of x^2 or |x|
+__device__ __forceinline__ float add_col(float s, float x, bool sq) { return sq ? fmaf(x, x, s) : __fadd_rn(s, fabsf(x)); }
 
 // ---- layer 0 and activation 1: centre c_1 and the three input rows I_1 = diag(h) W_0^T (written where
 //      given: the output layer of a one-hidden-layer net reads both, the float32 centre GEMM the centre), their
@@ -131,8 +141,7 @@ __global__ void __launch_bounds__(256) k_rows_input_act(CellSource src, int64_t 
       iv[e][0] = h[0] * w0;
       iv[e][1] = h[1] * w1;
       iv[e][2] = h[2] * w2;
-      const float rad = clt ? sqrtf(iv[e][0] * iv[e][0] + iv[e][1] * iv[e][1] + iv[e][2] * iv[e][2])
-                            : fabsf(iv[e][0]) + fabsf(iv[e][1]) + fabsf(iv[e][2]);
+      const float rad = clt ? input_sigma(iv[e][0], iv[e][1], iv[e][2]) : input_sum(iv[e][0], iv[e][1], iv[e][2]);
       if (infl.on) {
         // c: three fused multiply-adds; the input rows: one product each
         const float ru = __fmul_ru(rad, 1.0f + 4.0f * kU32);
@@ -229,7 +238,7 @@ __global__ void __launch_bounds__(256, 4) k_rows_input_relu(CellSource src, int6
       for (int e = 0; e < 2; ++e) {
         mu[e] = fmaf(wv[e][2], xc[2], fmaf(wv[e][1], xc[1], fmaf(wv[e][0], xc[0], bv[e])));
         const float i0 = h[0] * wv[e][0], i1 = h[1] * wv[e][1], i2 = h[2] * wv[e][2];
-        const float sg = sqrtf(fmaf(i2, i2, fmaf(i0, i0, i1 * i1)));
+        const float sg = input_sigma(i0, i1, i2);
         const bool need = relu_clt_mixed(mu[e], sg);
         const unsigned bm = __ballot_sync(0xffffffffu, need);
         if (need) s.list[nq + __popc(bm & ((1u << lane) - 1u))] = (uint8_t)(64 * c + 2 * lane + e);
@@ -470,8 +479,8 @@ __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new(int nc, int sq, con
             const __nv_bfloat162 x = __floats2bfloat162_rn(gm * v[q][i], gm * v[q][i + 1]);
             h[i / 2] = *reinterpret_cast<const uint32_t*>(&x);
             const float2 f = __bfloat1622float2(x);
-            acc[c][i] += sq ? f.x * f.x : fabsf(f.x);
-            acc[c][i + 1] += sq ? f.y * f.y : fabsf(f.y);
+            acc[c][i] = add_col(acc[c][i], f.x, sq);
+            acc[c][i + 1] = add_col(acc[c][i + 1], f.y, sq);
           }
           IO::st(xp[c], h);
           xp[c] += w;
@@ -536,8 +545,8 @@ __global__ void __launch_bounds__(32 * kNewWarps) k_rows_new_one(int nc, int sq,
       const __nv_bfloat162 y = __floats2bfloat162_rn(g * x[i], g * x[i + 1]);
       h[i / 2] = *reinterpret_cast<const uint32_t*>(&y);
       const float2 f = __bfloat1622float2(y);
-      acc[i] = sq ? fmaf(f.x, f.x, acc[i]) : acc[i] + fabsf(f.x);
-      acc[i + 1] = sq ? fmaf(f.y, f.y, acc[i + 1]) : acc[i + 1] + fabsf(f.y);
+      acc[i] = add_col(acc[i], f.x, sq);
+      acc[i + 1] = add_col(acc[i + 1], f.y, sq);
     }
     IO::st(xp + (size_t)r * w, h);
   };
@@ -620,8 +629,8 @@ __global__ void __launch_bounds__(32 * kFewWarps) k_rows_new_few(int sq, const f
 #pragma unroll 8
       for (int r = 0; r < end; ++r) {
         const float2 f = __bfloat1622float2(sx[r][lane]);
-        a0 = sq ? fmaf(f.x, f.x, a0) : a0 + fabsf(f.x);
-        a1 = sq ? fmaf(f.y, f.y, a1) : a1 + fabsf(f.y);
+        a0 = add_col(a0, f.x, sq);
+        a1 = add_col(a1, f.y, sq);
       }
     }
     __syncthreads();

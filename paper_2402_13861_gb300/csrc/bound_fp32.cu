@@ -38,8 +38,8 @@ namespace isx {
 namespace {
 
 constexpr float kU = 5.9604645e-08f;        // 2^-24, float32 unit roundoff
-constexpr float kSafe = 1.0000010f;         // (1 + 2^-20): slack for evaluating error formulas
-constexpr float kOutSafe = 1.0000020f;      // (1 + 32 u): the output layer's sums take at most 23 roundings (w = 512)
+constexpr float kSafe = 1.0000010f;         // (1 + 16 u): slack for evaluating error formulas, and for the output layer's
+                                            // sums, which take at most 13 roundings of a term
 constexpr float kInvSqrt3 = 0.57735026918962576f;
 
 __host__ __device__ __forceinline__ float gamma_k(int k) { return (k * kU) / (1.0f - k * kU); }
@@ -562,16 +562,23 @@ __global__ void __launch_bounds__(256)
   }
   if (u > 0 || cell >= nc) return;
   // symbols of the last activation, y_m = gamma_m w_m, and the centre
-  float v[4] = {0.f, 0.f, 0.f, 0.f};               // sum |y| or y^2, w . c, and the two error sums (inflate)
-  for (int m = lane; m < w; m += 32) {
-    const size_t i = (size_t)cell * w + m;
-    const float y = GAMMA[i] * wout[m];
-    v[0] = sq ? fmaf(y, y, v[0]) : v[0] + fabsf(y);
-    v[1] = fmaf(wout[m], C[i], v[1]);
-    if (inflate) {
-      v[2] = fmaf(fabsf(wout[m]), fabsf(C[i]), v[2]);
-      v[3] = fmaf(fabsf(wout[m]), fmaf(ALPHA[i], RAD[i], GAMMA[i]), v[3]);
+  // sum |y| or y^2, w . c, and the two error sums (inflate): a lane's terms in groups of four, so that none of the sums
+  // takes more than 13 roundings of a term (sixteen one after the other took 23 at w = 512)
+  float v[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int m0 = 0; m0 < w; m0 += 128) {
+    float g[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int m = m0 + lane; m < min(w, m0 + 128); m += 32) {
+      const size_t i = (size_t)cell * w + m;
+      const float y = GAMMA[i] * wout[m];
+      g[0] = sq ? fmaf(y, y, g[0]) : g[0] + fabsf(y);
+      g[1] = fmaf(wout[m], C[i], g[1]);
+      if (inflate) {
+        g[2] = fmaf(fabsf(wout[m]), fabsf(C[i]), g[2]);
+        g[3] = fmaf(fabsf(wout[m]), fmaf(ALPHA[i], RAD[i], GAMMA[i]), g[3]);
+      }
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] += g[q];
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q)
@@ -584,7 +591,7 @@ __global__ void __launch_bounds__(256)
       sp = tot;
       if (inflate) {
         float ge = gamma_k(w + 1) + kU;
-        sp = __fadd_ru(__fmul_ru(sp, kOutSafe), (ge * v[3] + gamma_k(w + 2) * (v[2] + fabsf(bout))) * 1.01f);
+        sp = __fadd_ru(__fmul_ru(sp, kSafe), (ge * v[3] + gamma_k(w + 2) * (v[2] + fabsf(bout))) * 1.01f);
       }
     } else if (mode == ISX_BOUND_CLT) {
       sp = sqrtf(tot);
@@ -771,7 +778,7 @@ __global__ void __launch_bounds__(kSmallT) k_bound_small(CellSource src, int64_t
           sp = tot;
           if (inflate) {
             float ge = gamma_k(w + 1) + kU;
-            sp = __fadd_ru(__fmul_ru(sp, kOutSafe), (ge * v[3] + gamma_k(w + 2) * (v[2] + fabsf(net.bout))) * 1.01f);
+            sp = __fadd_ru(__fmul_ru(sp, kSafe), (ge * v[3] + gamma_k(w + 2) * (v[2] + fabsf(net.bout))) * 1.01f);
           }
         } else if (mode == ISX_BOUND_CLT) {
           sp = sqrtf(tot);

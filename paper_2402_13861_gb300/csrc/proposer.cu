@@ -271,8 +271,11 @@ __global__ void __launch_bounds__(kTB) k_prop_forward(const __nv_bfloat16* pb, N
 constexpr int kGS = 64, kGP = kGS + 4, kGT = 256;
 constexpr size_t kGradSmemFloats = kWtFloats + 2 * kH * kH + kF * kGP + 5 * kH * kGP + kGS + 32;
 
-// dW[o][i] += sum_s dZ[o][s] A[i][s] for o = og + 16 r, i = ig + 16 c, and db[o] (threads with ig = 0)
+// dW[o][i] += sum_s dZ[o][s] A[i][s] for o = og + 16 r, i = ig + 16 c, and db[o] (threads with ig = 0).  The tile's
+// samples are summed by themselves first: one sum over all of a block's samples would take as many roundings as it has
+// samples (2^20 equal ones: up to 1.0e-4 of an entry, instead of 4e-6).
 __device__ __forceinline__ void grad_layer(const float* dZ, const float* A, int og, int ig, float (&dw)[4][4], float (&db)[4]) {
+  float tw[4][4] = {}, tb[4] = {};
 #pragma unroll 4
   for (int s = 0; s < kGS; s += 4) {
     float4 z[4], a[4];
@@ -285,9 +288,15 @@ __device__ __forceinline__ void grad_layer(const float* dZ, const float* A, int 
     for (int r = 0; r < 4; ++r) {
 #pragma unroll
       for (int c = 0; c < 4; ++c)
-        dw[r][c] = fmaf(z[r].w, a[c].w, fmaf(z[r].z, a[c].z, fmaf(z[r].y, a[c].y, fmaf(z[r].x, a[c].x, dw[r][c]))));
-      if (ig == 0) db[r] = (((db[r] + z[r].x) + z[r].y) + z[r].z) + z[r].w;
+        tw[r][c] = fmaf(z[r].w, a[c].w, fmaf(z[r].z, a[c].z, fmaf(z[r].y, a[c].y, fmaf(z[r].x, a[c].x, tw[r][c]))));
+      if (ig == 0) tb[r] = (((tb[r] + z[r].x) + z[r].y) + z[r].z) + z[r].w;
     }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) dw[r][c] += tw[r][c];
+    db[r] += tb[r];
   }
 }
 
@@ -352,12 +361,16 @@ __global__ void __launch_bounds__(kGT) k_prop_grad(const __nv_bfloat16* pb, Norm
       const int i = k / kGS, q = k % kGS;
       Za[i * kGP + q] = A3[i * kGP + q] > 0.f ? dz4[q] * vec[3 * kH + i] : 0.f;
     }
-    if (t < kH)
+    if (t < kH) {
+      float tw = 0.f, tb = 0.f;
 #pragma unroll 8
       for (int q = 0; q < kGS; ++q) {
-        dw4 = fmaf(dz4[q], A3[t * kGP + q], dw4);
-        db4 += dz4[q];
+        tw = fmaf(dz4[q], A3[t * kGP + q], tw);
+        tb += dz4[q];
       }
+      dw4 += tw;
+      db4 += tb;
+    }
     __syncthreads();
     // ---- dW3, db3; dZ2 = (W3^T dZ3) masked by A2 > 0 ----
     grad_layer(Za, A2, og, ig, dw3, db3);
@@ -375,12 +388,16 @@ __global__ void __launch_bounds__(kGT) k_prop_grad(const __nv_bfloat16* pb, Norm
     {
       const float* z = Za + (t >> 2) * kGP;
       const float* a = A0 + 2 * (t & 3) * kGP;
+      float tw[2] = {}, tb = 0.f;
 #pragma unroll 8
       for (int q = 0; q < kGS; ++q) {
-        dw1[0] = fmaf(z[q], a[q], dw1[0]);
-        dw1[1] = fmaf(z[q], a[kGP + q], dw1[1]);
-        db1 += z[q];
+        tw[0] = fmaf(z[q], a[q], tw[0]);
+        tw[1] = fmaf(z[q], a[kGP + q], tw[1]);
+        tb += z[q];
       }
+      dw1[0] += tw[0];
+      dw1[1] += tw[1];
+      db1 += tb;
     }
   }
 #pragma unroll

@@ -838,20 +838,21 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   const int64_t Sprev = H > 1 ? Smax - w : 0;
   const size_t per_cell = (size_t)(Smax + Sprev) * w * sizeof(float);
   const int64_t fit = std::min<int64_t>((int64_t)1 << 16, std::max<int64_t>(1, (int64_t)((6ull << 30) / per_cell)));
-  const int64_t chunks = (n + fit - 1) / fit, full_cells = (n + chunks - 1) / chunks;
+  const int64_t chunks = (n + fit - 1) / fit, chunk = (n + chunks - 1) / chunks;
+  const int64_t cap = std::min(n, fit);            // workspace: not the chunk, so that a shorter list never needs more
   auto& ws = inr->ws;
   const Slot xs[2] = {WS_X0, WS_X1}, rc[2] = {WS_R_RC0, WS_R_RC1}, ns[2] = {WS_R_CNT0, WS_R_CNT1},
              os[2] = {WS_R_OFF0, WS_R_OFF1};
   for (int i = 0; i < 2; ++i) {
-    const size_t rows = (size_t)full_cells * ((i == 0) == (H % 2 == 1) ? Smax : Sprev);   // layer j's go to buffer (j - 1) % 2
+    const size_t rows = (size_t)cap * ((i == 0) == (H % 2 == 1) ? Smax : Sprev);   // layer j's go to buffer (j - 1) % 2
     ISX_TRY(ws[xs[i]].ensure(rows * w * sizeof(float), "rows"));
     ISX_TRY(ws[rc[i]].ensure(rows * sizeof(int), "row cells"));
   }
   for (Slot s : {WS_C, WS_R_A, WS_RAD, WS_ALPHA, WS_GAMMA, WS_DELTA})
-    ISX_TRY(ws[s].ensure((size_t)full_cells * w * sizeof(float), "per-neuron"));
-  for (Slot s : {WS_R_CNT0, WS_R_CNT1}) ISX_TRY(ws[s].ensure((size_t)full_cells * sizeof(int), "row counts"));
-  for (Slot s : {WS_R_OFF0, WS_R_OFF1}) ISX_TRY(ws[s].ensure((size_t)full_cells * sizeof(int64_t), "row offsets"));
-  ISX_TRY(ws[WS_R_TOT].ensure(rows::scan_bytes(full_cells), "row total and scan block sums"));
+    ISX_TRY(ws[s].ensure((size_t)cap * w * sizeof(float), "per-neuron"));
+  for (Slot s : {WS_R_CNT0, WS_R_CNT1}) ISX_TRY(ws[s].ensure((size_t)cap * sizeof(int), "row counts"));
+  for (Slot s : {WS_R_OFF0, WS_R_OFF1}) ISX_TRY(ws[s].ensure((size_t)cap * sizeof(int64_t), "row offsets"));
+  ISX_TRY(ws[WS_R_TOT].ensure(rows::scan_bytes(cap), "row total and scan block sums"));
   int64_t* d_tot = ws[WS_R_TOT].as<int64_t>();
   float* RAD = ws[WS_RAD].as<float>();
   float* AL = ws[WS_ALPHA].as<float>();
@@ -859,8 +860,8 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   float* DE = ws[WS_DELTA].as<float>();
   const int sms = inr->sms;
   const CellBlock cb(w);
-  for (int64_t first = 0; first < n; first += full_cells) {
-    const int nc = (int)std::min<int64_t>(full_cells, n - first);
+  for (int64_t first = 0; first < n; first += chunk) {
+    const int nc = (int)std::min<int64_t>(chunk, n - first);
     float* C = ws[WS_C].as<float>();
     float* C2 = ws[WS_R_A].as<float>();
     // few cells: a whole block per cell in the kernels that walk over a cell's rows (up to 8 cells per SM, or 64 where

@@ -36,3 +36,21 @@ def test_fp32_bounds_only_enqueue(pkg, w, H, n, mode, inflate):
         stream.synchronize()
         assert torch.equal(c, c0) and torch.equal(s, s0)
     net.close()
+
+
+@pytest.mark.parametrize("w,H,long,short", [(16, 2, 70001, 65536), (256, 5, 4001, 3000)])
+def test_a_shorter_list_needs_no_more_workspace(pkg, w, H, long, short):
+    """A capture may not allocate: after a list of several chunks any shorter one, also of one larger chunk, can be
+    captured."""
+    net = pkg.Inr(inr.random_inr([3] + [w] * H + [1], 145 + w))
+    lo, hi = (torch.tensor(x, device="cuda") for x in boxes.random_boxes(long, 146, -10, -4))
+    c0, s0 = net.bound_cells(lo, hi, mode="clt", prec="fp32")
+    c, s = torch.zeros(short, device="cuda"), torch.zeros(short, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        net.bound_cells(lo[:short], hi[:short], mode="clt", prec="fp32", center=c, spread=s)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(c, c0[:short]) and torch.equal(s, s0[:short])
+    net.close()

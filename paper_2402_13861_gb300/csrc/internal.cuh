@@ -92,8 +92,8 @@ namespace isx {
 
 // ---- launch accounting (prof.cu) --------------------------------------------------------------
 enum KernelId {
-  K_INPUT, K_RELU, K_GEMV, K_GEMM_FP32, K_FRESH, K_REDUCE, K_OUTPUT, K_CULL, K_SCAN, K_SCATTER, K_MARK,
-  K_FLAGCOUNT, K_SCATTER_FLAGS, K_EVAL_FP32, K_MC_COUNT, K_MC_EMIT, K_IOTA, K_BOUND_TC, K_TC_PREP, K_TC_OUTPUT,
+  K_INPUT, K_GEMV, K_GEMM_FP32, K_FRESH, K_REDUCE, K_OUTPUT, K_CULL, K_SCAN, K_SCATTER, K_MARK,
+  K_FLAGCOUNT, K_SCATTER_FLAGS, K_EVAL_FP32, K_MC_COUNT, K_MC_EMIT, K_IOTA, K_BOUND_TC,
   K_EVAL_TC, K_PROP_GATE, K_PROP_MERGE, K_PROP_FWD, K_PROP_GRAD, K_PROP_ADAM, K_BOUND_RAFIXED, K_ROWS_GEMM, K_ROWS_AUX,
   K_ROWS_ACT, K_ROWS_NEW, K_ROWS_SPLIT, K_ROWS_REDUCE, K_ROWS_OUT, K_BOUND_SMALL, K_COUNT
 };

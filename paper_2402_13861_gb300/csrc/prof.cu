@@ -21,14 +21,13 @@ struct Acc {
   double ms = 0, flops = 0, bytes = 0;
 };
 Acc acc[K_COUNT];
-const char* names[K_COUNT] = {"input_layer",   "relu",          "center_gemv",   "gemm_fp32",    "fresh_rows",
-                              "reduce",        "output",        "cull_count",    "scan_counts",  "scatter_cells",
-                              "mark_corners",  "flag_count",    "scatter_flags", "eval_fp32",    "mc_count",
-                              "mc_emit",       "iota",          "bound_tc",      "tc_prep",      "tc_output",
-                              "eval_tc",       "prop_gate",     "prop_merge",   "prop_forward",
-                              "prop_grad",     "prop_adam",     "bound_rafixed", "rows_gemm",     "rows_aux",
-                              "rows_act",      "rows_new",      "rows_split",    "rows_reduce",  "rows_out",
-                              "bound_small"};
+const char* names[K_COUNT] = {"input_layer",   "center_gemv",   "gemm_fp32",     "fresh_rows",   "reduce",
+                              "output",        "cull_count",    "scan_counts",   "scatter_cells", "mark_corners",
+                              "flag_count",    "scatter_flags", "eval_fp32",     "mc_count",     "mc_emit",
+                              "iota",          "bound_tc",      "eval_tc",       "prop_gate",    "prop_merge",
+                              "prop_forward",  "prop_grad",     "prop_adam",     "bound_rafixed", "rows_gemm",
+                              "rows_aux",      "rows_act",      "rows_new",      "rows_split",   "rows_reduce",
+                              "rows_out",      "bound_small"};
 
 void drain_locked() {
   for (auto& r : pending) {

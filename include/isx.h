@@ -8,7 +8,9 @@
  *    library never frees them.  Host pointers (descriptors, iso-value arrays) are read during the
  *    call only.
  *  - `stream` is a cudaStream_t passed as void* (NULL = legacy default stream).  Work is enqueued
- *    on it; entry points that must read counts back (extraction) synchronise it before returning.
+ *    on it; entry points that must read counts or a status back (extraction, and bounds and point values in
+ *    BF16) synchronise it before returning.  Float32 and RA-Fixed bounds, float32 point values and the proposer
+ *    only enqueue, but for the first call of a size, which may allocate and time tile shapes.
  *  - Every entry point returns an isx_status; nothing throws across this interface.  On failure
  *    isx_last_error() returns a message for the calling thread.  A capacity shortfall returns
  *    ISX_ERR_CAPACITY after filling in the required sizes, without writing past any capacity.

@@ -12,7 +12,7 @@
 //         r = sum |y_i| (Eq. 2) or sigma^2 = sum y_i^2 (Eq. 7), RA-UA: sigma^2 / 3 (Sec. IV-A).
 // A symbol whose coefficient gamma_n is exactly 0 has an all-zero row in every later layer and is never
 // created.  Bound by the FP32 FMA rate of the row GEMM: 20003 random cells of levels 5-9 of the fitted
-// 3 -> 256 x 5 -> 1 network take 15.6 ms (43 TFLOP/s in the GEMM), where carrying all 1027 rows of every
+// 3 -> 256 x 5 -> 1 network take 16.0 ms (43 TFLOP/s in the GEMM), where carrying all 1027 rows of every
 // cell took 142.6 ms; with every symbol alive (ELU, 3 -> 128 x 4 -> 1, 5003 boxes) 2.3 ms against 4.0 ms.
 // A cell's result depends neither on the chunking nor on the launch shapes.
 //

@@ -16,7 +16,7 @@
 // the ReLU is applied in registers and written back in place after a block barrier.  Bound by FP32 FMA
 // issue and the shared-memory return bandwidth: two neighbouring cells share a 64-bit accumulator
 // (fma.rn.f32x2, the same results as two fmaf) and 28 values read feed 160 multiply-adds; W^T streams
-// through the cp.async ring of sgemm.cuh.  131075 cells of the 3 -> 256 x 5 -> 1 network: 6.63 ms, 52 TFLOP/s
+// through the cp.async ring of sgemm.cuh.  131075 cells of the 3 -> 256 x 5 -> 1 network: 6.38 ms, 54 TFLOP/s
 // (8.05 ms with 4 x 4 tiles that read 36 values per 80 multiply-adds, the weights from global memory).
 //
 // Rounding-error inflation (inflate != 0): every float32 rounding is charged to r, which is a

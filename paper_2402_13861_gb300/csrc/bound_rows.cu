@@ -16,7 +16,8 @@
 // operand is W_j itself, loaded once per CTA and shared by the rows of every cell: rows of many
 // cells fill each 128-row MMA tile (rows_gemm.cu).  Per chunk and layer this file runs:
 //   k_rows_input_act (layer 0 and activation 1);
-//   k_rows_scan_*: row offsets of the next layer (the host reads the total to size the buffers);
+//   k_rows_scan_*: row offsets of the next layer (the host reads the total to size the buffers, but for calls
+//     so short that buffers for every symbol alive are small);
 //   the row GEMM and k_rows_new, _one or _few (the new rows);
 //   k_rows_layer (rows_layer.cu): centre and input rows on the tensor cores, and in its epilogue r = sum |x|
 //     (sound) or sigma^2 = sum x^2 (UP) per (cell, neuron) over the stored rows and the input rows, the

@@ -21,10 +21,9 @@
 //    overlaps the next tile's first MMAs.
 // With one 128-thread warpgroup that issued, waited and drained in turn 2.1 M points of 3 -> 256 x 5 -> 1 took
 // 3.62 ms; this form takes 2.42 ms: of 11.2 k cycles per layer the MMAs take 6.1 k, 3.3 k go by waiting for
-// weights and 1.8 k until the first chunk of the next layer's operand is ready.  Halving the L2 reads with clusters
-// of two CTAs that multicast the weights to each other changes nothing: the 80 KB of the ring, all that
-// fits, cover too little of the load latency.  Every wait is bounded (2 s): on timeout the kernel records
-// ISX_ERR_TIMEOUT, lets copies land, frees TMEM and returns.
+// weights (the 80 KB of the ring, all that fits, cover too little of the load latency) and 1.8 k until the
+// first chunk of the next layer's operand is ready.  Every wait is bounded (2 s): on timeout the kernel
+// records ISX_ERR_TIMEOUT, lets copies land, frees TMEM and returns.
 #include "internal.cuh"
 #include "tc_ptx.cuh"
 #include "linearise.cuh"
@@ -74,9 +73,11 @@ struct EvSmem {
   static constexpr size_t bytes(int H, int ns) {
     return 1024 + 2 * kA + ns * kS + (size_t)(3 * W + (size_t)H * W + W + 2 * (G - 1) * kT) * 4 + kBars * 8 + 16;
   }
-  // stages that fit: five up to H = 11 at w = 256
-  static constexpr int stages(int H) { return bytes(H, NS) <= 227 * 1024 ? NS : NS - 1; }
+  // stages that fit: five up to H = 10 at w = 256, four at the most layers
+  static constexpr int stages(int H) { return bytes(H, NS) <= kMaxSmem ? NS : NS - 1; }
 };
+static_assert(EvSmem<256>::stages(10) == 5 && EvSmem<256>::stages(11) == 4 && EvSmem<256>::bytes(12, 4) <= kMaxSmem &&
+              EvSmem<128>::bytes(12, 2) <= kMaxSmem);
 
 __device__ __forceinline__ uint32_t aoff(int row, int k) {  // byte offset of (row, k..k+7), k % 8 == 0
   return (uint32_t)((k >> 6) * kT * 128 + row * 128 + ((((k & 63) >> 3) ^ (row & 7)) << 4));

@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(kTB) k_prop_forward(const __nv_bfloat16* pb, N
 
 // Forward and backward of the mean BCE over n samples: grad += dL/dtheta, loss += L.  Tiles of 64 samples, 256
 // threads with 4 x 4 register tiles: a training batch of 8192 gives 128 blocks.  Parameter gradients stay in
-// registers over a block's tiles.  8192 samples: 49 us (one thread per sample
-// in 64 blocks of 128 threads: 113 us); 2 M samples 3.2 ms (8.4 ms).
+// registers over a block's tiles.  8192 samples: 30 us a call, the two clears included (one thread per sample
+// in 64 blocks of 128 threads: 96 us); 2 M samples 3.27 ms (8.4 ms).
 constexpr int kGS = 64, kGP = kGS + 4, kGT = 256;
 constexpr size_t kGradSmemFloats = kWtFloats + 2 * kH * kH + kF * kGP + 5 * kH * kGP + kGS + 32;
 

@@ -32,7 +32,9 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: 
 //  - the producer warp streams the rows of G by TMA, one 64-wide K chunk of a tile per stage of an NS-stage
 //    ring, in the 128-byte-swizzled K-major layout of the MMA's B operand;
 //  - the scaler warps scale each staged chunk in place: one, two or four threads per row multiply its
-//    64 columns by its cell's alpha (rows past R stay the TMA's zero fill).  With one thread per row (four warps) the scaling
+//    64 columns by its cell's alpha.  Rows past R may hold anything (the TMA's zero fill, or with a row count in device
+//    memory what an earlier call left): each reaches its own column of the accumulator alone, which no epilogue
+//    thread reads.  With one thread per row (four warps) the scaling
 //    set the pace: 821 us for 3.5 M rows (4.4 TB/s) at w = 256, against 711 us (5.1 TB/s) with two; without
 //    any scaling the kernel takes 632 us, without scaling and epilogue 361 us;
 //  - the MMA warp loads W_j (bf16, [MW][W], K-major) once by TMA, owns TMEM and issues the MMAs (M = 128

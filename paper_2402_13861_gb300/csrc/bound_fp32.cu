@@ -12,7 +12,7 @@
 //         r = sum |y_i| (Eq. 2) or sigma^2 = sum y_i^2 (Eq. 7), RA-UA: sigma^2 / 3 (Sec. IV-A).
 // A symbol whose coefficient gamma_n is exactly 0 has an all-zero row in every later layer and is never
 // created.  Bound by the FP32 FMA rate of the row GEMM: 20003 random cells of levels 5-9 of the fitted
-// 3 -> 256 x 5 -> 1 network take 16.0 ms (43 TFLOP/s in the GEMM), where carrying all 1027 rows of every
+// 3 -> 256 x 5 -> 1 network take 17.0 ms (42 TFLOP/s in the GEMM), where carrying all 1027 rows of every
 // cell took 142.6 ms; with every symbol alive (ELU, 3 -> 128 x 4 -> 1, 5003 boxes) 2.3 ms against 4.0 ms.
 // A cell's result depends neither on the chunking nor on the launch shapes.
 //
@@ -833,8 +833,8 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   // The two row buffers take at most ~6 GB: even chunks of as many cells as fit with every symbol alive, so that the
   // host needs no row count and a call only enqueues.  (Chunks of as many cells as the rows that exist allow need one
   // count per layer on the host, which waits for the stream: 20003 cells of the 3 -> 256 x 5 -> 1 network 15.7 ms
-  // against 16.8, but 30000 of 3 -> 128 x 4 -> 1 with inflation 12.5 against 8.9, for the chunks that it starts over.)
-  // The last layer's rows go to one buffer, fewer to the other.
+  // against 17.0, but 30000 of 3 -> 128 x 4 -> 1 with inflation 12.4 against 8.9, for the chunks that it starts over.
+  // Twice the memory would make it 16.1 ms.)  The last layer's rows go to one buffer, fewer to the other.
   const int64_t Sprev = H > 1 ? Smax - w : 0;
   const size_t per_cell = (size_t)(Smax + Sprev) * w * sizeof(float);
   const int64_t fit = std::min<int64_t>((int64_t)1 << 16, std::max<int64_t>(1, (int64_t)((6ull << 30) / per_cell)));

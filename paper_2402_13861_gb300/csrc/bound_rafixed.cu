@@ -348,12 +348,13 @@ isx_status bound_rafixed(isx_inr inr, const CellSource& src, int64_t n, int infl
   const int L = inr->n_layers - 1;
   // Cells per CTA: 128 threads' worth of four cells each (eight warps on the SM's two CTAs keep the multiply-adds
   // fed); with fewer than that for every SM one CTA each, of at least 64 threads (they share the weight stream).  Two
-  // smaller ones would put two warps on the same sub-partition of the SM: 2600 cells of w = 144 in 251 us, not 169.
+  // smaller ones may put two warps on the same sub-partition of the SM: 4300 cells of w = 144 in 182 us, not 125.
   const int sms = inr->sms;
   // At small widths the input and output layers weigh more and twice the warps with two cells each hide more of their
-  // latency (w = 64, two hidden layers, 10^5 cells: 165 us against 199).  So do they while one CTA of 128 threads
-  // per SM takes all cells, where a CTA's own chain is the time (w = 512, eight layers, up to 608 cells: 505 us against
-  // 713; w = 256, five: 149 against 202 up to 1216 cells; beyond, four: 2400 cells of w = 512 in 995 us against 1107).
+  // latency (w = 64, two hidden layers, 5000 cells: 41 us against 45, 39000 cells 72 against 77).  So do they while one
+  // CTA of 128 threads per SM takes all cells, where a CTA's own chain is the time (w = 512, eight layers, up to 608
+  // cells: 480 us against 609; w = 256, five: 137 against 185 up to 1216 cells; beyond, four: 2400 cells of w = 512 in
+  // 970 us against 1071).
   const int few_cells = 2 * (128 * kRaCols / w);
   const bool few = few_cells > 0 && n <= (int64_t)sms * few_cells;
   const int cpt = w <= 64 || few ? 2 : 4;

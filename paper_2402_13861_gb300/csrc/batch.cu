@@ -134,13 +134,15 @@ isx_status isx_batch_run(isx_batch b, isx_mesh* meshes, void* stream) {
     for (int g = next++; g < (int)b->groups.size(); g = next++)
       for (int i : b->groups[g]) {
         isx_inr inr = b->inrs[i];
-        // lend the worker's workspace and chunk size to the entry's INR for the call
+        // lend the worker's workspace and chunk sizes to the entry's INR for the call
         std::swap(inr->ws, b->workers[w].ws);
-        const int64_t rb = inr->row_budget;
+        const int64_t rb = inr->row_budget, fb = inr->fp32_row_bytes;
         inr->row_budget = b->row_budget;
+        inr->fp32_row_bytes = kFp32RowBytesLess;   // there are several workers
         status[i] = isx_extract_isosurface(inr, &b->params[i], &meshes[i], b->streams[w]);
         if (status[i] != ISX_OK) message[i] = isx_last_error();
         inr->row_budget = rb;
+        inr->fp32_row_bytes = fb;
         std::swap(inr->ws, b->workers[w].ws);
       }
   };

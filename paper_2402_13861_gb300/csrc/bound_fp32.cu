@@ -12,7 +12,7 @@
 //         r = sum |y_i| (Eq. 2) or sigma^2 = sum y_i^2 (Eq. 7), RA-UA: sigma^2 / 3 (Sec. IV-A).
 // A symbol whose coefficient gamma_n is exactly 0 has an all-zero row in every later layer and is never
 // created.  Bound by the FP32 FMA rate of the row GEMM: 20003 random cells of levels 5-9 of the fitted
-// 3 -> 256 x 5 -> 1 network take 17.0 ms (42 TFLOP/s in the GEMM), where carrying all 1027 rows of every
+// 3 -> 256 x 5 -> 1 network take 16.1 ms (43 TFLOP/s in the GEMM), where carrying all 1027 rows of every
 // cell took 142.6 ms; with every symbol alive (ELU, 3 -> 128 x 4 -> 1, 5003 boxes) 2.3 ms against 4.0 ms.
 // A cell's result depends neither on the chunking nor on the launch shapes.
 //
@@ -830,29 +830,44 @@ isx_status bound_fp32(isx_inr inr, const CellSource& src, int64_t n, isx_bound_m
   const bool elu = inr->act == ISX_ACT_ELU;
   const int pad = elu ? kPad - 1 : 0, rs = elu ? kPad : 3;   // row alignment - 1, rows kept for the input's three
   const int Smax = rs + w * (H - 1);
-  // The two row buffers take at most ~6 GB: even chunks of as many cells as fit with every symbol alive, so that the
-  // host needs no row count and a call only enqueues.  (Chunks of as many cells as the rows that exist allow need one
-  // count per layer on the host, which waits for the stream: 20003 cells of the 3 -> 256 x 5 -> 1 network 15.7 ms
-  // against 17.0, but 30000 of 3 -> 128 x 4 -> 1 with inflation 12.4 against 8.9, for the chunks that it starts over.
-  // Twice the memory would make it 16.1 ms.)  The last layer's rows go to one buffer, fewer to the other.
+  // Even chunks of as many cells as the two row buffers hold with every symbol alive, so that the host needs no row
+  // count and a call only enqueues.  (Chunks of as many cells as the rows that exist allow need one count per layer
+  // on the host, which waits for the stream: 20003 cells of the 3 -> 256 x 5 -> 1 network 15.7 ms against 16.1, but 30000
+  // of 3 -> 128 x 4 -> 1 with inflation 12.4 against 8.9, for the chunks that it starts over.)  The last layer's rows
+  // go to one buffer, fewer to the other.  They take at most 12 GB (with 6 GB those 20003 cells take 17.0 ms), or 6
+  // for good on a device that does not have them.
   const int64_t Sprev = H > 1 ? Smax - w : 0;
   const size_t per_cell = (size_t)(Smax + Sprev) * w * sizeof(float);
-  const int64_t fit = std::min<int64_t>((int64_t)1 << 16, std::max<int64_t>(1, (int64_t)((6ull << 30) / per_cell)));
-  const int64_t chunks = (n + fit - 1) / fit, chunk = (n + chunks - 1) / chunks;
-  const int64_t cap = std::min(n, fit);            // workspace: not the chunk, so that a shorter list never needs more
   auto& ws = inr->ws;
   const Slot xs[2] = {WS_X0, WS_X1}, rc[2] = {WS_R_RC0, WS_R_RC1}, ns[2] = {WS_R_CNT0, WS_R_CNT1},
              os[2] = {WS_R_OFF0, WS_R_OFF1};
-  for (int i = 0; i < 2; ++i) {
-    const size_t rows = (size_t)cap * ((i == 0) == (H % 2 == 1) ? Smax : Sprev);   // layer j's go to buffer (j - 1) % 2
-    ISX_TRY(ws[xs[i]].ensure(rows * w * sizeof(float), "rows"));
-    ISX_TRY(ws[rc[i]].ensure(rows * sizeof(int), "row cells"));
+  int64_t chunk = 0;
+  auto reserve = [&]() -> isx_status {
+    const int64_t fit = std::min<int64_t>((int64_t)1 << 16, std::max<int64_t>(1, inr->fp32_row_bytes / (int64_t)per_cell));
+    const int64_t chunks = (n + fit - 1) / fit;
+    const int64_t cap = std::min(n, fit);          // not the chunk, so that a shorter list never needs more
+    chunk = (n + chunks - 1) / chunks;
+    for (int i = 0; i < 2; ++i) {
+      const size_t rows = (size_t)cap * ((i == 0) == (H % 2 == 1) ? Smax : Sprev);   // layer j's go to buffer (j - 1) % 2
+      ISX_TRY(ws[xs[i]].ensure(rows * w * sizeof(float), "rows"));
+      ISX_TRY(ws[rc[i]].ensure(rows * sizeof(int), "row cells"));
+    }
+    for (Slot s : {WS_C, WS_R_A, WS_RAD, WS_ALPHA, WS_GAMMA, WS_DELTA})
+      ISX_TRY(ws[s].ensure((size_t)cap * w * sizeof(float), "per-neuron"));
+    for (Slot s : {WS_R_CNT0, WS_R_CNT1}) ISX_TRY(ws[s].ensure((size_t)cap * sizeof(int), "row counts"));
+    for (Slot s : {WS_R_OFF0, WS_R_OFF1}) ISX_TRY(ws[s].ensure((size_t)cap * sizeof(int64_t), "row offsets"));
+    return ws[WS_R_TOT].ensure(rows::scan_bytes(cap), "row total and scan block sums");
+  };
+  isx_status reserved = reserve();
+  if (reserved == ISX_ERR_NOMEM && inr->fp32_row_bytes > kFp32RowBytesLess) {
+    for (int i = 0; i < 2; ++i) {
+      ws[xs[i]].release();
+      ws[rc[i]].release();
+    }
+    inr->fp32_row_bytes = kFp32RowBytesLess;
+    reserved = reserve();
   }
-  for (Slot s : {WS_C, WS_R_A, WS_RAD, WS_ALPHA, WS_GAMMA, WS_DELTA})
-    ISX_TRY(ws[s].ensure((size_t)cap * w * sizeof(float), "per-neuron"));
-  for (Slot s : {WS_R_CNT0, WS_R_CNT1}) ISX_TRY(ws[s].ensure((size_t)cap * sizeof(int), "row counts"));
-  for (Slot s : {WS_R_OFF0, WS_R_OFF1}) ISX_TRY(ws[s].ensure((size_t)cap * sizeof(int64_t), "row offsets"));
-  ISX_TRY(ws[WS_R_TOT].ensure(rows::scan_bytes(cap), "row total and scan block sums"));
+  ISX_TRY(reserved);
   int64_t* d_tot = ws[WS_R_TOT].as<int64_t>();
   float* RAD = ws[WS_RAD].as<float>();
   float* AL = ws[WS_ALPHA].as<float>();

@@ -61,6 +61,10 @@ enum Slot {
 
 }  // namespace isx
 
+namespace isx {
+constexpr int64_t kFp32RowBytesLess = (int64_t)6 << 30;   // fp32_row_bytes once the device did not have more
+}
+
 // The opaque INR handle.
 struct isx_inr_s {
   int device = 0;
@@ -84,6 +88,7 @@ struct isx_inr_s {
   std::vector<std::vector<float>> hW, hb;  // host copies
   isx::Buf ws[isx::WS_N_SLOTS];
   int64_t row_budget = (int64_t)1 << 24;  // symbol rows per chunk of the row-batched bound path
+  int64_t fp32_row_bytes = (int64_t)12 << 30;  // both row buffers of the float32 bound path, at most
   float* h_pinned = nullptr;            // small pinned host buffer for count read-back
   int* h_pinned_i = nullptr;
 };
